@@ -130,18 +130,18 @@ int pvt_vstep_select(const pvt_layer* layer, uint64_t k, uint32_t* idx_out, void
  * completely at start-up, a component living inside a host application that
  * owns all device memory, or a thread that must not enter an allocator (a
  * cudaMalloc would also synchronise the device).  Such callers cannot supply the
- * ~5 bytes per group of workspace that pvt_vstep_select asks for.  Here the
+ * 4 bytes per group (and 1 MiB) of workspace that pvt_vstep_select asks for.  Here the
  * scratch is a fixed array inside the library image instead; the caller passes
  * only the layer, k and the outputs.
  *
  * Limits and rules
  *   - At most PVT_NOALLOC_MAX_GROUPS groups (2^21, e.g. one 4096 x 4096 layer);
  *     a larger layer is rejected with PVT_ETOOLARGE before anything is enqueued.
- *   - The array (about 10.03 MiB) is held on every GPU on which the library's
+ *   - The array (about 9.6 MiB) is held on every GPU on which the library's
  *     device code has been loaded, until the process exits.  The CUDA runtime may
  *     load that code lazily: then it is the first call of this function on a
  *     device that makes the array resident (and that load may synchronise the
- *     device and needs those 10 MiB to be free).
+ *     device and needs those 9.6 MiB to be free).
  *   - The first call on each device also looks up the array's device address (a
  *     host-side runtime query; the device must be current).  Make that first
  *     call at start-up -- before the memory is handed out completely and outside

@@ -20,13 +20,19 @@ int fail_cuda(cudaError_t e) {
   return PVT_ECUDA;
 }
 
+// asked of the driver once per device
 int sm_count() {
-  int dev = 0, n = 0;
+  static std::atomic<int> known[kMaxDevices];
+  const int slot = device_slot();
+  int n = slot >= 0 ? known[slot].load(std::memory_order_relaxed) : 0;
+  if (n > 0) return n;
+  int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
       n <= 0) {
     (void)cudaGetLastError();
     return kSmCountFallback;
   }
+  if (slot >= 0) known[slot].store(n, std::memory_order_relaxed);
   return n;
 }
 
@@ -79,6 +85,15 @@ Timing& timing() {
 }
 
 }  // namespace
+
+int device_slot() {
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return -1;
+  }
+  return dev >= 0 && dev < kMaxDevices ? dev : -1;
+}
 
 void record_cuda_error(cudaError_t e) { g_last_cuda = e; }
 

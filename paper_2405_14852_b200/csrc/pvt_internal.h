@@ -2,6 +2,8 @@
 // launchers, workspace layout, small device helpers).  Not part of the ABI.
 #pragma once
 
+#include <atomic>
+
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -14,37 +16,28 @@ constexpr int kGroupDim = 8;
 constexpr int kSmCountFallback = 148;
 
 // ---- workspace layout -------------------------------------------------------
-// [0, 256)            header: status word (u32 at 0), selection state, counters
+// [0, 256)            header: status word (u32 at 0)
 // [256, ...)          region shared by select and encode (they run one after the
 //                     other on a stream and never need each other's scratch)
 constexpr size_t kWsHeaderBytes = 256;
 constexpr size_t kWsAlign = 256;
 
 // selection -------------------------------------------------------------------
-constexpr int kSelTile = 4096;      // groups per block of the select kernels
-constexpr int kSelThreads = 256;    // 16 groups per thread
-constexpr int kSelBins0 = 2048;     // key bits [30:20]
-constexpr int kSelBins1 = 2048;     // key bits [19:9]
-constexpr int kSelBins2 = 512;      // key bits [8:0]
-
-struct SelectState {        // lives in the header at byte 64
-  uint32_t digit0, digit1;  // threshold digits found so far
-  uint32_t threshold;       // full threshold key once the last digit is known
-  uint32_t need_eq;         // how many groups with key == threshold are taken (lowest indices)
-  uint64_t k_left;          // groups still to be taken from the current bucket
-  uint32_t done[4];         // block-completion counters of the passes
-  uint32_t cand_count;      // keys found inside the threshold bucket of the first digit
-};
-constexpr size_t kSelStateOffset = 64;
+constexpr int kSelThreads = 1024;     // passes over the keys
+constexpr int kNormThreads = 512;     // pass over g
+constexpr int kNormCtas = 2;          // its CTAs per SM
+constexpr int kSelBins0 = 8192;       // key bits [30:18]
+constexpr int kSelBins1 = 512;        // key bits [17:9]
+constexpr int kSelBins2 = 512;        // key bits [8:0]
+constexpr uint32_t kSelMaxCtas = 1024;
+// counts per CTA, state, the histograms
+constexpr uint32_t kSelScratchWords = 2 * kSelMaxCtas + 16 + kSelBins0 + kSelBins1 + kSelBins1 * kSelBins2;
 
 struct SelectLayout {
-  size_t hist_off;   // u32 [2048 + 2048 + 512]
-  size_t keys_off;   // u32 [G]
-  size_t tiles_off;  // u32 [2 * ntiles]: (greater, equal) counts, later exclusive offsets
-  size_t cand_off;   // u32 [cand_cap]: keys of the threshold bucket, any order
-  uint32_t cand_cap;
-  size_t bytes;      // end of the region (from the workspace base)
-  uint32_t ntiles;
+  size_t scratch_off;  // u32 [kSelScratchWords]
+  size_t keys_off;     // u32 [G]
+  size_t masks_off;    // u32 [G / 32][2]
+  size_t bytes;        // end of the region (from the workspace base)
 };
 SelectLayout select_layout(uint64_t G);
 
@@ -219,6 +212,32 @@ void record_cuda_error(cudaError_t e);
 
 // multiprocessors of the current device
 int device_sm_count();
+
+// ordinal of the current device below kMaxDevices, or -1: for what is set up once per device
+constexpr int kMaxDevices = 64;
+int device_slot();
+
+// Lets a kernel take all the dynamic shared memory there is; the driver is asked once per kernel and device.
+#ifdef __CUDACC__
+template <typename... KArgs>
+cudaError_t allow_smem(void (*kernel)(KArgs...)) {
+  static std::atomic<void*> done[kMaxDevices][8];  // kernels of one signature share these slots
+  const int dev = device_slot();
+  if (dev >= 0)
+    for (auto& d : done[dev])
+      if (d.load(std::memory_order_relaxed) == reinterpret_cast<void*>(kernel)) return cudaSuccess;
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(227 * 1024 - fa.sharedSizeBytes));
+  if (e != cudaSuccess || dev < 0) return e;
+  for (auto& d : done[dev]) {
+    void* none = nullptr;
+    if (d.compare_exchange_strong(none, reinterpret_cast<void*>(kernel))) break;
+  }
+  return cudaSuccess;
+}
+#endif
 
 // number of kernels launched by this process through the library (a claim the benchmark reports)
 void count_launches(int n);

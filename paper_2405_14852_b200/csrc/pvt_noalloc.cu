@@ -20,19 +20,16 @@ namespace pvt {
 namespace {
 
 // Largest layer the built-in scratch serves: 2^21 groups of 8 weights, e.g. a
-// 4096 x 4096 matrix.  Layout needs: 256 B header + 18 KiB histograms + 4 B per
-// group (keys) + 8 B per tile of 4096 groups + 1 B per group (candidate list of a
-// quarter of the groups), each part rounded up to 256 B.
+// 4096 x 4096 matrix.  Layout needs: 256 B header + 1.05 MiB counters and histograms
+// + 4.25 B per group (keys, masks), each part rounded up to 256 B.
 constexpr uint64_t kNoAllocMaxGroups = 1ull << 21;
-constexpr size_t kNoAllocScratchBytes =
-    256 + 18432 + 4 * kNoAllocMaxGroups + 8 * (kNoAllocMaxGroups / kSelTile) + kNoAllocMaxGroups + 1280;
+constexpr size_t kNoAllocScratchBytes = 4 * kNoAllocMaxGroups + kNoAllocMaxGroups / 4 + (9 << 17);
 
 // File-scope device array.  In host code this name is only a handle for the
 // runtime's symbol table, not a device address: the address is looked up with
 // cudaGetSymbolAddress below and only that pointer is given to kernels.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
 
-constexpr int kMaxDevices = 64;
 std::mutex g_setup_mu;
 void* g_scratch_ptr[kMaxDevices] = {};  // device address of the array, per device ordinal
 
@@ -77,7 +74,7 @@ extern "C" int pvt_vstep_select_noalloc(const pvt_layer* layer, uint64_t k, uint
   void* ws = nullptr;
   cudaError_t e = scratch_for_current_device(&ws);
   // the array keeps whatever the previous call left: the status word must start at zero
-  // (launch_select clears the selection state and the histograms itself)
+  // (launch_select clears the histograms itself)
   if (e == cudaSuccess) e = cudaMemsetAsync(ws, 0, sizeof(uint32_t), stream);
   if (e == cudaSuccess) e = launch_select(*layer, G, k, idx_out, ws, device_sm_count(), stream);
   if (e == cudaSuccess && status_out)

@@ -3,36 +3,31 @@
 // then an exact top-k by radix select on the binary32 bit patterns, ties at the
 // threshold resolved towards the lowest group index, result in ascending order.
 //
-// Passes (all on one stream, no host round trip, no inter-block waiting):
-//   1. norm_hist:   persistent grid; read g once (32 B per group), write the key of
-//                   every group, histogram key bits [30:20]
-//   2. refine_mid:  read the keys; those inside the threshold bucket are
-//                   histogrammed on bits [19:9] and copied to a compact candidate
-//                   list (usually a few per cent of the groups)
-//   3. refine_low:  histogram bits [8:0] of the candidates that match both digits
-//   4. tile_count:  per tile of 4096 groups: how many keys > threshold, == threshold
-//   5. scatter:     ordered compaction: position = (#greater before) +
-//                   min(#equal before, number of ties to take)
-// In passes 1-4 the block that finishes last (atomic ticket, no spinning) turns
-// the histogram into the next threshold digit, or the tile counts into offsets.
+// Four kernels, each launched before the one ahead of it has finished.  What bounds them is the one pass over g (32 B
+// per group); the others read keys that are in the L2 and cost little more than their launches:
+//   0. clear:  zeroes the histograms, beside pass 1
+//   1. keys:   32 bytes per thread and load, four groups in flight per thread; writes the key of every group and sums
+//              up key bits [30:18] -- 32 bins per octave, so that the threshold bin of ordinary updates holds a
+//              fraction of a per cent of the groups
+//   2. bin:    every CTA finds the threshold bin and writes two bits per group, above it and inside it; the members of
+//              the bin are counted by their lower 18 bits, in a table of all 2^18 of them (few members: few atomics) and
+//              in one of the upper nine of these bits
+//   3. write:  every CTA reads the threshold from those two tables, looks up the keys inside the bin, counts what it
+//              takes, waits for the counts of the CTAs before it and writes its part of the list by ballots:
+//              position = (#greater before) + min(#equal before, ties to take)
+// Measured as graph replays, 4096 x 4096 / 11008 x 4096 / 28672 x 8192: 29 / 54 / 236 us, of which pass 1 alone takes
+// 14 / 32 / 180 us (5.6 TB/s of g, 6.3 with the keys).  Five passes with one bin per eighth of an octave took
+// 45 / 74 / 344 us.  One cooperative kernel with the keys in shared memory takes 33 us, and about 10 us more to launch.
 #include "pvt_internal.h"
 
 namespace pvt {
 
 SelectLayout select_layout(uint64_t G) {
   SelectLayout s;
-  s.ntiles = (uint32_t)((G + kSelTile - 1) / kSelTile);
-  // candidates: a quarter of the groups is far more than a threshold bucket of real gradients holds; when
-  // it is not enough (many equal norms) the low pass reads the keys instead
-  uint64_t cap = G / 4;
-  if (cap < 65536) cap = 65536;
-  if (cap > G) cap = G;
-  s.cand_cap = (uint32_t)cap;
-  s.hist_off = kWsHeaderBytes;
-  s.keys_off = align_up(s.hist_off + sizeof(uint32_t) * (kSelBins0 + kSelBins1 + kSelBins2), kWsAlign);
-  s.tiles_off = align_up(s.keys_off + sizeof(uint32_t) * G, kWsAlign);
-  s.cand_off = align_up(s.tiles_off + sizeof(uint32_t) * 2 * (size_t)s.ntiles, kWsAlign);
-  s.bytes = align_up(s.cand_off + sizeof(uint32_t) * (size_t)s.cand_cap, kWsAlign);
+  s.scratch_off = kWsHeaderBytes;
+  s.keys_off = align_up(s.scratch_off + sizeof(uint32_t) * kSelScratchWords, kWsAlign);
+  s.masks_off = align_up(s.keys_off + sizeof(uint32_t) * G, kWsAlign);
+  s.bytes = align_up(s.masks_off + 8 * ((G + 31) / 32), kWsAlign);
   return s;
 }
 
@@ -40,80 +35,6 @@ namespace {
 
 // Keys: n_j = ||eta * g_j||^2 in binary32: u = eta*g_i rounded once, acc = fma(u, u, acc)
 // in index order from 0.  Non-negative, so the bit pattern orders like the value.
-
-// Block-wide: true in every thread of the block that took the last ticket.
-__device__ __forceinline__ bool last_block_done(uint32_t* counter) {
-  __shared__ bool is_last;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const uint32_t ticket = atomicAdd(counter, 1u);
-    is_last = (ticket == gridDim.x - 1);
-  }
-  __syncthreads();
-  if (is_last) __threadfence();
-  return is_last;
-}
-
-// Inclusive scan of one value per thread over a block of kSelThreads threads.
-__device__ __forceinline__ uint64_t block_inclusive_scan(uint64_t v, uint64_t* sh /*[kSelThreads/32]*/) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint64_t n = __shfl_up_sync(0xffffffffu, v, o);
-    if (lane >= o) v += n;
-  }
-  __syncthreads();
-  if (lane == 31) sh[warp] = v;
-  __syncthreads();
-  uint64_t base = 0;
-  for (int w = 0; w < warp; ++w) base += sh[w];
-  return v + base;
-}
-
-// Walk a histogram from its top bin downwards and find the bin that holds the
-// k_left-th largest key.  Exactly one thread of the block finds it and writes
-// *digit and *k_new (= how many keys must still be taken from inside that bin).
-template <int NBINS>
-__device__ void find_digit(const uint32_t* hist, uint64_t k_left, uint32_t* digit, uint64_t* k_new,
-                           uint64_t* sh_scan) {
-  constexpr int PER = NBINS / kSelThreads;
-  // thread t owns the bins [hi - PER + 1, hi], hi descending with t
-  const int hi = NBINS - 1 - threadIdx.x * PER;
-  uint32_t c[PER];
-  uint64_t mine = 0;
-#pragma unroll
-  for (int i = 0; i < PER; ++i) {
-    c[i] = __ldcg(hist + hi - i);
-    mine += c[i];
-  }
-  const uint64_t incl = block_inclusive_scan(mine, sh_scan);
-  uint64_t above = incl - mine;  // keys in bins above this thread's bins
-#pragma unroll
-  for (int i = 0; i < PER; ++i) {
-    if (above < k_left && k_left <= above + c[i]) {
-      *digit = (uint32_t)(hi - i);
-      *k_new = k_left - above;
-    }
-    above += c[i];
-  }
-}
-
-constexpr int kNormPer = 8;                              // 16-byte loads per thread and iteration of the norm pass
-
-// LP adjacent lanes share a group (LP = group size / 4: 2 or 4), lane q of them holding elements 4q..4q+3,
-// so a warp reads 512 contiguous bytes per load instruction.  The sum is a single chain in index order:
-// lane 0 runs its four steps from 0 and hands the partial sum to lane 1, which runs the next four, and so
-// on; every lane computes every round (the work is free, the pass is bound by memory), the value is
-// kept only where it is the group's own partial sum.
-__device__ __forceinline__ float norm_chain(float acc, const float4& a, float eta) {
-  float u;
-  u = __fmul_rn(eta, a.x); acc = __fmaf_rn(u, u, acc);
-  u = __fmul_rn(eta, a.y); acc = __fmaf_rn(u, u, acc);
-  u = __fmul_rn(eta, a.z); acc = __fmaf_rn(u, u, acc);
-  u = __fmul_rn(eta, a.w); acc = __fmaf_rn(u, u, acc);
-  return acc;
-}
 
 // ---- random subspace rules (appendix on small-scale experiments: subspaces drawn uniformly at random, or at
 // random in proportion to the size of the gradient entries) --------------------------------------------------
@@ -154,6 +75,17 @@ __device__ __forceinline__ double neglog_u32(uint32_t r) {
   return __fma_rn((double)(32 - e), 0.6931471805599453, -lnm);
 }
 
+template <int DG>
+__device__ __forceinline__ float norm_of(const float* v, float eta) {
+  float acc = 0.0f;
+#pragma unroll
+  for (int i = 0; i < DG; ++i) {
+    const float u = __fmul_rn(eta, v[i]);
+    acc = __fmaf_rn(u, u, acc);
+  }
+  return acc;
+}
+
 // What the first pass computes per group (everything after the keys is the same top-k):
 //   kKeyNorm          key = squared update norm (the greedy rule of the V step)
 //   kKeyNormBuffer    the same, and the straight-through buffer takes the step: buffer = fma(-eta, g, buffer)
@@ -161,307 +93,373 @@ __device__ __forceinline__ double neglog_u32(uint32_t r) {
 //   kKeyProportional  key = (float)(norm / E), E the exponential clock of the group's random word
 enum KeyMode { kKeyNorm = 0, kKeyNormBuffer = 1, kKeyUniform = 2, kKeyProportional = 3 };
 
-template <int LP, int MODE>
-__global__ void __launch_bounds__(kSelThreads) norm_hist_kernel(const float* __restrict__ g, uint64_t G, float eta,
-                                                                 uint64_t k, uint32_t* __restrict__ keys,
-                                                                 uint32_t* __restrict__ hist0, SelectState* st,
-                                                                 float* __restrict__ buffer, uint64_t seed) {
-  pdl_trigger();
-  pdl_wait();
-  constexpr int kTile = kSelThreads * kNormPer / LP;  // groups per block and iteration
-  __shared__ uint32_t sh_hist[kSelBins0];
-  __shared__ uint64_t sh_scan[kSelThreads / 32];
-  for (int b = threadIdx.x; b < kSelBins0; b += kSelThreads) sh_hist[b] = 0;
-  __syncthreads();
-  const float4* g4 = reinterpret_cast<const float4*>(g);
-  float4* buf4 = reinterpret_cast<float4*>(buffer);
-  const uint64_t F = (uint64_t)LP * G;  // 16-byte pieces
-  const uint32_t n_tiles = (uint32_t)((G + kTile - 1) / kTile);
-  const int q = threadIdx.x & (LP - 1);  // position of this lane within its group
-  for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    const uint64_t f0 = (uint64_t)tile * (LP * kTile) + threadIdx.x;
-    float4 a[kNormPer];
+struct SelParams {
+  const float* g;
+  float* buffer;
+  uint64_t G, k, seed;
+  uint32_t words;        // words of 32 groups per CTA of passes 2 and 3
+  float eta;
+  uint32_t* idx_out;
+  uint32_t* status;
+  uint32_t* keys;        // [G]
+  uint2* masks;          // per word of 32 groups: above the threshold bin, inside it (pass 3: above, equal the threshold)
+  uint32_t* hist0;       // sum over the CTAs: key bits [30:18]
+  uint32_t* hist1;       // members of the threshold bin: key bits [17:9]
+  uint32_t* fine;        // members of the threshold bin: key bits [17:0]
+  uint32_t* state;       // [0] threshold bin, [1] keys still to be taken from it, [2] ticket
+  uint64_t* counts;      // per CTA of the last pass: ready << 62 | equal << 31 | greater
+};
+
+// 32 bytes that are not read again: one 256-bit load where the pointer allows it
+__device__ __forceinline__ void load8(const float* p, bool wide, float* v) {
+  if (wide) {
+    asm volatile("ld.global.L1::no_allocate.L2::evict_first.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "l"(p));
+  } else {
+    const float4 a = __ldcs(reinterpret_cast<const float4*>(p)), b = __ldcs(reinterpret_cast<const float4*>(p) + 1);
+    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+  }
+}
+__device__ __forceinline__ void store8(float* p, bool wide, const float* v) {
+  if (wide) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+                 "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                 : "memory");
+  } else {
+    __stcs(reinterpret_cast<float4*>(p), make_float4(v[0], v[1], v[2], v[3]));
+    __stcs(reinterpret_cast<float4*>(p) + 1, make_float4(v[4], v[5], v[6], v[7]));
+  }
+}
+
+// inclusive scan over a block of 1024 threads; `sh` has one word per warp
+__device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* sh) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int i = 0; i < kNormPer; ++i) {  // all loads of the iteration first
-      const uint64_t f = f0 + (uint64_t)i * kSelThreads;
-      a[i] = (MODE != kKeyUniform && f < F) ? __ldcs(g4 + f) : make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t n = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += n;
+  }
+  __syncthreads();
+  if (lane == 31) sh[warp] = v;
+  __syncthreads();
+  const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? sh[lane] : 0u);
+  return v + before;
+}
+
+// Walk a histogram from its top bin downwards to the bin that holds the k_left-th largest key; found[0] = that bin,
+// found[1] = how many keys are still to be taken from inside it.  A block of 1024 threads.
+template <int NBINS>
+__device__ __forceinline__ void find_digit(const uint32_t* hist, uint32_t k_left, uint32_t* sh, uint32_t* found) {
+  constexpr int PER = NBINS >= kSelThreads ? NBINS / kSelThreads : 1;
+  const bool own = threadIdx.x < NBINS / PER;
+  const int hi = NBINS - 1 - (int)threadIdx.x * PER;
+  uint32_t c[PER], mine = 0;
+  if (PER >= 4 && own) {
+#pragma unroll
+    for (int i = 0; i < PER; i += 4) {
+      const uint4 q = __ldcg(reinterpret_cast<const uint4*>(hist + hi + 1 - PER) + (PER - 4 - i) / 4);
+      c[i] = q.w, c[i + 1] = q.z, c[i + 2] = q.y, c[i + 3] = q.x;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < PER; ++i) c[i] = own ? __ldcg(hist + hi - i) : 0u;
+  }
+#pragma unroll
+  for (int i = 0; i < PER; ++i) mine += c[i];
+  if (threadIdx.x == 0) found[0] = found[1] = 0;  // (nothing found: an inconsistent histogram, reported at the end)
+  uint32_t above = block_scan(mine, sh) - mine;
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    if (above < k_left && k_left - above <= c[i]) {
+      found[0] = (uint32_t)(hi - i);
+      found[1] = k_left - above;
+    }
+    above += c[i];
+  }
+  __syncthreads();
+}
+
+// The same for 512 bins by one warp (16 bins per lane); every lane gets the answer.
+__device__ __forceinline__ void find_digit_warp(const uint32_t* hist, uint32_t k_left, uint32_t* digit, uint32_t* left) {
+  const int lane = threadIdx.x & 31;
+  const uint4* q = reinterpret_cast<const uint4*>(hist + 512 - 16 * (lane + 1));  // this lane's bins, ascending
+  uint4 v[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) v[i] = __ldcg(q + i);
+  const uint32_t c[16] = {v[3].w, v[3].z, v[3].y, v[3].x, v[2].w, v[2].z, v[2].y, v[2].x,
+                          v[1].w, v[1].z, v[1].y, v[1].x, v[0].w, v[0].z, v[0].y, v[0].x};  // descending
+  uint32_t mine = 0;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) mine += c[i];
+  uint32_t above = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t n = __shfl_up_sync(0xffffffffu, above, o);
+    if (lane >= o) above += n;
+  }
+  above -= mine;
+  uint32_t d = 0, l = 0;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    if (above < k_left && k_left - above <= c[i]) {
+      d = (uint32_t)(511 - 16 * lane - i);
+      l = k_left - above;
+    }
+    above += c[i];
+  }
+  const uint32_t owner = __ballot_sync(0xffffffffu, l != 0);
+  const int src = owner ? __ffs(owner) - 1 : 0;  // (no owner: an inconsistent histogram, reported at the end)
+  *digit = __shfl_sync(0xffffffffu, d, src);
+  *left = __shfl_sync(0xffffffffu, l, src);
+}
+
+// ---- 0. everything the passes count in starts at zero
+__global__ void __launch_bounds__(kSelThreads) select_clear_kernel(uint4* scratch, uint32_t n16) {
+  pdl_trigger();
+  for (uint32_t i = blockIdx.x * kSelThreads + threadIdx.x; i < n16; i += gridDim.x * kSelThreads)
+    scratch[i] = make_uint4(0, 0, 0, 0);
+}
+
+// ---- 1. keys and the histogram of their upper bits: the one pass over g
+template <int DG, int MODE>
+__global__ void __launch_bounds__(kNormThreads, kNormCtas) select_keys_kernel(const SelParams p) {
+  __shared__ uint32_t hist[kSelBins0];
+  const uint32_t tid = threadIdx.x;
+  pdl_trigger();
+  for (uint32_t i = tid; i < kSelBins0; i += kNormThreads) hist[i] = 0;
+  __syncthreads();
+  constexpr int U = (DG == 16 ? 2 : 4) / (MODE == kKeyNormBuffer ? 2 : 1);  // groups in flight per thread
+  const bool wide = ((reinterpret_cast<uintptr_t>(p.g) |
+                      (MODE == kKeyNormBuffer ? reinterpret_cast<uintptr_t>(p.buffer) : 0)) & 31u) == 0;
+  const uint64_t stride = (uint64_t)gridDim.x * (U * kNormThreads);
+  for (uint64_t j0 = (uint64_t)blockIdx.x * (U * kNormThreads) + tid; j0 < p.G; j0 += stride) {
+    float v[U][DG];
+    if (MODE != kKeyUniform) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint64_t j = j0 + u * kNormThreads;
+        if (j < p.G) {
+#pragma unroll
+          for (int part = 0; part < DG / 8; ++part) load8(p.g + j * DG + 8 * part, wide, &v[u][8 * part]);
+        }
+      }
     }
     if (MODE == kKeyNormBuffer) {  // the straight-through buffer takes the step of every weight (Appendix E)
-      float4 b[kNormPer];
+      float b[U][DG];
 #pragma unroll
-      for (int i = 0; i < kNormPer; ++i) {
-        const uint64_t f = f0 + (uint64_t)i * kSelThreads;
-        b[i] = f < F ? __ldcs(buf4 + f) : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int u = 0; u < U; ++u) {
+        const uint64_t j = j0 + u * kNormThreads;
+        if (j < p.G) {
+#pragma unroll
+          for (int part = 0; part < DG / 8; ++part) load8(p.buffer + j * DG + 8 * part, wide, &b[u][8 * part]);
+        }
       }
-      const float neg_eta = -eta;
 #pragma unroll
-      for (int i = 0; i < kNormPer; ++i) {
-        const uint64_t f = f0 + (uint64_t)i * kSelThreads;
-        if (f < F)
-          __stcs(buf4 + f, make_float4(__fmaf_rn(neg_eta, a[i].x, b[i].x), __fmaf_rn(neg_eta, a[i].y, b[i].y),
-                                       __fmaf_rn(neg_eta, a[i].z, b[i].z), __fmaf_rn(neg_eta, a[i].w, b[i].w)));
-      }
-    }
+      for (int u = 0; u < U; ++u) {
+        const uint64_t j = j0 + u * kNormThreads;
+        if (j < p.G) {
 #pragma unroll
-    for (int i = 0; i < kNormPer; ++i) {
-      const uint64_t f = f0 + (uint64_t)i * kSelThreads;
-      float acc = norm_chain(0.0f, a[i], eta);  // valid on lane 0 of the group
+          for (int i = 0; i < DG; ++i) b[u][i] = __fmaf_rn(-p.eta, v[u][i], b[u][i]);
 #pragma unroll
-      for (int r = 1; r < LP; ++r) {
-        const float in = __shfl_up_sync(0xffffffffu, acc, 1);  // lane r: the sum over elements 0..4r-1
-        const float next = norm_chain(in, a[i], eta);
-        acc = q >= r ? next : acc;
-      }
-      if (q == LP - 1 && f < F) {
-        uint32_t key = __float_as_uint(acc);
-        if (MODE == kKeyUniform) key = __float_as_uint((float)(philox_first_word(f / LP, seed) >> 8));
-        if (MODE == kKeyProportional)
-          key = acc > 0.0f ? __float_as_uint(__double2float_rn(
-                                 __ddiv_rn((double)acc, neglog_u32(philox_first_word(f / LP, seed)))))
-                           : 0u;
-        keys[f / LP] = key;
-        atomicAdd(&sh_hist[key >> 20], 1u);
+          for (int part = 0; part < DG / 8; ++part) store8(p.buffer + j * DG + 8 * part, wide, &b[u][8 * part]);
+        }
       }
     }
-  }
-  __syncthreads();
-  for (int b = threadIdx.x; b < kSelBins0; b += kSelThreads)
-    if (sh_hist[b]) atomicAdd(&hist0[b], sh_hist[b]);
-  if (last_block_done(&st->done[0])) find_digit<kSelBins0>(hist0, k, &st->digit0, &st->k_left, sh_scan);
-}
-
-// Keys whose bits [30:20] equal digit0: histogram of bits [19:9], and a compact copy
-// (order irrelevant) for the last refinement.  Bucket members are first collected in
-// shared memory; a block reserves room in the global list with one atomic per flush.
-constexpr int kMidStage = 2048;  // bucket members a block collects before it flushes
-
-__global__ void __launch_bounds__(kSelThreads) refine_mid_kernel(const uint32_t* __restrict__ keys, uint64_t G,
-                                                                  uint32_t* __restrict__ hist1,
-                                                                  uint32_t* __restrict__ cand, uint32_t cand_cap,
-                                                                  SelectState* st) {
-  pdl_trigger();
-  pdl_wait();
-  __shared__ uint32_t sh_hist[kSelBins1];
-  __shared__ uint64_t sh_scan[kSelThreads / 32];
-  __shared__ uint32_t sh_stage[kMidStage + 8 * kSelThreads];  // room for one more iteration after the check
-  __shared__ uint32_t sh_n, sh_base;
-  for (int b = threadIdx.x; b < kSelBins1; b += kSelThreads) sh_hist[b] = 0;
-  if (threadIdx.x == 0) sh_n = 0;
-  __syncthreads();
-  const uint32_t prefix = st->digit0;
-  const uint64_t n_quads = (G + 3) / 4;
-  const uint64_t stride = (uint64_t)gridDim.x * kSelThreads;
-
-  auto flush = [&]() {  // called by the whole block
-    __syncthreads();
-    const uint32_t n = sh_n;
-    if (threadIdx.x == 0 && n) sh_base = atomicAdd(&st->cand_count, n);
-    __syncthreads();
-    const uint32_t base = sh_base;
-    for (uint32_t i = threadIdx.x; i < n; i += kSelThreads)
-      if (base + i < cand_cap) cand[base + i] = sh_stage[i];
-    __syncthreads();
-    if (threadIdx.x == 0) sh_n = 0;
-    __syncthreads();
-  };
-
-  for (uint64_t q0 = (uint64_t)blockIdx.x * kSelThreads; q0 < n_quads; q0 += 2 * stride) {
-    // two independent 16-byte loads per thread and iteration
-    uint32_t key[8];
-    uint32_t have[2] = {0, 0};
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const uint64_t q = q0 + (uint64_t)h * stride + threadIdx.x;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) key[4 * h + i] = 0;
-      if (q < n_quads) {
-        if (4 * q + 4 <= G) {
-          const uint4 v = *reinterpret_cast<const uint4*>(keys + 4 * q);
-          key[4 * h] = v.x; key[4 * h + 1] = v.y; key[4 * h + 2] = v.z; key[4 * h + 3] = v.w;
-          have[h] = 4;
+    for (int u = 0; u < U; ++u) {
+      const uint64_t j = j0 + u * kNormThreads;
+      if (j < p.G) {
+        uint32_t key;
+        if (MODE == kKeyUniform) {
+          key = __float_as_uint((float)(philox_first_word(j, p.seed) >> 8));
         } else {
-          have[h] = (uint32_t)(G - 4 * q);
-          for (uint32_t i = 0; i < have[h]; ++i) key[4 * h + i] = keys[4 * q + i];
+          const float acc = norm_of<DG>(v[u], p.eta);
+          key = __float_as_uint(acc);
+          if (MODE == kKeyProportional)
+            key = acc > 0.0f ? __float_as_uint(__double2float_rn(
+                                   __ddiv_rn((double)acc, neglog_u32(philox_first_word(j, p.seed)))))
+                             : 0u;
+        }
+        p.keys[j] = key;
+        atomicAdd(&hist[key >> 18], 1u);
+      }
+    }
+  }
+  __syncthreads();
+  pdl_wait();  // the sums have been cleared
+  for (uint32_t i = tid; i < kSelBins0; i += kNormThreads)
+    if (hist[i]) atomicAdd(&p.hist0[i], hist[i]);
+}
+
+// ---- 2. the threshold bin: two bits per group (above it, inside it), and its members by their lower bits
+__global__ void __launch_bounds__(kSelThreads) select_bin_kernel(const SelParams p) {
+  __shared__ uint32_t hist[kSelBins1], sh[32], found[2];
+  const uint32_t tid = threadIdx.x, lane = tid & 31;
+  pdl_trigger();
+  if (tid < kSelBins1) hist[tid] = 0;
+  const uint64_t w_lo = (uint64_t)blockIdx.x * p.words, n_words = (p.G + 31) / 32;
+  const uint64_t w_hi = w_lo + p.words < n_words ? w_lo + p.words : n_words;
+  pdl_wait();
+  find_digit<kSelBins0>(p.hist0, (uint32_t)p.k, sh, found);
+  const uint32_t bin = found[0];
+  constexpr uint32_t U = 16;  // words of 32 groups per warp and trip, all their keys in flight
+  for (uint64_t w0 = w_lo + U * (tid >> 5); w0 < w_hi; w0 += U * (kSelThreads / 32)) {
+    uint32_t key[U];
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) {
+      const uint64_t j = (w0 + u) * 32 + lane;
+      key[u] = w0 + u < w_hi && j < p.G ? __ldcg(p.keys + j) : 0u;
+    }
+    uint32_t above = 0, inside = 0;
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u) {
+      const bool real = w0 + u < w_hi && (w0 + u) * 32 + lane < p.G;
+      const uint32_t m_gt = __ballot_sync(0xffffffffu, real && (key[u] >> 18) > bin);
+      const uint32_t m_in = __ballot_sync(0xffffffffu, real && (key[u] >> 18) == bin);
+      if (lane == u) {
+        above = m_gt;
+        inside = m_in;
+      }
+      if (m_in) {
+        // equal keys of a warp add up first: many equal norms must not queue at one address
+        const bool in = (m_in >> lane) & 1u;
+        const uint32_t same = __match_any_sync(0xffffffffu, in ? key[u] : 0xffffffffu);
+        if (in && lane == (uint32_t)__ffs(same) - 1) {
+          atomicAdd(&hist[(key[u] >> 9) & 511u], (uint32_t)__popc(same));
+          atomicAdd(&p.fine[key[u] & 0x3ffffu], (uint32_t)__popc(same));
         }
       }
     }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if ((uint32_t)i < have[h] && (key[4 * h + i] >> 20) == prefix) {
-          atomicAdd(&sh_hist[(key[4 * h + i] >> 9) & 0x7ffu], 1u);
-          sh_stage[atomicAdd(&sh_n, 1u)] = key[4 * h + i];
-        }
+    if (lane < U && w0 + lane < w_hi) p.masks[w0 + lane] = make_uint2(above, inside);
+  }
+  __syncthreads();
+  if (tid < kSelBins1 && hist[tid]) atomicAdd(&p.hist1[tid], hist[tid]);
+  if (blockIdx.x == 0 && tid == 0) {
+    p.state[0] = bin;
+    p.state[1] = found[1];
+  }
+}
+
+// ---- 3. threshold, and the ordered list of what is taken
+// A CTA needs to know what the CTAs before it take.  It waits for their counts, and only for theirs: numbers are drawn
+// at the start, so whoever is waited for is already running (and waits for nobody after it).  The wait is bounded.
+constexpr uint32_t kSelMaxPolls = 1u << 21;
+
+__global__ void __launch_bounds__(kSelThreads) select_write_kernel(const SelParams p) {
+  __shared__ uint32_t sh[32], ticket, sh_threshold, sh_need, sum_gt, sum_eq, all_gt, all_eq;
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_trigger();
+  pdl_wait();
+  if (tid == 32) {
+    ticket = atomicAdd(&p.state[2], 1u);
+    sum_gt = sum_eq = all_gt = all_eq = 0;
+  }
+  if (warp == 0) {
+    const uint32_t bin = __ldcg(p.state), in_bin = __ldcg(p.state + 1);
+    uint32_t d1, d2, left;
+    find_digit_warp(p.hist1, in_bin, &d1, &left);
+    find_digit_warp(p.fine + 512 * d1, left, &d2, &left);
+    if (lane == 0) {
+      sh_threshold = (bin << 18) | (d1 << 9) | d2;
+      sh_need = left;
+    }
+  }
+  __syncthreads();
+  const uint32_t cta = ticket, threshold = sh_threshold, need_eq = sh_need;
+  const uint64_t w_lo = (uint64_t)cta * p.words, n_words = (p.G + 31) / 32;
+  const uint64_t w_hi = w_lo + p.words < n_words ? w_lo + p.words : n_words;
+
+  // one word of 32 groups per thread and trip; the members of the threshold bin (few) are looked up
+  auto resolve = [&](uint64_t w) {
+    uint2 m = __ldcg(p.masks + w);
+    uint32_t gt = m.x, eq = 0;
+    for (uint32_t in = m.y; in; in &= in - 1) {
+      const uint32_t b = (uint32_t)__ffs(in) - 1;
+      const uint32_t key = __ldcg(p.keys + w * 32 + b);
+      gt |= key > threshold ? 1u << b : 0u;
+      eq |= key == threshold ? 1u << b : 0u;
+    }
+    return make_uint2(gt, eq);
+  };
+  uint2 first = make_uint2(0, 0);  // the first trip's answer stays in registers, those of further trips go back
+  uint32_t n_gt = 0, n_eq = 0;
+  for (uint64_t w = w_lo + tid; w < w_hi; w += kSelThreads) {
+    const uint2 m = resolve(w);
+    if (w == w_lo + tid)
+      first = m;
+    else
+      p.masks[w] = m;
+    n_gt += __popc(m.x);
+    n_eq += __popc(m.y);
+  }
+  n_gt = __reduce_add_sync(0xffffffffu, n_gt);
+  n_eq = __reduce_add_sync(0xffffffffu, n_eq);
+  if (lane == 0 && n_gt) atomicAdd(&all_gt, n_gt);
+  if (lane == 0 && n_eq) atomicAdd(&all_eq, n_eq);
+  __syncthreads();
+  if (tid == 0) {
+    const uint64_t mine = (1ull << 63) | ((uint64_t)all_eq << 31) | all_gt;  // a CTA has fewer than 2^31 groups
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p.counts + cta), "l"(mine) : "memory");
+  }
+  bool ok = true;
+  uint32_t prev_gt = 0, prev_eq = 0;
+  for (uint32_t b = tid; b < cta; b += kSelThreads) {
+    uint64_t c = 0;
+    for (uint32_t i = 0; i < kSelMaxPolls && !(c >> 63); ++i)
+      asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(c) : "l"(p.counts + b) : "memory");
+    ok &= (c >> 63) != 0;
+    prev_gt += (uint32_t)c & 0x7fffffffu;
+    prev_eq += (uint32_t)(c >> 31) & 0x7fffffffu;
+  }
+  prev_gt = __reduce_add_sync(0xffffffffu, prev_gt);
+  prev_eq = __reduce_add_sync(0xffffffffu, prev_eq);
+  if (lane == 0 && prev_gt) atomicAdd(&sum_gt, prev_gt);
+  if (lane == 0 && prev_eq) atomicAdd(&sum_eq, prev_eq);
+  if (!__syncthreads_and(ok)) {
+    if (tid == 0) atomicOr(p.status, PVT_DEV_WAIT_EXPIRED);
+    return;
+  }
+  uint32_t at_gt = sum_gt, at_eq = sum_eq;  // what comes before the trip
+  // all greater keys plus the ties taken must be exactly k
+  if (cta == gridDim.x - 1 && tid == 0 && (uint64_t)at_gt + all_gt + min(at_eq + all_eq, need_eq) != p.k)
+    atomicOr(p.status, PVT_DEV_INTERNAL);
+  for (uint64_t w0 = w_lo; w0 < w_hi; w0 += kSelThreads) {
+    const uint64_t w = w0 + tid;
+    uint2 m = make_uint2(0, 0);
+    if (w < w_hi) m = w0 == w_lo ? first : __ldcg(p.masks + w);
+    // both counts in one scan: a trip has 2^15 groups
+    const uint32_t mine = (uint32_t)__popc(m.x) | ((uint32_t)__popc(m.y) << 16);
+    const uint32_t incl = block_scan(mine, sh);
+    uint32_t my_gt = at_gt + ((incl - mine) & 0xffffu), my_eq = at_eq + ((incl - mine) >> 16);
+    if (tid == kSelThreads - 1) {
+      sum_gt = at_gt + (incl & 0xffffu);
+      sum_eq = at_eq + (incl >> 16);
+    }
+    const uint32_t most = __reduce_max_sync(0xffffffffu, (uint32_t)__popc(m.x | m.y));
+    if (most <= 6) {  // few bits: every lane writes its own word's
+      for (uint32_t both = m.x | m.y; both; both &= both - 1) {
+        const uint32_t b = (uint32_t)__ffs(both) - 1;
+        const bool is_gt = (m.x >> b) & 1u;
+        const uint32_t pos = my_gt + min(my_eq, need_eq);
+        if ((is_gt || my_eq < need_eq) && pos < p.k) p.idx_out[pos] = (uint32_t)(w * 32) + b;
+        my_gt += is_gt;
+        my_eq += !is_gt;
+      }
+    } else {          // the warp writes one word after the other, a lane per group
+      for (uint32_t left = __ballot_sync(0xffffffffu, (m.x | m.y) != 0); left; left &= left - 1) {
+        const int src = __ffs(left) - 1;
+        const uint32_t gt = __shfl_sync(0xffffffffu, m.x, src), eq = __shfl_sync(0xffffffffu, m.y, src);
+        const uint32_t b_gt = __shfl_sync(0xffffffffu, my_gt, src), b_eq = __shfl_sync(0xffffffffu, my_eq, src);
+        const uint32_t below = (1u << lane) - 1u;
+        const uint32_t e = b_eq + __popc(eq & below), pos = b_gt + __popc(gt & below) + min(e, need_eq);
+        const bool take = ((gt >> lane) & 1u) || (((eq >> lane) & 1u) && e < need_eq);
+        if (take && pos < p.k) p.idx_out[pos] = (uint32_t)((w0 + 32 * warp + src) * 32) + lane;
       }
     }
     __syncthreads();
-    const uint32_t collected = sh_n;  // the same value in every thread
-    __syncthreads();                  // nobody adds to it again before everybody has read it
-    if (collected >= (uint32_t)kMidStage) flush();
-  }
-  flush();
-  for (int b = threadIdx.x; b < kSelBins1; b += kSelThreads)
-    if (sh_hist[b]) atomicAdd(&hist1[b], sh_hist[b]);
-  if (last_block_done(&st->done[1])) {
-    const uint64_t k_left = st->k_left;
-    __syncthreads();
-    find_digit<kSelBins1>(hist1, k_left, &st->digit1, &st->k_left, sh_scan);
-  }
-}
-
-// Bits [8:0] of the candidates that match (digit0, digit1); reads the candidate list, or
-// all keys if the list did not hold every bucket member.
-__global__ void __launch_bounds__(kSelThreads) refine_low_kernel(const uint32_t* __restrict__ keys, uint64_t G,
-                                                                  const uint32_t* __restrict__ cand,
-                                                                  uint32_t cand_cap, uint32_t* __restrict__ hist2,
-                                                                  SelectState* st) {
-  pdl_trigger();
-  pdl_wait();
-  __shared__ uint32_t sh_hist[kSelBins2];
-  __shared__ uint64_t sh_scan[kSelThreads / 32];
-  for (int b = threadIdx.x; b < kSelBins2; b += kSelThreads) sh_hist[b] = 0;
-  __syncthreads();
-  const uint32_t prefix = (st->digit0 << 11) | st->digit1;
-  const uint32_t n_cand = st->cand_count;
-  const bool listed = n_cand <= cand_cap;
-  const uint32_t* src = listed ? cand : keys;
-  const uint64_t n = listed ? (uint64_t)n_cand : G;
-  for (uint64_t i = (uint64_t)blockIdx.x * kSelThreads + threadIdx.x; i < n; i += (uint64_t)gridDim.x * kSelThreads) {
-    const uint32_t key = src[i];
-    if ((key >> 9) == prefix) atomicAdd(&sh_hist[key & 0x1ffu], 1u);
-  }
-  __syncthreads();
-  for (int b = threadIdx.x; b < kSelBins2; b += kSelThreads)
-    if (sh_hist[b]) atomicAdd(&hist2[b], sh_hist[b]);
-  if (last_block_done(&st->done[2])) {
-    const uint64_t k_left = st->k_left;
-    __shared__ uint32_t d2;
-    __shared__ uint64_t kn;
-    __syncthreads();
-    find_digit<kSelBins2>(hist2, k_left, &d2, &kn, sh_scan);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      st->threshold = (st->digit0 << 20) | (st->digit1 << 9) | d2;
-      st->need_eq = (uint32_t)kn;
-    }
-  }
-}
-
-__global__ void __launch_bounds__(kSelThreads) tile_count_kernel(const uint32_t* __restrict__ keys, uint64_t G,
-                                                                  uint32_t* __restrict__ tiles, uint32_t ntiles,
-                                                                  uint64_t k, SelectState* st, uint32_t* status) {
-  pdl_trigger();
-  pdl_wait();
-  __shared__ uint32_t sh_gt, sh_eq;
-  __shared__ uint64_t sh_scan[kSelThreads / 32];
-  if (threadIdx.x == 0) sh_gt = sh_eq = 0;
-  __syncthreads();
-  const uint32_t T = st->threshold;
-  const uint64_t j0 = (uint64_t)blockIdx.x * kSelTile;
-  constexpr int QUADS = kSelTile / (4 * kSelThreads);  // 16-byte loads per thread, all issued before use
-  uint32_t gt = 0, eq = 0;
-  if (j0 + kSelTile <= G) {
-    uint4 v[QUADS];
-#pragma unroll
-    for (int i = 0; i < QUADS; ++i)
-      v[i] = *reinterpret_cast<const uint4*>(keys + j0 + 4 * ((uint64_t)i * kSelThreads + threadIdx.x));
-#pragma unroll
-    for (int i = 0; i < QUADS; ++i) {
-      gt += (v[i].x > T) + (v[i].y > T) + (v[i].z > T) + (v[i].w > T);
-      eq += (v[i].x == T) + (v[i].y == T) + (v[i].z == T) + (v[i].w == T);
-    }
-  } else {
-    for (uint64_t j = j0 + threadIdx.x; j < G; j += kSelThreads) {
-      const uint32_t key = keys[j];
-      gt += key > T;
-      eq += key == T;
-    }
-  }
-  gt = __reduce_add_sync(0xffffffffu, gt);
-  eq = __reduce_add_sync(0xffffffffu, eq);
-  if ((threadIdx.x & 31) == 0) {
-    if (gt) atomicAdd(&sh_gt, gt);
-    if (eq) atomicAdd(&sh_eq, eq);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    tiles[2 * blockIdx.x] = sh_gt;
-    tiles[2 * blockIdx.x + 1] = sh_eq;
-  }
-  if (last_block_done(&st->done[3])) {
-    // exclusive scan of the tile counts, in place; consecutive tiles per thread
-    const uint32_t per = (ntiles + kSelThreads - 1) / kSelThreads;
-    const uint32_t lo = min(threadIdx.x * per, ntiles), hi = min(lo + per, ntiles);
-    uint64_t sg = 0, se = 0;
-    for (uint32_t t = lo; t < hi; ++t) {
-      sg += __ldcg(tiles + 2 * t);
-      se += __ldcg(tiles + 2 * t + 1);
-    }
-    const uint64_t ig = block_inclusive_scan(sg, sh_scan);
-    __syncthreads();
-    const uint64_t ie = block_inclusive_scan(se, sh_scan);
-    uint64_t rg = ig - sg, re = ie - se;
-    for (uint32_t t = lo; t < hi; ++t) {
-      const uint32_t cg = __ldcg(tiles + 2 * t), ce = __ldcg(tiles + 2 * t + 1);
-      tiles[2 * t] = (uint32_t)rg;
-      tiles[2 * t + 1] = (uint32_t)re;
-      rg += cg;
-      re += ce;
-    }
-    if (threadIdx.x == kSelThreads - 1) {
-      // all greater keys plus the ties taken must be exactly k
-      const uint64_t taken_eq = ie < st->need_eq ? ie : st->need_eq;
-      if (ig + taken_eq != k) atomicOr(status, PVT_DEV_INTERNAL);
-    }
-  }
-}
-
-__global__ void __launch_bounds__(kSelThreads) scatter_kernel(const uint32_t* __restrict__ keys, uint64_t G,
-                                                               const uint32_t* __restrict__ tiles,
-                                                               const SelectState* st, uint64_t k,
-                                                               uint32_t* __restrict__ idx_out) {
-  pdl_trigger();
-  pdl_wait();
-  __shared__ uint64_t sh_scan[kSelThreads / 32];
-  const uint32_t T = st->threshold, need_eq = st->need_eq;
-  constexpr int PER = kSelTile / kSelThreads;  // consecutive groups per thread: keeps index order
-  const uint64_t jt = (uint64_t)blockIdx.x * kSelTile + (uint64_t)threadIdx.x * PER;
-  uint32_t key[PER];
-  if (jt + PER <= G) {
-    const uint4* p = reinterpret_cast<const uint4*>(keys + jt);
-#pragma unroll
-    for (int i = 0; i < PER / 4; ++i) {
-      const uint4 v = p[i];
-      key[4 * i] = v.x; key[4 * i + 1] = v.y; key[4 * i + 2] = v.z; key[4 * i + 3] = v.w;
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < PER; ++i) key[i] = (jt + i < G) ? keys[jt + i] : 0u;
-  }
-  uint32_t gt = 0, eq = 0;
-#pragma unroll
-  for (int i = 0; i < PER; ++i) {
-    const bool in = jt + i < G;
-    gt += in && key[i] > T;
-    eq += in && key[i] == T;
-  }
-  // one scan for both counts: each fits 16 bits inside a tile of 4096
-  const uint64_t packed = (uint64_t)gt | ((uint64_t)eq << 32);
-  const uint64_t incl = block_inclusive_scan(packed, sh_scan);
-  uint64_t GT = (uint64_t)tiles[2 * blockIdx.x] + (uint32_t)(incl - packed);
-  uint64_t EQ = (uint64_t)tiles[2 * blockIdx.x + 1] + (uint32_t)((incl - packed) >> 32);
-#pragma unroll
-  for (int i = 0; i < PER; ++i) {
-    if (jt + i < G) {
-      const bool is_gt = key[i] > T, is_eq = key[i] == T;
-      if (is_gt || (is_eq && EQ < need_eq)) {
-        const uint64_t pos = GT + (EQ < need_eq ? EQ : need_eq);
-        if (pos < k) idx_out[pos] = (uint32_t)(jt + i);
-      }
-      GT += is_gt;
-      EQ += is_eq;
-    }
+    at_gt = sum_gt;
+    at_eq = sum_eq;
   }
 }
 
@@ -474,29 +472,20 @@ __global__ void iota_kernel(uint32_t* idx_out, uint64_t k) {
 
 namespace {
 
-template <int LP, int MODE>
-cudaError_t launch_norm(const pvt_layer& L, uint64_t G, uint64_t k, uint32_t* keys, uint32_t* hist0, SelectState* st,
-                        float* buffer, uint64_t seed, int sm_count, cudaStream_t stream) {
-  int per_sm = 0;
-  cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, norm_hist_kernel<LP, MODE>, kSelThreads, 0);
-  if (err != cudaSuccess) return err;
-  const uint64_t tile = (uint64_t)kSelThreads * kNormPer / LP;
-  const uint64_t tiles = (G + tile - 1) / tile;
-  const uint64_t resident = (uint64_t)sm_count * (uint64_t)(per_sm > 0 ? per_sm : 1);  // a persistent grid
-  norm_hist_kernel<LP, MODE><<<(unsigned)(tiles < resident ? tiles : resident), kSelThreads, 0, stream>>>(
-      L.g, G, L.eta, k, keys, hist0, st, buffer, seed);
-  return cudaGetLastError();
+template <int DG, int MODE>
+cudaError_t launch_keys(const SelParams& p, int sm_count, cudaStream_t stream) {
+  const uint64_t blocks = (p.G + 2 * kNormThreads - 1) / (2 * kNormThreads), resident = (uint64_t)sm_count * kNormCtas;
+  return launch_dependent(select_keys_kernel<DG, MODE>, (unsigned)(blocks < resident ? blocks : resident), kNormThreads, 0,
+                          stream, p);
 }
 
-template <int LP>
-cudaError_t launch_norm_mode(int mode, const pvt_layer& L, uint64_t G, uint64_t k, uint32_t* keys, uint32_t* hist0,
-                             SelectState* st, float* buffer, uint64_t seed, int sm_count, cudaStream_t stream) {
+template <int DG>
+cudaError_t launch_group(int mode, const SelParams& p, int sm_count, cudaStream_t stream) {
   switch (mode) {
-    case kKeyNormBuffer: return launch_norm<LP, kKeyNormBuffer>(L, G, k, keys, hist0, st, buffer, seed, sm_count, stream);
-    case kKeyUniform: return launch_norm<LP, kKeyUniform>(L, G, k, keys, hist0, st, buffer, seed, sm_count, stream);
-    case kKeyProportional:
-      return launch_norm<LP, kKeyProportional>(L, G, k, keys, hist0, st, buffer, seed, sm_count, stream);
-    default: return launch_norm<LP, kKeyNorm>(L, G, k, keys, hist0, st, buffer, seed, sm_count, stream);
+    case kKeyNormBuffer: return launch_keys<DG, kKeyNormBuffer>(p, sm_count, stream);
+    case kKeyUniform: return launch_keys<DG, kKeyUniform>(p, sm_count, stream);
+    case kKeyProportional: return launch_keys<DG, kKeyProportional>(p, sm_count, stream);
+    default: return launch_keys<DG, kKeyNorm>(p, sm_count, stream);
   }
 }
 
@@ -510,51 +499,47 @@ cudaError_t launch_select(const pvt_layer& L, uint64_t G, uint64_t k, uint32_t* 
 cudaError_t launch_select_keyed(const pvt_layer& L, uint64_t G, uint64_t k, uint32_t* idx_out, void* ws, int sm_count,
                                 cudaStream_t stream, int key_mode, float* buffer, uint64_t seed) {
   timing_begin(kKernSelect, stream);
-  cudaError_t err = cudaSuccess;
+  cudaError_t err;
   if (k == G && key_mode != kKeyNormBuffer) {  // every group is taken: the ascending index list itself
     iota_kernel<<<(unsigned)((k + 255) / 256), 256, 0, stream>>>(idx_out, k);
     err = cudaGetLastError();
-    count_launches(1);
-    timing_end(kKernSelect, stream);
-    return err;
+  } else {
+    const SelectLayout lay = select_layout(G);
+    char* base = static_cast<char*>(ws);
+    SelParams p;
+    p.g = L.g;
+    p.buffer = buffer;
+    p.G = G;
+    p.k = k;
+    p.seed = seed;
+    p.eta = L.eta;
+    p.idx_out = idx_out;
+    p.status = reinterpret_cast<uint32_t*>(base);
+    p.keys = reinterpret_cast<uint32_t*>(base + lay.keys_off);
+    p.masks = reinterpret_cast<uint2*>(base + lay.masks_off);
+    uint32_t* scratch = reinterpret_cast<uint32_t*>(base + lay.scratch_off);
+    p.counts = reinterpret_cast<uint64_t*>(scratch);
+    p.state = scratch + 2 * kSelMaxCtas;
+    p.hist0 = p.state + 16;
+    p.hist1 = p.hist0 + kSelBins0;
+    p.fine = p.hist1 + kSelBins1;
+    // the passes over the keys: a CTA per SM, fewer for small layers (at least two groups per thread)
+    uint64_t n_cta = (G + 2 * kSelThreads - 1) / (2 * kSelThreads);
+    const uint64_t most = sm_count < (int)kSelMaxCtas ? (uint64_t)sm_count : kSelMaxCtas;
+    if (n_cta > most) n_cta = most;
+    p.words = (uint32_t)(((G + n_cta - 1) / n_cta + 31) / 32);
+    constexpr uint32_t n16 = kSelScratchWords / 4;
+    select_clear_kernel<<<(n16 + kSelThreads - 1) / kSelThreads, kSelThreads, 0, stream>>>(
+        reinterpret_cast<uint4*>(scratch), n16);
+    err = cudaGetLastError();
+    if (err == cudaSuccess)
+      err = L.group_dim == 16 ? launch_group<16>(key_mode, p, sm_count, stream)
+                              : launch_group<8>(key_mode, p, sm_count, stream);
+    if (err == cudaSuccess) err = launch_dependent(select_bin_kernel, (unsigned)n_cta, kSelThreads, 0, stream, p);
+    if (err == cudaSuccess) err = launch_dependent(select_write_kernel, (unsigned)n_cta, kSelThreads, 0, stream, p);
+    count_launches(3);
   }
-  const SelectLayout lay = select_layout(G);
-  char* base = static_cast<char*>(ws);
-  uint32_t* status = reinterpret_cast<uint32_t*>(base);
-  SelectState* st = reinterpret_cast<SelectState*>(base + kSelStateOffset);
-  uint32_t* hist0 = reinterpret_cast<uint32_t*>(base + lay.hist_off);
-  uint32_t* hist1 = hist0 + kSelBins0;
-  uint32_t* hist2 = hist1 + kSelBins1;
-  uint32_t* keys = reinterpret_cast<uint32_t*>(base + lay.keys_off);
-  uint32_t* tiles = reinterpret_cast<uint32_t*>(base + lay.tiles_off);
-  // selection state (header, from byte 64) and the three histograms are adjacent: one clear
-  static_assert(kSelStateOffset + sizeof(SelectState) <= kWsHeaderBytes, "selection state must fit the header");
-  if ((err = cudaMemsetAsync(st, 0, (kWsHeaderBytes - kSelStateOffset) +
-                                        sizeof(uint32_t) * (kSelBins0 + kSelBins1 + kSelBins2), stream)) !=
-      cudaSuccess)
-    return err;
-  uint32_t* cand = reinterpret_cast<uint32_t*>(base + lay.cand_off);
-  // persistent grids: exactly the blocks that are resident at once
-  int mid_per_sm = 0;
-  if ((err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&mid_per_sm, refine_mid_kernel, kSelThreads, 0)) !=
-      cudaSuccess)
-    return err;
-  const uint64_t quad_blocks = ((G + 3) / 4 + 2 * kSelThreads - 1) / (2 * kSelThreads);
-  const uint64_t mid_res = (uint64_t)sm_count * (uint64_t)(mid_per_sm > 0 ? mid_per_sm : 1);
-  const unsigned mid_grid = (unsigned)(quad_blocks < mid_res ? quad_blocks : mid_res);
-  err = L.group_dim == 16 ? launch_norm_mode<4>(key_mode, L, G, k, keys, hist0, st, buffer, seed, sm_count, stream)
-                          : launch_norm_mode<2>(key_mode, L, G, k, keys, hist0, st, buffer, seed, sm_count, stream);
-  if (err != cudaSuccess) return err;
-  err = launch_dependent(refine_mid_kernel, mid_grid, kSelThreads, 0, stream, keys, G, hist1, cand, lay.cand_cap, st);
-  if (err != cudaSuccess) return err;
-  const unsigned low_grid = (unsigned)(lay.cand_cap / 8192 < (uint32_t)sm_count ? lay.cand_cap / 8192 + 1 : sm_count);
-  err = launch_dependent(refine_low_kernel, low_grid, kSelThreads, 0, stream, keys, G, cand, lay.cand_cap, hist2, st);
-  if (err != cudaSuccess) return err;
-  err = launch_dependent(tile_count_kernel, lay.ntiles, kSelThreads, 0, stream, keys, G, tiles, lay.ntiles, k, st, status);
-  if (err != cudaSuccess) return err;
-  err = launch_dependent(scatter_kernel, lay.ntiles, kSelThreads, 0, stream, keys, G, tiles, st, k, idx_out);
-  if (err == cudaSuccess) err = cudaGetLastError();
-  count_launches(5);
+  count_launches(1);
   timing_end(kKernSelect, stream);
   return err;
 }
