@@ -172,6 +172,31 @@ __device__ __forceinline__ uint32_t fast_div(uint32_t n, const FastDiv& f) {
 }
 #endif
 
+// ---- 32 bytes per thread --------------------------------------------------------------------------------
+#ifdef __CUDACC__
+// 32 bytes that are not read again: one 256-bit load where the pointer allows it
+__device__ __forceinline__ void load8(const float* p, bool wide, float* v) {
+  if (wide) {
+    asm volatile("ld.global.L1::no_allocate.L2::evict_first.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "l"(p));
+  } else {
+    const float4 a = __ldcs(reinterpret_cast<const float4*>(p)), b = __ldcs(reinterpret_cast<const float4*>(p) + 1);
+    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+  }
+}
+__device__ __forceinline__ void store8(float* p, bool wide, const float* v) {
+  if (wide) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+                 "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                 : "memory");
+  } else {
+    __stcs(reinterpret_cast<float4*>(p), make_float4(v[0], v[1], v[2], v[3]));
+    __stcs(reinterpret_cast<float4*>(p) + 1, make_float4(v[4], v[5], v[6], v[7]));
+  }
+}
+#endif
+
 // ---- programmatic dependent launch --------------------------------------------------------------------
 // Consecutive kernels of a call depend on one another, so between two of them the GPU would idle for a launch
 // latency.  A kernel launched with launch_dependent() may be scheduled while the kernel before it on the stream

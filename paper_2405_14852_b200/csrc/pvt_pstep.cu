@@ -9,10 +9,10 @@
 // Every product of two binary32 numbers is exact in binary64 and the sums are accumulated in binary64 with
 // atomic adds, so the result differs from a sequential sum only by the order of binary64 roundings.
 //
-// One streaming pass over g (two threads per group, 512 contiguous bytes per warp load).  Small codebooks
-// (M K <= 512 codewords) are accumulated in shared memory per block and flushed once; large ones go straight
-// to the L2 with one reduction per element.  Scale gradients are summed over a warp first when the warp
-// lies inside one row.
+// One streaming pass over g.  Small codebooks (M K <= 2048 codewords) are accumulated in shared memory per CTA and
+// flushed once; large ones go straight to the L2.  Between 1024 and 4096 codewords the two take about the same time
+// (4096 x 4096: 87 us for 1024 in shared memory, 56 us for 4096 in the L2, where fewer codewords queue up).  Scale
+// gradients are summed over a warp first when the warp lies inside one row.
 #include <cuda_fp16.h>
 
 #include "pvt_internal.h"
@@ -21,337 +21,368 @@ namespace pvt {
 namespace {
 
 constexpr int kPsThreads = 256;
-constexpr int kPsSmemCodewords = 512;
-
-// elements 4*half .. 4*half+3 of a codeword of 4*PARTS elements (PARTS = 2 for groups of 8 weights, 4 for 16)
-template <bool CB_F16, int PARTS = 2>
-__device__ __forceinline__ float4 half_codeword(const void* book, uint32_t code, uint32_t half) {
-  if (CB_F16) {
-    const uint2 raw = __ldg(reinterpret_cast<const uint2*>(book) + PARTS * (size_t)code + half);
-    const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&raw.x));
-    const float2 hi = __half22float2(*reinterpret_cast<const __half2*>(&raw.y));
-    return make_float4(lo.x, lo.y, hi.x, hi.y);
-  } else {
-    return __ldg(reinterpret_cast<const float4*>(book) + PARTS * (size_t)code + half);
-  }
-}
+constexpr size_t kPsMaxSmem = 226 * 1024;
+constexpr int kPsSmallBins = 2048;   // M K up to here: sums in shared memory, above it in the L2
 
 __device__ __forceinline__ void red_add_f64(double* p, double v) {
   asm volatile("red.global.add.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
 }
 
-template <int M, bool CB_F16, bool CODE_U16, bool SMEM_ACC, int PARTS = 2>
+// v = the codeword of a group (codebooks added left to right, each sum rounded once), from global or shared memory
+template <int M, bool CB_F16, int DG>
+__device__ __forceinline__ void group_codeword(const uint4* book, const uint32_t (&b)[M], uint32_t K, float (&v)[DG]) {
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+    const uint4* row = book + (size_t)(m * K + b[m]) * (DG / (CB_F16 ? 8 : 4));
+    float c[DG];
+#pragma unroll
+    for (int part = 0; part < DG / (CB_F16 ? 8 : 4); ++part) {
+      const uint4 raw = row[part];
+      const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (CB_F16) {
+          const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[i]));
+          c[8 * part + 2 * i] = f.x;
+          c[8 * part + 2 * i + 1] = f.y;
+        } else {
+          c[4 * part + i] = __uint_as_float(w[i]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < DG; ++i) v[i] = m == 0 ? c[i] : __fadd_rn(v[i], c[i]);
+  }
+}
+
+template <int M, bool CODE_U16>
+__device__ __forceinline__ void group_codes(const void* codes, uint64_t j, uint32_t (&b)[M]) {
+  if (!CODE_U16 && M == 2) {
+    const uint32_t both = __ldg(reinterpret_cast<const uint16_t*>(codes) + j);
+    b[0] = both & 0xffu;
+    b[M - 1] = both >> 8;
+  } else {
+#pragma unroll
+    for (int m = 0; m < M; ++m)
+      b[m] = CODE_U16 ? __ldg(reinterpret_cast<const uint16_t*>(codes) + j * M + m)
+                      : __ldg(reinterpret_cast<const uint8_t*>(codes) + j * M + m);
+  }
+}
+
+// sum over i of g_i v_i: the products are exact, one rounding each as for a sum
+template <int DG>
+__device__ __forceinline__ double dot_exact(const double (&g)[DG], const float (&v)[DG]) {
+  double d = g[0] * (double)v[0];
+#pragma unroll
+  for (int i = 1; i < DG; ++i) d = __fma_rn(g[i], (double)v[i], d);
+  return d;
+}
+
+// the exact products s * g of a group as one row of doubles; lanes start at different pieces (no bank conflict)
+template <int DG>
+__device__ __forceinline__ void put_products(double* row, uint32_t lane, double s, const double (&g)[DG]) {
+  double2* dst = reinterpret_cast<double2*>(row);
+#pragma unroll
+  for (int q = 0; q < DG / 2; q += 2) {
+    const double2 lo = make_double2(s * g[2 * q], s * g[2 * q + 1]), hi = make_double2(s * g[2 * q + 2], s * g[2 * q + 3]);
+    const uint32_t first = (lane >> 1) & 1u;
+    dst[q + first] = first ? hi : lo;
+    dst[q + (first ^ 1u)] = first ? lo : hi;
+  }
+}
+
+// Large codebooks: one reduction per element in the L2.  A lane takes a group: its 32 bytes of g, its codeword, its
+// share of the scale's gradient; the products then change places through shared memory so that the DG elements of a
+// group are added by DG adjacent lanes: an L2 slice takes the four binary64 values of a sector that one instruction
+// brings as one operation.  4096 x 4096: 48 us; with four elements of a group in a thread, four instructions to
+// the same sector, 107 us; with a lane per element from the start (three conversions and a codeword load per
+// element) 59 us.
+template <int M, bool CB_F16, bool CODE_U16, int DG>
 __global__ void __launch_bounds__(kPsThreads) pstep_grad_kernel(const float* __restrict__ g,
                                                                  const float* __restrict__ scale,
                                                                  const void* __restrict__ codes,
                                                                  const void* __restrict__ codebooks, uint64_t G,
-                                                                 uint32_t gpr, uint32_t K,
+                                                                 FastDiv gpr, uint32_t K,
                                                                  double* __restrict__ grad_books,
                                                                  double* __restrict__ grad_scale, uint32_t* status) {
-  __shared__ double sh_acc[SMEM_ACC ? kPsSmemCodewords * 8 : 1];
-  if (SMEM_ACC) {
-    for (uint32_t i = threadIdx.x; i < (uint32_t)M * K * 8; i += kPsThreads) sh_acc[i] = 0.0;
-    __syncthreads();
-  }
-  const uint64_t H = (uint64_t)PARTS * G;  // PARTS threads per group, four weights each
-  const float4* g4 = reinterpret_cast<const float4*>(g);
-  const int lane = threadIdx.x & 31;
-  for (uint64_t h0 = (uint64_t)blockIdx.x * kPsThreads; h0 < H; h0 += (uint64_t)gridDim.x * kPsThreads) {
-    const uint64_t h = h0 + threadIdx.x;
-    const bool valid = h < H;
-    const uint32_t j = (uint32_t)(h / PARTS), half = (uint32_t)h & (uint32_t)(PARTS - 1);
-    uint32_t row = 0xffffffffu;
+  __shared__ __align__(16) double sh_prod[kPsThreads / 32][32][DG];
+  constexpr uint32_t kFull = 0xffffffffu;
+  constexpr int PER = 32 / DG;  // groups per instruction of the reductions
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane / DG, e = lane % DG;
+  const bool wide = (reinterpret_cast<uintptr_t>(g) & 31u) == 0;
+  const uint64_t stride = 32 * (uint64_t)gridDim.x * (kPsThreads / 32);
+  uint64_t j0 = 32 * ((uint64_t)blockIdx.x * (kPsThreads / 32) + warp);
+  float gv[DG];
+  uint32_t b[M];
+  auto fetch = [&](uint64_t at) {
+#pragma unroll
+    for (int i = 0; i < DG; ++i) gv[i] = 0.0f;
+#pragma unroll
+    for (int m = 0; m < M; ++m) b[m] = 0;
+    if (at + lane < G) {
+#pragma unroll
+      for (int part = 0; part < DG / 8; ++part) load8(g + (at + lane) * DG + 8 * part, wide, &gv[8 * part]);
+      group_codes<M, CODE_U16>(codes, at + lane, b);
+    }
+  };
+  fetch(j0);
+  for (; j0 < G; j0 += stride) {
+    const bool mine = j0 + lane < G;
+    const uint32_t row = mine ? fast_div((uint32_t)(j0 + lane), gpr) : kFull;
+    const double s = mine ? (double)__ldg(scale + row) : 0.0;
+    bool bad = false;
+#pragma unroll
+    for (int m = 0; m < M; ++m) bad |= b[m] >= K;
+    if (bad && status) atomicOr(status, PVT_DEV_BAD_CODE);
+    const bool ok = mine && !bad;  // a group with a bad code contributes nothing
+    double gd[DG];
+#pragma unroll
+    for (int i = 0; i < DG; ++i) gd[i] = (double)gv[i];
+    uint32_t code[M];
+#pragma unroll
+    for (int m = 0; m < M; ++m) code[m] = b[m];
     double ds = 0.0;
-    if (valid) {
-      const float4 gv = __ldcs(g4 + h);
-      row = j / gpr;
-      const float s = __ldg(scale + row);
-      uint32_t b[M];
-      if (CODE_U16) {
-        const uint16_t* c = reinterpret_cast<const uint16_t*>(codes) + (size_t)j * M;
+    if (grad_scale && ok) {
+      float v[DG];
+      group_codeword<M, CB_F16, DG>(reinterpret_cast<const uint4*>(codebooks), code, K, v);
+      ds = dot_exact<DG>(gd, v);
+    }
+    put_products<DG>(sh_prod[warp][lane], lane, s, gd);
+    __syncwarp();
+    fetch(j0 + stride);  // beside the reductions
+    const uint32_t use = __ballot_sync(kFull, ok);
 #pragma unroll
-        for (int m = 0; m < M; ++m) b[m] = __ldg(c + m);
-      } else if (M == 2) {
-        const uint16_t both = __ldg(reinterpret_cast<const uint16_t*>(codes) + j);
-        b[0] = both & 0xffu;
-        b[M - 1] = both >> 8;
-      } else {
-        const uint8_t* c = reinterpret_cast<const uint8_t*>(codes) + (size_t)j * M;
-#pragma unroll
-        for (int m = 0; m < M; ++m) b[m] = __ldg(c + m);
-      }
-      bool bad = false;
+    for (int u = 0; u < DG; ++u) {
+      const int src = PER * u + sub;
+      const double p = sh_prod[warp][src][e];
 #pragma unroll
       for (int m = 0; m < M; ++m) {
-        if (b[m] >= K) {
-          bad = true;
-          b[m] = 0;
-        }
-      }
-      if (bad) {
-        if (status) atomicOr(status, PVT_DEV_BAD_CODE);
-      } else {
-        // codebook gradients: s * g, exact in binary64
-        const double sd = (double)s;
-        const double p0 = sd * (double)gv.x, p1 = sd * (double)gv.y, p2 = sd * (double)gv.z, p3 = sd * (double)gv.w;
-#pragma unroll
-        for (int m = 0; m < M; ++m) {
-          const size_t at = ((size_t)m * K + b[m]) * (4 * PARTS) + half * 4;
-          if (SMEM_ACC) {
-            atomicAdd(&sh_acc[at], p0);
-            atomicAdd(&sh_acc[at + 1], p1);
-            atomicAdd(&sh_acc[at + 2], p2);
-            atomicAdd(&sh_acc[at + 3], p3);
-          } else {
-            red_add_f64(grad_books + at, p0);
-            red_add_f64(grad_books + at + 1, p1);
-            red_add_f64(grad_books + at + 2, p2);
-            red_add_f64(grad_books + at + 3, p3);
-          }
-        }
-        if (grad_scale) {
-          float4 v = half_codeword<CB_F16, PARTS>(codebooks, b[0], half);
-#pragma unroll
-          for (int m = 1; m < M; ++m) {
-            const float4 v2 = half_codeword<CB_F16, PARTS>(codebooks, m * K + b[m], half);
-            v.x = __fadd_rn(v.x, v2.x);
-            v.y = __fadd_rn(v.y, v2.y);
-            v.z = __fadd_rn(v.z, v2.z);
-            v.w = __fadd_rn(v.w, v2.w);
-          }
-          ds = (double)gv.x * (double)v.x;
-          ds = __dadd_rn(ds, (double)gv.y * (double)v.y);
-          ds = __dadd_rn(ds, (double)gv.z * (double)v.z);
-          ds = __dadd_rn(ds, (double)gv.w * (double)v.w);
-        }
+        const uint32_t c = __shfl_sync(kFull, code[m], src);
+        if ((use >> src) & 1u) red_add_f64(grad_books + ((size_t)m * K + c) * DG + e, p);
       }
     }
+    __syncwarp();
     if (grad_scale) {
-      // a warp that lies inside one row adds its 32 contributions with one reduction
-      const uint32_t row0 = __shfl_sync(0xffffffffu, row, 0);
-      if (__all_sync(0xffffffffu, row == row0)) {
+      // a warp that lies inside one row adds its contributions with one reduction
+      const uint32_t row0 = __shfl_sync(kFull, row, 0);
+      if (__all_sync(kFull, row == row0)) {
 #pragma unroll
-        for (int o = 16; o; o >>= 1) ds = __dadd_rn(ds, __shfl_xor_sync(0xffffffffu, ds, o));
-        if (lane == 0 && row0 != 0xffffffffu) red_add_f64(grad_scale + row0, ds);
-      } else if (row != 0xffffffffu) {
+        for (int o = 16; o; o >>= 1) ds = __dadd_rn(ds, __shfl_xor_sync(kFull, ds, o));
+        if (lane == 0) red_add_f64(grad_scale + row0, ds);
+      } else if (ok) {
         red_add_f64(grad_scale + row, ds);
       }
     }
   }
-  if (SMEM_ACC) {
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < (uint32_t)M * K * 8; i += kPsThreads)
-      if (sh_acc[i] != 0.0) red_add_f64(grad_books + i, sh_acc[i]);
-  }
 }
 
 
-// Small codebooks with one-byte codes (M K <= 512): no floating-point atomics in the block.  A block takes tiles
-// of 512 groups; per tile it stages the exact products s * g in shared memory, counting-sorts the tile's groups by
-// code (integer shared-memory atomics hand out the slots), and then every accumulator (codebook, code, element)
-// is owned by one thread, which adds the products of the code's groups in binary64 with plain
-// additions.  The accumulators go to the L2 once per block.
-constexpr int kPsTile = 512;
+// Small codebooks: the sums stay in shared memory.  A CTA takes tiles of 1024 groups.  Per tile it stages the exact
+// products s * g, sorts the tile's (codebook, code) pairs by counting (integer shared-memory atomics hand out the
+// slots) and lets the team of four lanes that owns a pair, two elements each, add up its products in registers.
+// The next tile's loads are in flight
+// meanwhile.  What bounds it are the wavefronts of shared memory (73 % busy): a quarter of them rows of products in
+// sorted order, the rest products, lists, counters, codewords.  11008 x 4096 with two codebooks of 256: 167 us; with
+// tiles of 512 groups and no loads ahead 283 us; four codebooks of 256 332 us, in the L2 1930 us.
+constexpr int kPsSmallThreads = 512;
+constexpr int kPsTile = 1024;
+constexpr int kPsTeams = kPsSmallThreads / 4;
 
 template <int M, bool CB_F16>
-__global__ void __launch_bounds__(kPsThreads) pstep_grad_sorted_kernel(const float* __restrict__ g,
-                                                                        const float* __restrict__ scale,
-                                                                        const uint8_t* __restrict__ codes,
-                                                                        const void* __restrict__ codebooks, uint64_t G,
-                                                                        uint32_t gpr, uint32_t K,
-                                                                        double* __restrict__ grad_books,
-                                                                        double* __restrict__ grad_scale,
-                                                                        uint32_t* status) {
-  extern __shared__ __align__(16) unsigned char ps_smem[];
-  double* sh_acc = reinterpret_cast<double*>(ps_smem);                       // [M*K*8]
-  double* sh_p = sh_acc + (size_t)M * K * 8;                                 // [tile][8]: the exact products s * g
-  uint32_t* sh_cnt = reinterpret_cast<uint32_t*>(sh_p + kPsTile * 8);        // [M][256] counts
-  uint32_t* sh_start = sh_cnt + M * 256;                                     // [M][256]
-  uint16_t* sh_sorted = reinterpret_cast<uint16_t*>(sh_start + M * 256);     // [M][tile]
-  uint16_t* sh_slot = sh_sorted + M * kPsTile;                               // [M][tile]: slot of group in its bin
-  uint8_t* sh_code = reinterpret_cast<uint8_t*>(sh_slot + M * kPsTile);      // [M][tile]
+constexpr size_t small_smem(uint32_t K) {
+  const uint32_t bins = (M * K + kPsSmallThreads - 1) / kPsSmallThreads * kPsSmallThreads;
+  return (sizeof(double) * 8 + (CB_F16 ? 16 : 32)) * M * (size_t)K + sizeof(double) * 8 * kPsTile + sizeof(uint32_t) * (bins + 32) + sizeof(uint16_t) * M * kPsTile;
+}
 
-  for (uint32_t i = threadIdx.x; i < (uint32_t)M * K * 8; i += kPsThreads) sh_acc[i] = 0.0;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const float4* g4 = reinterpret_cast<const float4*>(g);
+template <int M, bool CB_F16, bool CODE_U16>
+__global__ void __launch_bounds__(kPsSmallThreads, 2) pstep_grad_small_kernel(const float* __restrict__ g,
+                                                                              const float* __restrict__ scale,
+                                                                              const void* __restrict__ codes,
+                                                                              const void* __restrict__ codebooks,
+                                                                              uint64_t G, FastDiv gpr, uint32_t K,
+                                                                              double* __restrict__ grad_books,
+                                                                              double* __restrict__ grad_scale,
+                                                                              uint32_t* status) {
+  extern __shared__ __align__(16) unsigned char ps_smem[];
+  constexpr uint32_t kFull = 0xffffffffu;
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t n_bins = M * K, per = (n_bins + kPsSmallThreads - 1) / kPsSmallThreads;
+  double* acc = reinterpret_cast<double*>(ps_smem);              // [M K][8]
+  double* prod = acc + (size_t)n_bins * 8;                       // [tile][8]: the exact products s * g
+  uint4* book = reinterpret_cast<uint4*>(prod + kPsTile * 8);    // [M K]: the codebooks
+  uint32_t* bin = reinterpret_cast<uint32_t*>(book + (size_t)n_bins * (CB_F16 ? 1 : 2));  // [M K, padded]: counts, then starts
+  uint32_t* part = bin + per * kPsSmallThreads + 1;              // [31]
+  uint16_t* list = reinterpret_cast<uint16_t*>(part + 31);       // [M tile]: the groups by (codebook, code)
+  for (uint32_t i = tid; i < n_bins * 8; i += kPsSmallThreads) acc[i] = 0.0;
+  constexpr uint32_t kRowPieces = CB_F16 ? 1 : 2;
+  if (grad_scale) {
+    for (uint32_t i = tid; i < n_bins * kRowPieces; i += kPsSmallThreads)
+      book[i] = __ldg(reinterpret_cast<const uint4*>(codebooks) + i);
+  }
   const uint64_t n_tiles = (G + kPsTile - 1) / kPsTile;
+  const bool wide = (reinterpret_cast<uintptr_t>(g) & 31u) == 0;
+  constexpr uint32_t kIter = kPsTile / kPsSmallThreads, kRun = 32 * kIter;  // groups of a thread, of a warp
+  const uint32_t slot0 = warp * kRun + lane;
+  float gv[kIter][8];
+  uint32_t b[kIter][M];
+  auto fetch = [&](uint64_t tile) {  // all loads of a tile, before the first use and beside the walk of the tile before it
+#pragma unroll
+    for (uint32_t it = 0; it < kIter; ++it) {
+      const uint64_t j = tile * kPsTile + slot0 + 32 * it;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) gv[it][i] = 0.0f;
+#pragma unroll
+      for (int m = 0; m < M; ++m) b[it][m] = 0;
+      if (j < G) {
+        load8(g + j * 8, wide, gv[it]);
+        group_codes<M, CODE_U16>(codes, j, b[it]);
+      }
+    }
+  };
+  fetch(blockIdx.x);
   for (uint64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
     const uint64_t j0 = tile * kPsTile;
     const uint32_t n_here = (uint32_t)(G - j0 < (uint64_t)kPsTile ? G - j0 : (uint64_t)kPsTile);
-    __syncthreads();  // the previous tile has been consumed
-    for (uint32_t i = threadIdx.x; i < (uint32_t)M * 256; i += kPsThreads) sh_cnt[i] = 0;
-    __syncthreads();
-    // stage the tile: two threads per group (512 contiguous bytes per warp load); all loads of the tile are
-    // issued before the first use, the pass is bound by memory latency otherwise
-    constexpr int kIter = 2 * kPsTile / kPsThreads;  // 8 half-groups per thread
-    float4 gv_all[kIter];
-    uint32_t b_all[kIter][M];
+    for (uint32_t i = tid; i < per * kPsSmallThreads; i += kPsSmallThreads) bin[i] = 0;
+    __syncthreads();  // (the previous tile has been consumed, too)
+    // rows of the warp's first and last group: usually the same, and then one scale and one sum serve all iterations
+    const uint32_t w_lo = warp * kRun, w_hi = min(w_lo + kRun, n_here);
+    const uint32_t row_lo = w_lo < n_here ? fast_div((uint32_t)(j0 + w_lo), gpr) : 0u;
+    const uint32_t row_hi = w_lo < n_here ? fast_div((uint32_t)(j0 + w_hi - 1), gpr) : 0u;
+    const bool one_row = row_lo == row_hi;
+    const double s_row = (double)__ldg(scale + row_lo);
+    double ds = 0.0;
+    uint32_t rank[kIter][M];  // slot of the pair within its bin
 #pragma unroll
-    for (int it = 0; it < kIter; ++it) {
-      const uint32_t hh = it * kPsThreads + threadIdx.x, slot = hh >> 1, half = hh & 1u;
-      gv_all[it] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (uint32_t it = 0; it < kIter; ++it) {
+      const uint32_t slot = slot0 + 32 * it;
+      const bool valid = slot < n_here;
+      bool bad = false;
 #pragma unroll
-      for (int m = 0; m < M; ++m) b_all[it][m] = 0;
-      if (slot < n_here) {
-        const uint64_t j = j0 + slot;
-        gv_all[it] = __ldcs(g4 + 2 * j + half);
-#pragma unroll
-        for (int m = 0; m < M; ++m) b_all[it][m] = __ldg(codes + j * M + m);
+      for (int m = 0; m < M; ++m) {
+        if (b[it][m] >= K) {
+          bad = true;
+          b[it][m] = 0;
+        }
+        if (valid) rank[it][m] = atomicAdd(&bin[m * K + b[it][m]], 1u);
       }
-    }
+      if (bad && status) atomicOr(status, PVT_DEV_BAD_CODE);
+      const uint32_t row = one_row || !valid ? row_lo : fast_div((uint32_t)(j0 + slot), gpr);
+      const double sd = bad ? 0.0 : one_row ? s_row : (double)__ldg(scale + row);  // a bad code's group contributes nothing
+      double gd[8];
 #pragma unroll
-    for (int it = 0; it < kIter; ++it) {
-      const uint32_t hh = it * kPsThreads + threadIdx.x, slot = hh >> 1, half = hh & 1u;
-      const uint64_t j = j0 + slot;
-      uint32_t row = 0xffffffffu;
-      double ds = 0.0;
-      if (slot < n_here) {
-        const float4 gv = gv_all[it];
-        row = (uint32_t)j / gpr;
-        uint32_t b[M];
-        bool bad = false;
-#pragma unroll
-        for (int m = 0; m < M; ++m) {
-          b[m] = b_all[it][m];
-          if (b[m] >= K) {
-            bad = true;
-            b[m] = 0;
-          }
-        }
-        {
-          const double sd = bad ? 0.0 : (double)__ldg(scale + row);  // a group with a bad code contributes nothing
-          double* dst = &sh_p[slot * 8 + half * 4];
-          dst[0] = sd * (double)gv.x;
-          dst[1] = sd * (double)gv.y;
-          dst[2] = sd * (double)gv.z;
-          dst[3] = sd * (double)gv.w;
-        }
-        if (half == 0) {
-#pragma unroll
-          for (int m = 0; m < M; ++m) {
-            sh_code[m * kPsTile + slot] = (uint8_t)b[m];
-            sh_slot[m * kPsTile + slot] = (uint16_t)atomicAdd(&sh_cnt[m * 256 + b[m]], 1u);
-          }
-        }
-        if (bad) {
-          if (status) atomicOr(status, PVT_DEV_BAD_CODE);
-        } else if (grad_scale) {
-          float4 v = half_codeword<CB_F16>(codebooks, b[0], half);
-#pragma unroll
-          for (int m = 1; m < M; ++m) {
-            const float4 v2 = half_codeword<CB_F16>(codebooks, m * K + b[m], half);
-            v.x = __fadd_rn(v.x, v2.x);
-            v.y = __fadd_rn(v.y, v2.y);
-            v.z = __fadd_rn(v.z, v2.z);
-            v.w = __fadd_rn(v.w, v2.w);
-          }
-          ds = (double)gv.x * (double)v.x;
-          ds = __dadd_rn(ds, (double)gv.y * (double)v.y);
-          ds = __dadd_rn(ds, (double)gv.z * (double)v.z);
-          ds = __dadd_rn(ds, (double)gv.w * (double)v.w);
-        }
-      }
+      for (int i = 0; i < 8; ++i) gd[i] = (double)gv[it][i];
+      put_products<8>(&prod[slot * 8], lane, sd, gd);
       if (grad_scale) {
-        const uint32_t row0 = __shfl_sync(0xffffffffu, row, 0);
-        if (__all_sync(0xffffffffu, row == row0)) {
-#pragma unroll
-          for (int o = 16; o; o >>= 1) ds = __dadd_rn(ds, __shfl_xor_sync(0xffffffffu, ds, o));
-          if (lane == 0 && row0 != 0xffffffffu) red_add_f64(grad_scale + row0, ds);
-        } else if (row != 0xffffffffu) {
-          red_add_f64(grad_scale + row, ds);
+        double d = 0.0;
+        if (valid && !bad) {
+          float v[8];
+          group_codeword<M, CB_F16, 8>(book, b[it], K, v);
+          d = dot_exact<8>(gd, v);
         }
+        if (one_row)
+          ds = __dadd_rn(ds, d);
+        else if (valid)
+          red_add_f64(grad_scale + row, d);
       }
     }
-    __syncthreads();
-    // exclusive prefix of the counts per codebook: one warp per codebook, eight bins per lane
-    if (warp < M) {
-      uint32_t c[8], sum = 0;
+    if (grad_scale && one_row) {
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        c[q] = sh_cnt[warp * 256 + lane * 8 + q];
-        sum += c[q];
-      }
+      for (int o = 16; o; o >>= 1) ds = __dadd_rn(ds, __shfl_xor_sync(kFull, ds, o));
+      if (lane == 0 && w_lo < n_here) red_add_f64(grad_scale + row_lo, ds);
+    }
+    __syncthreads();
+    // starts of the bins: every thread owns `per` adjacent ones
+    {
+      uint32_t sum = 0;
+      for (uint32_t i = 0; i < per; ++i) sum += bin[tid * per + i];
       uint32_t incl = sum;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t up = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += up;
+        const uint32_t up = __shfl_up_sync(kFull, incl, o);
+        if (lane >= (uint32_t)o) incl += up;
       }
-      uint32_t run = incl - sum;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        sh_start[warp * 256 + lane * 8 + q] = run;
-        run += c[q];
+      if (lane == 31) part[warp] = incl;
+      __syncthreads();
+      const uint32_t before = __reduce_add_sync(kFull, lane < warp ? part[lane] : 0u);
+      uint32_t run = before + incl - sum;
+      for (uint32_t i = 0; i < per; ++i) {
+        const uint32_t c = bin[tid * per + i];
+        bin[tid * per + i] = run;
+        run += c;
       }
+      if (tid == kPsSmallThreads - 1) bin[tid * per + per] = run;
     }
     __syncthreads();
 #pragma unroll
-    for (int m = 0; m < M; ++m)
-      for (uint32_t slot = threadIdx.x; slot < n_here; slot += kPsThreads) {
-        const uint32_t code = sh_code[m * kPsTile + slot];
-        sh_sorted[m * kPsTile + sh_start[m * 256 + code] + sh_slot[m * kPsTile + slot]] = (uint16_t)slot;
-      }
-    __syncthreads();
-    // every accumulator (codebook, code, element) is owned by one thread: plain binary64 additions over the
-    // code's groups; eight adjacent threads share a code, so its group list is a broadcast load
+    for (uint32_t it = 0; it < kIter; ++it) {
+      const uint32_t slot = slot0 + 32 * it;
+      if (slot < n_here) {
 #pragma unroll
-    for (int m = 0; m < M; ++m)
-      for (uint32_t bin = threadIdx.x; bin < K * 8; bin += kPsThreads) {
-        const uint32_t code = bin >> 3, e = bin & 7u;
-        const uint32_t cnt = sh_cnt[m * 256 + code];
-        if (cnt == 0) continue;
-        const uint16_t* list = &sh_sorted[m * kPsTile + sh_start[m * 256 + code]];
-        double acc = 0.0;
-        for (uint32_t i = 0; i < cnt; ++i) acc = __dadd_rn(acc, sh_p[(uint32_t)list[i] * 8 + e]);
-        sh_acc[((size_t)m * K + code) * 8 + e] += acc;
+        for (int m = 0; m < M; ++m) list[bin[m * K + b[it][m]] + rank[it][m]] = (uint16_t)slot;
       }
+    }
+    __syncthreads();
+    fetch(tile + gridDim.x);
+    // a team of four lanes, two elements each, owns every (codebook, code) pair
+    {
+      const double2* rows = reinterpret_cast<const double2*>(prod) + (tid & 3u);
+      for (uint32_t c = tid >> 2; c < n_bins; c += kPsTeams) {
+        uint32_t i = bin[c];
+        const uint32_t end = bin[c + 1];
+        if (i == end) continue;
+        double2* at = reinterpret_cast<double2*>(acc) + 4 * c + (tid & 3u);
+        double2 sum = *at;
+        do {
+          const double2 x = rows[4 * (uint32_t)list[i]];
+          sum.x = __dadd_rn(sum.x, x.x);
+          sum.y = __dadd_rn(sum.y, x.y);
+        } while (++i < end);
+        *at = sum;
+      }
+    }
+    __syncthreads();
   }
   __syncthreads();
-  for (uint32_t i = threadIdx.x; i < (uint32_t)M * K * 8; i += kPsThreads)
-    if (sh_acc[i] != 0.0) red_add_f64(grad_books + i, sh_acc[i]);
+  for (uint32_t i = tid; i < n_bins * 8; i += kPsSmallThreads)
+    if (acc[i] != 0.0) red_add_f64(grad_books + i, acc[i]);
 }
 
-template <int M, bool CB_F16>
-cudaError_t launch_grad_sorted(const pvt_layer& L, uint64_t G, double* grad_books, double* grad_scale, uint32_t* status,
-                               int sm_count, cudaStream_t stream) {
-  const uint32_t gpr = (uint32_t)(L.cols / kGroupDim), K = (uint32_t)L.codebook_size;
-  const size_t smem = sizeof(double) * M * K * 8 + sizeof(double) * kPsTile * 8 + sizeof(uint32_t) * M * 512 +
-                      sizeof(uint16_t) * M * kPsTile * 2 + (size_t)M * kPsTile;
-  cudaError_t e = cudaFuncSetAttribute(pstep_grad_sorted_kernel<M, CB_F16>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <int M, bool CB_F16, bool CODE_U16>
+cudaError_t launch_grad_small(const pvt_layer& L, uint64_t G, double* grad_books, double* grad_scale, uint32_t* status,
+                              int sm_count, cudaStream_t stream) {
+  const uint32_t K = (uint32_t)L.codebook_size;
+  const size_t smem = small_smem<M, CB_F16>(K);
+  const cudaError_t e = allow_smem(pstep_grad_small_kernel<M, CB_F16, CODE_U16>);
   if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pstep_grad_sorted_kernel<M, CB_F16>, kPsThreads, smem);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) per_sm = 1;
-  const uint64_t tiles = (G + kPsTile - 1) / kPsTile, cap = (uint64_t)sm_count * per_sm;
-  pstep_grad_sorted_kernel<M, CB_F16><<<(unsigned)(tiles < cap ? tiles : cap), kPsThreads, smem, stream>>>(
-      L.g, L.scale, static_cast<const uint8_t*>(L.codes), L.codebooks, G, gpr, K, grad_books, grad_scale, status);
+  const uint64_t tiles = (G + kPsTile - 1) / kPsTile, cap = (uint64_t)sm_count * (smem <= 112 * 1024 ? 2 : 1);
+  pstep_grad_small_kernel<M, CB_F16, CODE_U16><<<(unsigned)(tiles < cap ? tiles : cap), kPsSmallThreads, smem, stream>>>(
+      L.g, L.scale, L.codes, L.codebooks, G, make_fast_div((uint32_t)(L.cols / kGroupDim)), K, grad_books, grad_scale,
+      status);
+  return cudaGetLastError();
+}
+
+template <int M, bool CB_F16, bool CODE_U16, int DG>
+cudaError_t launch_grad_large(const pvt_layer& L, uint64_t G, double* grad_books, double* grad_scale, uint32_t* status,
+                              int sm_count, cudaStream_t stream) {
+  const uint64_t want = (G + kPsThreads - 1) / kPsThreads, cap = (uint64_t)sm_count * 8;
+  pstep_grad_kernel<M, CB_F16, CODE_U16, DG><<<(unsigned)(want < cap ? want : cap), kPsThreads, 0, stream>>>(
+      L.g, L.scale, L.codes, L.codebooks, G, make_fast_div((uint32_t)(L.cols / DG)), (uint32_t)L.codebook_size, grad_books,
+      grad_scale, status);
   return cudaGetLastError();
 }
 
 template <int M, bool CB_F16, bool CODE_U16>
 cudaError_t launch_grad(const pvt_layer& L, uint64_t G, double* grad_books, double* grad_scale, uint32_t* status,
                         int sm_count, cudaStream_t stream) {
-  const uint32_t gpr = (uint32_t)(L.cols / kGroupDim), K = (uint32_t)L.codebook_size;
-  if (L.group_dim == 16) {  // groups of 16 weights (one codebook): four threads per group, reductions in the L2
-    const uint64_t want16 = (4 * G + kPsThreads - 1) / kPsThreads, cap16 = (uint64_t)sm_count * 8;
-    pstep_grad_kernel<M, CB_F16, CODE_U16, false, 4><<<(unsigned)(want16 < cap16 ? want16 : cap16), kPsThreads, 0, stream>>>(
-        L.g, L.scale, L.codes, L.codebooks, G, (uint32_t)(L.cols / 16), K, grad_books, grad_scale, status);
-    return cudaGetLastError();
+  if (L.group_dim == 16) {  // groups of 16 weights: one codebook
+    if constexpr (M == 1)
+      return launch_grad_large<1, CB_F16, CODE_U16, 16>(L, G, grad_books, grad_scale, status, sm_count, stream);
   }
-  const bool smem_acc = (uint32_t)M * K <= (uint32_t)kPsSmemCodewords;
-  if (smem_acc && !CODE_U16) return launch_grad_sorted<M, CB_F16>(L, G, grad_books, grad_scale, status, sm_count, stream);
-  const uint64_t want = (2 * G + kPsThreads - 1) / kPsThreads;
-  const uint64_t cap = (uint64_t)sm_count * (smem_acc ? 4 : 8);
-  const unsigned blocks = (unsigned)(want < cap ? want : cap);
-  if (smem_acc)
-    pstep_grad_kernel<M, CB_F16, CODE_U16, true><<<blocks, kPsThreads, 0, stream>>>(
-        L.g, L.scale, L.codes, L.codebooks, G, gpr, K, grad_books, grad_scale, status);
-  else
-    pstep_grad_kernel<M, CB_F16, CODE_U16, false><<<blocks, kPsThreads, 0, stream>>>(
-        L.g, L.scale, L.codes, L.codebooks, G, gpr, K, grad_books, grad_scale, status);
-  return cudaGetLastError();
+  if ((uint32_t)M * (uint32_t)L.codebook_size <= (uint32_t)kPsSmallBins &&
+      small_smem<M, CB_F16>((uint32_t)L.codebook_size) <= kPsMaxSmem)
+    return launch_grad_small<M, CB_F16, CODE_U16>(L, G, grad_books, grad_scale, status, sm_count, stream);
+  return launch_grad_large<M, CB_F16, CODE_U16, 8>(L, G, grad_books, grad_scale, status, sm_count, stream);
 }
 
 // One Adam update, binary32, each operation rounded once, in the order stated in pvt.h.
