@@ -382,7 +382,7 @@ def search_roofline(engine, pairs_per_step, enc_ms, enc_n, steps, peaks, traffic
              "epilogue_bound_is": "one accumulator read per pair: 128 lanes per SM per clock at the maximum SM clock"}
     else:
         r = {"kernel": "encode_m1_kernel (exhaustive search, FP32 pipe)" if engine == "fp32"
-             else "encode_m2_kernel (beam search)", "bound": "alu", "peak": peaks["alu_tflops"],
+             else "encode_beam_kernel (beam search)", "bound": "alu", "peak": peaks["alu_tflops"],
              "frac": achieved / peaks["alu_tflops"],
              "peak_is": f"{peaks['sm_count']} SMs x 128 FP32 lanes x 2 flop x {peaks['sm_max_mhz_used']:.0f} MHz "
                         f"(derived; no measured FP32 peak)"}

@@ -150,10 +150,9 @@ namespace {
 
 // workspace of pvt_vstep_encode for k groups of this layer
 size_t encode_bytes(const pvt_layer& L, uint64_t k, int sms) {
-  if (L.num_codebooks >= 3) return encode_m2_workspace_bytes();  // header + the codebooks' image
+  if (L.num_codebooks >= 2) return encode_beam_workspace_bytes();  // header + the codebooks' image
   if (L.group_dim == 16)
     return encode_m1_use_tc(L, k) ? encode_m1_tc_layout((uint32_t)L.codebook_size, k, sms, 16).bytes : kWsHeaderBytes;
-  if (L.num_codebooks != 1) return encode_m2_workspace_bytes();
   return encode_m1_use_tc(L, k)
              ? encode_m1_tc_layout((uint32_t)L.codebook_size, k, sms).bytes
              : encode_m1_layout((uint32_t)L.codebook_size, k, sms, encode_m1_targets_per_thread(k, sms)).bytes;
@@ -258,15 +257,11 @@ int pvt_vstep_encode(const pvt_layer* layer, const uint32_t* idx, uint64_t k, fl
         encode_m1_layout((uint32_t)layer->codebook_size, k, sms, encode_m1_targets_per_thread(k, sms));
     if (ws_bytes < lay.bytes) return PVT_EWORKSPACE;
     e = launch_encode_m1(*layer, G, idx, k, err_out, ws, sms, static_cast<cudaStream_t>(cuda_stream));
-  } else if (layer->num_codebooks == 2) {
+  } else {
     if (layer->code_dtype != PVT_U8) return PVT_EUNSUPPORTED;
     if (layer->beam < 1 || layer->beam > 8) return PVT_EUNSUPPORTED;
-    if (ws_bytes < encode_m2_workspace_bytes()) return PVT_EWORKSPACE;
-    e = launch_encode_m2(*layer, G, idx, k, err_out, ws, sms, static_cast<cudaStream_t>(cuda_stream));
-  } else {
-    if (layer->beam < 1 || layer->beam > 8) return PVT_EUNSUPPORTED;
-    if (ws_bytes < encode_m2_workspace_bytes()) return PVT_EWORKSPACE;
-    e = launch_encode_mx(*layer, G, idx, k, err_out, ws, static_cast<cudaStream_t>(cuda_stream));
+    if (ws_bytes < encode_beam_workspace_bytes()) return PVT_EWORKSPACE;
+    e = launch_encode_beam(*layer, G, idx, k, err_out, ws, sms, static_cast<cudaStream_t>(cuda_stream));
   }
   return e == cudaSuccess ? PVT_OK : fail_cuda(e);
 }

@@ -1,0 +1,923 @@
+// Beam search of the V step for two to four additive codebooks (Appendix C: the code combination is found by beam
+// search; Appendix J: 8-bit codebooks, group size 8, beam size 8, target = gradient-updated dequantised weight; Eq. 8
+// for the target; Lemma 3.3 for keeping the previous tuple in the pool).
+//
+//   stage m (m = 1..M): each kept partial tuple (one empty tuple before stage 1) is extended by every codeword of
+//     codebook m; the score of an extension is ||t - c^1 - ... - c^m||^2;
+//   after stages 1..M-1 the `beam` smallest extensions under (score, tuple) are kept;
+//   the result is the smallest member of the last stage's extensions and the previous tuple.
+//
+// A warp handles four targets at a time; the codebooks live in shared memory; three CTAs (24 warps) share an SM.
+//   stage 1 (per target, the whole warp): lane l owns codewords l, l+32, ..., l+224 of codebook 1:
+//            score1 = ||c1||^2/2 - <t, c1> for 256 codewords (8 per lane, packed f32x2); the `beam` smallest are
+//            extracted with warp-wide integer minimum reductions on (score bits | code) keys.
+//   further stages (four targets x eight kept tuples = 32 residuals, one per lane): fast scores
+//            ||r||^2/2 + ||c||^2/2 - <r, c> of all residuals against all codewords, on the tensor pipe for fp16
+//            codebooks (mma.sync, the residuals as rows), on the FP32 pipe otherwise; only the minimum of each
+//            (residual, 32 codewords) cell is kept: 64 cells per target.
+//   a stage in the middle: the `beam`-th smallest of a target's 64 cell minima bounds its `beam`-th smallest score, so
+//            only cells within the rounding margin of it -- usually `beam` of them -- are scored again, a codeword per
+//            lane; what is within the margin goes on a short list, of which the `beam` smallest are kept.
+//   last stage: cells within the margin of the smallest are revisited, and what is within the margin gets its
+//            binary64 distance.
+// Fast scores are binary32.  Every decision they cannot settle within twice their rounding-error bound (membership of
+// the beam, the final argmin) is taken on binary64 distances accumulated in index order (the residual carried through
+// the codebooks in order), so the result is the argmin of (distance, tuple) over the pool exactly as defined.
+// What bounds it is instruction issue (about 800 warp instructions per target with two codebooks).  56 360
+// targets of an 11008 x 4096 layer, two / three / four fp16 codebooks of 256: 72 / 151 / 257 us; three binary32
+// codebooks 221 us.  (A warp per target, with two passes over all extensions in every stage and every decision in
+// binary64: 415 / 522 us for three / four, 992 us for three binary32 codebooks.)
+#include <cuda_fp16.h>
+
+#include "pvt_internal.h"
+
+namespace pvt {
+
+// header + the image of the codebooks (at most four binary32 codebooks: under 76 KiB)
+size_t encode_beam_workspace_bytes() { return kWsHeaderBytes + 77824; }
+
+namespace {
+
+constexpr int kBsThreads = 256;
+constexpr int kBsWarps = kBsThreads / 32;
+constexpr int kBsCtasPerSm = 3;  // resident CTAs per SM the kernel is compiled for (registers) and launched as
+constexpr int kBsK = 256;        // codebooks are padded to this many codewords
+constexpr int kBsGroup = 4;      // targets per warp iteration: 4 targets x 8 kept tuples = 32 lanes
+constexpr int kBsList = 32;      // extensions per target that a middle stage's list holds
+constexpr float kPadHalfNorm = 3.0e38f;
+constexpr float kInf = __builtin_huge_valf();
+constexpr long long kInfBits = 0x7ff0000000000000ll;
+
+struct BeamParams {
+  const float* W;
+  const float* g;
+  const float* scale;
+  const uint32_t* idx;
+  uint64_t k, G;
+  FastDiv gpr;
+  float eta;
+  const void* books;
+  uint32_t K, beam;
+  uint8_t* codes;  // M adjacent bytes per group
+  float* err_out;
+  uint32_t* status;
+};
+
+// Everything the kernel derives from the codebooks, in the byte order it has in shared memory.  One small kernel writes
+// it once per call into the workspace; every CTA of the search fetches it with a single bulk copy (cp.async.bulk,
+// completion on an mbarrier; no multicast).
+template <bool TC>
+struct StageImage;
+template <>
+struct StageImage<true> {  // tensor pipe: B fragments, word [n-tile][lane] = halves (c[8 nt + lane/4][2 (lane%4)], [.. + 1])
+  uint32_t b[kBsK / 8][32];
+  alignas(8) float h[kBsK];  // ||c||^2/2
+};
+template <>
+struct StageImage<false> {  // FP32 pipe
+  alignas(16) float x[kBsK / 2][16];  // pair p holds (c[2p][0], c[2p+1][0], c[2p][1], ...)
+  alignas(8) float h[kBsK];           // ||c||^2/2 (in pairs, too)
+};
+template <int M, bool TC>
+struct BeamImage {
+  alignas(16) float c[M][kBsK][8];
+  alignas(16) uint64_t p1[4][8][32];  // stage-1 operands: (c1[l+64q][i], c1[l+64q+32][i])
+  uint64_t h1[4][32];                 // (||c1||^2/2) pairs in the same order
+  StageImage<TC> st[M - 1];
+  float smax[4];                      // largest norm per codebook
+};
+
+struct BeamScratch {  // per warp
+  alignas(16) float r[32][8];                  // residuals, one per lane
+  union {
+    alignas(16) float wmin[32][8];             // cell minima on their way to the lanes that own the residuals
+    alignas(8) uint2 list[kBsGroup][kBsList];  // a middle stage's extensions within the margin: score bits, tuple
+  };
+  alignas(16) float t[kBsGroup][8];            // the targets of the group
+  alignas(16) uint32_t kept[kBsGroup][8];      // their kept tuples: code of codebook q in bits [31 - 8 q : 24 - 8 q]
+};
+template <int M, bool TC>
+struct BeamSmem {
+  BeamImage<M, TC> img;
+  BeamScratch w[kBsWarps];
+  alignas(8) uint64_t img_bar;  // completion of the image copy
+};
+
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float d;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+// D = A (16 x 16, rows = residuals) x B (16 x 8, columns = codewords) + C, fp16 operands, fp32 accumulation
+__device__ __forceinline__ void mma_16x8x16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1, float c0,
+                                            float c1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+      "{%10, %11, %10, %11};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(c0), "f"(c1));
+}
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  return (uint64_t)__float_as_uint(lo) | ((uint64_t)__float_as_uint(hi) << 32);
+}
+__device__ __forceinline__ float lo_of(uint64_t v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float hi_of(uint64_t v) { return __uint_as_float((uint32_t)(v >> 32)); }
+// order-preserving map binary32 -> u32
+__device__ __forceinline__ uint32_t ord(float f) {
+  const uint32_t b = __float_as_uint(f);
+  return b ^ ((b >> 31) ? 0xffffffffu : 0x80000000u);
+}
+__device__ __forceinline__ float unord(uint32_t o) {
+  return __uint_as_float(o ^ ((o >> 31) ? 0x80000000u : 0xffffffffu));
+}
+
+// ||t - c_1 - ... - c_n||^2 in binary64: the residual through the codebooks in order, the terms in element order;
+// code q of the tuple sits in bits [31 - 8 q : 24 - 8 q]
+template <int N>
+__device__ __forceinline__ double exact_tuple(const float* t, const float (*books)[kBsK][8], uint32_t key) {
+  double d = 0.0;
+#pragma unroll
+  for (int half = 0; half < 2; ++half) {
+    const float4 tt = *reinterpret_cast<const float4*>(t + 4 * half);
+    double e0 = (double)tt.x, e1 = (double)tt.y, e2 = (double)tt.z, e3 = (double)tt.w;
+#pragma unroll
+    for (int m = 0; m < N; ++m) {
+      const float4 c = *reinterpret_cast<const float4*>(&books[m][(key >> (24 - 8 * m)) & 0xffu][4 * half]);
+      e0 = __dsub_rn(e0, (double)c.x);
+      e1 = __dsub_rn(e1, (double)c.y);
+      e2 = __dsub_rn(e2, (double)c.z);
+      e3 = __dsub_rn(e3, (double)c.w);
+    }
+    d = __dadd_rn(d, __dmul_rn(e0, e0));
+    d = __dadd_rn(d, __dmul_rn(e1, e1));
+    d = __dadd_rn(d, __dmul_rn(e2, e2));
+    d = __dadd_rn(d, __dmul_rn(e3, e3));
+  }
+  return d;
+}
+// the same for the first n codes of a tuple (rarely needed: not inlined)
+__device__ __noinline__ double exact_partial(const float* t, const float (*books)[kBsK][8], uint32_t key, int n) {
+  double d = 0.0;
+#pragma unroll 1
+  for (int i = 0; i < 8; ++i) {
+    double e = (double)t[i];
+#pragma unroll 1
+    for (int m = 0; m < n; ++m) e = __dsub_rn(e, (double)books[m][(key >> (24 - 8 * m)) & 0xffu][i]);
+    d = __dadd_rn(d, __dmul_rn(e, e));
+  }
+  return d;
+}
+// ||t - c||^2 in binary64, the operations of the definition in index order
+__device__ __forceinline__ double exact1(const float* t, const float* c) {
+  double d = 0.0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const double e = __dsub_rn((double)t[i], (double)c[i]);
+    d = __dadd_rn(d, __dmul_rn(e, e));
+  }
+  return d;
+}
+
+template <bool CB_F16>
+__device__ __forceinline__ float load_cb(const void* books, uint32_t m, uint32_t kappa, uint32_t K, int i) {
+  const size_t off = ((size_t)m * K + kappa) * 8 + i;
+  return CB_F16 ? __half2float(reinterpret_cast<const __half*>(books)[off]) : reinterpret_cast<const float*>(books)[off];
+}
+
+// ---- PTX helpers of the image copy ----------------------------------------------------------------------------
+constexpr uint32_t kBsMaxSpins = 1u << 22;  // polls after which the wait for the image gives up
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ bool mbar_try_wait0(uint32_t bar) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar)
+      : "memory");
+  return ok != 0;
+}
+// One bulk copy global -> shared of the whole image (16-byte aligned on both sides, a multiple of 16 bytes),
+// issued by one thread; every thread then waits, a bounded number of polls, for its completion.  Returns false
+// (after recording PVT_DEV_WAIT_EXPIRED) if the copy has not landed by then: the CTA must leave without reading it.
+__device__ __forceinline__ bool fetch_image(void* dst, const void* src, uint32_t bytes, uint64_t* bar, uint32_t* status) {
+  const uint32_t b = smem_addr(bar);
+  if (threadIdx.x == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b));
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_addr(dst)),
+                 "l"(src), "r"(bytes), "r"(b)
+                 : "memory");
+  }
+  __syncthreads();  // the barrier is initialised before anybody polls it
+  bool ok = false;
+  for (uint32_t spin = 0; spin < kBsMaxSpins && !ok; ++spin) {
+    ok = mbar_try_wait0(b);
+    if (!ok && spin > 4096) __nanosleep(64);
+  }
+  if (!ok) atomicOr(status, PVT_DEV_WAIT_EXPIRED);
+  // everybody agrees (a thread that gave up makes the whole CTA leave)
+  return __syncthreads_and(ok) != 0;
+}
+
+// ---- the codebook image: one block, one codeword of every codebook per thread (K <= 256 = block size) ----
+template <int M, bool TC>
+__global__ void __launch_bounds__(kBsThreads) beam_image_kernel(const BeamParams p, BeamImage<M, TC>* __restrict__ img) {
+  __shared__ float red[kBsWarps][4];
+  pdl_trigger();
+  BeamImage<M, TC>& sm = *img;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool real = (uint32_t)tid < p.K;
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+    float c[8], n2 = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      c[i] = real ? load_cb<TC>(p.books, m, tid, p.K, i) : 0.0f;
+      n2 = __fmaf_rn(c[i], c[i], n2);
+      sm.c[m][tid][i] = c[i];
+    }
+    const float h = real ? 0.5f * n2 : kPadHalfNorm;
+    if (m == 0) {
+      // codeword tid = l + 32*jj, jj = 2q + half
+      const int jj = tid >> 5, q = jj >> 1, half = jj & 1;
+      float* p1f = reinterpret_cast<float*>(&sm.p1[0][0][0]);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) p1f[(((q * 8 + i) * 32) + lane) * 2 + half] = c[i];
+      reinterpret_cast<float*>(&sm.h1[0][0])[(q * 32 + lane) * 2 + half] = h;
+    } else {
+      StageImage<TC>& st = sm.st[m - 1];
+      if constexpr (TC) {
+#pragma unroll
+        for (int qq = 0; qq < 4; ++qq) {
+          const __half2 v = __floats2half2_rn(c[2 * qq], c[2 * qq + 1]);  // exact: the codebook is fp16
+          st.b[tid >> 3][4 * (tid & 7) + qq] = *reinterpret_cast<const uint32_t*>(&v);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) st.x[tid >> 1][2 * i + (tid & 1)] = c[i];
+      }
+      st.h[tid] = h;
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) n2 = fmaxf(n2, __shfl_xor_sync(0xffffffffu, n2, o));
+    if (lane == 0) red[warp][m] = n2;
+  }
+  __syncthreads();
+  if (tid < 4) {
+    float a = 0.0f;
+    if (tid < M)
+      for (int w = 0; w < kBsWarps; ++w) a = fmaxf(a, red[w][tid]);
+    sm.smax[tid] = sqrtf(a);
+  }
+}
+
+// compare-exchange network of eight keys (19 exchanges), of four (5)
+#define PVT_CE(a, b)                          \
+  {                                           \
+    const uint32_t lo_ = min(key[a], key[b]); \
+    key[b] = max(key[a], key[b]);             \
+    key[a] = lo_;                             \
+  }
+__device__ __forceinline__ void sort8(uint32_t (&key)[8]) {
+  PVT_CE(0, 2) PVT_CE(1, 3) PVT_CE(4, 6) PVT_CE(5, 7)
+  PVT_CE(0, 4) PVT_CE(1, 5) PVT_CE(2, 6) PVT_CE(3, 7)
+  PVT_CE(0, 1) PVT_CE(2, 3) PVT_CE(4, 5) PVT_CE(6, 7)
+  PVT_CE(2, 4) PVT_CE(3, 5)
+  PVT_CE(1, 4) PVT_CE(3, 6)
+  PVT_CE(1, 2) PVT_CE(3, 4) PVT_CE(5, 6)
+}
+__device__ __forceinline__ void sort4(uint32_t (&key)[4]) {
+  PVT_CE(0, 1) PVT_CE(2, 3) PVT_CE(0, 2) PVT_CE(1, 3) PVT_CE(1, 2)
+}
+#undef PVT_CE
+// minimum over the eight lanes of a target
+__device__ __forceinline__ uint32_t team_min(uint32_t v) {
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+// drops the head of the sorted list if it is `head` (keys are distinct where they matter)
+template <int N>
+__device__ __forceinline__ void pop_if(uint32_t (&key)[N], uint32_t head) {
+  const bool own = key[0] == head;
+#pragma unroll
+  for (int i = 0; i < N - 1; ++i) key[i] = own ? key[i + 1] : key[i];
+  key[N - 1] = own ? 0xffffffffu : key[N - 1];
+}
+// lexicographic minimum of (distance, tuple) over the eight lanes of a target
+__device__ __forceinline__ void team_min_exact(double& d, uint32_t& key) {
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) {
+    const double od = __shfl_xor_sync(0xffffffffu, d, o);
+    const uint32_t ok = __shfl_xor_sync(0xffffffffu, key, o);
+    if (od < d || (od == d && ok < key)) {
+      d = od;
+      key = ok;
+    }
+  }
+}
+
+// One further stage's fast scores for the lane's residual (target my_q, kept tuple my_b; rho = ||r||^2/2): the minimum
+// of every 32 codewords.  The residuals of all lanes are in w.r.  Returns what the tensor path adds to the margin.
+template <bool TC>
+__device__ __forceinline__ float stage_minima(const StageImage<TC>& st, BeamScratch& w, const float (&r)[8], float rho,
+                                              bool active, float smax, float (&sub_min)[8]) {
+  const uint32_t lane = threadIdx.x & 31;
+  if constexpr (TC) {
+    // The 32 residuals are the rows of two 16-row A tiles, each row [ -hi(2^e r) | -lo(2^e r) ] in fp16 (hi + lo keeps 22
+    // significant bits of r, or all bits above 2^-25 in scaled units); the columns of B are the codewords, [ c | c ]; C
+    // starts at 2^e ||c||^2/2.  e is common to the group: the largest residual element becomes [1/2, 1).  A thread
+    // holds elements 2 qd, 2 qd + 1 of rows g8, g8 + 8 of each tile.
+    const uint32_t g8 = lane >> 2, qd = lane & 3u;
+    float2 nr[4];
+    float rmax = 0.0f;
+#pragma unroll
+    for (int r4 = 0; r4 < 4; ++r4) {
+      nr[r4] = *reinterpret_cast<const float2*>(&w.r[16 * (r4 >> 1) + 8 * (r4 & 1) + g8][2 * qd]);
+      rmax = fmaxf(rmax, fmaxf(fabsf(nr[r4].x), fabsf(nr[r4].y)));
+    }
+    const uint32_t rbits = __reduce_max_sync(0xffffffffu, __float_as_uint(rmax));  // non-negative floats order as u32
+    int e = 126 - (int)((rbits >> 23) & 0xffu);
+    e = e > 15 ? 15 : (e < -100 ? -100 : e);
+    const float sc = __uint_as_float((uint32_t)(e + 127) << 23), inv = __uint_as_float((uint32_t)(127 - e) << 23);
+    uint32_t a[2][4];
+#pragma unroll
+    for (int r4 = 0; r4 < 4; ++r4) {
+      const float x = nr[r4].x * -sc, y = nr[r4].y * -sc;
+      const __half2 hi = __floats2half2_rn(x, y);
+      const float2 back = __half22float2(hi);
+      const __half2 lo = __floats2half2_rn(x - back.x, y - back.y);
+      a[r4 >> 1][r4 & 1] = *reinterpret_cast<const uint32_t*>(&hi);
+      a[r4 >> 1][2 + (r4 & 1)] = *reinterpret_cast<const uint32_t*>(&lo);
+    }
+#pragma unroll 2
+    for (int sub = 0; sub < 8; ++sub) {
+      float m[4] = {kInf, kInf, kInf, kInf};
+#pragma unroll
+      for (int n4 = 0; n4 < 4; ++n4) {
+        const int nt = 4 * sub + n4;
+        const uint32_t b = st.b[nt][lane];
+        const float2 hh = *reinterpret_cast<const float2*>(&st.h[8 * nt + 2 * qd]);
+        const float hx = hh.x * sc, hy = hh.y * sc;
+        float d0[4], d1[4];
+        mma_16x8x16(d0, a[0], b, b, hx, hy);
+        mma_16x8x16(d1, a[1], b, b, hx, hy);
+        m[0] = min3(m[0], d0[0], d0[1]);
+        m[1] = min3(m[1], d0[2], d0[3]);
+        m[2] = min3(m[2], d1[0], d1[1]);
+        m[3] = min3(m[3], d1[2], d1[3]);
+      }
+#pragma unroll
+      for (int r4 = 0; r4 < 4; ++r4) {
+        m[r4] = fminf(m[r4], __shfl_xor_sync(0xffffffffu, m[r4], 1));
+        m[r4] = fminf(m[r4], __shfl_xor_sync(0xffffffffu, m[r4], 2));
+      }
+      if (qd == 0) {
+#pragma unroll
+        for (int r4 = 0; r4 < 4; ++r4) w.wmin[16 * (r4 >> 1) + 8 * (r4 & 1) + g8][sub] = m[r4];
+      }
+    }
+    __syncwarp();
+    const float4 ma = *reinterpret_cast<const float4*>(&w.wmin[lane][0]);
+    const float4 mb = *reinterpret_cast<const float4*>(&w.wmin[lane][4]);
+    const float mm[8] = {ma.x, ma.y, ma.z, ma.w, mb.x, mb.y, mb.z, mb.w};
+#pragma unroll
+    for (int sub = 0; sub < 8; ++sub) sub_min[sub] = active ? __fmaf_rn(mm[sub], inv, rho) : kInf;
+    // the halves' absolute rounding floor (2^-25 per element in scaled units), doubled, with a factor 4 to spare
+    return 4.76837158203125e-7f /* 2^-21 */ * inv * smax;
+  } else {
+    uint64_t nrd[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) nrd[i] = pack2(-r[i], -r[i]);
+    const uint64_t rho2 = pack2(rho, rho);
+#pragma unroll
+    for (int sub = 0; sub < 8; ++sub) {
+      float cmin = kInf;
+      const ulonglong2* vals = reinterpret_cast<const ulonglong2*>(&st.x[0][0]) + sub * 16 * 4;
+      const uint64_t* norms = reinterpret_cast<const uint64_t*>(&st.h[0]) + sub * 16;
+#pragma unroll 4
+      for (int pr = 0; pr < 16; ++pr) {
+        const ulonglong2 q0 = vals[4 * pr], q1 = vals[4 * pr + 1], q2 = vals[4 * pr + 2], q3 = vals[4 * pr + 3];
+        uint64_t acc = add2(norms[pr], rho2);
+        acc = fma2(nrd[0], q0.x, acc);
+        acc = fma2(nrd[1], q0.y, acc);
+        acc = fma2(nrd[2], q1.x, acc);
+        acc = fma2(nrd[3], q1.y, acc);
+        acc = fma2(nrd[4], q2.x, acc);
+        acc = fma2(nrd[5], q2.y, acc);
+        acc = fma2(nrd[6], q3.x, acc);
+        acc = fma2(nrd[7], q3.y, acc);
+        cmin = min3(cmin, lo_of(acc), hi_of(acc));
+      }
+      sub_min[sub] = active ? cmin : kInf;
+    }
+    return 0.0f;
+  }
+}
+
+// The target's 64 (kept tuple, sub-chunk) flags from its lanes' eight: byte b belongs to kept tuple b.
+__device__ __forceinline__ uint64_t team_flags(uint32_t mine, uint32_t my_b) {
+  uint32_t lo = my_b < 4 ? mine << (8 * my_b) : 0u, hi = my_b >= 4 ? mine << (8 * (my_b - 4)) : 0u;
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) {
+    lo |= __shfl_xor_sync(0xffffffffu, lo, o);
+    hi |= __shfl_xor_sync(0xffffffffu, hi, o);
+  }
+  return ((uint64_t)hi << 32) | lo;
+}
+
+template <int M, bool TC>
+__global__ void __launch_bounds__(kBsThreads, kBsCtasPerSm) encode_beam_kernel(const BeamParams p,
+                                                                               const BeamImage<M, TC>* __restrict__ image) {
+  extern __shared__ __align__(16) unsigned char beam_smem[];
+  BeamSmem<M, TC>& smem = *reinterpret_cast<BeamSmem<M, TC>*>(beam_smem);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_wait();
+  if (!fetch_image(&smem.img, image, (uint32_t)sizeof(BeamImage<M, TC>), &smem.img_bar, p.status)) return;
+  const BeamImage<M, TC>& sm = smem.img;
+  BeamScratch& w = smem.w[warp];
+  const float s1max = sm.smax[0];
+  float sall_books = 0.0f;
+#pragma unroll
+  for (int m = 0; m < M; ++m) sall_books += sm.smax[m];
+
+  const uint64_t nwarps = (uint64_t)gridDim.x * kBsWarps;
+  const uint64_t n_groups = (p.k + kBsGroup - 1) / kBsGroup;
+  const uint32_t my_q = (uint32_t)lane >> 3, my_b = (uint32_t)lane & 7u;
+  constexpr uint32_t kFull = 0xffffffffu;
+
+  for (uint64_t gi = (uint64_t)blockIdx.x * kBsWarps + warp; gi < n_groups; gi += nwarps) {
+    uint32_t B = p.beam < p.K ? p.beam : p.K;  // tuples kept after the stage
+    // what this lane needs of its own target (target my_q of the group)
+    uint32_t my_j = kFull, my_prev = 0;
+    float my_sall = 0.0f;
+
+    // the four targets of the group, one element per lane (lane = 8 * target + element): index, W, g, row scale
+    // and previous tuple are fetched for all four at once, one fma and one division per lane (binary32)
+    uint32_t lane_j = kFull, lane_prev = 0;
+    {
+      const uint64_t n_mine = gi * kBsGroup + my_q;
+      if (n_mine < p.k) lane_j = __ldg(p.idx + n_mine);
+      float tv = 0.0f;
+      if (lane_j < p.G) {
+        const float wv = __ldg(p.W + (size_t)lane_j * 8 + my_b), gv = __ldg(p.g + (size_t)lane_j * 8 + my_b);
+        const float sc = __ldg(p.scale + fast_div(lane_j, p.gpr));
+        if (M == 2) {
+          const uint32_t both = reinterpret_cast<const uint16_t*>(p.codes)[lane_j];
+          lane_prev = (both << 24) | ((both >> 8) << 16);
+        } else {
+#pragma unroll
+          for (int m = 0; m < M; ++m) lane_prev |= (uint32_t)p.codes[(size_t)lane_j * M + m] << (24 - 8 * m);
+        }
+        tv = __fdiv_rn(__fmaf_rn(-p.eta, gv, wv), sc);
+      }
+      w.t[my_q][my_b] = tv;
+    }
+    __syncwarp();
+
+    // ---- stage 1, one target after the other, the whole warp on each
+#pragma unroll 1
+    for (uint32_t q = 0; q < (uint32_t)kBsGroup; ++q) {
+      const uint64_t n = gi * kBsGroup + q;
+      if (n >= p.k) break;
+      const uint32_t j = __shfl_sync(kFull, lane_j, 8 * q);
+      const uint32_t prev = __shfl_sync(kFull, lane_prev, 8 * q);
+      if (j >= p.G) {
+        if (lane == 0) atomicOr(p.status, PVT_DEV_BAD_INDEX);
+        continue;
+      }
+      float t[8];
+      {
+        const float4 ta = *reinterpret_cast<const float4*>(&w.t[q][0]);
+        const float4 tb = *reinterpret_cast<const float4*>(&w.t[q][4]);
+        t[0] = ta.x, t[1] = ta.y, t[2] = ta.z, t[3] = ta.w, t[4] = tb.x, t[5] = tb.y, t[6] = tb.z, t[7] = tb.w;
+      }
+      float nt2 = 0.0f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) nt2 = fmaf(t[i], t[i], nt2);
+      const float tnorm = sqrtf(nt2);
+      // twice the rounding-error bound of the fast score (factor >= 2 to spare), u = 2^-24:
+      //   |score1_fl - score1| <= 16.1 u (||c1||^2/2 + ||t|| ||c1||)
+      const float margin1 = 3.8146973e-6f /* 2^-18 */ * (0.5f * s1max * s1max + tnorm * s1max) + 1e-30f;
+
+      // 256 scores, 8 per lane
+      float f[8];
+      {
+        uint64_t acc[4];
+#pragma unroll
+        for (int qq = 0; qq < 4; ++qq) acc[qq] = sm.h1[qq][lane];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const uint64_t ntd = pack2(-t[i], -t[i]);
+#pragma unroll
+          for (int qq = 0; qq < 4; ++qq) acc[qq] = fma2(ntd, sm.p1[qq][i][lane], acc[qq]);
+        }
+#pragma unroll
+        for (int qq = 0; qq < 4; ++qq) {
+          f[2 * qq] = lo_of(acc[qq]);
+          f[2 * qq + 1] = hi_of(acc[qq]);
+        }
+      }
+      // extract the B smallest (score truncated to 24 bits | code): a first guess of the beam.  Every lane sorts
+      // its eight keys once; a round is then one warp minimum of the lanes' heads and a shift of the winning lane's list.
+      uint32_t key[8];
+#pragma unroll
+      for (int jj = 0; jj < 8; ++jj) key[jj] = (ord(f[jj]) & 0xffffff00u) | (uint32_t)(lane + 32 * jj);
+      sort8(key);
+      uint32_t beam_code[8];
+      uint32_t last = 0;  // the key extracted last
+#pragma unroll
+      for (int b = 0; b < 8; ++b) {
+        beam_code[b] = 0;
+        if ((uint32_t)b < B) {
+          last = __reduce_min_sync(kFull, key[0]);
+          beam_code[b] = last & 0xffu;
+          pop_if(key, last);  // keys are distinct: they end in the code
+        }
+      }
+      // is that guess provably the exact beam?  theta = an upper bound of the scores in the guess (the top of the
+      // truncation bucket of the key extracted last); every member of the exact beam scores <= theta + margin1; if
+      // exactly B codewords do, they are the guess and the exact beam at once.
+      {
+        uint32_t cnt = 0;
+        const float theta = unord(last | 0xffu);
+        const float limit1 = theta + margin1;
+        uint32_t member = 0;
+#pragma unroll
+        for (int jj = 0; jj < 8; ++jj) {
+          const bool in = f[jj] <= limit1 && (uint32_t)(lane + 32 * jj) < p.K;
+          member |= in ? (1u << jj) : 0u;
+          cnt += in;
+        }
+        cnt = __reduce_add_sync(kFull, cnt);
+        if (cnt != B) {
+          // undecided: order the shortlisted codewords by (binary64 distance, code)
+          for (uint32_t b = 0; b < B; ++b) {
+            double ld = __longlong_as_double(kInfBits);
+            uint32_t lk = kFull;
+#pragma unroll
+            for (int jj = 0; jj < 8; ++jj) {
+              if (member & (1u << jj)) {
+                const uint32_t kap = lane + 32 * jj;
+                const double d = exact1(t, sm.c[0][kap]);
+                if (d < ld || (d == ld && kap < lk)) {
+                  ld = d;
+                  lk = kap;
+                }
+              }
+            }
+            // warp-wide lexicographic minimum of (ld, lk); distances are >= 0 so their bits order like u64
+            const uint64_t bits = (uint64_t)__double_as_longlong(ld);
+            const uint32_t hi = (uint32_t)(bits >> 32), lo = (uint32_t)bits;
+            const uint32_t mhi = __reduce_min_sync(kFull, hi);
+            const uint32_t mlo = __reduce_min_sync(kFull, hi == mhi ? lo : kFull);
+            const uint32_t mk = __reduce_min_sync(kFull, (hi == mhi && lo == mlo) ? lk : kFull);
+            const uint32_t chosen = mk < (uint32_t)kBsK ? mk : 0u;
+#pragma unroll
+            for (int bb = 0; bb < 8; ++bb)
+              if ((uint32_t)bb == b) beam_code[bb] = chosen;
+            if ((chosen & 31u) == (uint32_t)lane) member &= ~(1u << (chosen >> 5));
+          }
+        }
+      }
+      // hand the beam to the lanes of the further stages
+      if (lane == 0) {
+        *reinterpret_cast<uint4*>(&w.kept[q][0]) =
+            make_uint4(beam_code[0] << 24, beam_code[1] << 24, beam_code[2] << 24, beam_code[3] << 24);
+        *reinterpret_cast<uint4*>(&w.kept[q][4]) =
+            make_uint4(beam_code[4] << 24, beam_code[5] << 24, beam_code[6] << 24, beam_code[7] << 24);
+      }
+      if (my_q == q) {
+        my_j = j;
+        my_prev = prev;
+        my_sall = tnorm + sall_books;
+      }
+    }
+    __syncwarp();
+
+    // ---- further stages: lane = (target my_q, kept tuple my_b)
+    double bd = __longlong_as_double(kInfBits);  // the best extension of the last stage: distance and tuple
+    uint32_t bk = kFull;
+#pragma unroll
+    for (int m = 1; m < M; ++m) {
+      const bool active = my_j != kFull && my_b < B;
+      const StageImage<TC>& st = sm.st[m - 1];
+      float r[8], rho = 0.0f;
+      {
+        const float4 ta = *reinterpret_cast<const float4*>(&w.t[my_q][0]);
+        const float4 tb = *reinterpret_cast<const float4*>(&w.t[my_q][4]);
+        r[0] = ta.x, r[1] = ta.y, r[2] = ta.z, r[3] = ta.w, r[4] = tb.x, r[5] = tb.y, r[6] = tb.z, r[7] = tb.w;
+        const uint32_t tuple = active ? w.kept[my_q][my_b] : 0u;  // (that of a skipped target was never written)
+#pragma unroll
+        for (int q = 0; q < m; ++q) {
+          const float* c = &sm.c[q][(tuple >> (24 - 8 * q)) & 0xffu][0];
+          const float4 ca = *reinterpret_cast<const float4*>(c), cb = *reinterpret_cast<const float4*>(c + 4);
+          const float cv[8] = {ca.x, ca.y, ca.z, ca.w, cb.x, cb.y, cb.z, cb.w};
+#pragma unroll
+          for (int i = 0; i < 8; ++i) r[i] = __fsub_rn(r[i], cv[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          r[i] = active ? r[i] : 0.0f;
+          rho = __fmaf_rn(r[i], r[i], rho);
+        }
+        rho = __fmul_rn(0.5f, rho);
+        *reinterpret_cast<float4*>(&w.r[lane][0]) = make_float4(r[0], r[1], r[2], r[3]);
+        *reinterpret_cast<float4*>(&w.r[lane][4]) = make_float4(r[4], r[5], r[6], r[7]);
+      }
+      __syncwarp();
+      float sub_min[8];
+      // twice the rounding-error bound of a fast score, with a factor 2 to spare (u = 2^-24; R = the target's largest
+      // residual, C = the largest codeword, S = the target plus the largest codeword of every codebook): 26 u (R + C)^2
+      // for its evaluation, (M - 1) u S (R + C) for the residual's own roundings
+      float rho_max = rho;
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) rho_max = fmaxf(rho_max, __shfl_xor_sync(kFull, rho_max, o));
+      const float reach = sqrtf(2.0f * rho_max) + sm.smax[m];
+      const float margin = (7.6293945e-6f /* 2^-17 */ * reach + 9.5367432e-7f /* 2^-20 */ * my_sall) * reach + 1e-30f +
+                           stage_minima<TC>(st, w, r, rho, active, sm.smax[m], sub_min);
+
+      // the limit up to which fast scores matter: the smallest score, or the keep-th smallest cell minimum (keep
+      // different extensions score no more than that), plus the margin
+      const uint32_t keep = m == M - 1 ? 1u : (p.beam < B * p.K ? p.beam : B * p.K);
+      float limit;
+      if (m == M - 1) {
+        float gmin = sub_min[0];
+#pragma unroll
+        for (int sub = 1; sub < 8; ++sub) gmin = fminf(gmin, sub_min[sub]);
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) gmin = fminf(gmin, __shfl_xor_sync(kFull, gmin, o));
+        limit = gmin + margin;
+      } else {
+        uint32_t key[8];
+#pragma unroll
+        for (int sub = 0; sub < 8; ++sub) key[sub] = (ord(sub_min[sub]) & ~63u) | (my_b * 8 + sub);
+        sort8(key);
+        uint32_t last = 0;
+        for (uint32_t b = 0; b < keep; ++b) {
+          last = team_min(key[0]);
+          pop_if(key, last);
+        }
+        // fewer cells than `keep` (or padding among them): no limit
+        limit = last >= ord(1.0e38f) ? kInf : unord(last | 63u) + margin;
+      }
+      auto flag_cells = [&]() {
+        uint32_t hits = 0;
+#pragma unroll
+        for (int sub = 0; sub < 8; ++sub) hits |= (active && sub_min[sub] <= limit) ? (1u << sub) : 0u;
+        return team_flags(hits, my_b);
+      };
+      uint64_t flags = flag_cells();
+      uint32_t n_list = 0;  // the same in the target's eight lanes
+      __syncwarp();         // the cell minima have been read: the list takes their place
+
+      // Revisit the flagged cells one after the other, four codewords per lane, the four targets of the group side by
+      // side.  (The fast score is evaluated again here, in another order: both evaluations lie within half the margin
+      // of the true score, so what the definition selects passes both tests.)
+#pragma unroll 1
+      for (int pass = 0;; ++pass) {
+        while (__any_sync(kFull, flags != 0)) {
+          const bool work = flags != 0;
+          const uint32_t pos = work ? (uint32_t)__ffsll((long long)flags) - 1u : 0u;
+          flags &= flags - 1;
+          const uint32_t hb = pos >> 3, hsub = pos & 7u;
+          const uint32_t tuple = work ? w.kept[my_q][hb] : 0u;
+          float sr[8], srho = 0.0f;
+          {
+            const float4 ra = *reinterpret_cast<const float4*>(&w.r[8 * my_q + hb][0]);
+            const float4 rb = *reinterpret_cast<const float4*>(&w.r[8 * my_q + hb][4]);
+            sr[0] = ra.x, sr[1] = ra.y, sr[2] = ra.z, sr[3] = ra.w, sr[4] = rb.x, sr[5] = rb.y, sr[6] = rb.z, sr[7] = rb.w;
+          }
+#pragma unroll
+          for (int i = 0; i < 8; ++i) srho = __fmaf_rn(sr[i], sr[i], srho);
+          srho = __fmul_rn(0.5f, srho);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const uint32_t k2 = hsub * 32u + 8u * c + my_b;
+            const float4 ca = *reinterpret_cast<const float4*>(&sm.c[m][k2][0]);
+            const float4 cb = *reinterpret_cast<const float4*>(&sm.c[m][k2][4]);
+            const float cv[8] = {ca.x, ca.y, ca.z, ca.w, cb.x, cb.y, cb.z, cb.w};
+            float s2 = __fadd_rn(st.h[k2], srho);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) s2 = __fmaf_rn(-sr[i], cv[i], s2);
+            const bool in = work && s2 <= limit && k2 < p.K;
+            const uint32_t key = tuple | (k2 << (24 - 8 * m));
+            if (m == M - 1) {
+              if (in) {
+                const double d = exact_tuple<M>(w.t[my_q], sm.c, key);
+                if (d < bd || (d == bd && key < bk)) {
+                  bd = d;
+                  bk = key;
+                }
+              }
+            } else {
+              const uint32_t who = (__ballot_sync(kFull, in) >> (8 * my_q)) & 0xffu;
+              const uint32_t at = n_list + __popc(who & ((1u << my_b) - 1u));
+              if (in && at < (uint32_t)kBsList) w.list[my_q][at] = make_uint2(__float_as_uint(s2), key);
+              n_list += __popc(who);
+            }
+          }
+        }
+        if (m == M - 1) break;
+        // More extensions within the limit than the list holds (one target in fifty): the keep-th smallest of those it
+        // holds is a lower limit.  Equal scores in that number are left to the exact path below.
+        const bool over = n_list > (uint32_t)kBsList;
+        if (pass == 3 || !__any_sync(kFull, over)) break;
+        __syncwarp();
+        uint32_t key[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) key[i] = over ? (ord(__uint_as_float(w.list[my_q][8 * i + my_b].x)) & ~31u) | (8 * i + my_b) : kFull;
+        sort4(key);
+        uint32_t last = 0;
+        for (uint32_t b = 0; b < keep; ++b) {
+          last = team_min(key[0]);
+          pop_if(key, last);
+        }
+        const float lower = unord(last | 31u) + margin;
+        const bool again = over && lower < limit;
+        if (!__any_sync(kFull, again)) break;
+        if (again) {
+          limit = lower;
+          n_list = 0;
+        }
+        flags = flag_cells();
+        if (!again) flags = 0;
+        __syncwarp();
+      }
+      if (m < M - 1) {
+        // the `keep` smallest of the list: eight lanes per target, up to four entries each
+        __syncwarp();
+        float es[4];
+        uint32_t ek[4], key[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const uint32_t at = 8 * i + my_b;
+          const bool have = at < n_list && n_list <= (uint32_t)kBsList;
+          const uint2 entry = have ? w.list[my_q][at] : make_uint2(0x7f800000u, kFull);
+          es[i] = __uint_as_float(entry.x);
+          ek[i] = entry.y;
+          key[i] = have ? (ord(es[i]) & ~31u) | at : kFull;
+        }
+        sort4(key);
+        uint32_t pick = kFull, last = 0;  // the list entry that becomes kept tuple my_b
+        for (uint32_t b = 0; b < keep; ++b) {
+          last = team_min(key[0]);
+          if (my_b == b) pick = last & 31u;
+          pop_if(key, last);
+        }
+        // exactly `keep` entries up to the last one's bucket plus the margin: provably the exact ones
+        const float sure = unord(last | 31u) + margin;
+        uint32_t near = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) near += ek[i] != kFull && es[i] <= sure;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) near += __shfl_xor_sync(kFull, near, o);
+        uint32_t next = my_b < keep && pick < n_list ? w.list[my_q][pick].y : 0u;
+        const bool target = my_j != kFull;
+        const bool all = n_list > (uint32_t)kBsList;  // many equal extensions: every one of them gets its distance
+        const bool unsure = target && !all && near != keep;
+        auto partial = [&](uint32_t tuple) { return exact_partial(w.t[my_q], sm.c, tuple, m + 1); };
+        if (__any_sync(kFull, unsure)) {
+          double ed[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            ed[i] = unsure && ek[i] != kFull ? partial(ek[i]) : __longlong_as_double(kInfBits);
+          for (uint32_t b = 0; b < keep; ++b) {
+            double d = ed[0];
+            uint32_t k = ek[0];
+#pragma unroll
+            for (int i = 1; i < 4; ++i)
+              if (ed[i] < d || (ed[i] == d && ek[i] < k)) d = ed[i], k = ek[i];
+            team_min_exact(d, k);
+            if (unsure && my_b == b) next = k;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (ek[i] == k) ed[i] = __longlong_as_double(kInfBits), ek[i] = kFull;
+          }
+        }
+        if (__any_sync(kFull, target && all)) {
+          double ld = -1.0;  // the (distance, tuple) taken last
+          uint32_t lk = 0;
+          for (uint32_t b = 0; b < keep; ++b) {
+            double d = __longlong_as_double(kInfBits);
+            uint32_t k = kFull;
+            for (uint32_t e = my_b; e < B * p.K; e += 8) {
+              if (!(target && all)) break;
+              const uint32_t key2 = w.kept[my_q][e / p.K] | ((e % p.K) << (24 - 8 * m));
+              const double x = partial(key2);
+              const bool later = x > ld || (x == ld && (key2 > lk || b == 0));
+              if (later && (x < d || (x == d && key2 < k))) d = x, k = key2;
+            }
+            __syncwarp();
+            team_min_exact(d, k);
+            if (target && all && my_b == b) next = k;
+            ld = d;
+            lk = k;
+          }
+        }
+        __syncwarp();  // everybody has read the tuples that are replaced now
+        if (target) w.kept[my_q][my_b] = next;
+        B = keep;
+        __syncwarp();
+      }
+    }
+    if (my_b == 0 && my_j != kFull) {  // the previous tuple joins the pool
+      bool ok = true;
+#pragma unroll
+      for (int m = 0; m < M; ++m) ok &= ((my_prev >> (24 - 8 * m)) & 0xffu) < p.K;
+      if (ok) {
+        const double d = exact_tuple<M>(w.t[my_q], sm.c, my_prev);
+        if (d < bd || (d == bd && my_prev < bk)) {
+          bd = d;
+          bk = my_prev;
+        }
+      } else {
+        atomicOr(p.status, PVT_DEV_BAD_CODE);
+      }
+    }
+    __syncwarp();
+    team_min_exact(bd, bk);
+    if (my_b == 0 && my_j != kFull) {
+      if (bd < __longlong_as_double(kInfBits)) {
+        if (M == 2) {
+          reinterpret_cast<uint16_t*>(p.codes)[my_j] = (uint16_t)((bk >> 24) | ((bk >> 8) & 0xff00u));
+        } else {
+#pragma unroll
+          for (int m = 0; m < M; ++m) p.codes[(size_t)my_j * M + m] = (uint8_t)(bk >> (24 - 8 * m));
+        }
+        if (p.err_out) p.err_out[gi * kBsGroup + my_q] = (float)bd;
+      } else if (M > 2) {
+        atomicOr(p.status, PVT_DEV_INTERNAL);
+      }
+    }
+    __syncwarp();  // the group's scratch is rewritten by the next iteration
+  }
+}
+
+template <int M, bool TC>
+cudaError_t launch_beam(const BeamParams& p, unsigned char* image_at, int sm_count, cudaStream_t stream) {
+  using Image = BeamImage<M, TC>;
+  static_assert(sizeof(Image) % 16 == 0, "the bulk copy moves multiples of 16 bytes");
+  static_assert(sizeof(Image) <= 77824, "the workspace reserves 76 KiB for the image");
+  constexpr size_t smem = sizeof(BeamSmem<M, TC>);
+  cudaError_t err = allow_smem(encode_beam_kernel<M, TC>);
+  if (err != cudaSuccess) return err;
+  Image* image = reinterpret_cast<Image*>(image_at);
+  timing_begin(kKernEncodeAux, stream);
+  beam_image_kernel<M, TC><<<1, kBsThreads, 0, stream>>>(p, image);
+  timing_end(kKernEncodeAux, stream);
+  if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  constexpr uint64_t fit = (228 * 1024) / (smem + 1024);
+  constexpr uint64_t per_sm = fit < kBsCtasPerSm ? fit : kBsCtasPerSm;  // persistent: the resident CTAs
+  const uint64_t groups = (p.k + kBsGroup - 1) / kBsGroup, want = (groups + kBsWarps - 1) / kBsWarps;
+  const uint64_t most = per_sm * (uint64_t)sm_count;
+  timing_begin(kKernEncodeMain, stream);
+  err = launch_dependent(encode_beam_kernel<M, TC>, (unsigned)(want < most ? want : most), kBsThreads, smem, stream, p,
+                         (const Image*)image);
+  count_launches(2);
+  timing_end(kKernEncodeMain, stream);
+  return err;
+}
+
+}  // namespace
+
+cudaError_t launch_encode_beam(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out, void* ws,
+                               int sm_count, cudaStream_t stream) {
+  BeamParams p;
+  p.W = L.W;
+  p.g = L.g;
+  p.scale = L.scale;
+  p.idx = idx;
+  p.k = k;
+  p.G = G;
+  p.gpr = make_fast_div((uint32_t)(L.cols / kGroupDim));
+  p.eta = L.eta;
+  p.books = L.codebooks;
+  p.K = (uint32_t)L.codebook_size;
+  p.beam = (uint32_t)L.beam;
+  p.codes = static_cast<uint8_t*>(L.codes);
+  p.err_out = err_out;
+  p.status = static_cast<uint32_t*>(ws);
+  unsigned char* image = static_cast<unsigned char*>(ws) + kWsHeaderBytes;
+  const bool f16 = L.codebook_dtype == PVT_F16;
+  switch (L.num_codebooks) {
+    case 2: return f16 ? launch_beam<2, true>(p, image, sm_count, stream) : launch_beam<2, false>(p, image, sm_count, stream);
+    case 3: return f16 ? launch_beam<3, true>(p, image, sm_count, stream) : launch_beam<3, false>(p, image, sm_count, stream);
+    default: return f16 ? launch_beam<4, true>(p, image, sm_count, stream) : launch_beam<4, false>(p, image, sm_count, stream);
+  }
+}
+
+}  // namespace pvt

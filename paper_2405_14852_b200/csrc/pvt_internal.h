@@ -76,7 +76,7 @@ struct EncodeM1Layout {
 };
 EncodeM1Layout encode_m1_layout(uint32_t K, uint64_t k, int sm_count, int targets_per_thread);
 int encode_m1_targets_per_thread(uint64_t k, int sm_count);  // 4 or 8
-size_t encode_m2_workspace_bytes();
+size_t encode_beam_workspace_bytes();
 
 // encode, M = 1 on the tensor cores (fp16 codebooks of at least 1024 codewords)
 struct EncodeM1TcLayout {
@@ -105,10 +105,8 @@ cudaError_t launch_encode_m1(const pvt_layer& L, uint64_t G, const uint32_t* idx
                              void* ws, int sm_count, cudaStream_t stream);
 cudaError_t launch_encode_m1_tc(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
                                 void* ws, int sm_count, cudaStream_t stream);
-cudaError_t launch_encode_m2(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
-                             void* ws, int sm_count, cudaStream_t stream);
-cudaError_t launch_encode_mx(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
-                             void* ws, cudaStream_t stream);
+cudaError_t launch_encode_beam(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
+                               void* ws, int sm_count, cudaStream_t stream);
 cudaError_t launch_encode_g16(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
                               void* ws, cudaStream_t stream);
 cudaError_t launch_dequant(const pvt_layer& L, uint64_t G, void* W_hat, int32_t out_dtype, uint32_t* status,

@@ -1,0 +1,32 @@
+"""Beam search over three and four codebooks where a middle stage's short list changes its way: codebooks of a few
+codewords (fewer cells than kept tuples), sizes around 32, lists that overflow because codewords nearly coincide, and
+because they do."""
+import numpy as np
+import pytest
+
+from paper_2405_14852_b200 import synth
+from test_gpu_parity import check_encode, oracle_nearest
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M", [3, 4])
+@pytest.mark.parametrize("K,beam,f16", [
+    (2, 8, True), (3, 3, False), (7, 8, True), (8, 8, False), (9, 8, True), (31, 7, True), (33, 8, False), (255, 2, True),
+])
+def test_small_and_ragged_codebooks(M, K, beam, f16):
+    L = synth.make_layer(16, 264, cfg=300 + M, num_codebooks=M, codebook_size=K, codebook_fp16=f16, beam=beam,
+                         nearest=oracle_nearest)
+    check_encode(L, np.arange(3, L.num_groups, 2, dtype=np.uint32))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M", [3, 4])
+@pytest.mark.parametrize("copies,jitter,f16", [(16, 1e-3, True), (16, 0.0, True), (32, 1e-6, False), (5, 0.0, False)])
+def test_clustered_codewords(M, copies, jitter, f16):
+    L = synth.make_layer(16, 256, cfg=310 + M, num_codebooks=M, codebook_size=256, codebook_fp16=f16,
+                         nearest=oracle_nearest)
+    rng = np.random.default_rng(copies)
+    for m in range(1, M):
+        base = L.codebooks[m].astype(np.float32)[np.arange(256) // copies]
+        L.codebooks[m] = (base + rng.normal(0.0, jitter, size=base.shape)).astype(L.codebooks.dtype)
+    check_encode(L, np.arange(L.num_groups, dtype=np.uint32))
