@@ -28,6 +28,9 @@ PVT_M1_AUTO, PVT_M1_FP32, PVT_M1_TENSOR = 0, 1, 2
 PVT_SAMPLE_UNIFORM, PVT_SAMPLE_PROPORTIONAL = 0, 1
 
 
+_OUT_DTYPE = {torch.float32: PVT_F32, torch.float16: PVT_F16}
+
+
 class pvt_layer(ctypes.Structure):
     _fields_ = [
         ("rows", ctypes.c_int32), ("cols", ctypes.c_int32), ("group_dim", ctypes.c_int32),
@@ -136,9 +139,16 @@ def _check(code: int, what: str) -> None:
         raise PvtError(code, what)
 
 
+# the current stream's handle without building a Stream object, where this torch has that query
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
@@ -249,8 +259,7 @@ def pvt_vstep_refine(layer: pvt_layer, idx: torch.Tensor, k: int, max_moves: int
 
 
 def pvt_dequant(layer: pvt_layer, W_hat: torch.Tensor, status: Optional[torch.Tensor] = None, stream=None) -> None:
-    out_dtype = {torch.float32: PVT_F32, torch.float16: PVT_F16}[W_hat.dtype]
-    _check(lib().pvt_dequant(ctypes.byref(layer), W_hat.data_ptr(), out_dtype, _ptr(status), _stream_ptr(stream)),
+    _check(lib().pvt_dequant(ctypes.byref(layer), W_hat.data_ptr(), _OUT_DTYPE[W_hat.dtype], _ptr(status), _stream_ptr(stream)),
            "pvt_dequant")
 
 
@@ -272,7 +281,7 @@ class Block:
             if len(dts) > 1:
                 raise ValueError("the dequantised matrices of a block share one dtype")
             if dts:
-                self.out_dtype = {torch.float32: PVT_F32, torch.float16: PVT_F16}[dts.pop()]
+                self.out_dtype = _OUT_DTYPE[dts.pop()]
         self._keep = (list(idx_outs), list(W_hats) if W_hats is not None else None)
 
     def workspace_bytes(self) -> int:
@@ -280,6 +289,27 @@ class Block:
         if need == 0:
             raise PvtError(PVT_EINVAL, "pvt_block_workspace_bytes")
         return need
+
+
+class OneLayer:
+    """pvt_vstep_block for one layer: the call's one-entry host arrays."""
+
+    def __init__(self):
+        self._k = (ctypes.c_uint64 * 1)()
+        self._idx = (ctypes.c_void_p * 1)()
+        self._W_hat = (ctypes.c_void_p * 1)()
+
+    def step(self, layer: pvt_layer, k: int, idx_out: torch.Tensor, W_hat: Optional[torch.Tensor], ws: torch.Tensor,
+             stream=None) -> None:
+        """select -> encode -> dequantise (the last if W_hat is given), one C call."""
+        self._k[0] = k
+        self._idx[0] = idx_out.data_ptr()
+        out, dtype = None, PVT_F32
+        if W_hat is not None:
+            self._W_hat[0] = W_hat.data_ptr()
+            out, dtype = self._W_hat, _OUT_DTYPE[W_hat.dtype]
+        _check(lib().pvt_vstep_block(ctypes.byref(layer), self._k, 1, self._idx, out, dtype, ws.data_ptr(),
+                                     ws.numel() * ws.element_size(), _stream_ptr(stream)), "pvt_vstep_block")
 
 
 def pvt_vstep_block(block: Block, ws: torch.Tensor, stream=None) -> None:

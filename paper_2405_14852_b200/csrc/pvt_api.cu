@@ -153,8 +153,9 @@ size_t encode_bytes(const pvt_layer& L, uint64_t k, int sms) {
   if (L.num_codebooks >= 2) return encode_beam_workspace_bytes();  // header + the codebooks' image
   if (L.group_dim == 16)
     return encode_m1_use_tc(L, k) ? encode_m1_tc_layout((uint32_t)L.codebook_size, k, sms, 16).bytes : kWsHeaderBytes;
-  return encode_m1_use_tc(L, k)
-             ? encode_m1_tc_layout((uint32_t)L.codebook_size, k, sms).bytes
+  if (encode_m1_use_tc(L, k)) return encode_m1_tc_layout((uint32_t)L.codebook_size, k, sms).bytes;
+  return (uint32_t)L.codebook_size <= kM1SmallCodebook
+             ? kM1SmallWorkspace
              : encode_m1_layout((uint32_t)L.codebook_size, k, sms, encode_m1_targets_per_thread(k, sms)).bytes;
 }
 
@@ -252,6 +253,9 @@ int pvt_vstep_encode(const pvt_layer* layer, const uint32_t* idx, uint64_t k, fl
   } else if (layer->num_codebooks == 1 && encode_m1_use_tc(*layer, k)) {
     if (ws_bytes < encode_m1_tc_layout((uint32_t)layer->codebook_size, k, sms).bytes) return PVT_EWORKSPACE;
     e = launch_encode_m1_tc(*layer, G, idx, k, err_out, ws, sms, static_cast<cudaStream_t>(cuda_stream));
+  } else if (layer->num_codebooks == 1 && (uint32_t)layer->codebook_size <= kM1SmallCodebook) {
+    if (ws_bytes < kM1SmallWorkspace) return PVT_EWORKSPACE;
+    e = launch_encode_m1_small(*layer, G, idx, k, err_out, ws, sms, static_cast<cudaStream_t>(cuda_stream));
   } else if (layer->num_codebooks == 1) {
     const EncodeM1Layout lay =
         encode_m1_layout((uint32_t)layer->codebook_size, k, sms, encode_m1_targets_per_thread(k, sms));

@@ -327,30 +327,6 @@ __global__ void __launch_bounds__(kEncThreads + 32, 1) encode_m1_kernel(const En
 }
 
 // ---- rescoring --------------------------------------------------------------------
-template <bool CB_F16, int DG>
-__device__ __forceinline__ void load_codeword(const void* book, uint32_t kappa, float* c) {
-  if (CB_F16) {
-#pragma unroll
-    for (int part = 0; part < DG / 8; ++part) {
-      const uint4 raw = __ldg(reinterpret_cast<const uint4*>(book) + (size_t)kappa * (DG / 8) + part);
-      const __half2* h = reinterpret_cast<const __half2*>(&raw);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float2 f = __half22float2(h[i]);
-        c[8 * part + 2 * i] = f.x;
-        c[8 * part + 2 * i + 1] = f.y;
-      }
-    }
-  } else {
-    const float4* q = reinterpret_cast<const float4*>(book) + (size_t)kappa * (DG / 4);
-#pragma unroll
-    for (int part = 0; part < DG / 4; ++part) {
-      const float4 a = __ldg(q + part);
-      c[4 * part] = a.x; c[4 * part + 1] = a.y; c[4 * part + 2] = a.z; c[4 * part + 3] = a.w;
-    }
-  }
-}
-
 // Eight lanes per target, four targets per warp: the kernel is a chain of dependent memory round trips
 // ((index, global minimum, margin, records) -> (W, g, scale) -> codewords), so what counts is how many targets
 // are in flight per warp, not how fast one of them is evaluated.

@@ -29,6 +29,7 @@ struct EncM1Params {
   const uint32_t* idx;
   uint64_t k, G;
   uint32_t gpr;
+  FastDiv gpr_div;  // the same as a divisor
   uint32_t dg;  // weights per group: 8, or 16 (tensor engine and rescoring only)
   float eta;
   const float* cbx;
@@ -90,6 +91,31 @@ __device__ __forceinline__ void form_target16(const EncM1Params& p, uint32_t j, 
     t[4 * q + 1] = __fdiv_rn(__fmaf_rn(neg_eta, gg.y, w.y), sc);
     t[4 * q + 2] = __fdiv_rn(__fmaf_rn(neg_eta, gg.z, w.z), sc);
     t[4 * q + 3] = __fdiv_rn(__fmaf_rn(neg_eta, gg.w, w.w), sc);
+  }
+}
+
+// one codeword of DG elements, widened to binary32
+template <bool CB_F16, int DG>
+__device__ __forceinline__ void load_codeword(const void* book, uint32_t kappa, float* c) {
+  if (CB_F16) {
+#pragma unroll
+    for (int part = 0; part < DG / 8; ++part) {
+      const uint4 raw = __ldg(reinterpret_cast<const uint4*>(book) + (size_t)kappa * (DG / 8) + part);
+      const __half2* h = reinterpret_cast<const __half2*>(&raw);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 f = __half22float2(h[i]);
+        c[8 * part + 2 * i] = f.x;
+        c[8 * part + 2 * i + 1] = f.y;
+      }
+    }
+  } else {
+    const float4* q = reinterpret_cast<const float4*>(book) + (size_t)kappa * (DG / 4);
+#pragma unroll
+    for (int part = 0; part < DG / 4; ++part) {
+      const float4 a = __ldg(q + part);
+      c[4 * part] = a.x; c[4 * part + 1] = a.y; c[4 * part + 2] = a.z; c[4 * part + 3] = a.w;
+    }
   }
 }
 

@@ -91,6 +91,8 @@ struct EncodeM1TcLayout {
   uint32_t n_ctas;
 };
 bool encode_m1_use_tc(const pvt_layer& L, uint64_t k);
+constexpr uint32_t kM1SmallCodebook = 1024;  // without the tensor engine: codebooks up to here stay in shared memory
+constexpr size_t kM1SmallWorkspace = kWsHeaderBytes + kWsAlign;
 void set_m1_search(int mode);
 EncodeM1TcLayout encode_m1_tc_layout(uint32_t K, uint64_t k, int sm_count, int group_dim = 8);
 
@@ -103,6 +105,8 @@ cudaError_t launch_select_keyed(const pvt_layer& L, uint64_t G, uint64_t k, uint
                                 cudaStream_t stream, int key_mode, float* buffer, uint64_t seed);
 cudaError_t launch_encode_m1(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
                              void* ws, int sm_count, cudaStream_t stream);
+cudaError_t launch_encode_m1_small(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
+                                   void* ws, int sm_count, cudaStream_t stream);
 cudaError_t launch_encode_m1_tc(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
                                 void* ws, int sm_count, cudaStream_t stream);
 cudaError_t launch_encode_beam(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,

@@ -30,7 +30,7 @@ class VStepLayer:
         self.desc = B.make_layer(self.rows, self.cols, W, g, scale, codebooks, codes, eta=self.eta, beam=self.beam,
                                  group_dim=self.group_dim)
         self._ws = None
-        self._ws_k = 0
+        self._one = B.OneLayer()
         if max_k is not None:
             self.reserve(max_k)
 
@@ -49,27 +49,35 @@ class VStepLayer:
             B.pvt_workspace_init(self._ws)
         return self._ws
 
+    def _with_workspace(self, k: int, call):
+        """call(workspace) with the workspace at hand; only a call that finds it too small makes it grow (the library
+        checks its size before it enqueues anything)."""
+        if self._ws is not None:
+            try:
+                return call(self._ws)
+            except B.PvtError as e:
+                if e.code != B.PVT_EWORKSPACE:
+                    raise
+        return call(self.reserve(k))
+
     def select(self, k: int, idx_out: Optional[torch.Tensor] = None) -> torch.Tensor:
-        ws = self.reserve(k)
         if idx_out is None:
             idx_out = torch.empty(k, dtype=torch.int32, device=self.W.device)
-        B.pvt_vstep_select(self.desc, k, idx_out, ws)
+        self._with_workspace(k, lambda ws: B.pvt_vstep_select(self.desc, k, idx_out, ws))
         return idx_out
 
     def select_ste(self, buffer: torch.Tensor, k: int, idx_out: Optional[torch.Tensor] = None) -> torch.Tensor:
         """Selection while the straight-through buffer takes the step (Appendix E): buffer -= eta * g in place."""
-        ws = self.reserve(k)
         if idx_out is None:
             idx_out = torch.empty(k, dtype=torch.int32, device=self.W.device)
-        B.pvt_vstep_select_ste(self.desc, buffer, k, idx_out, ws)
+        self._with_workspace(k, lambda ws: B.pvt_vstep_select_ste(self.desc, buffer, k, idx_out, ws))
         return idx_out
 
     def sample(self, k: int, rule: int, seed: int, idx_out: Optional[torch.Tensor] = None) -> torch.Tensor:
         """A random subspace (B.PVT_SAMPLE_UNIFORM / B.PVT_SAMPLE_PROPORTIONAL) instead of the greedy one."""
-        ws = self.reserve(k)
         if idx_out is None:
             idx_out = torch.empty(k, dtype=torch.int32, device=self.W.device)
-        B.pvt_vstep_sample(self.desc, k, rule, seed, idx_out, ws)
+        self._with_workspace(k, lambda ws: B.pvt_vstep_sample(self.desc, k, rule, seed, idx_out, ws))
         return idx_out
 
     def encode_against(self, buffer: torch.Tensor, idx: torch.Tensor, err_out: Optional[torch.Tensor] = None) -> None:
@@ -77,11 +85,11 @@ class VStepLayer:
         k = int(idx.numel())
         desc = B.make_layer(self.rows, self.cols, buffer, self.g, self.scale, self.codebooks, self.codes, eta=0.0,
                             beam=self.beam, group_dim=self.group_dim)
-        B.pvt_vstep_encode(desc, idx, k, err_out, self.reserve(k))
+        self._with_workspace(k, lambda ws: B.pvt_vstep_encode(desc, idx, k, err_out, ws))
 
     def encode(self, idx: torch.Tensor, err_out: Optional[torch.Tensor] = None) -> None:
         k = int(idx.numel())
-        B.pvt_vstep_encode(self.desc, idx, k, err_out, self.reserve(k))
+        self._with_workspace(k, lambda ws: B.pvt_vstep_encode(self.desc, idx, k, err_out, ws))
 
     def dequant(self, out: Optional[torch.Tensor] = None, dtype=torch.float32) -> torch.Tensor:
         if out is None:
@@ -91,6 +99,11 @@ class VStepLayer:
 
     def step(self, k: int, idx_out=None, W_hat=None, err_out=None):
         """One V step followed by the dequantisation that opens the next step."""
+        if err_out is None:  # the three calls as one
+            if idx_out is None:
+                idx_out = torch.empty(k, dtype=torch.int32, device=self.W.device)
+            self._with_workspace(k, lambda ws: self._one.step(self.desc, k, idx_out, W_hat, ws))
+            return idx_out, W_hat
         idx = self.select(k, idx_out)
         self.encode(idx, err_out)
         return idx, self.dequant(W_hat) if W_hat is not None else None
