@@ -309,16 +309,13 @@ __global__ void __launch_bounds__(kEncThreads + 32, 1) encode_m1_kernel(const En
         const uint32_t cnt = sm.list_cnt[s];
         CandRecord r;
         r.best = best[tt];
-        r.pad = 0;
+        r.w[0] = r.w[1] = r.w[2] = 0;
         uint32_t m = 0;
 #pragma unroll
-        for (int v = 0; v < kListLen; ++v) {
-          r.sub[v] = 0;
-          if ((uint32_t)v < cnt && sm.list_min[v][s] <= limit) r.sub[m++] = sm.list_id[v][s];
-        }
-        r.cnt = (cnt > (uint32_t)kListLen && sm.evicted_min[s] <= limit) ? kCandOverflow : (uint16_t)m;
-        *reinterpret_cast<uint4*>(&p.rec[((size_t)tile * p.n_slices + sl) * TILE + s]) =
-            *reinterpret_cast<const uint4*>(&r);
+        for (int v = 0; v < kListLen; ++v)
+          if ((uint32_t)v < cnt && sm.list_min[v][s] <= limit) cand_add(r, m++, sm.list_id[v][s]);
+        r.w[0] |= ((cnt > (uint32_t)kListLen && sm.evicted_min[s] <= limit) ? kCandOverflow : m) << 24;
+        cand_write(&p.rec[((size_t)tile * p.n_slices + sl) * TILE + s], r);
         atomicMin(&p.gbest[n], ord(best[tt]));
         if (sl == 0) p.margin[n] = margin[tt];
       }
@@ -329,7 +326,8 @@ __global__ void __launch_bounds__(kEncThreads + 32, 1) encode_m1_kernel(const En
 // ---- rescoring --------------------------------------------------------------------
 // Eight lanes per target, four targets per warp: the kernel is a chain of dependent memory round trips
 // ((index, global minimum, margin, records) -> (W, g, scale) -> codewords), so what counts is how many targets
-// are in flight per warp, not how fast one of them is evaluated.
+// are in flight per warp, not how fast one of them is evaluated.  (With every candidate evaluated in binary64, 1048576
+// targets took 368 us, 20971 15.3.)
 constexpr int kRsLanes = 8;
 constexpr int kRsPerWarp = 32 / kRsLanes;
 constexpr int kRsPerBlock = 8 * kRsPerWarp;  // 256 threads
@@ -343,13 +341,17 @@ __global__ void __launch_bounds__(256) rescore_m1_kernel(const EncM1Params p) {
   const int gshift = grp * kRsLanes;
   const uint64_t n = ((uint64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * kRsPerWarp + grp;
   bool active = n < p.k;
+  pdl_wait();
   uint32_t j = 0;
   float limit = 0.0f;
   uint4 raw0 = make_uint4(0x7f800000u, 0, 0, 0), raw1 = raw0;  // best = +inf: never within the limit
   if (active) {
     const uint32_t tile = (uint32_t)(n / p.tile), s = (uint32_t)(n % p.tile);
     j = __ldg(p.idx + n);
-    limit = unord(p.gbest[n]) + p.margin[n];
+    const float least = unord(p.gbest[n]);
+    limit = p.margin[n];
+    // (a least score of minus infinity marks a target that is rescored against the whole codebook)
+    limit = fabsf(least) < 3.0e38f ? least + fmaf(p.rel_margin, fabsf(least), limit) : least;
     const uint4* rec = reinterpret_cast<const uint4*>(p.rec);
     if ((uint32_t)l < p.n_slices) raw0 = __ldg(&rec[((size_t)tile * p.n_slices + l) * p.tile + s]);
     if ((uint32_t)l + kRsLanes < p.n_slices)
@@ -386,10 +388,25 @@ __global__ void __launch_bounds__(256) rescore_m1_kernel(const EncM1Params p) {
       best_code = kappa;
     }
   };
-  auto visit = [&](uint32_t sub) {
-    for (uint32_t w = l; w < sub_cw; w += kRsLanes) {
-      const uint32_t kappa = sub * sub_cw + w;
-      if (kappa < p.K) score(kappa);
+  // Binary32 decides which codewords the binary64 evaluation can turn on: a sum of at most 16 squares of differences is off
+  // by less than 20 2^-24 of itself, so that the winner, and all that tie with it, lie within 2^-18 of the least.  A lane
+  // remembers its least distance and the one after it; if that is inside as well (two codewords of one lane that near, or
+  // equal), or the least is no number of the range, every candidate of the target is evaluated in binary64.
+  float near1 = __uint_as_float(0x7f800000u), near2 = near1;
+  uint32_t near_code = 0;
+  auto estimate = [&](uint32_t kappa) {
+    float c[DG];
+    load_codeword<CB_F16, DG>(p.book, kappa, c);
+    float d = 0.0f;
+#pragma unroll
+    for (int i = 0; i < DG; ++i) {
+      const float e = t[i] - c[i];
+      d = fmaf(e, e, d);
+    }
+    near2 = fminf(near2, fmaxf(near1, d));
+    if (d < near1) {
+      near1 = d;
+      near_code = kappa;
     }
   };
 
@@ -398,37 +415,60 @@ __global__ void __launch_bounds__(256) rescore_m1_kernel(const EncM1Params p) {
   // shuffles are executed by the whole warp.
   const uint32_t in0 = __ballot_sync(kFull, active && __uint_as_float(raw0.x) <= limit);
   const uint32_t in1 = __ballot_sync(kFull, active && __uint_as_float(raw1.x) <= limit);
-  uint32_t live = ((in0 >> gshift) & 0xffu) | (((in1 >> gshift) & 0xffu) << kRsLanes);
-  while (__any_sync(kFull, live != 0)) {
-    const bool has = live != 0;
-    const int sl = has ? __ffs(live) - 1 : 0;
-    live &= live - 1;
-    const int src = gshift + (sl & (kRsLanes - 1));
-    const bool upper = sl >= kRsLanes;
-    const uint32_t y0 = __shfl_sync(kFull, raw0.y, src), y1 = __shfl_sync(kFull, raw1.y, src);
-    const uint32_t z0 = __shfl_sync(kFull, raw0.z, src), z1 = __shfl_sync(kFull, raw1.z, src);
-    const uint32_t w0 = __shfl_sync(kFull, raw0.w, src), w1 = __shfl_sync(kFull, raw1.w, src);
-    if (!has) continue;
-    const uint32_t s01 = upper ? y1 : y0, s23 = upper ? z1 : z0;
-    const uint32_t cnt = (upper ? w1 : w0) & 0xffffu;
-    if (cnt == kCandOverflow) {
-      uint32_t u_lo, u_hi;
-      slice_units(p, (uint32_t)sl, &u_lo, &u_hi);
-      for (uint32_t sub = u_lo * subs_per_unit; sub < u_hi * subs_per_unit; ++sub) visit(sub);
-    } else {
-      if (cnt > 0) visit(s01 & 0xffffu);
-      if (cnt > 1) visit(s01 >> 16);
-      if (cnt > 2) visit(s23 & 0xffffu);
-      if (cnt > 3) visit(s23 >> 16);
+  const uint32_t slices = ((in0 >> gshift) & 0xffu) | (((in1 >> gshift) & 0xffu) << kRsLanes);
+  auto sweep = [&](bool on, auto&& take) {
+    auto visit = [&](uint32_t sub) {
+      for (uint32_t w = l; w < sub_cw; w += kRsLanes) {
+        const uint32_t kappa = sub * sub_cw + w;
+        if (kappa < p.K) take(kappa);
+      }
+    };
+    uint32_t live = on ? slices : 0;
+    while (__any_sync(kFull, live != 0)) {
+      const bool has = live != 0;
+      const int sl = has ? __ffs(live) - 1 : 0;
+      live &= live - 1;
+      const int src = gshift + (sl & (kRsLanes - 1));
+      const bool upper = sl >= kRsLanes;
+      const uint32_t y0 = __shfl_sync(kFull, raw0.y, src), y1 = __shfl_sync(kFull, raw1.y, src);
+      const uint32_t z0 = __shfl_sync(kFull, raw0.z, src), z1 = __shfl_sync(kFull, raw1.z, src);
+      const uint32_t w0 = __shfl_sync(kFull, raw0.w, src), w1 = __shfl_sync(kFull, raw1.w, src);
+      if (!has) continue;
+      uint32_t ids[3] = {upper ? y1 : y0, upper ? z1 : z0, upper ? w1 : w0};
+      const uint32_t cnt = ids[0] >> 24;
+      if (cnt == kCandOverflow) {
+        uint32_t u_lo, u_hi;
+        slice_units(p, (uint32_t)sl, &u_lo, &u_hi);
+        for (uint32_t sub = u_lo * subs_per_unit; sub < u_hi * subs_per_unit; ++sub) visit(sub);
+      } else {
+        for (uint32_t q = 0; q < cnt; ++q) {
+          visit(ids[0] & 0xfffu);
+          if (q & 1u) {
+            ids[0] = ids[1];
+            ids[1] = ids[2];
+          } else {
+            ids[0] = (ids[0] >> 12) & 0xfffu;
+          }
+        }
+      }
     }
-  }
-  if (p.exc_count && active) {  // codewords whose fast score is not trustworthy: always evaluated
-    const uint32_t n_exc = __ldg(p.exc_count);
-    for (uint32_t e = l; e < n_exc && e < p.K; e += kRsLanes) {
-      const uint32_t kappa = __ldg(p.exc_list + e);
-      if (kappa < p.K) score(kappa);
+    if (p.exc_count && on) {  // codewords whose fast score is not trustworthy: always evaluated
+      const uint32_t n_exc = __ldg(p.exc_count);
+      for (uint32_t e = l; e < n_exc && e < p.K; e += kRsLanes) {
+        const uint32_t kappa = __ldg(p.exc_list + e);
+        if (kappa < p.K) take(kappa);
+      }
     }
-  }
+  };
+  sweep(active, estimate);
+  float least = near1;
+#pragma unroll
+  for (int off = kRsLanes / 2; off > 0; off >>= 1) least = fminf(least, __shfl_xor_sync(kFull, least, off));
+  const float inside = fmaf(least, 3.814697265625e-6f /* 2^-18 */, least) + 1e-36f;
+  const uint32_t again = __ballot_sync(kFull, active && (near2 <= inside || !(least < 1e38f)));
+  const bool all = (again >> gshift) & 0xffu;
+  if (active && !all && near1 <= inside) score(near_code);
+  if (again) sweep(active && all, score);
   // lexicographic minimum of (distance, code) over the eight lanes of the target; distances are >= 0 so their
   // bits order like u64
   const uint64_t bits = (uint64_t)__double_as_longlong(best_d);
@@ -483,6 +523,7 @@ cudaError_t launch_encode_m1(const pvt_layer& L, uint64_t G, const uint32_t* idx
   p.k = k;
   p.G = G;
   p.gpr = (uint32_t)(L.cols / kGroupDim);
+  p.gpr_div = make_fast_div(p.gpr);
   p.dg = kGroupDim;
   p.eta = L.eta;
   p.cbx = reinterpret_cast<const float*>(base + lay.cbx_off);
@@ -490,6 +531,7 @@ cudaError_t launch_encode_m1(const pvt_layer& L, uint64_t G, const uint32_t* idx
   p.n_units = lay.n_chunks;
   p.unit_cw = kChunkCodewords;
   p.sub_cw = kSubCodewords;
+  p.rel_margin = 0.0f;
   p.exc_count = nullptr;
   p.exc_list = nullptr;
   p.K = (uint32_t)L.codebook_size;
@@ -531,16 +573,17 @@ cudaError_t launch_encode_m1(const pvt_layer& L, uint64_t G, const uint32_t* idx
 cudaError_t launch_rescore_m1(const EncM1Params& p, bool codebook_f16, cudaStream_t stream) {
   timing_begin(kKernEncodeRescore, stream);
   const unsigned blocks = (unsigned)((p.k + kRsPerBlock - 1) / kRsPerBlock);
+  cudaError_t err;
   if (p.dg == 16) {  // groups of 16 weights come from the tensor engine only: fp16 codebooks
-    rescore_m1_kernel<true, 16><<<blocks, 256, 0, stream>>>(p);
+    err = launch_dependent(rescore_m1_kernel<true, 16>, blocks, 256, 0, stream, p);
   } else if (codebook_f16) {
-    rescore_m1_kernel<true, 8><<<blocks, 256, 0, stream>>>(p);
+    err = launch_dependent(rescore_m1_kernel<true, 8>, blocks, 256, 0, stream, p);
   } else {
-    rescore_m1_kernel<false, 8><<<blocks, 256, 0, stream>>>(p);
+    err = launch_dependent(rescore_m1_kernel<false, 8>, blocks, 256, 0, stream, p);
   }
   count_launches(1);
   timing_end(kKernEncodeRescore, stream);
-  return cudaGetLastError();
+  return err;
 }
 
 }  // namespace pvt

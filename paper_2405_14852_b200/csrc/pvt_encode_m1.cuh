@@ -40,7 +40,8 @@ struct EncM1Params {
   const uint32_t* exc_count;  // codewords the fast score cannot represent: always rescored (may be null)
   const uint32_t* exc_list;
   uint32_t* gbest;
-  float* margin;
+  float* margin;      // rounding-error margin of each target's fast scores, to which
+  float rel_margin;   // this share of the score is added
   CandRecord* rec;
   const void* book;  // the caller's codebook [K][dg]
   void* codes;
@@ -66,7 +67,7 @@ __device__ __forceinline__ void form_target(const EncM1Params& p, uint32_t j, fl
   const float4* g4 = reinterpret_cast<const float4*>(p.g);
   const float4 w0 = __ldg(W4 + 2 * (size_t)j), w1 = __ldg(W4 + 2 * (size_t)j + 1);
   const float4 g0 = __ldg(g4 + 2 * (size_t)j), g1 = __ldg(g4 + 2 * (size_t)j + 1);
-  const float sc = __ldg(p.scale + j / p.gpr);
+  const float sc = __ldg(p.scale + fast_div(j, p.gpr_div));
   const float neg_eta = -p.eta;
   t[0] = __fdiv_rn(__fmaf_rn(neg_eta, g0.x, w0.x), sc);
   t[1] = __fdiv_rn(__fmaf_rn(neg_eta, g0.y, w0.y), sc);
@@ -82,7 +83,7 @@ __device__ __forceinline__ void form_target(const EncM1Params& p, uint32_t j, fl
 __device__ __forceinline__ void form_target16(const EncM1Params& p, uint32_t j, float* t) {
   const float4* W4 = reinterpret_cast<const float4*>(p.W) + 4 * (size_t)j;
   const float4* g4 = reinterpret_cast<const float4*>(p.g) + 4 * (size_t)j;
-  const float sc = __ldg(p.scale + j / p.gpr);
+  const float sc = __ldg(p.scale + fast_div(j, p.gpr_div));
   const float neg_eta = -p.eta;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
@@ -163,6 +164,16 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   return false;
 }
 
+
+// candidate records: sub-chunks are added one by one, the count last
+__device__ __forceinline__ void cand_add(CandRecord& r, uint32_t n, uint32_t sub) {
+  const uint32_t bits = sub << (12 * (n & 1u));
+#pragma unroll
+  for (uint32_t q = 0; q < 3; ++q) r.w[q] |= (n >> 1) == q ? bits : 0u;
+}
+__device__ __forceinline__ void cand_write(CandRecord* to, const CandRecord& r) {
+  *reinterpret_cast<uint4*>(to) = make_uint4(__float_as_uint(r.best), r.w[0], r.w[1], r.w[2]);
+}
 
 // units [lo, hi) of slice sl
 __device__ __forceinline__ void slice_units(const EncM1Params& p, uint32_t sl, uint32_t* lo, uint32_t* hi) {

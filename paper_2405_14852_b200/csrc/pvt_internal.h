@@ -50,16 +50,16 @@ constexpr int kChunkCodewords = 256; // codewords per staged chunk (one bulk cop
 constexpr int kSubCodewords = 32;    // tracking granularity of the running minimum
 constexpr int kChunkBytes = kChunkCodewords * (kGroupDim * 4 + 4);  // 9216: pairs interleaved + half norms
 constexpr int kEncStages = 4;
-constexpr int kListLen = 4;          // remembered near-minimum sub-chunks per (target, slice)
+constexpr int kListLen = 4;          // near-minimum sub-chunks per (target, slice) that the FP32 engine remembers
 constexpr int kMaxSlices = 16;
-constexpr uint16_t kCandOverflow = 0xffffu;
 
 struct CandRecord {        // 16 bytes, one per (target, codebook slice)
   float best;              // smallest fast score of the slice
-  uint16_t sub[kListLen];  // sub-chunk ids whose minimum lies within the margin of `best`
-  uint16_t cnt;            // valid entries of sub[]; kCandOverflow: rescan the whole slice
-  uint16_t pad;
+  uint32_t w[3];           // up to six sub-chunk ids (12 bits each, two per word) whose minimum lies within the margin of
+                           // `best`; their number in the upper byte of w[0], kCandOverflow: rescan the whole slice
 };
+constexpr int kCandMost = 6;
+constexpr uint32_t kCandOverflow = 0xffu;
 
 struct EncodeM1Layout {
   size_t cbx_off;      // expanded codebook: n_chunks * kChunkBytes
