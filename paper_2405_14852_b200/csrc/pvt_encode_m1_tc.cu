@@ -708,7 +708,10 @@ cudaError_t launch_tc(const pvt_layer& L, const EncM1Params& p, const EncodeM1Tc
                       cudaStream_t stream) {
   timing_begin(kKernEncodeAux, stream);
   const uint32_t n_cw = lay.n_steps * kTcStepCw;
-  tc_prep_kernel<DG><<<(n_cw + 255) / 256, 256, 0, stream>>>(
+  // enough threads for one codeword each, and for no more than four of the initial minima each until the chip is full
+  const uint64_t fill = (p.k + 1023) / 1024 < 592 ? (p.k + 1023) / 1024 : 592;
+  const uint32_t image = (n_cw + 255) / 256;
+  tc_prep_kernel<DG><<<fill > image ? (unsigned)fill : image, 256, 0, stream>>>(
       reinterpret_cast<const uint4*>(L.codebooks), p.K, lay.n_steps,
       reinterpret_cast<unsigned char*>(base + lay.bimg_off), stats, reinterpret_cast<uint32_t*>(base + lay.exc_off),
       p.gbest, p.k);
