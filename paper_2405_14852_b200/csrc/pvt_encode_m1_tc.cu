@@ -327,6 +327,7 @@ struct TcSmem {
   uint64_t drain_bar[4];
   uint32_t list[kTcListLen][kTcEpiThreads];  // key of the maximum (upper half) and number of the sub-chunk
   float margin[kTcTile];   // per target; negative if it is out of range or absent
+  float seed[kTcTile];      // score of the stored code
   float odd_best[kTcTile];  // what the odd set leaves for the even one
   uint32_t odd_cnt[kTcTile], odd_evicted[kTcTile];
   uint32_t tmem_base;
@@ -529,6 +530,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
         float t[DG];
 #pragma unroll
         for (int i = 0; i < DG; ++i) t[i] = 0.0f;
+        float prev = -kNegInf;
         if (n < p.k) {
           const uint32_t j = p.idx[n];
           if (j < p.G) {  // an index out of range is reported by the rescoring kernel
@@ -537,6 +539,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
             else
               form_target16(p, j, t);
             have = true;
+            // the distance to the stored code: only what comes near it has to be remembered
+            const uint32_t code = p.code_u16 ? reinterpret_cast<const uint16_t*>(p.codes)[j]
+                                             : reinterpret_cast<const uint8_t*>(p.codes)[j];
+            if (code < p.K) {
+              float c[DG];
+              load_codeword<true, DG>(p.book, code, c);
+              float d = 0.0f;
+#pragma unroll
+              for (int i = 0; i < DG; ++i) d = fmaf(t[i] - c[i], t[i] - c[i], d);
+              if (d < 1e30f) prev = d;
+            }
           }
         }
         pdl_wait();  // the image's statistics (and the initial minima)
@@ -605,6 +618,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
                                          (norm * cnmax + hmax + nt2) +
                                      4.76837158203125e-7f /* 2^-21 */);
         sm.margin[own] = in_range ? margin : -1.0f;
+        sm.seed[own] = in_range ? -0.5f * sc * prev * 1.0001f : kNegInf;  // (minus infinity without a stored code)
       }
       epi_sync();
       const float margin = sm.margin[own];
@@ -618,7 +632,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
       // the list of remembered sub-chunks lives in shared memory, its fill count and the best evicted entry
       // in registers: the common case of an event is one store and no load
       uint32_t list_cnt = 0, evicted = 0xffffffffu;
-      uint32_t lim = 0xfc00u;  // keys up to this one are remembered
+      // keys up to this one are remembered: at first those that may reach the score of the stored code.  (With no bound to
+      // begin with, every thread remembers its first steps one after the other: 4096x4096 1x16, five units per CTA, 95 us instead of 90.)
+      const float seed = sm.seed[own];
+      uint32_t lim = key_limit(seed - fmaf(kRelMargin, fabsf(seed), margin));
       auto note = [&](uint32_t key, uint32_t sub) {
         if (key <= lim) {
           const uint32_t slot = list_cnt & (kTcListLen - 1);
@@ -626,7 +643,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
           sm.list[slot][tid] = (key << 16) | sub;
           ++list_cnt;
           best = fmaxf(best, key_score(key));
-          lim = key_limit(best - fmaf(kRelMargin, fabsf(best), margin));
+          lim = min(lim, key_limit(best - fmaf(kRelMargin, fabsf(best), margin)));
         }
       };
       for (uint32_t st = s_lo + ((it ^ set) & 1); st < s_hi && alive; st += 2, ++uses) {
@@ -665,7 +682,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
         if (in_range) {
           const uint32_t other_cnt = sm.odd_cnt[own];
           best = fmaxf(best, sm.odd_best[own]);
-          lim = key_limit(best - fmaf(kRelMargin, fabsf(best), margin));
+          lim = min(lim, key_limit(best - fmaf(kRelMargin, fabsf(best), margin)));
           uint32_t cnt_out = 0;
 #pragma unroll
           for (int q = 0; q < 2 * kTcListLen; ++q) {
@@ -690,9 +707,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
     }
   }
 
-  pdl_trigger();
   tc_fence_before();
   __syncthreads();
+  pdl_trigger();
   if (warp == kTcEpiWarps + 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);
