@@ -1,12 +1,14 @@
 // dequantize_weights (Algorithm 3, first line): W_hat = s_row * sum_m C_m[b_m] for
-// every weight group.  Streaming kernel, persistent grid: two threads per group (four
-// weights each), four half-groups in flight per thread, codes read coalesced,
-// codewords gathered from the L2-resident codebook (small codebooks are first copied
-// to shared memory), every store instruction of a warp covers whole 32-byte sectors.
+// every weight group.  Streaming kernel, persistent grid: one thread per 16 bytes of the
+// result, four of them in flight per thread, codes read coalesced, codewords gathered from
+// the L2-resident codebook (small codebooks are first copied to shared memory), and a
+// warp's stores contiguous: 512 bytes per instruction.
 //
 // Arithmetic per element, binary32, each step rounded once: v = c1 (+ c2);
 // w = s * v; fp16 output = round-to-nearest-even of w.
 #include <cuda_fp16.h>
+
+#include <atomic>
 
 #include "pvt_internal.h"
 
@@ -14,34 +16,50 @@ namespace pvt {
 namespace {
 
 constexpr int kDqThreads = 256;
-constexpr int kDqUnroll = 4;          // half-groups in flight per thread
-constexpr int kDqSmemCodewords = 512;  // M*K up to this many codewords are staged in shared memory
+constexpr int kDqUnroll = 4;             // pieces of 16 result bytes in flight per thread
+constexpr int kDqSmemBytes = 32 * 1024;  // codebooks of up to this size are staged in shared memory
 
-// elements 4*half .. 4*half+3 of one codeword of 4*PARTS elements, widened to binary32
-template <bool CB_F16, int PARTS>
-__device__ __forceinline__ float4 load_half_codeword(const void* book, uint32_t code, uint32_t half) {
+// elements EL*part .. EL*part+EL-1 of one codeword of EL*PARTS elements, widened to binary32
+template <bool CB_F16, int EL, int PARTS>
+__device__ __forceinline__ void load_part(const void* book, uint32_t code, uint32_t part, float* v) {
+  const size_t at = PARTS * (size_t)code + part;
   if (CB_F16) {
-    const uint2 raw = *(reinterpret_cast<const uint2*>(book) + PARTS * (size_t)code + half);
-    const float2 lo = __half22float2(*reinterpret_cast<const __half2*>(&raw.x));
-    const float2 hi = __half22float2(*reinterpret_cast<const __half2*>(&raw.y));
-    return make_float4(lo.x, lo.y, hi.x, hi.y);
+    uint32_t raw[EL / 2];
+    if (EL == 8)
+      *reinterpret_cast<uint4*>(raw) = reinterpret_cast<const uint4*>(book)[at];
+    else
+      *reinterpret_cast<uint2*>(raw) = reinterpret_cast<const uint2*>(book)[at];
+#pragma unroll
+    for (int i = 0; i < EL / 2; ++i) {
+      const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&raw[i]));
+      v[2 * i] = f.x;
+      v[2 * i + 1] = f.y;
+    }
   } else {
-    return *(reinterpret_cast<const float4*>(book) + PARTS * (size_t)code + half);
+#pragma unroll
+    for (int i = 0; i < EL / 4; ++i) {
+      const float4 a = reinterpret_cast<const float4*>(book)[at * (EL / 4) + i];
+      v[4 * i] = a.x, v[4 * i + 1] = a.y, v[4 * i + 2] = a.z, v[4 * i + 3] = a.w;
+    }
   }
 }
 
-// Two threads per group, four elements each: a warp then writes 512 (fp32) or 256 (fp16)
-// contiguous bytes per store instruction, i.e. whole 32-byte sectors.
-// (PARTS threads per group: 2 for groups of 8 weights, 4 for groups of 16.)
-template <int M, bool CB_F16, bool CODE_U16, bool OUT_F16, bool SMEM_BOOK, int PARTS>
+// 16 result bytes per thread, eight fp16 or four fp32 weights: DG / EL threads per group.
+// Bound by the stores where the codebook is in shared memory; a codebook of 2^16 codewords is gathered from L2 at no
+// more than one group per cycle and SM, since each lane's codeword is another line.  (fp16 results with four weights per
+// thread: 11008x4096 3x8 43.5 us instead of 29.8, 5120x5120 2x8 19.6 instead of 14.7.  fp32 results with eight:
+// 11008x4096 2x8 45 us instead of 31.7, 32 bytes per lane are stored more slowly.)
+template <int M, bool CB_F16, bool CODE_U16, bool OUT_F16, bool SMEM_BOOK, int DG>
 __global__ void __launch_bounds__(kDqThreads) dequant_kernel(const void* __restrict__ codebooks,
                                                               const void* __restrict__ codes,
                                                               const float* __restrict__ scale, uint64_t G,
                                                               FastDiv gpr, uint32_t K, void* __restrict__ W_hat,
                                                               uint32_t* status) {
-  constexpr int kCwBytes = (CB_F16 ? 8 : 16) * PARTS;
-  __shared__ __align__(16) unsigned char sh_book[SMEM_BOOK ? kDqSmemCodewords * kCwBytes : 16];
+  constexpr int EL = OUT_F16 ? 8 : 4, PARTS = DG / EL;
+  constexpr int kCwBytes = (CB_F16 ? 2 : 4) * DG;
+  __shared__ __align__(16) unsigned char sh_book[SMEM_BOOK ? kDqSmemBytes : 16];
   const void* book = codebooks;
+  pdl_wait();
   if (SMEM_BOOK) {
     const uint4* src = reinterpret_cast<const uint4*>(codebooks);
     uint4* dst = reinterpret_cast<uint4*>(sh_book);
@@ -50,18 +68,20 @@ __global__ void __launch_bounds__(kDqThreads) dequant_kernel(const void* __restr
     __syncthreads();
     book = sh_book;
   }
-  // kDqUnroll half-groups per thread and iteration, a block apart, all their loads issued
+  // kDqUnroll parts per thread and iteration, a block apart, all their loads issued
   // before the first use: the code -> codeword -> store chain of one group is two
   // dependent memory round trips, so several must be in flight per thread
   const uint64_t H = (uint64_t)PARTS * G;
   const uint64_t stride = (uint64_t)gridDim.x * (kDqThreads * kDqUnroll);
   for (uint64_t base = (uint64_t)blockIdx.x * (kDqThreads * kDqUnroll); base < H; base += stride) {
     uint32_t b[kDqUnroll][M];
+    float s[kDqUnroll];
     bool bad = false;
 #pragma unroll
     for (int u = 0; u < kDqUnroll; ++u) {
       const uint64_t h = base + (uint64_t)u * kDqThreads + threadIdx.x;
       const uint32_t j = (uint32_t)(h / PARTS);
+      s[u] = 0.0f;
 #pragma unroll
       for (int m = 0; m < M; ++m) b[u][m] = 0;
       if (h < H) {
@@ -69,15 +89,20 @@ __global__ void __launch_bounds__(kDqThreads) dequant_kernel(const void* __restr
           const uint16_t* c = reinterpret_cast<const uint16_t*>(codes) + (size_t)j * M;
 #pragma unroll
           for (int m = 0; m < M; ++m) b[u][m] = __ldg(c + m);
-        } else if (M == 2) {
-          const uint16_t both = __ldg(reinterpret_cast<const uint16_t*>(codes) + j);  // two adjacent bytes
-          b[u][0] = both & 0xffu;
-          b[u][M - 1] = both >> 8;
+        } else if (M % 2 == 0) {  // two adjacent bytes at a time
+          const uint16_t* c = reinterpret_cast<const uint16_t*>(codes) + (size_t)j * (M / 2);
+#pragma unroll
+          for (int m = 0; m < M; m += 2) {
+            const uint16_t both = __ldg(c + m / 2);
+            b[u][m] = both & 0xffu;
+            b[u][(m + 1) % M] = both >> 8;
+          }
         } else {
           const uint8_t* c = reinterpret_cast<const uint8_t*>(codes) + (size_t)j * M;
 #pragma unroll
           for (int m = 0; m < M; ++m) b[u][m] = __ldg(c + m);
         }
+        s[u] = __ldg(scale + fast_div(j, gpr));  // row of group j (G < 2^32)
 #pragma unroll
         for (int m = 0; m < M; ++m) {
           if (b[u][m] >= K) {
@@ -88,65 +113,70 @@ __global__ void __launch_bounds__(kDqThreads) dequant_kernel(const void* __restr
       }
     }
     if (bad && status) atomicOr(status, PVT_DEV_BAD_CODE);
-    float4 v[kDqUnroll];
-    float s[kDqUnroll];
+    float v[kDqUnroll][EL];
 #pragma unroll
-    for (int u = 0; u < kDqUnroll; ++u) {
-      const uint64_t h = base + (uint64_t)u * kDqThreads + threadIdx.x;
-      const uint32_t j = (uint32_t)(h / PARTS), half = (uint32_t)h & (uint32_t)(PARTS - 1);
-      v[u] = load_half_codeword<CB_F16, PARTS>(book, b[u][0], half);
+    for (int u = 0; u < kDqUnroll; ++u)
+      load_part<CB_F16, EL, PARTS>(book, b[u][0], threadIdx.x % PARTS, v[u]);
 #pragma unroll
-      for (int m = 1; m < M; ++m) {  // codebooks added left to right, each sum rounded once
-        const float4 v2 = load_half_codeword<CB_F16, PARTS>(book, m * K + b[u][m], half);
-        v[u].x = __fadd_rn(v[u].x, v2.x);
-        v[u].y = __fadd_rn(v[u].y, v2.y);
-        v[u].z = __fadd_rn(v[u].z, v2.z);
-        v[u].w = __fadd_rn(v[u].w, v2.w);
+    for (int m = 1; m < M; ++m) {  // codebooks added left to right, each sum rounded once
+#pragma unroll
+      for (int u = 0; u < kDqUnroll; ++u) {
+        float v2[EL];
+        load_part<CB_F16, EL, PARTS>(book, m * K + b[u][m], threadIdx.x % PARTS, v2);
+#pragma unroll
+        for (int i = 0; i < EL; ++i) v[u][i] = __fadd_rn(v[u][i], v2[i]);
       }
-      s[u] = h < H ? __ldg(scale + fast_div(j, gpr)) : 0.0f;  // row of group j (G < 2^32)
     }
 #pragma unroll
     for (int u = 0; u < kDqUnroll; ++u) {
       const uint64_t h = base + (uint64_t)u * kDqThreads + threadIdx.x;
       if (h >= H) continue;
-      const float4 w = make_float4(__fmul_rn(s[u], v[u].x), __fmul_rn(s[u], v[u].y), __fmul_rn(s[u], v[u].z),
-                                   __fmul_rn(s[u], v[u].w));
-      if (OUT_F16) {
-        const __half2 lo = __floats2half2_rn(w.x, w.y), hi = __floats2half2_rn(w.z, w.w);
-        __stcs(reinterpret_cast<uint2*>(W_hat) + h,
-               make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi)));
-      } else {
-        __stcs(reinterpret_cast<float4*>(W_hat) + h, w);
+#pragma unroll
+      for (int i = 0; i < EL; ++i) v[u][i] = __fmul_rn(s[u], v[u][i]);
+      uint32_t w[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (OUT_F16) {
+          const __half2 two = __floats2half2_rn(v[u][2 * i % EL], v[u][(2 * i + 1) % EL]);
+          w[i] = *reinterpret_cast<const uint32_t*>(&two);
+        } else {
+          w[i] = __float_as_uint(v[u][i]);
+        }
       }
+      __stcs(reinterpret_cast<uint4*>(W_hat) + h, make_uint4(w[0], w[1], w[2], w[3]));
     }
   }
 }
 
-template <int M, bool CB_F16, bool CODE_U16, bool OUT_F16, int PARTS = 2>
+template <int M, bool CB_F16, bool CODE_U16, bool OUT_F16, bool SMEM_BOOK, int DG>
+cudaError_t launch_s(const pvt_layer& L, uint64_t G, void* W_hat, uint32_t* status, int sm_count, cudaStream_t stream) {
+  const auto kernel = dequant_kernel<M, CB_F16, CODE_U16, OUT_F16, SMEM_BOOK, DG>;
+  // persistent grid: as many blocks as are resident at once (asked once per device)
+  static std::atomic<int> resident[kMaxDevices];
+  const int dev = device_slot();
+  int per_sm = dev >= 0 ? resident[dev].load(std::memory_order_relaxed) : 0;
+  if (per_sm < 1) {
+    const cudaError_t oe = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kDqThreads, 0);
+    if (oe != cudaSuccess) return oe;
+    if (per_sm < 1) per_sm = 1;
+    if (dev >= 0) resident[dev].store(per_sm, std::memory_order_relaxed);
+  }
+  const uint64_t per_block = (uint64_t)kDqThreads * kDqUnroll;
+  const uint64_t want = (DG / (OUT_F16 ? 8 : 4) * G + per_block - 1) / per_block;
+  const uint64_t cap = (uint64_t)sm_count * (uint64_t)per_sm;
+  return launch_dependent(kernel, (unsigned)(want < cap ? want : cap), kDqThreads, 0, stream, L.codebooks, L.codes, L.scale,
+                          G, make_fast_div((uint32_t)(L.cols / DG)), (uint32_t)L.codebook_size, W_hat, status);
+}
+
+template <int M, bool CB_F16, bool CODE_U16, bool OUT_F16, int DG = 8>
 cudaError_t launch_t(const pvt_layer& L, uint64_t G, void* W_hat, uint32_t* status, int sm_count,
                      cudaStream_t stream) {
-  const bool smem_book = (uint32_t)M * (uint32_t)L.codebook_size * (PARTS / 2) <= (uint32_t)kDqSmemCodewords;
-  // persistent grid: as many blocks as are resident at once
-  int per_sm = 0;
-  cudaError_t oe = smem_book ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                                   &per_sm, dequant_kernel<M, CB_F16, CODE_U16, OUT_F16, true, PARTS>, kDqThreads, 0)
-                             : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                                   &per_sm, dequant_kernel<M, CB_F16, CODE_U16, OUT_F16, false, PARTS>, kDqThreads, 0);
-  if (oe != cudaSuccess) return oe;
-  if (per_sm < 1) per_sm = 1;
-  const uint64_t per_block = (uint64_t)kDqThreads * kDqUnroll;
-  const uint64_t want = (PARTS * G + per_block - 1) / per_block;
-  const uint64_t cap = (uint64_t)sm_count * (uint64_t)per_sm;
-  const unsigned blocks = (unsigned)(want < cap ? want : cap);
-  const FastDiv gpr = make_fast_div((uint32_t)(L.cols / (4 * PARTS)));  // groups per row
-  const uint32_t K = (uint32_t)L.codebook_size;
-  if (smem_book)
-    dequant_kernel<M, CB_F16, CODE_U16, OUT_F16, true, PARTS>
-        <<<blocks, kDqThreads, 0, stream>>>(L.codebooks, L.codes, L.scale, G, gpr, K, W_hat, status);
-  else
-    dequant_kernel<M, CB_F16, CODE_U16, OUT_F16, false, PARTS>
-        <<<blocks, kDqThreads, 0, stream>>>(L.codebooks, L.codes, L.scale, G, gpr, K, W_hat, status);
-  return cudaGetLastError();
+  // 32 KB: all that two to four codebooks can take; of one codebook, what leaves six blocks per SM resident
+  if constexpr (M == 1) {
+    if ((uint64_t)L.codebook_size * ((CB_F16 ? 2 : 4) * DG) > (uint64_t)kDqSmemBytes)
+      return launch_s<M, CB_F16, CODE_U16, OUT_F16, false, DG>(L, G, W_hat, status, sm_count, stream);
+  }
+  return launch_s<M, CB_F16, CODE_U16, OUT_F16, true, DG>(L, G, W_hat, status, sm_count, stream);
 }
 
 template <int M, bool CB_F16, bool CODE_U16>
@@ -172,7 +202,7 @@ cudaError_t launch_dequant(const pvt_layer& L, uint64_t G, void* W_hat, int32_t 
   const bool f16 = L.codebook_dtype == PVT_F16;
   if (L.group_dim == 16) {  // groups of 16 weights: one codebook
     const bool u16 = L.code_dtype == PVT_U16, o16 = out_dtype == PVT_F16;
-#define PVT_DQ16(CB, CU, OF) launch_t<1, CB, CU, OF, 4>(L, G, W_hat, status, sm_count, stream)
+#define PVT_DQ16(CB, CU, OF) launch_t<1, CB, CU, OF, 16>(L, G, W_hat, status, sm_count, stream)
     if (f16)
       err = u16 ? (o16 ? PVT_DQ16(true, true, true) : PVT_DQ16(true, true, false))
                 : (o16 ? PVT_DQ16(true, false, true) : PVT_DQ16(true, false, false));

@@ -445,6 +445,7 @@ __global__ void __launch_bounds__(kBsThreads, kBsCtasPerSm) encode_beam_kernel(c
   extern __shared__ __align__(16) unsigned char beam_smem[];
   BeamSmem<M, TC>& smem = *reinterpret_cast<BeamSmem<M, TC>*>(beam_smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_trigger();
   pdl_wait();
   if (!fetch_image(&smem.img, image, (uint32_t)sizeof(BeamImage<M, TC>), &smem.img_bar, p.status)) return;
   const BeamImage<M, TC>& sm = smem.img;

@@ -341,6 +341,7 @@ __global__ void __launch_bounds__(256) rescore_m1_kernel(const EncM1Params p) {
   const int gshift = grp * kRsLanes;
   const uint64_t n = ((uint64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * kRsPerWarp + grp;
   bool active = n < p.k;
+  pdl_trigger();
   pdl_wait();
   uint32_t j = 0;
   float limit = 0.0f;

@@ -52,6 +52,7 @@ __global__ void __launch_bounds__(kSmThreads, 4) encode_m1_small_kernel(const En
   const uint32_t tid = threadIdx.x, l = tid & 7u, team = tid >> 3, n_teams = kSmThreads / 8;
   if (tid == 0) sm_n2max = 0;
   __syncthreads();
+  pdl_trigger();
   pdl_wait();
   {
     uint32_t n2bits = 0;

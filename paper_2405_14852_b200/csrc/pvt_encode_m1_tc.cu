@@ -632,8 +632,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
       // the list of remembered sub-chunks lives in shared memory, its fill count and the best evicted entry
       // in registers: the common case of an event is one store and no load
       uint32_t list_cnt = 0, evicted = 0xffffffffu;
-      // keys up to this one are remembered: at first those that may reach the score of the stored code.  (With no bound to
-      // begin with, every thread remembers its first steps one after the other: 4096x4096 1x16, five units per CTA, 95 us instead of 90.)
+      // keys up to this one are remembered: at first those that may reach the score of the stored code.  (With no bound
+      // to begin with, every thread remembers its first steps one after the other: 4096x4096 1x16, five units per CTA,
+      // 95 us instead of 90.)
       const float seed = sm.seed[own];
       uint32_t lim = key_limit(seed - fmaf(kRelMargin, fabsf(seed), margin));
       auto note = [&](uint32_t key, uint32_t sub) {

@@ -70,6 +70,8 @@ template <int M, bool CB_F16, bool CODE_U16, bool STAGED>
 __global__ void __launch_bounds__(kRfThreads) refine_kernel(const RefineParams p) {
   __shared__ __align__(16) float sh_book[STAGED ? kRfSmemCodewords * 8 : 8];
   const uint32_t K = p.K;
+  pdl_trigger();
+  pdl_wait();
   if (STAGED) {
     for (uint32_t row = threadIdx.x; row < M * K; row += kRfThreads) {
       float c[8];
@@ -209,12 +211,13 @@ __global__ void __launch_bounds__(kRfThreads) refine_kernel(const RefineParams p
 template <int M, bool CB_F16, bool CODE_U16>
 cudaError_t launch_staged(const RefineParams& p, cudaStream_t stream) {
   const unsigned blocks = (unsigned)((p.k + kRfThreads / 32 - 1) / (kRfThreads / 32));
+  cudaError_t err;
   if ((uint64_t)M * p.K <= (uint64_t)kRfSmemCodewords)
-    refine_kernel<M, CB_F16, CODE_U16, true><<<blocks, kRfThreads, 0, stream>>>(p);
+    err = launch_dependent(refine_kernel<M, CB_F16, CODE_U16, true>, blocks, kRfThreads, 0, stream, p);
   else
-    refine_kernel<M, CB_F16, CODE_U16, false><<<blocks, kRfThreads, 0, stream>>>(p);
+    err = launch_dependent(refine_kernel<M, CB_F16, CODE_U16, false>, blocks, kRfThreads, 0, stream, p);
   count_launches(1);
-  return cudaGetLastError();
+  return err;
 }
 
 }  // namespace
