@@ -1,7 +1,7 @@
 // dequantize_weights (Algorithm 3, first line): W_hat = s_row * sum_m C_m[b_m] for
 // every weight group.  Streaming kernel, persistent grid: one thread per 16 bytes of the
 // result, four of them in flight per thread, codes read coalesced, codewords gathered from
-// the L2-resident codebook (small codebooks are first copied to shared memory), and a
+// the L2-resident codebook (small ones are first copied to shared memory), and a
 // warp's stores contiguous: 512 bytes per instruction.
 //
 // Arithmetic per element, binary32, each step rounded once: v = c1 (+ c2);
@@ -17,7 +17,10 @@ namespace {
 
 constexpr int kDqThreads = 256;
 constexpr int kDqUnroll = 4;             // pieces of 16 result bytes in flight per thread
-constexpr int kDqSmemBytes = 32 * 1024;  // codebooks of up to this size are staged in shared memory
+// Codebooks of up to this size are staged in shared memory: two to four always (256 codewords each at most), one if it is
+// small.  No more than that is reserved, for it costs resident blocks (32 KB for all: 11008x4096 2x8 39 us after the
+// search instead of 32).
+__host__ __device__ constexpr int staged_bytes(int M, int cw_bytes) { return M == 1 ? 8192 : M * 256 * cw_bytes; }
 
 // elements EL*part .. EL*part+EL-1 of one codeword of EL*PARTS elements, widened to binary32
 template <bool CB_F16, int EL, int PARTS>
@@ -57,7 +60,7 @@ __global__ void __launch_bounds__(kDqThreads) dequant_kernel(const void* __restr
                                                               uint32_t* status) {
   constexpr int EL = OUT_F16 ? 8 : 4, PARTS = DG / EL;
   constexpr int kCwBytes = (CB_F16 ? 2 : 4) * DG;
-  __shared__ __align__(16) unsigned char sh_book[SMEM_BOOK ? kDqSmemBytes : 16];
+  __shared__ __align__(16) unsigned char sh_book[SMEM_BOOK ? staged_bytes(M, kCwBytes) : 16];
   const void* book = codebooks;
   pdl_wait();
   if (SMEM_BOOK) {
@@ -171,9 +174,9 @@ cudaError_t launch_s(const pvt_layer& L, uint64_t G, void* W_hat, uint32_t* stat
 template <int M, bool CB_F16, bool CODE_U16, bool OUT_F16, int DG = 8>
 cudaError_t launch_t(const pvt_layer& L, uint64_t G, void* W_hat, uint32_t* status, int sm_count,
                      cudaStream_t stream) {
-  // 32 KB: all that two to four codebooks can take; of one codebook, what leaves six blocks per SM resident
   if constexpr (M == 1) {
-    if ((uint64_t)L.codebook_size * ((CB_F16 ? 2 : 4) * DG) > (uint64_t)kDqSmemBytes)
+    constexpr int cw_bytes = (CB_F16 ? 2 : 4) * DG;
+    if ((uint64_t)L.codebook_size * cw_bytes > (uint64_t)staged_bytes(1, cw_bytes))
       return launch_s<M, CB_F16, CODE_U16, OUT_F16, false, DG>(L, G, W_hat, status, sm_count, stream);
   }
   return launch_s<M, CB_F16, CODE_U16, OUT_F16, true, DG>(L, G, W_hat, status, sm_count, stream);
