@@ -298,7 +298,6 @@ int pvt_vstep_trust(const pvt_layer* layer, uint64_t k_max, float ratio, uint32_
   timing_begin(kKernTrust, stream);
   if (e == cudaSuccess) e = launch_trust_rank(*layer, G, k_max, ws, t, stream);
   if (e == cudaSuccess) e = launch_trust_before_search(*layer, G, k_max, ws, t, stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(base + t.encode_off, 0, kWsHeaderBytes, stream);
   timing_end(kKernTrust, stream);
   if (e != cudaSuccess) return fail_cuda(e);
   rc = pvt_vstep_encode(layer, idx_sel, k_max, nullptr, base + t.encode_off, t.bytes - t.encode_off, cuda_stream);

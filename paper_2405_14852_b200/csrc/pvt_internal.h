@@ -131,13 +131,14 @@ struct TrustLayout {
   size_t idx_off;       // u32 [k]: the selection, ascending
   size_t pairs_a_off;   // u64 [k]: (inverted key, position) pairs; the sorted order ends here
   size_t pairs_b_off;   // u64 [k]: second sort buffer, afterwards f64 [k] squared changes by rank
-  size_t counts_off;    // u32 [256 * sort_blocks]
+  size_t counts_off;    // u32 [4 or 1][256][sort_stride], afterwards f64: the changes' sums by block
   size_t saved_off;     // u32 [k]: previous codes by position
   size_t partial_off;   // f64 [norm_blocks]
   size_t stats_off;     // f64 [2] + ticket
   size_t encode_off;    // workspace of the search kernels (own header)
   size_t bytes;
-  uint32_t sort_blocks, norm_blocks;
+  uint32_t sort_blocks, sort_stride, sort_rounds, norm_blocks;
+  bool sort_direct;     // few blocks: one kernel per digit, with counts of all four digits
 };
 TrustLayout trust_layout(uint64_t G, uint64_t k, size_t encode_bytes, int sm_count);
 cudaError_t launch_trust_rank(const pvt_layer& L, uint64_t G, uint64_t k, void* ws, const TrustLayout& t,

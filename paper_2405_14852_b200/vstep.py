@@ -117,8 +117,8 @@ class VStepLayer:
             self._ws = torch.empty(need, dtype=torch.uint8, device=self.W.device)
             B.pvt_workspace_init(self._ws)
         idx = torch.empty(k_max, dtype=torch.int32, device=self.W.device)
-        n = torch.zeros(1, dtype=torch.int64, device=self.W.device)
-        stats = torch.zeros(2, dtype=torch.float64, device=self.W.device)
+        n = torch.empty(1, dtype=torch.int64, device=self.W.device)
+        stats = torch.empty(2, dtype=torch.float64, device=self.W.device)
         B.pvt_vstep_trust(self.desc, k_max, ratio, idx, n, stats, self._ws)
         return idx, n, stats
 
