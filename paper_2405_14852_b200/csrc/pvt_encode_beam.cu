@@ -237,6 +237,7 @@ template <int M, bool TC>
 __global__ void __launch_bounds__(kBsThreads) beam_image_kernel(const BeamParams p, BeamImage<M, TC>* __restrict__ img) {
   __shared__ float red[kBsWarps][4];
   pdl_trigger();
+  pdl_wait();
   BeamImage<M, TC>& sm = *img;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool real = (uint32_t)tid < p.K;
@@ -878,9 +879,9 @@ cudaError_t launch_beam(const BeamParams& p, unsigned char* image_at, int sm_cou
   if (err != cudaSuccess) return err;
   Image* image = reinterpret_cast<Image*>(image_at);
   timing_begin(kKernEncodeAux, stream);
-  beam_image_kernel<M, TC><<<1, kBsThreads, 0, stream>>>(p, image);
+  err = launch_dependent(beam_image_kernel<M, TC>, 1, kBsThreads, 0, stream, p, image);
   timing_end(kKernEncodeAux, stream);
-  if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  if (err != cudaSuccess) return err;
   constexpr uint64_t fit = (228 * 1024) / (smem + 1024);
   constexpr uint64_t per_sm = fit < kBsCtasPerSm ? fit : kBsCtasPerSm;  // persistent: the resident CTAs
   const uint64_t groups = (p.k + kBsGroup - 1) / kBsGroup, want = (groups + kBsWarps - 1) / kBsWarps;

@@ -453,11 +453,13 @@ __global__ void __launch_bounds__(256) rescore_m1_kernel(const EncM1Params p) {
         }
       }
     }
-    if (p.exc_count && on) {  // codewords whose fast score is not trustworthy: always evaluated
-      const uint32_t n_exc = __ldg(p.exc_count);
-      for (uint32_t e = l; e < n_exc && e < p.K; e += kRsLanes) {
-        const uint32_t kappa = __ldg(p.exc_list + e);
-        if (kappa < p.K) take(kappa);
+    if (p.any_exc && on && __ldg(p.any_exc) != 0) {  // codewords whose fast score is not trustworthy: always evaluated
+      for (uint32_t b = 0; b < p.exc_blocks; ++b) {
+        const uint32_t n = __ldg(p.n_exc + b);
+        for (uint32_t e = l; e < n && e < p.exc_per_block; e += kRsLanes) {
+          const uint32_t kappa = __ldg(p.exc_list + (size_t)b * p.exc_per_block + e);
+          if (kappa < p.K) take(kappa);
+        }
       }
     }
   };
@@ -533,7 +535,7 @@ cudaError_t launch_encode_m1(const pvt_layer& L, uint64_t G, const uint32_t* idx
   p.unit_cw = kChunkCodewords;
   p.sub_cw = kSubCodewords;
   p.rel_margin = 0.0f;
-  p.exc_count = nullptr;
+  p.any_exc = nullptr;
   p.exc_list = nullptr;
   p.K = (uint32_t)L.codebook_size;
   p.n_tiles = lay.n_tiles;

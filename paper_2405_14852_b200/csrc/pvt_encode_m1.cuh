@@ -37,7 +37,10 @@ struct EncM1Params {
   uint32_t K, n_tiles, n_slices, tile;
   uint32_t n_units, unit_cw;  // the codebook is cut into n_units units of unit_cw codewords; a slice is a run of whole units
   uint32_t sub_cw;            // codewords per remembered sub-chunk (a multiple of 32 that divides unit_cw)
-  const uint32_t* exc_count;  // codewords the fast score cannot represent: always rescored (may be null)
+  // codewords the fast score cannot represent, always rescored: their number (may be null), and by block of codewords the
+  // number and the places in the list
+  const uint32_t *any_exc, *n_exc;
+  uint32_t exc_blocks, exc_per_block;
   const uint32_t* exc_list;
   uint32_t* gbest;
   float* margin;      // rounding-error margin of each target's fast scores, to which

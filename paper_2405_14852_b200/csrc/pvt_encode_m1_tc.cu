@@ -76,6 +76,15 @@ constexpr int kTcStages = 2;            // codebook stages (eight steps each: 32
 constexpr int kTcEpiThreads = 512;      // two sets of 256, one thread per target each: even and odd steps
 constexpr int kTcEpiWarps = kTcEpiThreads / 32;
 constexpr int kTcThreads = kTcEpiThreads + 160;  // + producer warp + one MMA warp per A block and accumulator buffer
+// What the search has to know of the codewords, by block of 256 of them: written by the kernel that prepares the image, so
+// that nothing has to be cleared before it.
+constexpr uint32_t kTcPrepCw = 256;
+static_assert(65536 / kTcPrepCw <= kTcTile, "one thread of the search per block");
+struct TcStats {
+  uint32_t any_exc;  // exceptions of all blocks
+  uint32_t n_exc[65536 / kTcPrepCw];  // exceptions of a block, listed from its first place in the list on
+  uint2 norms[65536 / kTcPrepCw];     // bit pattern of the largest ||c||^2; 0x7f800000 - that of the smallest (zero: none)
+};
 constexpr uint32_t kTmemCols = 512;
 constexpr float kMaxHalfNorm = 60000.0f;  // largest ||c||^2/2 the image represents
 constexpr float kNegInf = -__builtin_huge_valf();
@@ -136,7 +145,7 @@ EncodeM1TcLayout encode_m1_tc_layout(uint32_t K, uint64_t k, int sm_count, int g
   e.bimg_off = kWsHeaderBytes;
   e.stats_off = align_up(e.bimg_off + (size_t)e.n_steps * (group_dim == 16 ? TcDim<16>::kStepBytes : kTcStepBytes),
                          kWsAlign);
-  e.exc_off = e.stats_off + kWsAlign;
+  e.exc_off = align_up(e.stats_off + sizeof(TcStats), kWsAlign);
   e.gbest_off = align_up(e.exc_off + sizeof(uint32_t) * K, kWsAlign);
   e.margin_off = align_up(e.gbest_off + sizeof(uint32_t) * k, kWsAlign);
   e.rec_off = align_up(e.margin_off + sizeof(float) * k, kWsAlign);
@@ -146,21 +155,19 @@ EncodeM1TcLayout encode_m1_tc_layout(uint32_t K, uint64_t k, int sm_count, int g
 
 namespace {
 
-// stats block in the workspace: [0] bit pattern of max ||c||^2 over representable codewords, [1] exception count
-struct TcStats {
-  uint32_t n2max_bits;
-  uint32_t exc_count;
-  uint32_t n2min_inv;  // 0x7f800000 - bit pattern of the smallest ||c||^2 of those (zero: none)
-};
-
 // ---- codebook image ------------------------------------------------------------
 template <int DG>
-__global__ void __launch_bounds__(256) tc_prep_kernel(const uint4* __restrict__ book, uint32_t K, uint32_t n_steps,
+__global__ void __launch_bounds__(kTcPrepCw) tc_prep_kernel(const uint4* __restrict__ book, uint32_t K, uint32_t n_steps,
                                                        unsigned char* __restrict__ bimg, TcStats* stats,
                                                        uint32_t* __restrict__ exc_list, uint32_t* __restrict__ gbest,
                                                        uint64_t k) {
   using D = TcDim<DG>;
-  pdl_trigger();  // the search forms its targets meanwhile
+  __shared__ uint32_t sh_exc, sh_max, sh_inv;
+  if (threadIdx.x == 0) sh_exc = sh_max = sh_inv = 0;
+  pdl_wait();
+  // The search forms its targets meanwhile, from memory that this kernel does not write: so not before the wait.
+  pdl_trigger();
+  __syncthreads();
   for (uint64_t n = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; n < k; n += (uint64_t)gridDim.x * blockDim.x)
     gbest[n] = 0xffffffffu;
   const uint32_t kappa = blockIdx.x * blockDim.x + threadIdx.x;
@@ -187,8 +194,7 @@ __global__ void __launch_bounds__(256) tc_prep_kernel(const uint4* __restrict__ 
     }
     const bool rep = real && (0.5f * n2 <= kMaxHalfNorm);  // false for NaN / Inf as well
     if (real && !rep) {
-      const uint32_t pos = atomicAdd(&stats->exc_count, 1u);
-      if (pos < K) exc_list[pos] = kappa;
+      exc_list[blockIdx.x * kTcPrepCw + atomicAdd(&sh_exc, 1u)] = kappa;
     }
     if (rep) {
       n2bits = __float_as_uint(n2);
@@ -221,8 +227,13 @@ __global__ void __launch_bounds__(256) tc_prep_kernel(const uint4* __restrict__ 
   n2bits = __reduce_max_sync(0xffffffffu, n2bits);
   n2inv = __reduce_max_sync(0xffffffffu, n2inv);
   if ((threadIdx.x & 31) == 0) {
-    if (n2bits > __ldcg(&stats->n2max_bits)) atomicMax(&stats->n2max_bits, n2bits);
-    if (n2inv > __ldcg(&stats->n2min_inv)) atomicMax(&stats->n2min_inv, n2inv);
+    atomicMax(&sh_max, n2bits);
+    atomicMax(&sh_inv, n2inv);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && blockIdx.x * kTcPrepCw < n_steps * kTcStepCw) {
+    stats->n_exc[blockIdx.x] = sh_exc;
+    stats->norms[blockIdx.x] = make_uint2(sh_max, sh_inv);
   }
 }
 
@@ -332,12 +343,13 @@ struct TcSmem {
   uint32_t odd_cnt[kTcTile], odd_evicted[kTcTile];
   uint32_t tmem_base;
   uint32_t abort_flag;
+  uint32_t n2max_bits, n2min_inv, n_exc;  // over all codewords
 };
 
 template <int DG>
 __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1Params p,
                                                                       const unsigned char* __restrict__ bimg,
-                                                                      const TcStats* __restrict__ stats) {
+                                                                      TcStats* __restrict__ stats) {
   using D = TcDim<DG>;
   constexpr int kStepBytes = D::kStepBytes;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -347,6 +359,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
 
   if (tid == 0) {
     sm.abort_flag = 0;
+    sm.n2max_bits = sm.n2min_inv = sm.n_exc = 0;
     for (int s = 0; s < kTcStages; ++s) {
       mbar_init(smem_u32(&sm.full_bar[s]), 1);
       mbar_init(smem_u32(&sm.empty_bar[s]), 4);  // one commit per MMA warp, at the stage's last step
@@ -552,10 +565,24 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
             }
           }
         }
-        pdl_wait();  // the image's statistics (and the initial minima)
-        const float n2max = __uint_as_float(stats->n2max_bits);
+        if (u == blockIdx.x) {
+          pdl_wait();  // the image's statistics (and the initial minima)
+          const uint2 part = own < p.exc_blocks ? __ldcg(&stats->norms[own]) : make_uint2(0, 0);
+          const uint32_t n2bits = __reduce_max_sync(0xffffffffu, part.x), n2inv = __reduce_max_sync(0xffffffffu, part.y);
+          if (lane == 0) {
+            atomicMax(&sm.n2max_bits, n2bits);
+            atomicMax(&sm.n2min_inv, n2inv);
+          }
+          if (blockIdx.x == 0) {  // for the rescoring kernel
+            const uint32_t exc = __reduce_add_sync(0xffffffffu, own < p.exc_blocks ? __ldcg(&stats->n_exc[own]) : 0u);
+            if (lane == 0) atomicAdd(&sm.n_exc, exc);
+          }
+          asm volatile("bar.sync 2, %0;" ::"n"(kTcTile) : "memory");
+          if (blockIdx.x == 0 && own == 0) stats->any_exc = sm.n_exc;
+        }
+        const float n2max = __uint_as_float(sm.n2max_bits);
         const float cnmax = sqrtf(n2max), hmax = 0.5f * n2max;
-        const float cnmin = sqrtf(__uint_as_float(0x7f800000u - stats->n2min_inv));  // (infinite if there is none)
+        const float cnmin = sqrtf(__uint_as_float(0x7f800000u - sm.n2min_inv));  // (infinite if there is none)
         float m = 0.0f, nt2 = 0.0f;
 #pragma unroll
         for (int i = 0; i < DG; ++i) {
@@ -728,14 +755,13 @@ cudaError_t launch_tc(const pvt_layer& L, const EncM1Params& p, const EncodeM1Tc
   const uint32_t n_cw = lay.n_steps * kTcStepCw;
   // enough threads for one codeword each, and for no more than four of the initial minima each until the chip is full
   const uint64_t fill = (p.k + 1023) / 1024 < 592 ? (p.k + 1023) / 1024 : 592;
-  const uint32_t image = (n_cw + 255) / 256;
-  tc_prep_kernel<DG><<<fill > image ? (unsigned)fill : image, 256, 0, stream>>>(
-      reinterpret_cast<const uint4*>(L.codebooks), p.K, lay.n_steps,
-      reinterpret_cast<unsigned char*>(base + lay.bimg_off), stats, reinterpret_cast<uint32_t*>(base + lay.exc_off),
-      p.gbest, p.k);
+  const uint32_t image = (n_cw + kTcPrepCw - 1) / kTcPrepCw;
+  cudaError_t err = launch_dependent(tc_prep_kernel<DG>, fill > image ? (unsigned)fill : image, kTcPrepCw, 0, stream,
+                                     reinterpret_cast<const uint4*>(L.codebooks), p.K, lay.n_steps,
+                                     reinterpret_cast<unsigned char*>(base + lay.bimg_off), stats,
+                                     reinterpret_cast<uint32_t*>(base + lay.exc_off), p.gbest, p.k);
   count_launches(1);
   timing_end(kKernEncodeAux, stream);
-  cudaError_t err = cudaGetLastError();
   if (err != cudaSuccess) return err;
   const size_t smem = sizeof(TcSmem<DG>);
   if ((err = allow_smem(encode_m1_tc_kernel<DG>)) != cudaSuccess) return err;
@@ -767,7 +793,7 @@ cudaError_t launch_encode_m1_tc(const pvt_layer& L, uint64_t G, const uint32_t* 
   p.dg = (uint32_t)L.group_dim;
   p.eta = L.eta;
   p.cbx = nullptr;
-  p.n2max_bits = &stats->n2max_bits;
+  p.n2max_bits = nullptr;
   p.K = (uint32_t)L.codebook_size;
   p.n_tiles = lay.n_tiles;
   p.n_slices = lay.n_slices;
@@ -776,7 +802,10 @@ cudaError_t launch_encode_m1_tc(const pvt_layer& L, uint64_t G, const uint32_t* 
   p.unit_cw = kTcStepCw;
   p.sub_cw = kTcSubCw;
   p.rel_margin = rel_margin(L.group_dim);
-  p.exc_count = &stats->exc_count;
+  p.any_exc = &stats->any_exc;
+  p.n_exc = stats->n_exc;
+  p.exc_blocks = (lay.n_steps * kTcStepCw + kTcPrepCw - 1) / kTcPrepCw;
+  p.exc_per_block = kTcPrepCw;
   p.exc_list = reinterpret_cast<const uint32_t*>(base + lay.exc_off);
   p.gbest = reinterpret_cast<uint32_t*>(base + lay.gbest_off);
   p.margin = reinterpret_cast<float*>(base + lay.margin_off);
@@ -790,9 +819,8 @@ cudaError_t launch_encode_m1_tc(const pvt_layer& L, uint64_t G, const uint32_t* 
   p.max_spins = hook.max_spins;
   p.withhold_copy = hook.withhold_copy;
 
-  cudaError_t err = cudaMemsetAsync(stats, 0, sizeof(TcStats), stream);
-  if (err != cudaSuccess) return err;
-  err = L.group_dim == 16 ? launch_tc<16>(L, p, lay, base, stats, stream) : launch_tc<8>(L, p, lay, base, stats, stream);
+  const cudaError_t err =
+      L.group_dim == 16 ? launch_tc<16>(L, p, lay, base, stats, stream) : launch_tc<8>(L, p, lay, base, stats, stream);
   if (err != cudaSuccess) return err;
   return launch_rescore_m1(p, true, stream);
 }

@@ -108,6 +108,7 @@ __global__ void __launch_bounds__(kPsThreads) pstep_grad_kernel(const float* __r
   __shared__ __align__(16) double sh_prod[kPsThreads / 32][32][DG];
   constexpr uint32_t kFull = 0xffffffffu;
   constexpr int PER = 32 / DG;  // groups per instruction of the reductions
+  pdl_trigger();
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane / DG, e = lane % DG;
   const bool wide = (reinterpret_cast<uintptr_t>(g) & 31u) == 0;
   const uint64_t stride = 32 * (uint64_t)gridDim.x * (kPsThreads / 32);
@@ -205,6 +206,7 @@ __global__ void __launch_bounds__(kPsSmallThreads, 2) pstep_grad_small_kernel(co
                                                                               uint32_t* status) {
   extern __shared__ __align__(16) unsigned char ps_smem[];
   constexpr uint32_t kFull = 0xffffffffu;
+  pdl_trigger();
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t n_bins = M * K, per = (n_bins + kPsSmallThreads - 1) / kPsSmallThreads;
   double* acc = reinterpret_cast<double*>(ps_smem);              // [M K][8]
@@ -390,6 +392,8 @@ __global__ void __launch_bounds__(256) adam_kernel(float* __restrict__ param, __
                                                     const double* __restrict__ grad, float* __restrict__ exp_avg,
                                                     float* __restrict__ exp_avg_sq, uint64_t n, float lr, float beta1,
                                                     float beta2, float eps, float bias1, float bias2) {
+  pdl_trigger();
+  pdl_wait();
   const float omb1 = __fsub_rn(1.0f, beta1), omb2 = __fsub_rn(1.0f, beta2);
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
     const float gr = __double2float_rn(grad[i]);
@@ -411,6 +415,8 @@ __global__ void __launch_bounds__(256) adam_direction_kernel(const float4* __res
                                                               float4* __restrict__ exp_avg_sq, float4* __restrict__ dir,
                                                               uint64_t n4, float beta1, float beta2, float eps,
                                                               float bias1, float bias2) {
+  pdl_trigger();
+  pdl_wait();
   const float omb1 = __fsub_rn(1.0f, beta1), omb2 = __fsub_rn(1.0f, beta2);
   auto one = [&](float gr, float& m, float& v) {
     m = __fmaf_rn(beta1, m, __fmul_rn(omb1, gr));
@@ -437,12 +443,13 @@ cudaError_t launch_adam_direction(const float* grad, float* exp_avg, float* exp_
                                   cudaStream_t stream) {
   timing_begin(kKernAdam, stream);
   const uint64_t n4 = n / 4, want = (n4 + 255) / 256, cap = (uint64_t)sm_count * 8;
-  adam_direction_kernel<<<(unsigned)(want < cap ? want : cap), 256, 0, stream>>>(
-      reinterpret_cast<const float4*>(grad), reinterpret_cast<float4*>(exp_avg), reinterpret_cast<float4*>(exp_avg_sq),
-      reinterpret_cast<float4*>(dir), n4, beta1, beta2, eps, bias1, bias2);
+  const cudaError_t err = launch_dependent(
+      adam_direction_kernel, (unsigned)(want < cap ? want : cap), 256, 0, stream, reinterpret_cast<const float4*>(grad),
+      reinterpret_cast<float4*>(exp_avg), reinterpret_cast<float4*>(exp_avg_sq), reinterpret_cast<float4*>(dir), n4, beta1,
+      beta2, eps, bias1, bias2);
   count_launches(1);
   timing_end(kKernAdam, stream);
-  return cudaGetLastError();
+  return err;
 }
 
 cudaError_t launch_pstep_grad(const pvt_layer& L, uint64_t G, double* grad_books, double* grad_scale, uint32_t* status,
@@ -485,12 +492,12 @@ cudaError_t launch_adam(float* param, void* param_f16, const double* grad, float
                         int sm_count, cudaStream_t stream) {
   timing_begin(kKernAdam, stream);
   const uint64_t want = (n + 255) / 256, cap = (uint64_t)sm_count * 8;
-  adam_kernel<<<(unsigned)(want < cap ? want : cap), 256, 0, stream>>>(param, reinterpret_cast<__half*>(param_f16), grad,
-                                                                      exp_avg, exp_avg_sq, n, lr, beta1, beta2, eps,
-                                                                      bias1, bias2);
+  const cudaError_t err =
+      launch_dependent(adam_kernel, (unsigned)(want < cap ? want : cap), 256, 0, stream, param,
+                       reinterpret_cast<__half*>(param_f16), grad, exp_avg, exp_avg_sq, n, lr, beta1, beta2, eps, bias1, bias2);
   count_launches(1);
   timing_end(kKernAdam, stream);
-  return cudaGetLastError();
+  return err;
 }
 
 }  // namespace pvt

@@ -194,7 +194,8 @@ __device__ __forceinline__ void find_digit_warp(const uint32_t* hist, uint32_t k
 
 // ---- 0. everything the passes count in starts at zero
 __global__ void __launch_bounds__(kSelThreads) select_clear_kernel(uint4* scratch, uint32_t n16) {
-  pdl_trigger();
+  pdl_wait();
+  pdl_trigger();  // (after the wait: the next kernel reads g and writes keys before its own)
   for (uint32_t i = blockIdx.x * kSelThreads + threadIdx.x; i < n16; i += gridDim.x * kSelThreads)
     scratch[i] = make_uint4(0, 0, 0, 0);
 }
@@ -442,6 +443,8 @@ __global__ void __launch_bounds__(kSelThreads) select_write_kernel(const SelPara
 }
 
 __global__ void iota_kernel(uint32_t* idx_out, uint64_t k) {
+  pdl_trigger();
+  pdl_wait();
   const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < k) idx_out[i] = (uint32_t)i;
 }
@@ -479,8 +482,7 @@ cudaError_t launch_select_keyed(const pvt_layer& L, uint64_t G, uint64_t k, uint
   timing_begin(kKernSelect, stream);
   cudaError_t err;
   if (k == G && key_mode != kKeyNormBuffer) {  // every group is taken: the ascending index list itself
-    iota_kernel<<<(unsigned)((k + 255) / 256), 256, 0, stream>>>(idx_out, k);
-    err = cudaGetLastError();
+    err = launch_dependent(iota_kernel, (unsigned)((k + 255) / 256), 256, 0, stream, idx_out, k);
   } else {
     const SelectLayout lay = select_layout(G);
     char* base = static_cast<char*>(ws);
@@ -507,9 +509,8 @@ cudaError_t launch_select_keyed(const pvt_layer& L, uint64_t G, uint64_t k, uint
     if (n_cta > most) n_cta = most;
     p.words = (uint32_t)(((G + n_cta - 1) / n_cta + 31) / 32);
     constexpr uint32_t n16 = kSelScratchWords / 4;
-    select_clear_kernel<<<(n16 + kSelThreads - 1) / kSelThreads, kSelThreads, 0, stream>>>(
-        reinterpret_cast<uint4*>(scratch), n16);
-    err = cudaGetLastError();
+    err = launch_dependent(select_clear_kernel, (n16 + kSelThreads - 1) / kSelThreads, kSelThreads, 0, stream,
+                           reinterpret_cast<uint4*>(scratch), n16);
     if (err == cudaSuccess)
       err = L.group_dim == 16 ? launch_group<16>(key_mode, p, sm_count, stream)
                               : launch_group<8>(key_mode, p, sm_count, stream);
