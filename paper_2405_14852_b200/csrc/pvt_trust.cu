@@ -19,7 +19,8 @@
 //   cut            running sum of the blocks, first position that breaks the bound
 //   restore        previous codes for every position from the cut on
 // Bound by the latency of these short dependent kernels: each is launched while the one before it runs, and up to
-// kSortDirect blocks a radix pass is one kernel.  (Three plain launches per pass: step of 4096x4096, k = 20971, 306 us; now 218.)
+// kSortDirect blocks a radix pass is one kernel.  (Three plain launches per pass: step of 4096x4096, k = 20971, 306 us;
+// now 218.)
 #include <cuda_fp16.h>
 
 #include "pvt_internal.h"
