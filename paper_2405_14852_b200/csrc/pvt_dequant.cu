@@ -1,6 +1,6 @@
 // dequantize_weights (Algorithm 3, first line): W_hat = s_row * sum_m C_m[b_m] for
 // every weight group.  Streaming kernel, persistent grid: one thread per 16 bytes of the
-// result, four of them in flight per thread, codes read coalesced, codewords gathered from
+// result, two of them in flight per thread, codes read coalesced, codewords gathered from
 // the L2-resident codebook (small ones are first copied to shared memory), and a
 // warp's stores contiguous: 512 bytes per instruction.
 //
@@ -16,7 +16,7 @@ namespace pvt {
 namespace {
 
 constexpr int kDqThreads = 256;
-constexpr int kDqUnroll = 4;             // pieces of 16 result bytes in flight per thread
+constexpr int kDqUnroll = 2;  // pieces of 16 result bytes in flight per thread (5120x5120 2x8 fp16 14.0 us; four 14.8, eight 19.8)
 // Codebooks of up to this size are staged in shared memory: two to four always (256 codewords each at most), one if it is
 // small.  No more than that is reserved, for it costs resident blocks (32 KB for all: 11008x4096 2x8 39 us after the
 // search instead of 32).
