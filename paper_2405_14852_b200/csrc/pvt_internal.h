@@ -188,6 +188,11 @@ __device__ __forceinline__ void load8(const float* p, bool wide, float* v) {
     v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
   }
 }
+// Asks for `bytes` (a multiple of 16, from a 16-byte boundary) to be brought into the L2.  It reads nothing, so it may
+// stand before pdl_wait(): whoever writes there meanwhile writes in the same L2.
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void store8(float* p, bool wide, const float* v) {
   if (wide) {
     asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
@@ -203,9 +208,11 @@ __device__ __forceinline__ void store8(float* p, bool wide, const float* v) {
 // ---- programmatic dependent launch --------------------------------------------------------------------
 // Consecutive kernels of a call depend on one another, so between two of them the GPU would idle for a launch
 // latency.  A kernel launched with launch_dependent() may be scheduled while the kernel before it on the stream
-// is still running; it must execute pdl_wait() before its first access to global memory, which returns once
-// that kernel has completed and its writes are visible.  Every kernel of a chain calls pdl_trigger() at its
-// start to allow the one after it to be scheduled early.  Both are no-ops for a kernel launched the plain way.
+// is still running; every thread of it must execute pdl_wait() before its first access to global memory, which
+// returns once that kernel has completed and its writes are visible.  There is no exception for what an earlier
+// kernel of the chain wrote, or the caller: the wait is what makes it visible to this grid.  (A prefetch into the L2
+// is no access.)  Every kernel of a chain calls pdl_trigger() at its start to allow the one after it to be scheduled
+// early.  Both are no-ops for a kernel launched the plain way.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

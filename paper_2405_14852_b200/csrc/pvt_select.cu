@@ -5,7 +5,7 @@
 //
 // Four kernels, each launched before the one ahead of it has finished.  What bounds them is the one pass over g (32 B
 // per group); the others read keys that are in the L2 and cost little more than their launches:
-//   0. clear:  zeroes the histograms, beside pass 1
+//   0. clear:  zeroes the histograms; meanwhile the first 64 KB of g per block of pass 1 come to the L2
 //   1. keys:   32 bytes per thread and load, four groups in flight per thread; writes the key of every group and sums
 //              up key bits [30:18] -- 32 bins per octave, so that the threshold bin of ordinary updates holds a
 //              fraction of a per cent of the groups
@@ -192,10 +192,10 @@ __device__ __forceinline__ void find_digit_warp(const uint32_t* hist, uint32_t k
   *left = __shfl_sync(0xffffffffu, l, src);
 }
 
-// ---- 0. everything the passes count in starts at zero
+// ---- 0. what pass 1 adds to starts at zero
 __global__ void __launch_bounds__(kSelThreads) select_clear_kernel(uint4* scratch, uint32_t n16) {
+  pdl_trigger();
   pdl_wait();
-  pdl_trigger();  // (after the wait: the next kernel reads g and writes keys before its own)
   for (uint32_t i = blockIdx.x * kSelThreads + threadIdx.x; i < n16; i += gridDim.x * kSelThreads)
     scratch[i] = make_uint4(0, 0, 0, 0);
 }
@@ -207,8 +207,15 @@ __global__ void __launch_bounds__(kNormThreads, kNormCtas) select_keys_kernel(co
   const uint32_t tid = threadIdx.x;
   pdl_trigger();
   for (uint32_t i = tid; i < kSelBins0; i += kNormThreads) hist[i] = 0;
-  __syncthreads();
   constexpr int U = (DG == 16 ? 2 : 4) / (MODE == kKeyNormBuffer ? 2 : 1);  // groups in flight per thread
+  const uint64_t first = (uint64_t)blockIdx.x * (U * kNormThreads);
+  if (tid == 0 && MODE != kKeyUniform && first < p.G) {  // what the block reads first comes to the L2 while it waits
+    const uint64_t n = p.G - first < U * kNormThreads ? p.G - first : U * kNormThreads;
+    prefetch_l2(p.g + first * DG, (uint32_t)(n * DG * sizeof(float)));
+    if (MODE == kKeyNormBuffer) prefetch_l2(p.buffer + first * DG, (uint32_t)(n * DG * sizeof(float)));
+  }
+  __syncthreads();
+  pdl_wait();
   const bool wide = ((reinterpret_cast<uintptr_t>(p.g) |
                       (MODE == kKeyNormBuffer ? reinterpret_cast<uintptr_t>(p.buffer) : 0)) & 31u) == 0;
   const uint64_t stride = (uint64_t)gridDim.x * (U * kNormThreads);
@@ -266,7 +273,6 @@ __global__ void __launch_bounds__(kNormThreads, kNormCtas) select_keys_kernel(co
     }
   }
   __syncthreads();
-  pdl_wait();  // the sums have been cleared
   for (uint32_t i = tid; i < kSelBins0; i += kNormThreads)
     if (hist[i]) atomicAdd(&p.hist0[i], hist[i]);
 }
