@@ -164,9 +164,8 @@ __global__ void __launch_bounds__(kTcPrepCw) tc_prep_kernel(const uint4* __restr
   using D = TcDim<DG>;
   __shared__ uint32_t sh_exc, sh_max, sh_inv;
   if (threadIdx.x == 0) sh_exc = sh_max = sh_inv = 0;
-  pdl_wait();
-  // The search forms its targets meanwhile, from memory that this kernel does not write: so not before the wait.
   pdl_trigger();
+  pdl_wait();
   __syncthreads();
   for (uint64_t n = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; n < k; n += (uint64_t)gridDim.x * blockDim.x)
     gbest[n] = 0xffffffffu;
@@ -383,13 +382,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
   tc_fence_after();
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(&sm.tmem_base);
 
+  pdl_wait();
   const uint64_t units = (uint64_t)p.n_tiles * p.n_slices;
 
   if (warp == kTcEpiWarps) {
     // ------------------------------------------------------------ bulk-copy producer
     // (the whole warp runs the loop, lane 0 issues the copies: no lane waits at the final barrier meanwhile)
     {
-      pdl_wait();  // the image
       // total number of steps of this CTA (for the byte count of the last, partial stage)
       uint32_t total = 0;
       for (uint64_t u = blockIdx.x; u < units; u += gridDim.x) {
@@ -566,7 +565,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
           }
         }
         if (u == blockIdx.x) {
-          pdl_wait();  // the image's statistics (and the initial minima)
           const uint2 part = own < p.exc_blocks ? __ldcg(&stats->norms[own]) : make_uint2(0, 0);
           const uint32_t n2bits = __reduce_max_sync(0xffffffffu, part.x), n2inv = __reduce_max_sync(0xffffffffu, part.y);
           if (lane == 0) {

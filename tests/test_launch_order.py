@@ -49,7 +49,7 @@ def test_the_kernels_are_found():
     assert "dequant_kernel" in dependent_kernels(code_of("pvt_dequant.cu"))
 
 
-@pytest.mark.parametrize("name", ["pvt_select.cu"])
+@pytest.mark.parametrize("name", sources())
 def test_dependent_kernels_wait_before_they_touch_memory(name):
     for kernel, (params, body) in dependent_kernels(code_of(name)).items():
         at = body.find("pdl_wait()")
