@@ -53,11 +53,9 @@ __device__ __forceinline__ void load_part(const void* book, uint32_t code, uint3
 // thread: 11008x4096 3x8 43.5 us instead of 29.8, 5120x5120 2x8 19.6 instead of 14.7.  fp32 results with eight:
 // 11008x4096 2x8 45 us instead of 31.7, 32 bytes per lane are stored more slowly.)
 template <int M, bool CB_F16, bool CODE_U16, bool OUT_F16, bool SMEM_BOOK, int DG>
-__global__ void __launch_bounds__(kDqThreads) dequant_kernel(const void* __restrict__ codebooks,
-                                                              const void* __restrict__ codes,
-                                                              const float* __restrict__ scale, uint64_t G,
-                                                              FastDiv gpr, uint32_t K, void* __restrict__ W_hat,
-                                                              uint32_t* status) {
+__global__ void __launch_bounds__(kDqThreads) dequant_kernel(const void* codebooks, const void* codes,
+                                                              const float* scale, uint64_t G, FastDiv gpr, uint32_t K,
+                                                              void* __restrict__ W_hat, uint32_t* status) {
   constexpr int EL = OUT_F16 ? 8 : 4, PARTS = DG / EL;
   constexpr int kCwBytes = (CB_F16 ? 2 : 4) * DG;
   __shared__ __align__(16) unsigned char sh_book[SMEM_BOOK ? staged_bytes(M, kCwBytes) : 16];
@@ -73,13 +71,14 @@ __global__ void __launch_bounds__(kDqThreads) dequant_kernel(const void* __restr
   }
   // kDqUnroll parts per thread and iteration, a block apart, all their loads issued
   // before the first use: the code -> codeword -> store chain of one group is two
-  // dependent memory round trips, so several must be in flight per thread
+  // dependent memory round trips, so several must be in flight per thread; the codes
+  // and scales of the next iteration are asked for ahead of this one's stores (with the
+  // loads behind the stores 11008x4096 2x8 fp32 takes 9 us more)
   const uint64_t H = (uint64_t)PARTS * G;
   const uint64_t stride = (uint64_t)gridDim.x * (kDqThreads * kDqUnroll);
-  for (uint64_t base = (uint64_t)blockIdx.x * (kDqThreads * kDqUnroll); base < H; base += stride) {
-    uint32_t b[kDqUnroll][M];
-    float s[kDqUnroll];
-    bool bad = false;
+  uint32_t b[kDqUnroll][M];
+  float s[kDqUnroll];
+  auto fetch = [&](uint64_t base) {
 #pragma unroll
     for (int u = 0; u < kDqUnroll; ++u) {
       const uint64_t h = base + (uint64_t)u * kDqThreads + threadIdx.x;
@@ -91,32 +90,40 @@ __global__ void __launch_bounds__(kDqThreads) dequant_kernel(const void* __restr
         if (CODE_U16) {
           const uint16_t* c = reinterpret_cast<const uint16_t*>(codes) + (size_t)j * M;
 #pragma unroll
-          for (int m = 0; m < M; ++m) b[u][m] = __ldg(c + m);
+          for (int m = 0; m < M; ++m) b[u][m] = c[m];
         } else if (M % 2 == 0) {  // two adjacent bytes at a time
           const uint16_t* c = reinterpret_cast<const uint16_t*>(codes) + (size_t)j * (M / 2);
 #pragma unroll
           for (int m = 0; m < M; m += 2) {
-            const uint16_t both = __ldg(c + m / 2);
+            const uint16_t both = c[m / 2];
             b[u][m] = both & 0xffu;
             b[u][(m + 1) % M] = both >> 8;
           }
         } else {
           const uint8_t* c = reinterpret_cast<const uint8_t*>(codes) + (size_t)j * M;
 #pragma unroll
-          for (int m = 0; m < M; ++m) b[u][m] = __ldg(c + m);
+          for (int m = 0; m < M; ++m) b[u][m] = c[m];
         }
-        s[u] = __ldg(scale + fast_div(j, gpr));  // row of group j (G < 2^32)
+        s[u] = scale[fast_div(j, gpr)];  // row of group j (G < 2^32)
+      }
+    }
+  };
+  uint64_t base = (uint64_t)blockIdx.x * (kDqThreads * kDqUnroll);
+  fetch(base);
+  for (; base < H; base += stride) {
+    bool bad = false;
 #pragma unroll
-        for (int m = 0; m < M; ++m) {
-          if (b[u][m] >= K) {
-            bad = true;
-            b[u][m] = 0;
-          }
+    for (int u = 0; u < kDqUnroll; ++u) {
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        if (b[u][m] >= K) {
+          bad = true;
+          b[u][m] = 0;
         }
       }
     }
     if (bad && status) atomicOr(status, PVT_DEV_BAD_CODE);
-    float v[kDqUnroll][EL];
+    float v[kDqUnroll][EL], row_scale[kDqUnroll];
 #pragma unroll
     for (int u = 0; u < kDqUnroll; ++u)
       load_part<CB_F16, EL, PARTS>(book, b[u][0], threadIdx.x % PARTS, v[u]);
@@ -131,11 +138,14 @@ __global__ void __launch_bounds__(kDqThreads) dequant_kernel(const void* __restr
       }
     }
 #pragma unroll
+    for (int u = 0; u < kDqUnroll; ++u) row_scale[u] = s[u];
+    fetch(base + stride);
+#pragma unroll
     for (int u = 0; u < kDqUnroll; ++u) {
       const uint64_t h = base + (uint64_t)u * kDqThreads + threadIdx.x;
       if (h >= H) continue;
 #pragma unroll
-      for (int i = 0; i < EL; ++i) v[u][i] = __fmul_rn(s[u], v[u][i]);
+      for (int i = 0; i < EL; ++i) v[u][i] = __fmul_rn(row_scale[u], v[u][i]);
       uint32_t w[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {

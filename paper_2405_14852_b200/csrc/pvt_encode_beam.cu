@@ -234,7 +234,7 @@ __device__ __forceinline__ bool fetch_image(void* dst, const void* src, uint32_t
 
 // ---- the codebook image: one block, one codeword of every codebook per thread (K <= 256 = block size) ----
 template <int M, bool TC>
-__global__ void __launch_bounds__(kBsThreads) beam_image_kernel(const BeamParams p, BeamImage<M, TC>* __restrict__ img) {
+__global__ void __launch_bounds__(kBsThreads) beam_image_kernel(const BeamParams p, BeamImage<M, TC>* img) {
   __shared__ float red[kBsWarps][4];
   pdl_trigger();
   pdl_wait();
@@ -442,7 +442,7 @@ __device__ __forceinline__ uint64_t team_flags(uint32_t mine, uint32_t my_b) {
 
 template <int M, bool TC>
 __global__ void __launch_bounds__(kBsThreads, kBsCtasPerSm) encode_beam_kernel(const BeamParams p,
-                                                                               const BeamImage<M, TC>* __restrict__ image) {
+                                                                               const BeamImage<M, TC>* image) {
   extern __shared__ __align__(16) unsigned char beam_smem[];
   BeamSmem<M, TC>& smem = *reinterpret_cast<BeamSmem<M, TC>*>(beam_smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -472,11 +472,11 @@ __global__ void __launch_bounds__(kBsThreads, kBsCtasPerSm) encode_beam_kernel(c
     uint32_t lane_j = kFull, lane_prev = 0;
     {
       const uint64_t n_mine = gi * kBsGroup + my_q;
-      if (n_mine < p.k) lane_j = __ldg(p.idx + n_mine);
+      if (n_mine < p.k) lane_j = p.idx[n_mine];
       float tv = 0.0f;
       if (lane_j < p.G) {
-        const float wv = __ldg(p.W + (size_t)lane_j * 8 + my_b), gv = __ldg(p.g + (size_t)lane_j * 8 + my_b);
-        const float sc = __ldg(p.scale + fast_div(lane_j, p.gpr));
+        const float wv = p.W[(size_t)lane_j * 8 + my_b], gv = p.g[(size_t)lane_j * 8 + my_b];
+        const float sc = p.scale[fast_div(lane_j, p.gpr)];
         if (M == 2) {
           const uint32_t both = reinterpret_cast<const uint16_t*>(p.codes)[lane_j];
           lane_prev = (both << 24) | ((both >> 8) << 16);

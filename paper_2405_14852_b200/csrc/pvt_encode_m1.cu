@@ -348,15 +348,15 @@ __global__ void __launch_bounds__(256) rescore_m1_kernel(const EncM1Params p) {
   uint4 raw0 = make_uint4(0x7f800000u, 0, 0, 0), raw1 = raw0;  // best = +inf: never within the limit
   if (active) {
     const uint32_t tile = (uint32_t)(n / p.tile), s = (uint32_t)(n % p.tile);
-    j = __ldg(p.idx + n);
+    j = p.idx[n];
     const float least = unord(p.gbest[n]);
     limit = p.margin[n];
     // (a least score of minus infinity marks a target that is rescored against the whole codebook)
     limit = fabsf(least) < 3.0e38f ? least + fmaf(p.rel_margin, fabsf(least), limit) : least;
     const uint4* rec = reinterpret_cast<const uint4*>(p.rec);
-    if ((uint32_t)l < p.n_slices) raw0 = __ldg(&rec[((size_t)tile * p.n_slices + l) * p.tile + s]);
+    if ((uint32_t)l < p.n_slices) raw0 = rec[((size_t)tile * p.n_slices + l) * p.tile + s];
     if ((uint32_t)l + kRsLanes < p.n_slices)
-      raw1 = __ldg(&rec[((size_t)tile * p.n_slices + l + kRsLanes) * p.tile + s]);
+      raw1 = rec[((size_t)tile * p.n_slices + l + kRsLanes) * p.tile + s];
     if (j >= p.G) {
       if (l == 0) atomicOr(p.status, PVT_DEV_BAD_INDEX);
       active = false;
@@ -453,11 +453,11 @@ __global__ void __launch_bounds__(256) rescore_m1_kernel(const EncM1Params p) {
         }
       }
     }
-    if (p.any_exc && on && __ldg(p.any_exc) != 0) {  // codewords whose fast score is not trustworthy: always evaluated
+    if (p.any_exc && on && *p.any_exc != 0) {  // codewords whose fast score is not trustworthy: always evaluated
       for (uint32_t b = 0; b < p.exc_blocks; ++b) {
-        const uint32_t n = __ldg(p.n_exc + b);
+        const uint32_t n = p.n_exc[b];
         for (uint32_t e = l; e < n && e < p.exc_per_block; e += kRsLanes) {
-          const uint32_t kappa = __ldg(p.exc_list + (size_t)b * p.exc_per_block + e);
+          const uint32_t kappa = p.exc_list[(size_t)b * p.exc_per_block + e];
           if (kappa < p.K) take(kappa);
         }
       }

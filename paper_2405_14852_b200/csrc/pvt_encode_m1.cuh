@@ -68,9 +68,9 @@ __device__ __forceinline__ float unord(uint32_t o) {
 __device__ __forceinline__ void form_target(const EncM1Params& p, uint32_t j, float* t) {
   const float4* W4 = reinterpret_cast<const float4*>(p.W);
   const float4* g4 = reinterpret_cast<const float4*>(p.g);
-  const float4 w0 = __ldg(W4 + 2 * (size_t)j), w1 = __ldg(W4 + 2 * (size_t)j + 1);
-  const float4 g0 = __ldg(g4 + 2 * (size_t)j), g1 = __ldg(g4 + 2 * (size_t)j + 1);
-  const float sc = __ldg(p.scale + fast_div(j, p.gpr_div));
+  const float4 w0 = W4[2 * (size_t)j], w1 = W4[2 * (size_t)j + 1];
+  const float4 g0 = g4[2 * (size_t)j], g1 = g4[2 * (size_t)j + 1];
+  const float sc = p.scale[fast_div(j, p.gpr_div)];
   const float neg_eta = -p.eta;
   t[0] = __fdiv_rn(__fmaf_rn(neg_eta, g0.x, w0.x), sc);
   t[1] = __fdiv_rn(__fmaf_rn(neg_eta, g0.y, w0.y), sc);
@@ -86,11 +86,11 @@ __device__ __forceinline__ void form_target(const EncM1Params& p, uint32_t j, fl
 __device__ __forceinline__ void form_target16(const EncM1Params& p, uint32_t j, float* t) {
   const float4* W4 = reinterpret_cast<const float4*>(p.W) + 4 * (size_t)j;
   const float4* g4 = reinterpret_cast<const float4*>(p.g) + 4 * (size_t)j;
-  const float sc = __ldg(p.scale + fast_div(j, p.gpr_div));
+  const float sc = p.scale[fast_div(j, p.gpr_div)];
   const float neg_eta = -p.eta;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const float4 w = __ldg(W4 + q), gg = __ldg(g4 + q);
+    const float4 w = W4[q], gg = g4[q];
     t[4 * q + 0] = __fdiv_rn(__fmaf_rn(neg_eta, gg.x, w.x), sc);
     t[4 * q + 1] = __fdiv_rn(__fmaf_rn(neg_eta, gg.y, w.y), sc);
     t[4 * q + 2] = __fdiv_rn(__fmaf_rn(neg_eta, gg.z, w.z), sc);
@@ -104,7 +104,7 @@ __device__ __forceinline__ void load_codeword(const void* book, uint32_t kappa, 
   if (CB_F16) {
 #pragma unroll
     for (int part = 0; part < DG / 8; ++part) {
-      const uint4 raw = __ldg(reinterpret_cast<const uint4*>(book) + (size_t)kappa * (DG / 8) + part);
+      const uint4 raw = reinterpret_cast<const uint4*>(book)[(size_t)kappa * (DG / 8) + part];
       const __half2* h = reinterpret_cast<const __half2*>(&raw);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -117,7 +117,7 @@ __device__ __forceinline__ void load_codeword(const void* book, uint32_t kappa, 
     const float4* q = reinterpret_cast<const float4*>(book) + (size_t)kappa * (DG / 4);
 #pragma unroll
     for (int part = 0; part < DG / 4; ++part) {
-      const float4 a = __ldg(q + part);
+      const float4 a = q[part];
       c[4 * part] = a.x; c[4 * part + 1] = a.y; c[4 * part + 2] = a.z; c[4 * part + 3] = a.w;
     }
   }

@@ -88,14 +88,14 @@ __global__ void __launch_bounds__(kSmThreads, 4) encode_m1_small_kernel(const En
 #pragma unroll
     for (int tt = 0; tt < TT; ++tt) {
       const uint64_t n = tile * per_cta + (uint64_t)tt * n_teams + team;
-      j[tt] = n < p.k ? __ldg(p.idx + n) : kFull;
+      j[tt] = n < p.k ? p.idx[n] : kFull;
       mine[tt] = 0.0f;
     }
 #pragma unroll
     for (int tt = 0; tt < TT; ++tt) {
       if (j[tt] < p.G) {
-        const float w = __ldg(p.W + (size_t)j[tt] * 8 + l), gg = __ldg(p.g + (size_t)j[tt] * 8 + l);
-        mine[tt] = __fdiv_rn(__fmaf_rn(-p.eta, gg, w), __ldg(p.scale + fast_div(j[tt], p.gpr_div)));
+        const float w = p.W[(size_t)j[tt] * 8 + l], gg = p.g[(size_t)j[tt] * 8 + l];
+        mine[tt] = __fdiv_rn(__fmaf_rn(-p.eta, gg, w), p.scale[fast_div(j[tt], p.gpr_div)]);
       }
       nt2[tt] = 0.0f;
 #pragma unroll

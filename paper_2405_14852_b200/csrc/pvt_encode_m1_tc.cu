@@ -157,10 +157,9 @@ namespace {
 
 // ---- codebook image ------------------------------------------------------------
 template <int DG>
-__global__ void __launch_bounds__(kTcPrepCw) tc_prep_kernel(const uint4* __restrict__ book, uint32_t K, uint32_t n_steps,
-                                                       unsigned char* __restrict__ bimg, TcStats* stats,
-                                                       uint32_t* __restrict__ exc_list, uint32_t* __restrict__ gbest,
-                                                       uint64_t k) {
+__global__ void __launch_bounds__(kTcPrepCw) tc_prep_kernel(const uint4* book, uint32_t K, uint32_t n_steps,
+                                                       unsigned char* bimg, TcStats* stats, uint32_t* exc_list,
+                                                       uint32_t* gbest, uint64_t k) {
   using D = TcDim<DG>;
   __shared__ uint32_t sh_exc, sh_max, sh_inv;
   if (threadIdx.x == 0) sh_exc = sh_max = sh_inv = 0;
@@ -180,7 +179,7 @@ __global__ void __launch_bounds__(kTcPrepCw) tc_prep_kernel(const uint4* __restr
       raw[part] = make_uint4(0, 0, 0, 0);
       part2[part] = 0.0f;
       if (real) {
-        raw[part] = __ldg(book + (size_t)kappa * D::kPart + part);
+        raw[part] = book[(size_t)kappa * D::kPart + part];
         const __half2* h = reinterpret_cast<const __half2*>(&raw[part]);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -347,8 +346,7 @@ struct TcSmem {
 
 template <int DG>
 __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1Params p,
-                                                                      const unsigned char* __restrict__ bimg,
-                                                                      TcStats* __restrict__ stats) {
+                                                                      const unsigned char* bimg, TcStats* stats) {
   using D = TcDim<DG>;
   constexpr int kStepBytes = D::kStepBytes;
   extern __shared__ __align__(128) unsigned char smem_raw[];

@@ -211,8 +211,10 @@ __device__ __forceinline__ void store8(float* p, bool wide, const float* v) {
 // is still running; every thread of it must execute pdl_wait() before its first access to global memory, which
 // returns once that kernel has completed and its writes are visible.  There is no exception for what an earlier
 // kernel of the chain wrote, or the caller: the wait is what makes it visible to this grid.  (A prefetch into the L2
-// is no access.)  Every kernel of a chain calls pdl_trigger() at its start to allow the one after it to be scheduled
-// early.  Both are no-ops for a kernel launched the plain way.
+// is no access.)  Nor may such a kernel read through the read-only path (__ldg, const ... __restrict__): that promises
+// memory nobody writes as long as the kernel lives, while kernels ahead of it are still writing when it starts, and
+// lets the compiler move the load ahead of the wait.  Every kernel of a chain calls pdl_trigger() at its start to allow
+// the one after it to be scheduled early.  Both are no-ops for a kernel launched the plain way.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -388,10 +388,9 @@ cudaError_t launch_grad(const pvt_layer& L, uint64_t G, double* grad_books, doub
 }
 
 // One Adam update, binary32, each operation rounded once, in the order stated in pvt.h.
-__global__ void __launch_bounds__(256) adam_kernel(float* __restrict__ param, __half* __restrict__ param_f16,
-                                                    const double* __restrict__ grad, float* __restrict__ exp_avg,
-                                                    float* __restrict__ exp_avg_sq, uint64_t n, float lr, float beta1,
-                                                    float beta2, float eps, float bias1, float bias2) {
+__global__ void __launch_bounds__(256) adam_kernel(float* param, __half* param_f16, const double* grad, float* exp_avg,
+                                                    float* exp_avg_sq, uint64_t n, float lr, float beta1, float beta2,
+                                                    float eps, float bias1, float bias2) {
   pdl_trigger();
   pdl_wait();
   const float omb1 = __fsub_rn(1.0f, beta1), omb2 = __fsub_rn(1.0f, beta2);
@@ -412,9 +411,8 @@ __global__ void __launch_bounds__(256) adam_kernel(float* __restrict__ param, __
 // Adam-normalised update direction of the V step (Section 3.4): moments as in Adam, u = (m / bias1) /
 // (sqrt(v / bias2) + eps), binary32, each operation rounded once.  Four elements per thread (128-bit accesses).
 // Bound by HBM, three arrays read and three written.  32 bytes of each per thread and trip: 5120x5120 106 us (16 bytes: 113).
-__global__ void __launch_bounds__(256) adam_direction_kernel(const float* __restrict__ grad, float* __restrict__ exp_avg,
-                                                              float* __restrict__ exp_avg_sq, float* __restrict__ dir,
-                                                              uint64_t n4, float beta1, float beta2, float eps,
+__global__ void __launch_bounds__(256) adam_direction_kernel(const float* grad, float* exp_avg, float* exp_avg_sq,
+                                                              float* dir, uint64_t n4, float beta1, float beta2, float eps,
                                                               float bias1, float bias2) {
   pdl_trigger();
   pdl_wait();

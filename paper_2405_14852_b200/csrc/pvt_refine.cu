@@ -36,7 +36,7 @@ struct RefineParams {
 template <bool CB_F16>
 __device__ __forceinline__ void global_codeword(const void* books, uint32_t row, float c[8]) {
   if (CB_F16) {
-    const uint4 raw = __ldg(reinterpret_cast<const uint4*>(books) + row);
+    const uint4 raw = reinterpret_cast<const uint4*>(books)[row];
     const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -46,7 +46,7 @@ __device__ __forceinline__ void global_codeword(const void* books, uint32_t row,
     }
   } else {
     const float4* src = reinterpret_cast<const float4*>(books) + 2 * (size_t)row;
-    const float4 lo = __ldg(src), hi = __ldg(src + 1);
+    const float4 lo = src[0], hi = src[1];
     c[0] = lo.x, c[1] = lo.y, c[2] = lo.z, c[3] = lo.w, c[4] = hi.x, c[5] = hi.y, c[6] = hi.z, c[7] = hi.w;
   }
 }
@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(kRfThreads, M <= 2 ? 4 : 2) refine_kernel(cons
   // persistent blocks: the codebooks are staged once per block, not once per eight targets
   for (uint64_t n = (uint64_t)blockIdx.x * (kRfThreads / 32) + (threadIdx.x >> 5); n < p.k;
        n += (uint64_t)gridDim.x * (kRfThreads / 32)) {
-    const uint32_t j = __ldg(p.idx + n);
+    const uint32_t j = p.idx[n];
     if (j >= p.G) {
       if (lane == 0 && p.status) atomicOr(p.status, PVT_DEV_BAD_INDEX);
       continue;
@@ -104,8 +104,8 @@ __global__ void __launch_bounds__(kRfThreads, M <= 2 ? 4 : 2) refine_kernel(cons
     {
       const float4* W4 = reinterpret_cast<const float4*>(p.W) + 2 * (size_t)j;
       const float4* g4 = reinterpret_cast<const float4*>(p.g) + 2 * (size_t)j;
-      const float4 w0 = __ldg(W4), w1 = __ldg(W4 + 1), g0 = __ldg(g4), g1 = __ldg(g4 + 1);
-      const float s = __ldg(p.scale + j / p.gpr), ne = -p.eta;
+      const float4 w0 = W4[0], w1 = W4[1], g0 = g4[0], g1 = g4[1];
+      const float s = p.scale[j / p.gpr], ne = -p.eta;
       const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
       const float gg[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
 #pragma unroll

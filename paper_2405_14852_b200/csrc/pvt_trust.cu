@@ -76,7 +76,7 @@ __device__ __forceinline__ uint32_t digit_of(uint64_t pair, int pass) { return (
 
 template <int DG>
 __device__ __forceinline__ uint64_t rank_pair(const RankParams& p, uint64_t a) {
-  const uint32_t j = __ldg(p.idx + a);
+  const uint32_t j = p.idx[a];
   uint32_t key = 0, code = 0;
   if (j < p.G) {
     code = load_packed(p.codes, j, p.M, p.code_u16);
@@ -85,7 +85,7 @@ __device__ __forceinline__ uint64_t rank_pair(const RankParams& p, uint64_t a) {
     float acc = 0.0f;
 #pragma unroll
     for (int q = 0; q < DG / 4; ++q) {  // one chain over the DG elements in index order
-      const float4 x = __ldg(src + q);
+      const float4 x = src[q];
       float u;
       u = __fmul_rn(eta, x.x); acc = __fmaf_rn(u, u, acc);
       u = __fmul_rn(eta, x.y); acc = __fmaf_rn(u, u, acc);
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(kSortThreads) rank_init_kernel(const RankParam
 }
 
 // the counts of a later digit (more than kSortDirect blocks)
-__global__ void __launch_bounds__(kSortThreads) sort_count_kernel(const uint64_t* __restrict__ in, const RankParams p,
+__global__ void __launch_bounds__(kSortThreads) sort_count_kernel(const uint64_t* in, const RankParams p,
                                                                   int pass) {
   __shared__ uint32_t h[kSortBins];
   h[threadIdx.x] = 0;
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(kSortThreads) sort_count_kernel(const uint64_t
 }
 
 // exclusive prefix sum of n counters in place, one block; every thread owns a contiguous run
-__global__ void __launch_bounds__(kScanThreads) sort_scan_kernel(uint32_t* __restrict__ counts, uint32_t n) {
+__global__ void __launch_bounds__(kScanThreads) sort_scan_kernel(uint32_t* counts, uint32_t n) {
   __shared__ uint32_t part[kScanThreads];
   pdl_trigger();
   pdl_wait();
@@ -180,8 +180,7 @@ __global__ void __launch_bounds__(kScanThreads) sort_scan_kernel(uint32_t* __res
 // stable scatter: within a block the pairs are visited in position order (round, then thread); a pair's slot is
 // the block's start for its digit + the number of earlier pairs of the block with the same digit
 template <bool DIRECT>
-__global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const uint64_t* __restrict__ in,
-                                                                    uint64_t* __restrict__ out, const RankParams p,
+__global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const uint64_t* in, uint64_t* out, const RankParams p,
                                                                     int pass) {
   __shared__ uint32_t seen[kSortBins];               // pairs of earlier rounds, per digit, plus the block's start
   __shared__ uint32_t cnt[kSortWarps][kSortBins];    // this round: per warp and digit
@@ -276,7 +275,7 @@ __device__ __forceinline__ void codeword(const void* book, uint32_t code, float*
   if (CB_F16) {
 #pragma unroll
     for (int part = 0; part < DG / 8; ++part) {
-      const uint4 raw = __ldg(reinterpret_cast<const uint4*>(book) + (size_t)code * (DG / 8) + part);
+      const uint4 raw = reinterpret_cast<const uint4*>(book)[(size_t)code * (DG / 8) + part];
       const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -289,7 +288,7 @@ __device__ __forceinline__ void codeword(const void* book, uint32_t code, float*
     const float4* src = reinterpret_cast<const float4*>(book) + (size_t)code * (DG / 4);
 #pragma unroll
     for (int part = 0; part < DG / 4; ++part) {
-      const float4 x = __ldg(src + part);
+      const float4 x = src[part];
       c[4 * part] = x.x, c[4 * part + 1] = x.y, c[4 * part + 2] = x.z, c[4 * part + 3] = x.w;
     }
   }
@@ -360,7 +359,7 @@ __global__ void __launch_bounds__(kNormThreads) sq_norm_kernel(const TrustParams
     for (int u = 0; u < kFlight; ++u) {
       const uint64_t j = j0 + u * stride;
       packed[u] = j < p.G ? load_codes<CODE_U16>(p.codes, (uint32_t)j, p.M) : 0u;
-      s[u] = j < p.G ? __ldg(p.scale + fast_div((uint32_t)j, p.gpr)) : 0.0f;
+      s[u] = j < p.G ? p.scale[fast_div((uint32_t)j, p.gpr)] : 0.0f;
     }
 #pragma unroll
     for (int u = 0; u < kFlight; ++u)
@@ -435,10 +434,10 @@ __global__ void __launch_bounds__(kChangeThreads) change_kernel(const TrustParam
   pdl_trigger();
   pdl_wait();
   const uint32_t a = r < p.k ? (uint32_t)p.pairs[r] : 0xffffffffu;
-  uint32_t j = a < p.k ? __ldg(p.idx + a) : 0xffffffffu;
+  uint32_t j = a < p.k ? p.idx[a] : 0xffffffffu;
   double acc = 0.0;
   if (j < p.G) {
-    const float s = __ldg(p.scale + fast_div(j, p.gpr));
+    const float s = p.scale[fast_div(j, p.gpr)];
     float wo[DG], wn[DG];
     bool ok = group_weights<CB_F16, DG>(p.books, p.K, p.M, p.saved[a], CODE_U16, s, wo);
     ok &= group_weights<CB_F16, DG>(p.books, p.K, p.M, load_codes<CODE_U16>(p.codes, j, p.M), CODE_U16, s, wn);

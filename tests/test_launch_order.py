@@ -1,6 +1,7 @@
 """Kernels that are launched before the kernel ahead of them has finished: every one of them waits, in every thread and
-unconditionally, before anything that touches global memory (the rule stated at pdl_wait in csrc/pvt_internal.h).  Read
-from the sources, since a violation is a race that no run has to show."""
+unconditionally, before anything that touches global memory, and none reads through the read-only path, whose loads need
+not stay behind the wait (the rule stated at pdl_wait in csrc/pvt_internal.h).  Read from the sources, since a violation
+is a race that no run has to show."""
 import glob
 import os
 import re
@@ -63,3 +64,19 @@ def test_dependent_kernels_wait_before_they_touch_memory(name):
         for pattern in touch:
             hit = re.search(pattern, ahead)
             assert not hit, f"{kernel} touches memory ahead of its wait: {hit.group(0)!r}"
+
+
+@pytest.mark.parametrize("name", sources() + ["pvt_encode_m1.cuh"])
+def test_dependent_kernels_do_not_read_through_the_read_only_path(name):
+    text = code_of(name)
+    for kernel, (params, _) in dependent_kernels(text).items():
+        hit = re.search(r"const\s+[\w<>, ]+\*\s*__restrict__\s+\w+", params)
+        assert not hit, f"{kernel}: {hit.group(0)}"
+    # what is left of the file without the kernels that are launched the plain way and what only they call
+    late = dependent_kernels(text)
+    for kernel, (params, body) in kernels(text).items():
+        if kernel not in late:
+            text = text.replace(body, "")
+    if name == "pvt_pstep.cu":
+        text = re.sub(r"void group_codes\(.*?\n}\n", "", text, flags=re.S)
+    assert "__ldg" not in text
