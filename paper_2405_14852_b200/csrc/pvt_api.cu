@@ -72,6 +72,12 @@ int check_quantiser(const pvt_layer* L) {
   return PVT_OK;
 }
 
+// What the search over several codebooks asks for beyond that.
+int check_beam(const pvt_layer* L) {
+  if (L->num_codebooks < 2) return PVT_OK;
+  return L->code_dtype == PVT_U8 && L->beam >= 1 && L->beam <= 8 ? PVT_OK : PVT_EUNSUPPORTED;
+}
+
 // ---- optional timing ----------------------------------------------------------
 struct Timing {
   std::mutex mu;
@@ -262,8 +268,7 @@ int pvt_vstep_encode(const pvt_layer* layer, const uint32_t* idx, uint64_t k, fl
     if (ws_bytes < lay.bytes) return PVT_EWORKSPACE;
     e = launch_encode_m1(*layer, G, idx, k, err_out, ws, sms, static_cast<cudaStream_t>(cuda_stream));
   } else {
-    if (layer->code_dtype != PVT_U8) return PVT_EUNSUPPORTED;
-    if (layer->beam < 1 || layer->beam > 8) return PVT_EUNSUPPORTED;
+    if ((rc = check_beam(layer)) != PVT_OK) return rc;
     if (ws_bytes < encode_beam_workspace_bytes()) return PVT_EWORKSPACE;
     e = launch_encode_beam(*layer, G, idx, k, err_out, ws, sms, static_cast<cudaStream_t>(cuda_stream));
   }
@@ -284,10 +289,7 @@ int pvt_vstep_trust(const pvt_layer* layer, uint64_t k_max, float ratio, uint32_
   if ((reinterpret_cast<uintptr_t>(n_out) & 7u) || (reinterpret_cast<uintptr_t>(stats_out) & 7u)) return PVT_EINVAL;
   if (!codes_aligned(layer) || !aligned4(idx_out)) return PVT_EINVAL;
   if (reinterpret_cast<uintptr_t>(ws) & (kWsAlign - 1)) return PVT_EINVAL;
-  if (layer->num_codebooks >= 2) {
-    if (layer->code_dtype != PVT_U8 || layer->beam < 1 || layer->beam > 8) return PVT_EUNSUPPORTED;
-    if (layer->num_codebooks == 2 && (reinterpret_cast<uintptr_t>(layer->codes) & 1u)) return PVT_EINVAL;
-  }
+  if ((rc = check_beam(layer)) != PVT_OK) return rc;
   const int sms = sm_count();
   const TrustLayout t = trust_layout(G, k_max, encode_bytes(*layer, k_max, sms), sms);
   if (ws_bytes < t.bytes) return PVT_EWORKSPACE;
@@ -370,6 +372,8 @@ int pvt_vstep_block(const pvt_layer* layers, const uint64_t* k, int32_t n_layers
     if (!idx_out[i] || !aligned4(idx_out[i]) || !L.W || !L.g || !L.scale || !L.codebooks || !L.codes) return PVT_EINVAL;
     if (!aligned16(L.W) || !aligned16(L.g) || !aligned16(L.codebooks) || !codes_aligned(&L)) return PVT_EINVAL;
     if (W_hat && W_hat[i] && !aligned16(W_hat[i])) return PVT_EINVAL;
+    const int rc = check_beam(&L);
+    if (rc != PVT_OK) return rc;
   }
   if (W_hat && out_dtype != PVT_F32 && out_dtype != PVT_F16) return PVT_EINVAL;
   for (int32_t i = 0; i < n_layers; ++i) {

@@ -157,3 +157,14 @@ def test_block_call_validates_every_layer_before_launching():
     idx_bad = (ctypes.c_void_p * n)(0x2000, None)
     assert lib.pvt_vstep_block(arr, ks, n, idx_bad, None, B.PVT_F32, 0x4000, 1 << 30, None) == B.PVT_EINVAL
     assert lib.pvt_vstep_block(arr, ks, 0, idx, None, B.PVT_F32, 0x4000, 1 << 30, None) == B.PVT_EINVAL
+
+
+@pytest.mark.parametrize("kw", [dict(num_codebooks=2, code_dtype=B.PVT_U16), dict(num_codebooks=2, beam=0),
+                                dict(num_codebooks=3, beam=9)])
+def test_block_call_refuses_what_the_beam_search_does_not_take_before_launching(kw):
+    n = 2
+    arr = (B.pvt_layer * n)(_layer(), _layer(**kw))  # (without a device a call that launched anything says PVT_ECUDA)
+    ks, idx = (ctypes.c_uint64 * n)(4, 4), (ctypes.c_void_p * n)(0x2000, 0x3000)
+    before = B.pvt_launch_count()
+    rc = B.lib().pvt_vstep_block(arr, ks, n, idx, None, B.PVT_F32, 0x4000, 1 << 30, None)
+    assert rc == B.PVT_EUNSUPPORTED and B.pvt_launch_count() == before
