@@ -66,7 +66,8 @@ extern "C" {
 #define PVT_DEV_BAD_INDEX 1u    /* an entry of idx was >= G; that entry was skipped */
 #define PVT_DEV_BAD_CODE 2u     /* a stored code was >= K; treated as code 0 (dequant) or left out of the pool */
 #define PVT_DEV_WAIT_EXPIRED 4u /* a bounded wait on an on-chip barrier ran out; results of the call are invalid */
-#define PVT_DEV_INTERNAL 8u     /* an internal consistency check failed (selection count mismatch) */
+#define PVT_DEV_INTERNAL 8u     /* an internal consistency check failed (selection count mismatch), or a group has no finite
+                                   distance to any codeword (a target that is not finite): it keeps its codes */
 
 /*
  * One quantised linear layer and the update direction of this step.

@@ -861,8 +861,8 @@ __global__ void __launch_bounds__(kBsThreads, kBsCtasPerSm) encode_beam_kernel(c
           for (int m = 0; m < M; ++m) p.codes[(size_t)my_j * M + m] = (uint8_t)(bk >> (24 - 8 * m));
         }
         if (p.err_out) p.err_out[gi * kBsGroup + my_q] = (float)bd;
-      } else if (M > 2) {
-        atomicOr(p.status, PVT_DEV_INTERNAL);
+      } else {
+        atomicOr(p.status, PVT_DEV_INTERNAL);  // non-finite target: no distance compares below infinity
       }
     }
     __syncwarp();  // the group's scratch is rewritten by the next iteration

@@ -4,8 +4,10 @@ because they do."""
 import numpy as np
 import pytest
 
+from oracle import pvt_oracle as oracle
+from paper_2405_14852_b200 import binding as B
 from paper_2405_14852_b200 import synth
-from test_gpu_parity import check_encode, oracle_nearest
+from test_gpu_parity import check_encode, oracle_nearest, run_encode
 
 
 @pytest.mark.gpu
@@ -30,3 +32,22 @@ def test_clustered_codewords(M, copies, jitter, f16):
         base = L.codebooks[m].astype(np.float32)[np.arange(256) // copies]
         L.codebooks[m] = (base + rng.normal(0.0, jitter, size=base.shape)).astype(L.codebooks.dtype)
     check_encode(L, np.arange(L.num_groups, dtype=np.uint32))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,f16,value", [(2, True, np.nan), (2, False, np.nan), (2, True, np.inf), (3, True, np.nan)])
+def test_a_target_that_is_not_finite_is_reported_and_keeps_its_codes(M, f16, value):
+    L = synth.make_layer(16, 256, cfg=320 + M, num_codebooks=M, codebook_size=100, codebook_fp16=f16, nearest=oracle_nearest)
+    odd = [2, 3, 77, L.num_groups - 1]  # two of one group of four targets, alone among others, the last
+    idx = np.arange(L.num_groups, dtype=np.uint32)
+    t = oracle.targets(L.W, L.g, L.scale, L.eta, idx)
+    before = L.codes.reshape(-1, M).copy()
+    want = oracle.encode(t, L.codebooks, before, L.beam)
+    L.W.reshape(-1, 8)[odd, 5] = value
+    got, _, status = run_encode(L, idx)
+    assert status == B.PVT_DEV_INTERNAL
+    got = got.reshape(-1, M)
+    assert np.array_equal(got[odd], before[odd])
+    rest = np.setdiff1d(idx, odd)
+    decisive = (want.d_second - want.d_best)[rest] > 1e-6 * want.d_second[rest]
+    assert np.array_equal(got[rest][decisive], want.codes[rest][decisive])
