@@ -875,7 +875,7 @@ cudaError_t launch_beam(const BeamParams& p, unsigned char* image_at, int sm_cou
   static_assert(sizeof(Image) % 16 == 0, "the bulk copy moves multiples of 16 bytes");
   static_assert(sizeof(Image) <= 77824, "the workspace reserves 76 KiB for the image");
   constexpr size_t smem = sizeof(BeamSmem<M, TC>);
-  cudaError_t err = allow_smem(encode_beam_kernel<M, TC>);
+  cudaError_t err = allow_smem<encode_beam_kernel<M, TC>>();
   if (err != cudaSuccess) return err;
   Image* image = reinterpret_cast<Image*>(image_at);
   timing_begin(kKernEncodeAux, stream);

@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kSmThreads, 4) encode_m1_small_kernel(const En
 template <bool CB_F16, int TT>
 cudaError_t launch_small(const EncM1Params& p, int sm_count, cudaStream_t stream) {
   const size_t smem = small_smem_bytes(p.K);
-  const cudaError_t err = allow_smem(encode_m1_small_kernel<CB_F16, TT>);
+  const cudaError_t err = allow_smem<encode_m1_small_kernel<CB_F16, TT>>();
   if (err != cudaSuccess) return err;
   const uint64_t per_cta = kSmThreads / 8 * TT, tiles = (p.k + per_cta - 1) / per_cta;
   constexpr uint64_t kMost = 1024 / kSmThreads;  // 64 registers a thread

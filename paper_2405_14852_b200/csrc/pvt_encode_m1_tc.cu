@@ -760,7 +760,7 @@ cudaError_t launch_tc(const pvt_layer& L, const EncM1Params& p, const EncodeM1Tc
   timing_end(kKernEncodeAux, stream);
   if (err != cudaSuccess) return err;
   const size_t smem = sizeof(TcSmem<DG>);
-  if ((err = allow_smem(encode_m1_tc_kernel<DG>)) != cudaSuccess) return err;
+  if ((err = allow_smem<encode_m1_tc_kernel<DG>>()) != cudaSuccess) return err;
   timing_begin(kKernEncodeMain, stream);
   err = launch_dependent(encode_m1_tc_kernel<DG>, lay.n_ctas, kTcThreads, smem, stream, p,
                          reinterpret_cast<const unsigned char*>(base + lay.bimg_off), stats);

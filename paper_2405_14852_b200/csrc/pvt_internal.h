@@ -256,23 +256,17 @@ int device_slot();
 
 // Lets a kernel take all the dynamic shared memory there is; the driver is asked once per kernel and device.
 #ifdef __CUDACC__
-template <typename... KArgs>
-cudaError_t allow_smem(void (*kernel)(KArgs...)) {
-  static std::atomic<void*> done[kMaxDevices][8];  // kernels of one signature share these slots
+template <auto kernel>
+cudaError_t allow_smem() {
+  static std::atomic<bool> done[kMaxDevices];  // of this kernel: the instantiation is its own
   const int dev = device_slot();
-  if (dev >= 0)
-    for (auto& d : done[dev])
-      if (d.load(std::memory_order_relaxed) == reinterpret_cast<void*>(kernel)) return cudaSuccess;
+  if (dev >= 0 && done[dev].load(std::memory_order_relaxed)) return cudaSuccess;
   cudaFuncAttributes fa;
   cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(227 * 1024 - fa.sharedSizeBytes));
-  if (e != cudaSuccess || dev < 0) return e;
-  for (auto& d : done[dev]) {
-    void* none = nullptr;
-    if (d.compare_exchange_strong(none, reinterpret_cast<void*>(kernel))) break;
-  }
-  return cudaSuccess;
+  if (e == cudaSuccess && dev >= 0) done[dev].store(true, std::memory_order_relaxed);
+  return e;
 }
 #endif
 

@@ -355,7 +355,7 @@ cudaError_t launch_grad_small(const pvt_layer& L, uint64_t G, double* grad_books
                               int sm_count, cudaStream_t stream) {
   const uint32_t K = (uint32_t)L.codebook_size;
   const size_t smem = small_smem<M, CB_F16>(K);
-  const cudaError_t e = allow_smem(pstep_grad_small_kernel<M, CB_F16, CODE_U16>);
+  const cudaError_t e = allow_smem<pstep_grad_small_kernel<M, CB_F16, CODE_U16>>();
   if (e != cudaSuccess) return e;
   const uint64_t tiles = (G + kPsTile - 1) / kPsTile, cap = (uint64_t)sm_count * (smem <= 112 * 1024 ? 2 : 1);
   pstep_grad_small_kernel<M, CB_F16, CODE_U16><<<(unsigned)(tiles < cap ? tiles : cap), kPsSmallThreads, smem, stream>>>(
