@@ -8,8 +8,6 @@
 // w = s * v; fp16 output = round-to-nearest-even of w.
 #include <cuda_fp16.h>
 
-#include <atomic>
-
 #include "pvt_internal.h"
 
 namespace pvt {
@@ -163,20 +161,12 @@ __global__ void __launch_bounds__(kDqThreads) dequant_kernel(const void* codeboo
 
 template <int M, bool CB_F16, bool CODE_U16, bool OUT_F16, bool SMEM_BOOK, int DG>
 cudaError_t launch_s(const pvt_layer& L, uint64_t G, void* W_hat, uint32_t* status, int sm_count, cudaStream_t stream) {
-  const auto kernel = dequant_kernel<M, CB_F16, CODE_U16, OUT_F16, SMEM_BOOK, DG>;
-  // persistent grid: as many blocks as are resident at once (asked once per device)
-  static std::atomic<int> resident[kMaxDevices];
-  const int dev = device_slot();
-  int per_sm = dev >= 0 ? resident[dev].load(std::memory_order_relaxed) : 0;
-  if (per_sm < 1) {
-    const cudaError_t oe = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kDqThreads, 0);
-    if (oe != cudaSuccess) return oe;
-    if (per_sm < 1) per_sm = 1;
-    if (dev >= 0) resident[dev].store(per_sm, std::memory_order_relaxed);
-  }
+  constexpr auto kernel = dequant_kernel<M, CB_F16, CODE_U16, OUT_F16, SMEM_BOOK, DG>;
+  uint64_t cap = 0;
+  const cudaError_t e = resident_blocks<kernel>(kDqThreads, sm_count, &cap);
+  if (e != cudaSuccess) return e;
   const uint64_t per_block = (uint64_t)kDqThreads * kDqUnroll;
   const uint64_t want = (DG / (OUT_F16 ? 8 : 4) * G + per_block - 1) / per_block;
-  const uint64_t cap = (uint64_t)sm_count * (uint64_t)per_sm;
   return launch_dependent(kernel, (unsigned)(want < cap ? want : cap), kDqThreads, 0, stream, L.codebooks, L.codes, L.scale,
                           G, make_fast_div((uint32_t)(L.cols / DG)), (uint32_t)L.codebook_size, W_hat, status);
 }

@@ -268,6 +268,23 @@ cudaError_t allow_smem() {
   if (e == cudaSuccess && dev >= 0) done[dev].store(true, std::memory_order_relaxed);
   return e;
 }
+
+// Blocks of a kernel without dynamic shared memory that are resident at once on the device, the grid of a persistent
+// kernel; the driver is asked once per kernel and device.
+template <auto kernel>
+cudaError_t resident_blocks(int threads, int sm_count, uint64_t* blocks) {
+  static std::atomic<int> known[kMaxDevices];  // per SM
+  const int dev = device_slot();
+  int per_sm = dev >= 0 ? known[dev].load(std::memory_order_relaxed) : 0;
+  if (per_sm < 1) {
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) per_sm = 1;
+    if (dev >= 0) known[dev].store(per_sm, std::memory_order_relaxed);
+  }
+  *blocks = (uint64_t)sm_count * (uint64_t)per_sm;
+  return cudaSuccess;
+}
 #endif
 
 // number of kernels launched by this process through the library (a claim the benchmark reports)

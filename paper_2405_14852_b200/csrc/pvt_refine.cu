@@ -232,17 +232,25 @@ __global__ void __launch_bounds__(kRfThreads, M <= 2 ? 4 : 2) refine_kernel(cons
   }
 }
 
+template <int M, bool CB_F16, bool CODE_U16, bool STAGED>
+cudaError_t launch_resident(const RefineParams& p, cudaStream_t stream) {
+  constexpr auto kernel = refine_kernel<M, CB_F16, CODE_U16, STAGED>;
+  const uint64_t want = (p.k + kRfThreads / 32 - 1) / (kRfThreads / 32);
+  uint64_t most = 0;
+  const cudaError_t e = resident_blocks<kernel>(kRfThreads, device_sm_count(), &most);
+  if (e != cudaSuccess) return e;
+  // Staged codebooks: the resident blocks and no more, since each further wave stages them again (20011 targets of 2x251
+  // 27.7 us, with twice as many blocks 29.3).  Nothing staged: a second wave evens out the first (56360 targets of
+  // 1x4096 309 us, without it 324).
+  if (!STAGED) most *= 2;
+  count_launches(1);
+  return launch_dependent(kernel, (unsigned)(want < most ? want : most), kRfThreads, 0, stream, p);
+}
+
 template <int M, bool CB_F16, bool CODE_U16>
 cudaError_t launch_staged(const RefineParams& p, cudaStream_t stream) {
-  const uint64_t want = (p.k + kRfThreads / 32 - 1) / (kRfThreads / 32), most = 8 * (uint64_t)kSmCountFallback;
-  const unsigned blocks = (unsigned)(want < most ? want : most);
-  cudaError_t err;
-  if ((uint64_t)M * p.K <= (uint64_t)kRfSmemCodewords)
-    err = launch_dependent(refine_kernel<M, CB_F16, CODE_U16, true>, blocks, kRfThreads, 0, stream, p);
-  else
-    err = launch_dependent(refine_kernel<M, CB_F16, CODE_U16, false>, blocks, kRfThreads, 0, stream, p);
-  count_launches(1);
-  return err;
+  if ((uint64_t)M * p.K <= (uint64_t)kRfSmemCodewords) return launch_resident<M, CB_F16, CODE_U16, true>(p, stream);
+  return launch_resident<M, CB_F16, CODE_U16, false>(p, stream);
 }
 
 }  // namespace

@@ -539,7 +539,7 @@ TrustLayout trust_layout(uint64_t G, uint64_t k, size_t encode_bytes, int sm_cou
   t.sort_blocks = (uint32_t)((k + tile - 1) / tile);
   t.sort_direct = t.sort_blocks <= kSortDirect;
   t.sort_stride = t.sort_direct ? (t.sort_blocks + 3) / 4 * 4 : t.sort_blocks;
-  t.norm_blocks = (uint32_t)(4 * (sm_count > 0 ? sm_count : kSmCountFallback));
+  t.norm_blocks = (uint32_t)(4 * sm_count);
   t.idx_off = host_align(select_layout(G).bytes);
   t.pairs_a_off = host_align(t.idx_off + sizeof(uint32_t) * k);
   t.pairs_b_off = host_align(t.pairs_a_off + sizeof(uint64_t) * k);   // second sort buffer, later the changes

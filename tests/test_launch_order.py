@@ -80,3 +80,8 @@ def test_dependent_kernels_do_not_read_through_the_read_only_path(name):
     if name == "pvt_pstep.cu":
         text = re.sub(r"void group_codes\(.*?\n}\n", "", text, flags=re.S)
     assert "__ldg" not in text
+
+
+def test_grids_follow_the_device():
+    """The multiprocessor count that stands in when the device cannot be asked sizes no grid by itself."""
+    assert [f for f in sources() if "kSmCountFallback" in code_of(f)] == ["pvt_api.cu"]
