@@ -9,10 +9,9 @@
 // Every product of two binary32 numbers is exact in binary64 and the sums are accumulated in binary64 with
 // atomic adds, so the result differs from a sequential sum only by the order of binary64 roundings.
 //
-// One streaming pass over g.  Small codebooks (M K <= 2048 codewords) are accumulated in shared memory per CTA and
-// flushed once; large ones go straight to the L2.  Between 1024 and 4096 codewords the two take about the same time
-// (4096 x 4096: 87 us for 1024 in shared memory, 56 us for 4096 in the L2, where fewer codewords queue up).  Scale
-// gradients are summed over a warp first when the warp lies inside one row.
+// One streaming pass over g.  Small codebooks (M K <= 1024 codewords) are accumulated in shared memory per CTA and
+// flushed once; large ones go straight to the L2.  Scale gradients are summed over a warp first when the warp lies inside
+// one row.
 #include <cuda_fp16.h>
 
 #include "pvt_internal.h"
@@ -21,8 +20,12 @@ namespace pvt {
 namespace {
 
 constexpr int kPsThreads = 256;
-constexpr size_t kPsMaxSmem = 226 * 1024;
-constexpr int kPsSmallBins = 2048;   // M K up to here: sums in shared memory, above it in the L2
+constexpr size_t kPsMaxSmem = 227 * 1024;
+// M K up to here: sums in shared memory, above it in the L2.  Shared memory slows down with the codewords that a tile is
+// sorted into, the L2 speeds up with the codewords that its reductions spread over.  4096 x 4096, one fp16 codebook of
+// 512 / 1024 / 1500 / 1944 codewords: 59 / 89 / 99 / 114 us in shared memory, 163 / 115 / 70 / 59 us in the L2;
+// four codebooks of 256 (the most that several codebooks have): 161 and 470 us.
+constexpr int kPsSmallBins = 1024;
 
 __device__ __forceinline__ void red_add_f64(double* p, double v) {
   asm volatile("red.global.add.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
@@ -381,8 +384,8 @@ cudaError_t launch_grad(const pvt_layer& L, uint64_t G, double* grad_books, doub
     if constexpr (M == 1)
       return launch_grad_large<1, CB_F16, CODE_U16, 16>(L, G, grad_books, grad_scale, status, sm_count, stream);
   }
-  if ((uint32_t)M * (uint32_t)L.codebook_size <= (uint32_t)kPsSmallBins &&
-      small_smem<M, CB_F16>((uint32_t)L.codebook_size) <= kPsMaxSmem)
+  static_assert(small_smem<M, CB_F16>(kPsSmallBins / M) <= kPsMaxSmem, "a block holds every small codebook's sums");
+  if ((uint32_t)M * (uint32_t)L.codebook_size <= (uint32_t)kPsSmallBins)
     return launch_grad_small<M, CB_F16, CODE_U16>(L, G, grad_books, grad_scale, status, sm_count, stream);
   return launch_grad_large<M, CB_F16, CODE_U16, 8>(L, G, grad_books, grad_scale, status, sm_count, stream);
 }

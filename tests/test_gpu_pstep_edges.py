@@ -1,5 +1,8 @@
 """Gradients of the P step where the accumulation changes: sums in shared memory against sums in the L2, tiles and
 warps that are not full, rows that end inside a warp, an update matrix on a 16-byte boundary only."""
+import os
+import re
+
 import numpy as np
 import pytest
 import torch
@@ -8,18 +11,33 @@ from oracle import pvt_oracle as oracle
 from paper_2405_14852_b200 import binding as B
 
 
-@pytest.mark.gpu
-@pytest.mark.parametrize("M,K,f16,rows,per_row,gd,offset", [
-    (1, 2048, True, 41, 25, 8, 0),     # the largest codebook summed in shared memory; 1025 groups: one in the last tile
+CASES = [
+    (1, 1024, True, 41, 25, 8, 0),     # the largest codebook summed in shared memory; 1025 groups: one in the last tile
+    (1, 1024, False, 300, 129, 8, 4),
+    (4, 256, True, 41, 25, 8, 4),      # as many codewords in four codebooks
+    (1, 1025, True, 33, 31, 8, 4),     # the smallest summed in the L2; 1023 groups
+    (1, 1025, False, 41, 25, 8, 0),
+    (1, 2048, True, 41, 25, 8, 0),
     (1, 2048, False, 300, 129, 8, 4),
-    (1, 2049, True, 33, 31, 8, 4),     # the smallest summed in the L2; 1023 groups
+    (1, 2049, True, 33, 31, 8, 4),
     (2, 256, True, 1031, 33, 8, 4),    # several tiles per CTA, warps over two rows
     (2, 2, False, 3, 683, 8, 0),       # every group at two codewords; one group beyond two tiles
     (3, 250, True, 130, 64, 8, 0),
     (4, 256, False, 64, 70, 8, 4),
     (1, 2, True, 1, 1, 8, 0),          # one group
     (1, 300, True, 65, 17, 16, 4),     # groups of 16
-])
+]
+
+
+def test_the_cases_are_on_both_sides_of_the_rule():
+    source = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2405_14852_b200", "csrc", "pvt_pstep.cu")
+    line = int(re.search(r"kPsSmallBins = (\d+);", open(source).read()).group(1))
+    for f16 in (True, False):
+        assert {line, line + 1} <= {M * K for M, K, cb, _, _, gd, _ in CASES if cb == f16 and gd == 8}
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,K,f16,rows,per_row,gd,offset", CASES)
 def test_gradients_at_the_edges(M, K, f16, rows, per_row, gd, offset):
     rng = np.random.default_rng(M * 1000 + K)
     cols, G = per_row * gd, rows * per_row
