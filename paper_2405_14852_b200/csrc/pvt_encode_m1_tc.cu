@@ -117,7 +117,7 @@ bool encode_m1_use_tc(const pvt_layer& L, uint64_t k) {
   const int mode = g_m1_search.load(std::memory_order_relaxed);
   if (mode == PVT_M1_FP32) return false;
   if (mode == PVT_M1_TENSOR) return true;
-  return L.codebook_size >= 1024;  // below that the FP32 pipe with its larger target tiles is as fast
+  return L.codebook_size >= kM1TensorCodebook;
 }
 
 EncodeM1TcLayout encode_m1_tc_layout(uint32_t K, uint64_t k, int sm_count, int group_dim) {

@@ -91,7 +91,11 @@ struct EncodeM1TcLayout {
   uint32_t n_ctas;
 };
 bool encode_m1_use_tc(const pvt_layer& L, uint64_t k);
-constexpr uint32_t kM1SmallCodebook = 1024;  // without the tensor engine: codebooks up to here stay in shared memory
+// fp16 codebooks from here on: the tensor engine (the line that pvt.h states).  20971 / 500000 targets, 512 codewords:
+// small-codebook kernel 17 / 173 us, tensor engine 18 / 210; 768: 27 / 237 and 19 / 218; 1024: 29 / 299 and 19 / 224.
+constexpr int kM1TensorCodebook = 1024;
+// Without the tensor engine: codebooks up to here stay in shared memory (both sides measured at the kernel).
+constexpr uint32_t kM1SmallCodebook = 1024;
 constexpr size_t kM1SmallWorkspace = kWsHeaderBytes + kWsAlign;
 void set_m1_search(int mode);
 EncodeM1TcLayout encode_m1_tc_layout(uint32_t K, uint64_t k, int sm_count, int group_dim = 8);
