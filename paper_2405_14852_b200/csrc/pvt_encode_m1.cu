@@ -24,10 +24,10 @@
 //   5. at the end of the unit each thread writes, per target, the remembered
 //      sub-chunks that are still within the margin of the slice minimum, and folds
 //      the slice minimum into a per-target global minimum (atomic).
-// Rescoring.  One warp per target: every remembered sub-chunk of every slice whose
+// Rescoring.  Eight lanes per target: every remembered sub-chunk of every slice whose
 // minimum lies within the margin of the global minimum is revisited, the binary64
 // distance sum (t_i-c_i)^2 (index order) of each of its codewords is evaluated
-// from the caller's codebook, and the argmin of (distance, code) is written.
+// from the caller's codebook where the binary32 distance leaves it open, and the argmin of (distance, code) is written.
 // The margin bounds twice the rounding error of the fast score, so the codeword
 // that is nearest in exact arithmetic is always among those rescored.
 #include <cuda_fp16.h>

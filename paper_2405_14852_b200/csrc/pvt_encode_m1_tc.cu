@@ -27,9 +27,11 @@
 // codebook go through buffer 0, odd ones through buffer 1.  Warp 16 copies the codebook (two stages of eight steps).
 //
 // What bounds it: not a pipe but the ring each accumulator goes round - MMA issued, executed, completion seen, read out,
-// release seen - about 750 cycles for 128 x 128 scores, with all of tensor memory in flight (a fp16 accumulator takes a
-// 32-bit column too).  Measured at 1048576 targets x 65536 codewords, per 256 x 128 scores: 393 cycles; 363 with neither
-// minima nor comparisons; the tensor pipe is busy for 130 and the minima take 128 of the ALU's.  Against binary32
+// release seen -, with all of tensor memory in flight (a fp16 accumulator takes a 32-bit column too).  Measured at
+// 1048576 targets x 65536 codewords and 1965 MHz: 3223 us, that is 447 cycles per 256 x 128 scores (an accumulator comes
+// round once in two of these steps); 365 with neither minima nor comparisons.  The tensor pipe is busy for 130 of them
+// (31 % of the active cycles by its counter) and the minima take 128 of the ALU's; issue slots 44 %.  A small subspace runs
+// below that rate, for units begin, drain and end more often: 20971 targets 89 us, 616 cycles a step.  Against binary32
 // accumulators, two instructions per step, eight epilogue warps that alternate between the buffers and one issuing warp per
 // A block: 3245 us for 4556 us.  Of this, fp16 accumulators gave 4556 -> 3740; four issuing warps alone nothing; sixteen
 // epilogue warps with a buffer each 3900 -> 3300; an arrival by all threads of a warp instead of one behind a branch
@@ -636,6 +638,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
         // 2^e (||t|| ||c|| + h + ||t||^2) for the sum of products in binary32, rounded or truncated (twice the terms for
         // groups of 16); 2^-24 where a half is subnormal, and the split of h and of the bias.  Twice that is the margin, the
         // last terms with a factor 2 to spare: margin + kRelMargin |S|.
+        // How the tensor cores add and round is not documented: that a sum is formed to binary32 accuracy and is off by at
+        // most one unit of 2^-10 of itself per instruction as a half is an assumption.  What supports it are the tests, in
+        // which the codes are the same as those of binary64 distances.
         const float margin = 2.0f * (517.0f * r2 / (in_range ? sc : 1.0f) +
                                      (DG == 8 ? 3.814697265625e-6f /* 2^-18 */ : 7.62939453125e-6f) * sc *
                                          (norm * cnmax + hmax + nt2) +
@@ -656,8 +661,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
       // in registers: the common case of an event is one store and no load
       uint32_t list_cnt = 0, evicted = 0xffffffffu;
       // keys up to this one are remembered: at first those that may reach the score of the stored code.  (With no bound
-      // to begin with, every thread remembers its first steps one after the other: 4096x4096 1x16, five units per CTA,
-      // 95 us instead of 90.)
+      // to begin with, every thread remembers its first steps one after the other: 4096x4096 1x16 95 us instead of 90.)
       const float seed = sm.seed[own];
       uint32_t lim = key_limit(seed - fmaf(kRelMargin, fabsf(seed), margin));
       auto note = [&](uint32_t key, uint32_t sub) {
@@ -784,7 +788,6 @@ cudaError_t launch_encode_m1_tc(const pvt_layer& L, uint64_t G, const uint32_t* 
   p.k = k;
   p.G = G;
   p.gpr = (uint32_t)(L.cols / L.group_dim);
-  p.gpr_div = make_fast_div(p.gpr);
   p.gpr_div = make_fast_div(p.gpr);
   p.dg = (uint32_t)L.group_dim;
   p.eta = L.eta;

@@ -81,8 +81,8 @@ size_t encode_beam_workspace_bytes();
 // encode, M = 1 on the tensor cores (fp16 codebooks of at least 1024 codewords)
 struct EncodeM1TcLayout {
   size_t bimg_off;    // codebook image in operand order: n_steps * 4096 bytes
-  size_t stats_off;   // max ||c||^2 (bit pattern), exception count
-  size_t exc_off;     // u32 [K]: codewords the image cannot represent
+  size_t stats_off;   // TcStats: exceptions and extreme norms by block of codewords
+  size_t exc_off;     // u32 [K]: codewords the image cannot represent, by block
   size_t gbest_off, margin_off, rec_off;
   size_t bytes;
   uint32_t n_steps;   // 128-codeword steps

@@ -184,10 +184,10 @@ __global__ void __launch_bounds__(kPsThreads) pstep_grad_kernel(const float* __r
 // Small codebooks: the sums stay in shared memory.  A CTA takes tiles of 1024 groups.  Per tile it stages the exact
 // products s * g, sorts the tile's (codebook, code) pairs by counting (integer shared-memory atomics hand out the
 // slots) and lets the team of four lanes that owns a pair, two elements each, add up its products in registers.
-// The next tile's loads are in flight
-// meanwhile.  What bounds it are the wavefronts of shared memory (73 % busy): a quarter of them rows of products in
-// sorted order, the rest products, lists, counters, codewords.  11008 x 4096 with two codebooks of 256: 167 us; with
-// tiles of 512 groups and no loads ahead 283 us; four codebooks of 256 332 us, in the L2 1930 us.
+// The next tile's loads are in flight meanwhile.  What bounds it is shared memory (its pipe 71 % busy, 66 % of the cycles
+// with a wavefront of it): products, lists, counters and codewords, and the rows of products in sorted order.
+// 11008 x 4096, codes as a search leaves them, two / four codebooks of 256: 195 / 416 us, in the L2 843 / 1101 us.  With
+// uniformly random codes 166 / 332 us; there tiles of 512 groups with no loads ahead took 283 us for two codebooks.
 constexpr int kPsSmallThreads = 512;
 constexpr int kPsTile = 1024;
 constexpr int kPsTeams = kPsSmallThreads / 4;
@@ -412,8 +412,9 @@ __global__ void __launch_bounds__(256) adam_kernel(float* param, __half* param_f
 }
 
 // Adam-normalised update direction of the V step (Section 3.4): moments as in Adam, u = (m / bias1) /
-// (sqrt(v / bias2) + eps), binary32, each operation rounded once.  Four elements per thread (128-bit accesses).
-// Bound by HBM, three arrays read and three written.  32 bytes of each per thread and trip: 5120x5120 106 us (16 bytes: 113).
+// (sqrt(v / bias2) + eps), binary32, each operation rounded once.
+// Bound by HBM, three arrays read and three written.  Eight elements, 32 bytes of each, per thread and trip: 5120x5120
+// 106 us (16 bytes: 113).
 __global__ void __launch_bounds__(256) adam_direction_kernel(const float* grad, float* exp_avg, float* exp_avg_sq,
                                                               float* dir, uint64_t n4, float beta1, float beta2, float eps,
                                                               float bias1, float bias2) {

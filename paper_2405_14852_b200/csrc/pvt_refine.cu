@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(kRfThreads, M <= 2 ? 4 : 2) refine_kernel(cons
         for (int i = 0; i < 8; ++i) keep[i] = cw[m][i];
         // Only a neighbour below the current error matters, and binary32 says which may be: with r the target less the
         // other codewords, each difference rounded, the root of its error is off by no more than 2^-24 of r's and its
-        // intermediates' norms and of itself.  (Every neighbour in binary64: 46 us for 20011 targets of 2x251, now 25.)
+        // intermediates' norms and of itself.  (Every neighbour in binary64: 46 us for 20011 targets of 2x251, now 28.)
         float r[8], rr = 0.0f;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {

@@ -15,9 +15,9 @@
 //   3. write:  every CTA reads the threshold from those two tables, looks up the keys inside the bin, counts what it
 //              takes, waits for the counts of the CTAs before it and writes its part of the list by ballots:
 //              position = (#greater before) + min(#equal before, ties to take)
-// Measured as graph replays, 4096 x 4096 / 11008 x 4096 / 28672 x 8192: 29 / 54 / 236 us, of which pass 1 alone takes
-// 14 / 32 / 180 us (5.6 TB/s of g, 6.3 with the keys).  Five passes with one bin per eighth of an octave took
-// 45 / 74 / 344 us.  One cooperative kernel with the keys in shared memory takes 33 us, and about 10 us more to launch.
+// Measured as graph replays, 4096 x 4096 / 11008 x 4096 / 28672 x 8192: 32 / 53 / 245 us.  Of the first, by its counters,
+// pass 1 takes 16 us (4.2 TB/s of g from cold; 5.3 for the second), the others 4.5, 10 and 12.  Five passes with one bin per
+// eighth of an octave took 45 / 74 / 344 us.  One cooperative kernel with the keys in shared memory takes 33 us, and about 10 us more to launch.
 #include "pvt_internal.h"
 
 namespace pvt {
@@ -107,7 +107,7 @@ struct SelParams {
   uint32_t* hist1;       // members of the threshold bin: key bits [17:9]
   uint32_t* fine;        // members of the threshold bin: key bits [17:0]
   uint32_t* state;       // [0] threshold bin, [1] keys still to be taken from it, [2] ticket
-  uint64_t* counts;      // per CTA of the last pass: ready << 62 | equal << 31 | greater
+  uint64_t* counts;      // per CTA of the last pass: ready << 63 | equal << 31 | greater
 };
 
 // inclusive scan over a block of 1024 threads; `sh` has one word per warp
