@@ -70,3 +70,15 @@ def test_block_without_dequantisation_and_with_skipped_outputs():
     assert torch.equal(idxs[0], idxs[1])
     want = oracle.dequant(devs[1].codes.cpu().numpy(), L.codebooks, L.scale, 64, 256)
     assert out.cpu().numpy().tobytes() == want.tobytes()
+
+
+@pytest.mark.gpu
+def test_the_stream_is_the_current_one_with_and_without_the_quick_query(monkeypatch):
+    side = torch.cuda.Stream()
+    for stream in (torch.cuda.default_stream(), side):
+        with torch.cuda.stream(stream):
+            quick = B._stream_ptr(None)
+            with monkeypatch.context() as m:
+                m.setattr(B, "_raw_stream", None)  # a torch without it
+                assert B._stream_ptr(None) == quick == stream.cuda_stream
+    assert B._stream_ptr(side) == side.cuda_stream
