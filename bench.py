@@ -381,13 +381,15 @@ def search_roofline(engine, pairs_per_step, enc_ms, enc_n, steps, peaks, traffic
              "frac_of_epilogue_bound": common["pairs_per_s"] / peaks["epilogue_pairs_per_s"],
              "epilogue_bound_is": "one accumulator read per pair: 128 lanes per SM per clock at the maximum SM clock"}
     else:
-        r = {"kernel": "encode_m1_kernel (exhaustive search, FP32 pipe)" if engine == "fp32"
-             else "encode_beam_kernel (beam search)", "bound": "alu", "peak": peaks["alu_tflops"],
+        r = {"kernel": {"fp32": "encode_m1_kernel (exhaustive search, FP32 pipe)",
+                        "small": "encode_m1_small_kernel (exhaustive search, small codebook)",
+                        "beam": "encode_beam_kernel (beam search)"}[engine], "bound": "alu", "peak": peaks["alu_tflops"],
              "frac": achieved / peaks["alu_tflops"],
              "peak_is": f"{peaks['sm_count']} SMs x 128 FP32 lanes x 2 flop x {peaks['sm_max_mhz_used']:.0f} MHz "
                         f"(derived; no measured FP32 peak)"}
         if engine == "beam":
-            r["note"] = ("issue-bound; stage 2 (2048 of 2304 pairs per group) on the tensor pipe for fp16 codebooks; "
+            r["note"] = ("no unit full (issue slots and shared memory about two thirds); stage 2 (2048 of 2304 pairs per "
+                         "group) on the tensor pipe for fp16 codebooks; "
                          "the search as written needs 16 (K1 + K2) + 2 B K2 flop per group (B.K2 cross terms reuse "
                          "<t, c2>), the 16 flop per pair of the metric count every pair as a full dot product")
     r.update(common)
@@ -400,7 +402,7 @@ def engine_of(layer, search):
     f16 = layer.L.codebooks.dtype.itemsize == 2
     if f16 and (search == "tensor" or (search == "auto" and layer.K >= 1024)):
         return "tensor"
-    return "fp32"
+    return "small" if layer.K <= 1024 else "fp32"
 
 
 _PROFILE_OF = {"tensor": ("encode_m1_tc_kernel_8192x1024_1x16_tau1.0.md", ["pvt_encode_m1_tc.cu", "pvt_encode_m1.cuh"]),
@@ -587,8 +589,7 @@ def sub_record(args, dev, local, peaks, flush_l2, resident_layers):
         steps = 20
         t = runner.timed(steps, 3, flush_l2)
         enc_ms, enc_n = t["kern"][B.PVT_KERNEL_ENCODE_MAIN]
-        r = search_roofline(engine, runner.pairs, enc_ms, enc_n, steps, peaks, recorded_traffic(engine, runner.k)
-                            if engine == "fp32" else recorded_traffic(engine, runner.k))
+        r = search_roofline(engine, runner.pairs, enc_ms, enc_n, steps, peaks, recorded_traffic(engine, runner.k))
         st = stage_record(runner, t, steps, peaks, 4)
         out[engine] = {"ms_per_step": t["ms_per_step"], "groups_per_s": runner.k / (t["ms_per_step"] * 1e-3),
                        "pairs_per_s": runner.pairs / (t["ms_per_step"] * 1e-3), "graph_replay": t["graphed"],
@@ -753,7 +754,7 @@ def _time_oracle_encode(oracle, L, idx, codes2):
 
 
 def _oracle_sample(oracle, L, k, search_budget_s, probe=256):
-    """The CPU checker, as it stands, on one layer: norms and selection over all its groups, the search on the
+    """The CPU oracle, as it stands, on one layer: norms and selection over all its groups, the search on the
     first n selected groups (n sized for about `search_budget_s` seconds), dequantisation of the whole layer."""
     t0 = time.perf_counter()
     idx = oracle.select(oracle.group_norms(L.g, L.eta), k)
@@ -770,7 +771,7 @@ def _oracle_sample(oracle, L, k, search_budget_s, probe=256):
 
 
 def _extrapolate(sample_layer, k_sample, n, t_sel, t_enc, t_deq, G_total, k_total, pairs_total):
-    """Whole-workload step time of the checker from its timings on one layer: selection and dequantisation
+    """Whole-workload step time of the oracle from its timings on one layer: selection and dequantisation
     scale with the groups, the search with the codeword pairs."""
     pairs_n = n * sample_layer.pairs_per_group()
     return (t_sel + t_deq) * (G_total / sample_layer.num_groups) + t_enc * (pairs_total / pairs_n)
@@ -853,7 +854,7 @@ def host_layers(kind):
 
 
 def run_reference(args):
-    """The CPU checker timed as the reference arm: every step is one bounded sample of the workload (selection
+    """The CPU oracle timed as the reference arm: every step is one bounded sample of the workload (selection
     over all groups of its smallest layer, search of n of that layer's selected groups for about two seconds,
     dequantisation of that layer), extrapolated linearly to the whole workload; value = groups re-encoded per
     second of that step."""
@@ -886,7 +887,7 @@ def run_reference(args):
               "group_dim": 8, "groups": G_total, "num_codebooks": first.M, "codebook_size": first.K,
               "codebook_dtype": "f16" if first.K > 256 or first.M > 1 else "f32",
               "tau": first.tau, "k": k_total, "pairs_per_step": pairs_total,
-              "search_engine": "cpu checker (binary64)", "dequant_dtype": "f32",
+              "search_engine": "cpu oracle (binary64)", "dequant_dtype": "f32",
               "l2": "not applicable", "launch": "host threads", "parallelism": "host cores"}
     line = {"impl": "reference", "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": args.gpus,
             "steps": args.steps, "warmup": warm, "ms_per_step": t_step * 1e3, "higher_is_better": True,
