@@ -1,5 +1,5 @@
 /*
- * CPU checker for the discrete V step of PV-Tuning.  TEST INFRASTRUCTURE ONLY:
+ * CPU oracle for the discrete V step of PV-Tuning.  TEST INFRASTRUCTURE ONLY:
  * it defines what the GPU library must compute, it is deliberately plain and
  * slow, and it shares no code with the CUDA path.  Only the tests, the smoke
  * check and the benchmark's CPU-baseline leg may call it.

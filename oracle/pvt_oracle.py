@@ -1,8 +1,8 @@
-"""ctypes binding of the CPU checker (``pvt_oracle.c``).
+"""ctypes binding of the CPU oracle (``pvt_oracle.c``).
 
 TEST INFRASTRUCTURE ONLY: imported by the tests, the smoke check and the
 benchmark's CPU-baseline leg; never by the GPU library or its Python binding.
-The checker is compiled on first use with ``gcc -O2 -ffp-contract=off
+The oracle is compiled on first use with ``gcc -O2 -ffp-contract=off
 -fopenmp`` (no fused operations other than its explicit ``fmaf`` calls).
 """
 from __future__ import annotations
@@ -21,7 +21,7 @@ _lib = None
 
 
 def build(force: bool = False) -> str:
-    """Compile the checker into ``libpvt_oracle.so`` next to its source."""
+    """Compile the oracle into ``libpvt_oracle.so`` next to its source."""
     if force or not os.path.exists(_LIB) or os.path.getmtime(_LIB) < os.path.getmtime(_SRC):
         cmd = ["gcc", "-O2", "-ffp-contract=off", "-fopenmp", "-fPIC", "-shared", "-Wall",
                "-o", _LIB, _SRC, "-lm"]

@@ -4,7 +4,7 @@ This module only draws random numbers and lays them out; it performs none of
 the V step's own arithmetic (no norms, no selection, no codeword search, no
 dequantisation).  Where the recipe of an input needs a nearest-codeword
 assignment (the second residual codebook, "nearest" previous codes) the caller
-passes that routine in as ``nearest``; the CPU checker's tests pass theirs and
+passes that routine in as ``nearest``; the CPU oracle's tests pass theirs and
 the benchmark passes the GPU library's.
 
 Recipe (stand-ins for Llama-2 linear layers: only their shapes are real):
