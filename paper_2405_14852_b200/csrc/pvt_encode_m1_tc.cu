@@ -27,11 +27,11 @@
 // codebook go through buffer 0, odd ones through buffer 1.  Warp 16 copies the codebook (two stages of eight steps).
 //
 // What bounds it: not a pipe but the ring each accumulator goes round - MMA issued, executed, completion seen, read out,
-// release seen -, with all of tensor memory in flight (a fp16 accumulator takes a 32-bit column too).  Measured at
-// 1048576 targets x 65536 codewords and 1965 MHz: 3223 us, that is 447 cycles per 256 x 128 scores (an accumulator comes
-// round once in two of these steps); 365 with neither minima nor comparisons.  The tensor pipe is busy for 130 of them
-// (31 % of the active cycles by its counter) and the minima take 128 of the ALU's; issue slots 44 %.  A small subspace runs
-// below that rate, for units begin, drain and end more often: 20971 targets 89 us, 616 cycles a step.  Against binary32
+// release seen -, with all of tensor memory in flight (a fp16 accumulator takes a 32-bit column too).  Measured with the
+// SM's own clock counter (1845 MHz under this load), 1048576 targets x 65536 codewords: 3223 us, 414 cycles per 256 x 128
+// scores (an accumulator comes round once in two of these steps); 335 with neither minima nor comparisons.  The tensor pipe
+// is busy for 130 of them (31 % by its counter) and the minima take 128 of the ALU's; issue slots 44 %.  A small subspace
+// runs below that rate, for units begin, drain and end more often: 20971 targets 89 us, 525 cycles a step.  Against binary32
 // accumulators, two instructions per step, eight epilogue warps that alternate between the buffers and one issuing warp per
 // A block: 3245 us for 4556 us.  Of this, fp16 accumulators gave 4556 -> 3740; four issuing warps alone nothing; sixteen
 // epilogue warps with a buffer each 3900 -> 3300; an arrival by all threads of a warp instead of one behind a branch
