@@ -59,3 +59,19 @@ def test_gradients_at_the_edges(M, K, f16, rows, per_row, gd, offset):
     # n terms of magnitude <= a, added in another order
     assert np.abs(gb.cpu().numpy() - want_b).max() <= G * 1.5 * np.abs(g).max() * 2.0 ** -50
     assert np.abs(gs.cpu().numpy() - want_s).max() <= cols * np.abs(g).max() * np.abs(books.astype(np.float32)).max() * M * 2.0 ** -50
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,offset", [(4, 0), (8, 0), (12, 0), (2052, 4), (303112, 0)])
+def test_the_direction_may_take_the_place_of_the_gradient(n, offset):
+    rng = np.random.default_rng(n)
+    grad = rng.normal(0.0, 1e-3, size=n).astype(np.float32)
+    m, v = rng.normal(0.0, 1e-3, size=n).astype(np.float32), rng.uniform(0.0, 1e-6, size=n).astype(np.float32)
+    flat = [torch.zeros(n + offset, dtype=torch.float32, device="cuda")[offset:] for _ in range(3)]
+    for t, a in zip(flat, (grad, m, v)):
+        t.copy_(torch.from_numpy(a))
+    want = oracle.adam_direction(grad, m, v, 3)
+    B.pvt_adam_direction(flat[0], flat[1], flat[2], flat[0], 3)
+    torch.cuda.synchronize()
+    for t, a in zip(flat, (want, m, v)):
+        assert t.cpu().numpy().tobytes() == a.tobytes()

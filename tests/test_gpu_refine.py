@@ -102,3 +102,24 @@ def test_refine_rejects_bad_arguments():
         with pytest.raises(B.PvtError) as e:
             B.pvt_vstep_refine(dev.desc, idx, k, mm)
         assert e.value.code == B.PVT_EINVAL
+
+
+@pytest.mark.parametrize("M,K,f16,k", [
+    (2, 100, True, 9473),    # staged: more targets than twice the resident warps, one in the last trip
+    (3, 64, False, 5000),    # two resident blocks per SM
+    (1, 600, True, 19001),   # nothing staged: more than the doubled grid takes at once
+    (4, 200, True, 9500),
+])
+def test_refine_with_more_targets_than_resident_warps(M, K, f16, k):
+    L = synth.make_layer(320, 512, cfg=208, num_codebooks=M, codebook_size=K, codebook_fp16=f16, nearest=oracle_nearest)
+    G = L.num_groups
+    idx = np.sort(np.random.default_rng(k).choice(G, size=k, replace=False)).astype(np.uint32)
+    at = idx.astype(np.int64)
+    t = oracle.targets(L.W, L.g, L.scale, L.eta, idx)
+    want, d, want_moves = oracle.local_search(t, L.codebooks, L.codes.reshape(G, M)[at], 2)
+    codes, err, moves, status = gpu_refine(L, idx, 2)
+    assert status == 0
+    assert np.array_equal(codes.reshape(G, M)[at].astype(np.int32), want)
+    assert np.array_equal(moves, want_moves) and np.array_equal(err, d.astype(np.float32))
+    rest = np.setdiff1d(np.arange(G), at)
+    assert np.array_equal(codes.reshape(G, M)[rest], L.codes.reshape(G, M)[rest])
