@@ -16,8 +16,9 @@
 //              takes, waits for the counts of the CTAs before it and writes its part of the list by ballots:
 //              position = (#greater before) + min(#equal before, ties to take)
 // Measured as graph replays, 4096 x 4096 / 11008 x 4096 / 28672 x 8192: 32 / 53 / 245 us.  Of the first, by its counters,
-// pass 1 takes 16 us (4.2 TB/s of g from cold; 5.4 for the second), the others 4.5, 10 and 12.  Five passes with one bin per
-// eighth of an octave took 45 / 74 / 344 us.  One cooperative kernel with the keys in shared memory takes 33 us, and about 10 us more to launch.
+// pass 1 takes 16 us (4.2 TB/s of g from cold; 5.4 for the second), the others 4.5, 10 and 12.  Five passes with one bin
+// per eighth of an octave took 45 / 74 / 344 us.  One cooperative kernel with the keys in shared memory takes 33 us, and
+// about 10 us more to launch.
 #include "pvt_internal.h"
 
 namespace pvt {
@@ -192,7 +193,7 @@ __device__ __forceinline__ void find_digit_warp(const uint32_t* hist, uint32_t k
   *left = __shfl_sync(0xffffffffu, l, src);
 }
 
-// ---- 0. what pass 1 adds to starts at zero
+// ---- 0. everything the passes count in starts at zero
 __global__ void __launch_bounds__(kSelThreads) select_clear_kernel(uint4* scratch, uint32_t n16) {
   pdl_trigger();
   pdl_wait();
