@@ -24,10 +24,11 @@
 // the beam, the final argmin) is taken on binary64 distances accumulated in index order (the residual carried through
 // the codebooks in order), so the result is the argmin of (distance, tuple) over the pool exactly as defined.
 // What bounds it: no unit by itself.  With two / three codebooks 740 / 1470 warp instructions per target fill 64 / 60 % of
-// the issue slots and shared memory is busy 66 / 76 % of the time; the rest are the dependences of one target's chain (sort,
-// warp minima, acceptance), which six warps per scheduler do not hide.  56 360 targets of an 11008 x 4096 layer, two /
-// three / four fp16 codebooks of 256: 72 / 152 / 258 us; three binary32 codebooks 220 us.  (A warp per target, with two passes over all extensions in every stage and every decision in
-// binary64: 415 / 522 us for three / four, 992 us for three binary32 codebooks.)
+// the issue slots and shared memory is busy 66 / 76 % of the time; the rest are the dependences of one target's chain
+// (sort, warp minima, acceptance), which six warps per scheduler do not hide.  56 360 targets of an 11008 x 4096 layer,
+// two / three / four fp16 codebooks of 256: 72 / 152 / 258 us; three binary32 codebooks 220 us.  (A warp per target, with
+// two passes over all extensions in every stage and every decision in binary64: 415 / 522 us for three / four, 992 us for
+// three binary32 codebooks.)
 #include <cuda_fp16.h>
 
 #include "pvt_internal.h"
