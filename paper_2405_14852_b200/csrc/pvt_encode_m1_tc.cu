@@ -249,20 +249,43 @@ __device__ __forceinline__ void tmem_relinquish() {
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
 }
-// D[tmem] (+)= A[smem] * B[smem]^T, fp16 x fp16 -> fp16, M = 128, N = 128, K = 16;
-// accumulate == 0 overwrites D
-__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                         uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
+// One step of an accumulator, D[tmem] = A[smem] * B[smem]^T (fp16 x fp16 -> fp16, M = 128, N = 128, K = 16 per instruction,
+// the second, for groups of 16, onto the first), and the arrival on the mbarrier that follows its completion.  The whole
+// warp calls; one thread, always the same, is elected inside the statement.  (A branch on the lane in its place leaves the
+// compiler without the knowledge that one thread runs it, and the operands go through a loop over the active lanes: issue
+// and commit took 107 cycles by themselves, 310 to 370 beside the other warps, where this takes 9.)
+template <int MMAS>
+__device__ __forceinline__ void umma_step(uint32_t d_tmem, const uint64_t* a_desc, uint64_t b_desc, uint32_t idesc,
+                                          uint32_t bar) {
+  if constexpr (MMAS == 1) {
+    asm volatile(
+        "{\n\t.reg .pred one, onto;\n\t"
+        "elect.sync _|one, 0xffffffff;\n\t"
+        "setp.ne.b32 onto, 0, 0;\n\t"
+        "@one tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, onto;\n\t"
+        "@one tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%4];\n\t}" ::"r"(d_tmem),
+        "l"(a_desc[0]), "l"(b_desc), "r"(idesc), "r"(bar)
+        : "memory");
+  } else {
+    asm volatile(
+        "{\n\t.reg .pred one, onto;\n\t"
+        "elect.sync _|one, 0xffffffff;\n\t"
+        "setp.ne.b32 onto, 0, 0;\n\t"
+        "@one tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, onto;\n\t"
+        "setp.eq.b32 onto, 0, 0;\n\t"
+        "@one tcgen05.mma.cta_group::1.kind::f16 [%0], %5, %6, %3, onto;\n\t"
+        "@one tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%4];\n\t}" ::"r"(d_tmem),
+        "l"(a_desc[0]), "l"(b_desc), "r"(idesc), "r"(bar), "l"(a_desc[1]), "l"(b_desc + (uint64_t)(2 * (128 >> 4)))
+        : "memory");
+  }
 }
-// arrive on the mbarrier once all MMAs issued so far by this thread have completed
+// arrive on the mbarrier once all MMAs issued so far by the warp's elected thread have completed; called by the whole warp
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+  asm volatile(
+      "{\n\t.reg .pred one;\n\t"
+      "elect.sync _|one, 0xffffffff;\n\t"
+      "@one tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
+      : "memory");
 }
 // shared-memory operand descriptor: K-major, no swizzle, K chunks 128 B apart, 8-row groups group_bytes apart
 __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t group_bytes) {
@@ -492,28 +515,20 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
             if (alive) alive = wait_all(empty, (j & 1) ? 0u : 1u);
             if (alive) {
               tc_fence_after();
-              if (lane == 0) {
-                // two K chunks per instruction
-#pragma unroll
-                for (int m = 0; m < D::kMmas; ++m)
-                  umma_f16(d, a_desc[m], b_s + (uint64_t)(2 * j * (kStepBytes >> 4) + 2 * m * (128 >> 4)), kIdesc, m > 0);
-                umma_commit(full);  // the accumulator is ready
-              }
-              __syncwarp();
+              umma_step<D::kMmas>(d, a_desc, b_s + (uint64_t)(2 * j * (kStepBytes >> 4)), kIdesc, full);
             }
           }
         }
         // this warp has read the whole stage (the last stage is not reused)
-        if (alive && base + kTcGroupSteps < total && lane == 0) umma_commit(smem_u32(&sm.empty_bar[s]));
-        __syncwarp();
+        if (alive && base + kTcGroupSteps < total) umma_commit(smem_u32(&sm.empty_bar[s]));
         s = (s == (uint32_t)kTcStages - 1) ? 0 : s + 1;
         if (s == 0) stage_par ^= 1;
       }
-      if (!alive && lane == 0) {
+      if (!alive) {
         // wait (bounded) for whatever was issued before tensor memory is released
         umma_commit(smem_u32(&sm.drain_bar[2 * buf + q]));
         for (uint32_t spin = 0; spin < kMaxSpins; ++spin) {  // always the full limit: these MMAs do complete
-          if (mbar_try_wait(smem_u32(&sm.drain_bar[2 * buf + q]), 0)) break;
+          if (__all_sync(0xffffffffu, mbar_try_wait(smem_u32(&sm.drain_bar[2 * buf + q]), 0))) break;
           __nanosleep(64);
         }
       }
