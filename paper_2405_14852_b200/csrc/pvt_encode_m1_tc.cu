@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
       for (uint64_t u = blockIdx.x; u < units && alive; u += gridDim.x) {
         uint32_t s_lo, s_hi;
         slice_units(p, (uint32_t)(u % p.n_slices), &s_lo, &s_hi);
-        for (uint32_t st = s_lo; st < s_hi && alive; ++st, ++it) {
+        for (uint32_t st = s_lo; st < s_hi && alive;) {
           const uint32_t grp = it / kTcGroupSteps, sub = it % kTcGroupSteps, s = grp % kTcStages;
           const uint32_t fb = smem_u32(&sm.full_bar[s]);
           if (sub == 0) {
@@ -442,10 +442,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
               mbar_expect_tx(fb, (left < (uint32_t)kTcGroupSteps ? left : (uint32_t)kTcGroupSteps) * kStepBytes);
             __syncwarp();
           }
+          // the steps up to the end of the stage or of the unit lie one after the other on both sides: one copy
+          const uint32_t room = kTcGroupSteps - sub, n = s_hi - st < room ? s_hi - st : room;
           // test hook: a step that is never copied leaves its stage's barrier incomplete, so the MMA warps' wait
           // for that stage runs out
-          if (lane == 0 && it != p.withhold_copy)
-            bulk_g2s(smem_u32(&sm.b[s][sub][0]), bimg + (size_t)st * kStepBytes, kStepBytes, fb);
+          if (lane == 0 && p.withhold_copy - it >= n)
+            bulk_g2s(smem_u32(&sm.b[s][sub][0]), bimg + (size_t)st * kStepBytes, n * kStepBytes, fb);
+          st += n;
+          it += n;
         }
       }
       if (!alive && lane == 0) {
