@@ -329,19 +329,21 @@ __device__ __forceinline__ void tmem_ld_wait(uint32_t* v, uint32_t* w) {
 // taken does not matter (all are within the error bound of the best).  So the maxima are minima of unsigned 16-bit
 // halves: the three-operand minimum takes two registers per instruction, the two-operand f16x2 maximum one at twice the
 // rate - as fast, with half as many instructions.
-__device__ __forceinline__ uint32_t key_min64(const uint32_t* v) {
-  uint32_t m[4];
+// Which of 64 keys are below a cap, in 16 instructions: both halves of the result are the cap if none is, otherwise one of
+// them is the smallest key.
+__device__ __forceinline__ uint32_t key_min64(const uint32_t* v, uint32_t cap) {
+  uint32_t m[4] = {__vimin3_u16x2(v[0], v[1], cap), __vimin3_u16x2(v[2], v[3], v[4]), __vimin3_u16x2(v[5], v[6], v[7]),
+                   __vimin3_u16x2(v[8], v[9], v[10])};
 #pragma unroll
-  for (int i = 0; i < 4; ++i) m[i] = __vimin3_u16x2(v[i], v[i + 4], v[i + 8]);
+  for (int i = 11; i < 27; i += 8)
 #pragma unroll
-  for (int i = 12; i < 28; i += 8)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) m[q] = __vimin3_u16x2(m[q], v[i + q], v[i + 4 + q]);
-  m[0] = __vimin3_u16x2(m[0], v[28], v[29]);
-  m[1] = __vimin3_u16x2(m[1], v[30], v[31]);
-  const uint32_t x = __vimin3_u16x2(__vminu2(m[0], m[1]), m[2], m[3]);
-  return min(x & 0xffffu, x >> 16);
+    for (int q = 0; q < 4; ++q) m[q] = __vimin3_u16x2(m[q], v[i + 2 * q], v[i + 2 * q + 1]);
+  m[0] = __vimin3_u16x2(m[0], v[27], v[28]);
+  m[1] = __vimin3_u16x2(m[1], v[29], v[30]);
+  m[2] = __vimin3_u16x2(m[2], v[31], m[3]);
+  return __vimin3_u16x2(m[0], m[1], m[2]);
 }
+__device__ __forceinline__ uint32_t lower_half(uint32_t x) { return min(x & 0xffffu, x >> 16); }
 __device__ __forceinline__ float key_score(uint32_t key) { return __half2float(__ushort_as_half((unsigned short)key)); }
 // the key of the largest half not above a score, and of -0 from there on: every half that reaches the score passes
 __device__ __forceinline__ uint32_t key_limit(float score) {
@@ -683,6 +685,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
       // to begin with, every thread remembers its first steps one after the other: 4096x4096 1x16 95 us instead of 90.)
       const float seed = sm.seed[own];
       uint32_t lim = key_limit(seed - fmaf(kRelMargin, fabsf(seed), margin));
+      uint32_t cap = (lim + 1) * 0x10001u;  // (a key is a half with the sign bit: the limit is far below 0xffff)
       auto note = [&](uint32_t key, uint32_t sub) {
         if (key <= lim) {
           const uint32_t slot = list_cnt & (kTcListLen - 1);
@@ -691,6 +694,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
           ++list_cnt;
           best = fmaxf(best, key_score(key));
           lim = min(lim, key_limit(best - fmaf(kRelMargin, fabsf(best), margin)));
+          cap = (lim + 1) * 0x10001u;
         }
       };
       for (uint32_t st = s_lo + ((it ^ set) & 1); st < s_hi && alive; st += 2, ++uses) {
@@ -708,10 +712,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
         tmem_ld_wait(v, w);
         tc_fence_before();
         mbar_arrive(empty);
-        const uint32_t ka = key_min64(v), kb = key_min64(w);
-        if (min(ka, kb) <= lim) {
-          note(ka, 2 * st);
-          note(kb, 2 * st + 1);
+        const uint32_t xa = key_min64(v, cap), xb = key_min64(w, cap);
+        if ((xa ^ cap) | (xb ^ cap)) {
+          note(lower_half(xa), 2 * st);
+          note(lower_half(xb), 2 * st + 1);
         }
       }
       it += s_hi - s_lo;
