@@ -540,6 +540,7 @@ cudaError_t launch_encode_m1(const pvt_layer& L, uint64_t G, const uint32_t* idx
   p.K = (uint32_t)L.codebook_size;
   p.n_tiles = lay.n_tiles;
   p.n_slices = lay.n_slices;
+  p.slice_div = make_fast_div(lay.n_slices);
   p.tile = lay.tile;
   p.gbest = reinterpret_cast<uint32_t*>(base + lay.gbest_off);
   p.margin = reinterpret_cast<float*>(base + lay.margin_off);

@@ -36,6 +36,7 @@ struct EncM1Params {
   const uint32_t* n2max_bits;
   uint32_t K, n_tiles, n_slices, tile;
   uint32_t n_units, unit_cw;  // the codebook is cut into n_units units of unit_cw codewords; a slice is a run of whole units
+  FastDiv slice_div;          // n_slices as a divisor
   uint32_t sub_cw;            // codewords per remembered sub-chunk (a multiple of 32 that divides unit_cw)
   // codewords the fast score cannot represent, always rescored: their number (may be null), and by block of codewords the
   // number and the places in the list
@@ -180,8 +181,8 @@ __device__ __forceinline__ void cand_write(CandRecord* to, const CandRecord& r) 
 
 // units [lo, hi) of slice sl
 __device__ __forceinline__ void slice_units(const EncM1Params& p, uint32_t sl, uint32_t* lo, uint32_t* hi) {
-  *lo = (uint32_t)((uint64_t)sl * p.n_units / p.n_slices);
-  *hi = (uint32_t)((uint64_t)(sl + 1) * p.n_units / p.n_slices);
+  *lo = fast_div(sl * p.n_units, p.slice_div);  // (at most 16 slices of 512 units)
+  *hi = fast_div((sl + 1) * p.n_units, p.slice_div);
 }
 
 }  // namespace m1

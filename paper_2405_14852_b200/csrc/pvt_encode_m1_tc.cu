@@ -18,25 +18,28 @@
 // costs is (2^e t - hi) . (c - t), a small vector times the distance.  So one instruction of fp16 accuracy serves where
 // <t, c> - h needed t in two halves, two instructions and binary32 scores, and few sub-chunks come within the margin.
 // The codebook image is written once per call by a small kernel in exactly the shared-memory byte order, so every
-// 128-codeword step arrives with one 1-D bulk copy (4 KB); the A rows are written by the threads that own the targets.
+// 128-codeword step arrives with one 1-D bulk copy (4 KB); the A rows are written by threads of the CTA.
 // e_n is chosen per target so that max_i |2^e t_i| lies in [1/2, 1), smaller if the best score would not be a half.
 //
 // CTA = 256 targets (two 128-row A blocks) x a slice of the codebook, one CTA per SM, persistent over (tile, slice) units.
 // Tensor memory: 2 buffers x 2 A blocks x 128 columns = 512 columns.  Each of these four accumulators has one warp that
-// issues its MMAs (warps 17-20) and four that read it out (warps 0-15; warp w reads lanes 32 (w % 4) ..): even steps of the
-// codebook go through buffer 0, odd ones through buffer 1.  Warp 16 copies the codebook (two stages of eight steps).
+// issues its MMAs (warps 16-19) and four that read it out (warps 0-15; warp w reads lanes 32 (w % 4) ..): even steps of the
+// codebook go through buffer 0, odd ones through buffer 1.  Warp 20 copies the codebook (two stages of eight steps), warps
+// 21-23 form the targets of the next unit.  That is six warps on each scheduler; the ones that wait long sleep.
 //
-// What bounds it: not a pipe but the ring each accumulator goes round - MMA issued, executed, completion seen, read out,
-// release seen -, with all of tensor memory in flight (a fp16 accumulator takes a 32-bit column too).  Measured with the
-// SM's own clock counter (1845 MHz under this load), 1048576 targets x 65536 codewords: 3223 us, 414 cycles per 256 x 128
-// scores (an accumulator comes round once in two of these steps); 335 with neither minima nor comparisons.  The tensor pipe
-// is busy for 130 of them (31 % by its counter) and the minima take 128 of the ALU's; issue slots 44 %.  A small subspace
-// runs below that rate, for units begin, drain and end more often: 20971 targets 89 us, 525 cycles a step.  Against binary32
-// accumulators, two instructions per step, eight epilogue warps that alternate between the buffers and one issuing warp per
-// A block: 3245 us for 4556 us.  Of this, fp16 accumulators gave 4556 -> 3740; four issuing warps alone nothing; sixteen
-// epilogue warps with a buffer each 3900 -> 3300; an arrival by all threads of a warp instead of one behind a branch
-// 3300 -> 3245.  Tried and slower: the epilogue issuing its own MMAs (4533: its minima join the ring), the copies in an
-// issuing warp (3460), the issue loop in one thread (3570).
+// What bounds it: the ring each accumulator goes round - MMA issued, executed, completion seen, read out, release seen -,
+// with all of tensor memory in flight (a fp16 accumulator takes a 32-bit column too), and on it the instructions of the
+// warps that share a scheduler.  By the SM's own clock counter (1820 MHz under this load) 1048576 targets x 65536 codewords
+// take 298 cycles per 256 x 128 scores, an accumulator coming round once in two of these steps; MMAs and tensor-memory
+// loads together keep their pipe busy for 200 of them, the minima the ALU for 130.  20971 targets: 64 us.
+// Before, in us for 1048576 / 20971 targets: 3228 / 90.6.  The issuing thread elected inside the statement (umma_step):
+// 2990; one codebook copy per run of steps in place of one per step: 2510; the limit as a member of the minima: 2402 / 72.4;
+// the next unit's targets formed beside the search, units counted without 64-bit divisions: 2367 / 63.6.  (A unit used to
+// begin 7500 cycles after the end of the one before it.)
+// Tried and slower: two issuing warps (2800), the events of a step handled while the next one's columns are on their way
+// (2520: spills), the read-out warps issuing their own MMAs (a bare ring of this kind: 411 cycles for 250), 64-column
+// accumulators (344), mma.sync beside tcgen05 (they share a pipe), four or five codebook stages (no change).  Against
+// binary32 accumulators, two instructions per step and eight read-out warps: 4556.
 //
 // Codewords whose half squared norm exceeds the fp16 range get a sentinel row
 // that can never win and are listed as "exceptions": the rescoring kernel always
@@ -77,7 +80,11 @@ constexpr int kTcGroupSteps = 8;        // steps per codebook stage: the MMA war
 constexpr int kTcStages = 2;            // codebook stages (eight steps each: 32 KB, or 64 KB for groups of 16)
 constexpr int kTcEpiThreads = 512;      // two sets of 256, one thread per target each: even and odd steps
 constexpr int kTcEpiWarps = kTcEpiThreads / 32;
-constexpr int kTcThreads = kTcEpiThreads + 160;  // + producer warp + one MMA warp per A block and accumulator buffer
+constexpr int kTcMmaWarp = kTcEpiWarps;     // the first of four: one per A block and accumulator buffer
+constexpr int kTcCopyWarp = kTcMmaWarp + 4;
+constexpr int kTcFormWarp = kTcCopyWarp + 1;  // the first of three that form the next unit's targets
+constexpr int kTcFormers = 96;
+constexpr int kTcThreads = 32 * kTcFormWarp + kTcFormers;  // 24 warps, six per scheduler
 // What the search has to know of the codewords, by block of 256 of them: written by the kernel that prepares the image, so
 // that nothing has to be cleared before it.
 constexpr uint32_t kTcPrepCw = 256;
@@ -351,21 +358,24 @@ __device__ __forceinline__ uint32_t key_limit(float score) {
 }
 
 // ---- shared memory -----------------------------------------------------------------
+constexpr float kOutOfRange = -1.0f, kAbsent = -2.0f;  // in place of a margin
 template <int DG>
 struct TcSmem {
-  alignas(128) unsigned char a[2][TcDim<DG>::kABlockBytes];  // two A blocks of 128 targets
+  alignas(128) unsigned char a[2][2][TcDim<DG>::kABlockBytes];  // of this unit and the next: two A blocks of 128 targets
   alignas(128) unsigned char b[kTcStages][kTcGroupSteps][TcDim<DG>::kStepBytes];
   alignas(8) uint64_t full_bar[kTcStages];
   uint64_t empty_bar[kTcStages];
   uint64_t tmem_full[2][2];   // per buffer and A block
   uint64_t tmem_empty[2][2];
-  uint64_t a_ready;
+  uint64_t a_first;               // the first unit's rows
+  uint64_t a_ready[2], a_free[2];  // per unit parity
   uint64_t drain_bar[4];
-  uint32_t list[kTcListLen][kTcEpiThreads];  // key of the maximum (upper half) and number of the sub-chunk
-  float margin[kTcTile];   // per target; negative if it is out of range or absent
-  float seed[kTcTile];      // score of the stored code
-  float odd_best[kTcTile];  // what the odd set leaves for the even one
-  uint32_t odd_cnt[kTcTile], odd_evicted[kTcTile];
+  // key of the maximum (upper half) and number of the sub-chunk: of the even set, and of the odd one by unit parity
+  uint32_t list[3][kTcListLen][kTcTile];
+  float margin[2][kTcTile];   // per unit parity and target; kOutOfRange, kAbsent
+  float seed[2][kTcTile];     // score of the stored code
+  float odd_best[2][kTcTile];  // what the odd set leaves for the even one
+  uint32_t odd_cnt[2][kTcTile], odd_evicted[2][kTcTile];
   uint32_t tmem_base;
   uint32_t abort_flag;
   uint32_t n2max_bits, n2min_inv, n_exc;  // over all codewords
@@ -394,11 +404,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
         mbar_init(smem_u32(&sm.tmem_empty[b][q]), 128);  // every thread of the four warps
       }
     }
-    mbar_init(smem_u32(&sm.a_ready), kTcTile);
+    mbar_init(smem_u32(&sm.a_first), kTcTile);
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(smem_u32(&sm.a_ready[b]), kTcFormers);
+      mbar_init(smem_u32(&sm.a_free[b]), 4 + kTcEpiWarps);  // one commit per MMA warp, one arrival per read-out warp
+    }
     for (int i = 0; i < 4; ++i) mbar_init(smem_u32(&sm.drain_bar[i]), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == kTcEpiWarps + 1) {
+  if (warp == kTcMmaWarp) {
     tmem_alloc(smem_u32(&sm.tmem_base), kTmemCols);
     tmem_relinquish();
   }
@@ -408,35 +422,168 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(&sm.tmem_base);
 
   pdl_wait();
-  const uint64_t units = (uint64_t)p.n_tiles * p.n_slices;
+  // unit u is slice u % n_slices of tile u / n_slices
+  const uint32_t units = p.n_tiles * p.n_slices;
+  // (in 32 bits: at most 2^24 tiles of one slice, fewer of more; a 64-bit division takes a warp a thousand cycles)
+  auto unit_steps = [&](uint32_t u, uint32_t* lo, uint32_t* hi) {
+    const uint32_t tile = fast_div(u, p.slice_div);
+    slice_units(p, u - tile * p.n_slices, lo, hi);
+    return tile;
+  };
+  auto total_steps = [&] {  // of this CTA
+    uint32_t total = 0;
+    if (p.n_slices == 1) {
+      total = ((units - 1 - blockIdx.x) / gridDim.x + 1) * p.n_units;
+    } else {
+      for (uint32_t u = blockIdx.x; u < units; u += gridDim.x) {
+        uint32_t s_lo, s_hi;
+        unit_steps(u, &s_lo, &s_hi);
+        total += s_hi - s_lo;
+      }
+    }
+    return total;
+  };
+  // a wait whose answer is the same in every lane: one poll by all of them when the phase is already over, otherwise
+  // lane 0 polls, a bounded number of times, and tells the others (all threads polling one barrier slow every barrier
+  // operation of the CTA down)
+  auto wait_all = [&](uint32_t bar, uint32_t parity) -> bool {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    bool ok = true;
+    if (lane == 0) ok = mbar_wait(bar, parity, abort_flag, p.status, p.max_spins);
+    return __shfl_sync(0xffffffffu, ok, 0);
+  };
+  // the same for waits that are long: the warp sleeps between its polls, so that it takes no issue slots from the others
+  auto wait_asleep = [&](uint32_t bar, uint32_t parity, uint32_t ns) -> bool {
+    for (uint32_t spin = 0; spin < p.max_spins; ++spin) {
+      if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+      if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+      __nanosleep(ns);
+    }
+    if (lane == 0) {
+      *abort_flag = 1;
+      atomicOr(p.status, PVT_DEV_WAIT_EXPIRED);
+    }
+    return false;
+  };
 
-  if (warp == kTcEpiWarps) {
+  // the index of a tile's target (an impossible one beyond the last)
+  auto target_index = [&](uint32_t tile, uint32_t own) -> uint32_t {
+    const uint64_t n = (uint64_t)tile * kTcTile + own;
+    return n < p.k ? p.idx[n] : 0xffffffffu;
+  };
+  // Forms target `own` of a unit: the group's index j -> its A row, margin and seed.
+  auto form_row = [&](uint32_t j, uint32_t own, uint32_t par) {
+    const uint32_t rb = own >> 7, r = own & 127u;
+    unsigned char* a_row = &sm.a[par][rb][(r >> 3) * D::kAGroupBytes + (r & 7) * 16];
+    const float n2max = __uint_as_float(sm.n2max_bits);
+    const float cnmax = sqrtf(n2max), hmax = 0.5f * n2max;
+    const float cnmin = sqrtf(__uint_as_float(0x7f800000u - sm.n2min_inv));  // (infinite if there is none)
+    // the target of this thread, its scaling, its A row
+    float t[DG];
+#pragma unroll
+    for (int i = 0; i < DG; ++i) t[i] = 0.0f;
+    float prev = -kNegInf;
+    const bool have = j < p.G;  // an index out of range is reported by the rescoring kernel
+    if (have) {
+      // the distance to the stored code: only what comes near it has to be remembered
+      const uint32_t code = p.code_u16 ? reinterpret_cast<const uint16_t*>(p.codes)[j]
+                                       : reinterpret_cast<const uint8_t*>(p.codes)[j];
+      if (DG == 8)
+        form_target(p, j, t);
+      else
+        form_target16(p, j, t);
+      if (code < p.K) {
+        float c[DG];
+        load_codeword<true, DG>(p.book, code, c);
+        float d = 0.0f;
+#pragma unroll
+        for (int i = 0; i < DG; ++i) d = fmaf(t[i] - c[i], t[i] - c[i], d);
+        if (d < 1e30f) prev = d;
+      }
+    }
+    float m = 0.0f, nt2 = 0.0f;
+#pragma unroll
+    for (int i = 0; i < DG; ++i) {
+      m = fmaxf(m, fabsf(t[i]));
+      nt2 = fmaf(t[i], t[i], nt2);
+    }
+    bool in_range = (m < 256.0f) && (nt2 == nt2);  // also false for Inf / NaN
+    const float norm = sqrtf(nt2);
+    int e = 0;
+    if (in_range && m > 0.0f) {
+      e = -ilogbf(m) - 1;
+      e = e > 15 ? 15 : e;
+    }
+    // the best score, at least -2^e (||t|| + min ||c||)^2 / 2, has to be a half
+    // (and above that of the padding rows, -327520 2^e)
+    const float far = norm + cnmin, low = 0.5f * far * far;
+    in_range = in_range && low < 150000.0f;
+    if (in_range && low > 1.0f) e = min(e, 14 - ilogbf(low));
+    const float sc = in_range ? scalbnf(1.0f, e) : 0.0f;
+    float r2 = 0.0f;  // ||2^e t - hi||^2
+    {
+      const uint32_t sb = __half_as_ushort(__float2half_rn(sc));
+#pragma unroll
+      for (int part = 0; part < D::kPart; ++part) {
+        __half2 hi[4];
+        float bias = 0.0f;  // sum over i of (2^e t_i - hi_i) t_i - 2^e t_i^2 / 2 = -t_i (hi_i - 2^e t_i / 2)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float tx = in_range ? t[8 * part + 2 * i] : 0.0f, ty = in_range ? t[8 * part + 2 * i + 1] : 0.0f;
+          const float x = tx * sc, y = ty * sc;  // exact products
+          hi[i] = __floats2half2_rn(x, y);
+          const float2 back = __half22float2(hi[i]);
+          r2 = fmaf(x - back.x, x - back.x, r2);
+          r2 = fmaf(y - back.y, y - back.y, r2);
+          bias = fmaf(-tx, fmaf(-0.5f, x, back.x), bias);
+          bias = fmaf(-ty, fmaf(-0.5f, y, back.y), bias);
+        }
+        const __half b_hi = __float2half_rn(bias);
+        const float r1 = bias - __half2float(b_hi);
+        const __half b_lo = __float2half_rn(r1);
+        const __half b_lo2 = __float2half_rn(r1 - __half2float(b_lo));
+        *reinterpret_cast<uint4*>(a_row + 256 * part) = reinterpret_cast<const uint4*>(hi)[0];
+        *reinterpret_cast<uint4*>(a_row + 256 * part + 128) =
+            make_uint4(sb | (sb << 16), sb | ((uint32_t)__half_as_ushort(b_hi) << 16),
+                       (uint32_t)__half_as_ushort(b_lo) | ((uint32_t)__half_as_ushort(b_lo2) << 16), sb | (sb << 16));
+      }
+    }
+    // A score is S = -2^e ||t - c||^2 / 2 but for rounding: the bias takes 2^e ||t||^2 / 2 off and adds what the rounding
+    // of the target costs at c = t.  Error bound, in the score's units: 2^-10 of itself for the rounding to a half
+    // (rounded or truncated; twice for two instructions, whose parts have one sign); for the rest of the rounding of the
+    // target r ||t - c|| <= 2^-10 |S| + 2^9 r^2 2^-e with r = ||2^e t - hi||; 2^-19 of the sum of magnitudes
+    // 2^e (||t|| ||c|| + h + ||t||^2) for the sum of products in binary32, rounded or truncated (twice the terms for
+    // groups of 16); 2^-24 where a half is subnormal, and the split of h and of the bias.  Twice that is the margin, the
+    // last terms with a factor 2 to spare: margin + kRelMargin |S|.
+    // How the tensor cores add and round is not documented: that a sum is formed to binary32 accuracy and is off by at
+    // most one unit of 2^-10 of itself per instruction as a half is an assumption.  What supports it are the tests, in
+    // which the codes are the same as those of binary64 distances.
+    const float margin = 2.0f * (517.0f * r2 / (in_range ? sc : 1.0f) +
+                                 (DG == 8 ? 3.814697265625e-6f /* 2^-18 */ : 7.62939453125e-6f) * sc *
+                                     (norm * cnmax + hmax + nt2) +
+                                 4.76837158203125e-7f /* 2^-21 */);
+    sm.margin[par][own] = !have ? kAbsent : in_range ? margin : kOutOfRange;
+    sm.seed[par][own] = in_range ? -0.5f * sc * prev * 1.0001f : kNegInf;  // (minus infinity without a stored code)
+  };
+
+  if (warp == kTcCopyWarp) {
     // ------------------------------------------------------------ bulk-copy producer
     // (the whole warp runs the loop, lane 0 issues the copies: no lane waits at the final barrier meanwhile)
     {
       // total number of steps of this CTA (for the byte count of the last, partial stage)
-      uint32_t total = 0;
-      for (uint64_t u = blockIdx.x; u < units; u += gridDim.x) {
-        uint32_t s_lo, s_hi;
-        slice_units(p, (uint32_t)(u % p.n_slices), &s_lo, &s_hi);
-        total += s_hi - s_lo;
-      }
+      const uint32_t total = total_steps();
       uint32_t it = 0;
       bool alive = true;
-      for (uint64_t u = blockIdx.x; u < units && alive; u += gridDim.x) {
+      for (uint32_t u = blockIdx.x; u < units && alive; u += gridDim.x) {
         uint32_t s_lo, s_hi;
-        slice_units(p, (uint32_t)(u % p.n_slices), &s_lo, &s_hi);
+        unit_steps(u, &s_lo, &s_hi);
         for (uint32_t st = s_lo; st < s_hi && alive;) {
           const uint32_t grp = it / kTcGroupSteps, sub = it % kTcGroupSteps, s = grp % kTcStages;
           const uint32_t fb = smem_u32(&sm.full_bar[s]);
           if (sub == 0) {
             if (grp >= (uint32_t)kTcStages) {
               const uint32_t eb = smem_u32(&sm.empty_bar[s]), ep = ((grp / kTcStages) - 1) & 1;
-              if (!__all_sync(0xffffffffu, mbar_try_wait(eb, ep))) {
-                bool ok = true;
-                if (lane == 0) ok = mbar_wait(eb, ep, abort_flag, p.status, p.max_spins);
-                alive = __shfl_sync(0xffffffffu, ok, 0);
-              }
+              alive = wait_asleep(eb, ep, 200);
             }
             if (!alive) break;
             const uint32_t left = total - it;
@@ -468,38 +615,25 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
         }
       }
     }
-  } else if (warp > kTcEpiWarps) {
+  } else if (warp >= kTcMmaWarp && warp < kTcCopyWarp) {
     // ------------------------------------------------------------ MMA issuers: one warp per A block and accumulator buffer
     // The whole warp runs the loop, so that everything the instructions need (descriptors, addresses, parities) is
     // computed once per warp in converged code; one lane issues.  The loop is part of the ring of the accumulators, so it
     // is kept to the bare sequence: a codebook stage (eight steps, four of this warp's buffer) is one trip, its steps are
     // unrolled with constant parities and descriptor offsets, and a wait that is already over costs a single poll.
     {
-      const uint32_t iss = (uint32_t)(warp - kTcEpiWarps - 1), q = iss & 1u, buf = iss >> 1;
+      const uint32_t iss = (uint32_t)(warp - kTcMmaWarp), q = iss & 1u, buf = iss >> 1;
       uint64_t a_desc[D::kMmas];
 #pragma unroll
       for (int m = 0; m < D::kMmas; ++m)
-        a_desc[m] = smem_desc(smem_u32(&sm.a[q][0]), D::kAGroupBytes) + (uint64_t)(2 * m * (128 >> 4));
-      uint32_t total = 0;  // steps of this CTA
-      for (uint64_t u = blockIdx.x; u < units; u += gridDim.x) {
-        uint32_t s_lo, s_hi;
-        slice_units(p, (uint32_t)(u % p.n_slices), &s_lo, &s_hi);
-        total += s_hi - s_lo;
-      }
+        a_desc[m] = smem_desc(smem_u32(&sm.a[1][q][0]), D::kAGroupBytes) + (uint64_t)(2 * m * (128 >> 4));
+      const uint32_t total = total_steps();
       const uint64_t b_desc0 = smem_desc(smem_u32(&sm.b[0][0][0]), D::kBGroupBytes);
       const uint32_t full = smem_u32(&sm.tmem_full[buf][q]), empty = smem_u32(&sm.tmem_empty[buf][q]);
       const uint32_t d = tmem_base + q * 128 + buf * 256;
-      const uint32_t a_ready = smem_u32(&sm.a_ready);
-      // a wait whose answer is the same in every lane: one poll by all of them when the phase is already over,
-      // otherwise lane 0 polls (bounded) and tells the others
-      auto wait_all = [&](uint32_t bar, uint32_t parity) -> bool {
-        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-        bool ok = true;
-        if (lane == 0) ok = mbar_wait(bar, parity, abort_flag, p.status, p.max_spins);
-        return __shfl_sync(0xffffffffu, ok, 0);
-      };
+      constexpr uint64_t kAUnit = (2 * D::kABlockBytes) >> 4;  // from the rows of even units to those of odd ones
       bool alive = true;
-      uint64_t u = blockIdx.x;
+      uint32_t u = blockIdx.x;
       uint32_t unit_i = 0, unit_end = 0;  // units begun and their steps
       uint32_t s = 0, stage_par = 0;      // codebook stage of the trip and the parity of its barrier
       for (uint32_t base = 0; base < total && alive; base += kTcGroupSteps) {
@@ -511,10 +645,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
           if (it < total && alive) {
             while (it >= unit_end && alive) {  // the next unit begins: its A rows must be in place
               uint32_t s_lo, s_hi;
-              slice_units(p, (uint32_t)(u % p.n_slices), &s_lo, &s_hi);
+              unit_steps(u, &s_lo, &s_hi);
               unit_end += s_hi - s_lo;
               u += gridDim.x;
-              alive = wait_all(a_ready, unit_i & 1);
+              if (unit_i > 0) umma_commit(smem_u32(&sm.a_free[(unit_i - 1) & 1]));  // the unit before is behind this warp
+              alive = wait_all(smem_u32(&sm.a_ready[unit_i & 1]), (unit_i >> 1) & 1);
+#pragma unroll
+              for (int m = 0; m < D::kMmas; ++m) a_desc[m] = (unit_i & 1) ? a_desc[m] + kAUnit : a_desc[m] - kAUnit;
               ++unit_i;
             }
             // the buffer's use number base / 2 + j (base / 2 is even)
@@ -539,139 +676,75 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
         }
       }
     }
+  } else if (warp >= kTcFormWarp) {
+    // ------------------------------------------------------------ formers: the targets of the next unit
+    // The rows of one unit are formed while the search is at the one before, so that a unit begins with its first
+    // instruction and not with three dependent trips to memory.  (The first unit's are formed by the even set.)
+    const uint32_t first = (uint32_t)tid - 32 * kTcFormWarp;
+    bool alive = wait_all(smem_u32(&sm.a_first), 0);
+    __syncwarp();
+    mbar_arrive(smem_u32(&sm.a_ready[0]));
+    uint32_t unit_i = 1;
+    for (uint32_t u = blockIdx.x + gridDim.x; u < units && alive; u += gridDim.x, ++unit_i) {
+      const uint32_t par = unit_i & 1, tile = fast_div(u, p.slice_div);
+      constexpr int kRounds = (kTcTile + kTcFormers - 1) / kTcFormers;
+      uint32_t j[kRounds];
+#pragma unroll
+      for (int q = 0; q < kRounds; ++q) j[q] = first + q * kTcFormers < kTcTile ? target_index(tile, first + q * kTcFormers) : 0;
+      alive = wait_asleep(smem_u32(&sm.a_free[par]), ((unit_i >> 1) & 1) ^ 1, 500);
+      if (!alive) break;
+#pragma unroll 1
+      for (int q = 0; q < kRounds; ++q) {
+        if (first + q * kTcFormers < kTcTile) form_row(j[0], first + q * kTcFormers, par);
+#pragma unroll
+        for (int i = 0; i + 1 < kRounds; ++i) j[i] = j[i + 1];
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> visible to the MMA
+      mbar_arrive(smem_u32(&sm.a_ready[par]));
+    }
   } else {
-    // ------------------------------------------------------------ target owners / epilogue
-    const uint32_t set = (uint32_t)tid / kTcTile, own = (uint32_t)tid % kTcTile;
-    const uint32_t rb = own >> 7, r = own & 127u;
-    unsigned char* a_row = &sm.a[rb][(r >> 3) * D::kAGroupBytes + (r & 7) * 16];
+    // ------------------------------------------------------------ read-out
+    const uint32_t set = (uint32_t)tid / kTcTile, own = (uint32_t)tid % kTcTile, rb = own >> 7;
     const uint32_t acc = tmem_base + (((uint32_t)(warp & 3) * 32u) << 16) + set * 256 + rb * 128;
     const uint32_t full = smem_u32(&sm.tmem_full[set][rb]), empty = smem_u32(&sm.tmem_empty[set][rb]);
     constexpr float kRelMargin = rel_margin(DG);
-    auto epi_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(kTcEpiThreads) : "memory"); };
+    // A warp of the odd set and the one of the even set with the same targets meet once per unit, when the odd one has left
+    // what it found.  It goes on at once: its next unit writes to the other of two places.
+    auto pair_sync = [&] { asm volatile("bar.sync %0, 64;" ::"r"(1 + (warp & 7)) : "memory"); };
+    if (set == 0) {
+      const uint32_t j = target_index(fast_div(blockIdx.x, p.slice_div), own);
+      const uint2 part = own < p.exc_blocks ? __ldcg(&stats->norms[own]) : make_uint2(0, 0);
+      const uint32_t n2bits = __reduce_max_sync(0xffffffffu, part.x), n2inv = __reduce_max_sync(0xffffffffu, part.y);
+      if (lane == 0) {
+        atomicMax(&sm.n2max_bits, n2bits);
+        atomicMax(&sm.n2min_inv, n2inv);
+      }
+      if (blockIdx.x == 0) {  // for the rescoring kernel
+        const uint32_t exc = __reduce_add_sync(0xffffffffu, own < p.exc_blocks ? __ldcg(&stats->n_exc[own]) : 0u);
+        if (lane == 0) atomicAdd(&sm.n_exc, exc);
+      }
+      asm volatile("bar.sync 9, %0;" ::"n"(kTcTile) : "memory");
+      if (blockIdx.x == 0 && own == 0) stats->any_exc = sm.n_exc;
+      form_row(j, own, 0);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> visible to the MMA
+      mbar_arrive(smem_u32(&sm.a_first));
+    }
     uint32_t it = 0;    // steps of the CTA before the unit
     uint32_t uses = 0;  // of this set's buffer
-    bool alive = true;  // after a wait that ran out the set only keeps its turns at the two barriers of each unit
+    uint32_t unit_i = 0;
+    bool alive = true;  // after a wait that ran out the set only keeps its turn at the barrier of each unit
 
-    for (uint64_t u = blockIdx.x; u < units; u += gridDim.x) {
-      const uint32_t tile = (uint32_t)(u / p.n_slices), sl = (uint32_t)(u % p.n_slices);
+    for (uint32_t u = blockIdx.x; u < units; u += gridDim.x, ++unit_i) {
       uint32_t s_lo, s_hi;
-      slice_units(p, sl, &s_lo, &s_hi);
+      const uint32_t tile = unit_steps(u, &s_lo, &s_hi), sl = u - tile * p.n_slices, par = unit_i & 1;
       const uint64_t n = (uint64_t)tile * kTcTile + own;
-      bool have = false;
-      if (set == 0 && alive) {
-        // the target of this thread, its scaling, its A row
-        float t[DG];
-#pragma unroll
-        for (int i = 0; i < DG; ++i) t[i] = 0.0f;
-        float prev = -kNegInf;
-        if (n < p.k) {
-          const uint32_t j = p.idx[n];
-          if (j < p.G) {  // an index out of range is reported by the rescoring kernel
-            if (DG == 8)
-              form_target(p, j, t);
-            else
-              form_target16(p, j, t);
-            have = true;
-            // the distance to the stored code: only what comes near it has to be remembered
-            const uint32_t code = p.code_u16 ? reinterpret_cast<const uint16_t*>(p.codes)[j]
-                                             : reinterpret_cast<const uint8_t*>(p.codes)[j];
-            if (code < p.K) {
-              float c[DG];
-              load_codeword<true, DG>(p.book, code, c);
-              float d = 0.0f;
-#pragma unroll
-              for (int i = 0; i < DG; ++i) d = fmaf(t[i] - c[i], t[i] - c[i], d);
-              if (d < 1e30f) prev = d;
-            }
-          }
-        }
-        if (u == blockIdx.x) {
-          const uint2 part = own < p.exc_blocks ? __ldcg(&stats->norms[own]) : make_uint2(0, 0);
-          const uint32_t n2bits = __reduce_max_sync(0xffffffffu, part.x), n2inv = __reduce_max_sync(0xffffffffu, part.y);
-          if (lane == 0) {
-            atomicMax(&sm.n2max_bits, n2bits);
-            atomicMax(&sm.n2min_inv, n2inv);
-          }
-          if (blockIdx.x == 0) {  // for the rescoring kernel
-            const uint32_t exc = __reduce_add_sync(0xffffffffu, own < p.exc_blocks ? __ldcg(&stats->n_exc[own]) : 0u);
-            if (lane == 0) atomicAdd(&sm.n_exc, exc);
-          }
-          asm volatile("bar.sync 2, %0;" ::"n"(kTcTile) : "memory");
-          if (blockIdx.x == 0 && own == 0) stats->any_exc = sm.n_exc;
-        }
-        const float n2max = __uint_as_float(sm.n2max_bits);
-        const float cnmax = sqrtf(n2max), hmax = 0.5f * n2max;
-        const float cnmin = sqrtf(__uint_as_float(0x7f800000u - sm.n2min_inv));  // (infinite if there is none)
-        float m = 0.0f, nt2 = 0.0f;
-#pragma unroll
-        for (int i = 0; i < DG; ++i) {
-          m = fmaxf(m, fabsf(t[i]));
-          nt2 = fmaf(t[i], t[i], nt2);
-        }
-        bool in_range = (m < 256.0f) && (nt2 == nt2);  // also false for Inf / NaN
-        const float norm = sqrtf(nt2);
-        int e = 0;
-        if (in_range && m > 0.0f) {
-          e = -ilogbf(m) - 1;
-          e = e > 15 ? 15 : e;
-        }
-        // the best score, at least -2^e (||t|| + min ||c||)^2 / 2, has to be a half
-        // (and above that of the padding rows, -327520 2^e)
-        const float far = norm + cnmin, low = 0.5f * far * far;
-        in_range = in_range && low < 150000.0f;
-        if (in_range && low > 1.0f) e = min(e, 14 - ilogbf(low));
-        const float sc = in_range ? scalbnf(1.0f, e) : 0.0f;
-        float r2 = 0.0f;  // ||2^e t - hi||^2
-        {
-          const uint32_t sb = __half_as_ushort(__float2half_rn(sc));
-#pragma unroll
-          for (int part = 0; part < D::kPart; ++part) {
-            __half2 hi[4];
-            float bias = 0.0f;  // sum over i of (2^e t_i - hi_i) t_i - 2^e t_i^2 / 2 = -t_i (hi_i - 2^e t_i / 2)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const float tx = in_range ? t[8 * part + 2 * i] : 0.0f, ty = in_range ? t[8 * part + 2 * i + 1] : 0.0f;
-              const float x = tx * sc, y = ty * sc;  // exact products
-              hi[i] = __floats2half2_rn(x, y);
-              const float2 back = __half22float2(hi[i]);
-              r2 = fmaf(x - back.x, x - back.x, r2);
-              r2 = fmaf(y - back.y, y - back.y, r2);
-              bias = fmaf(-tx, fmaf(-0.5f, x, back.x), bias);
-              bias = fmaf(-ty, fmaf(-0.5f, y, back.y), bias);
-            }
-            const __half b_hi = __float2half_rn(bias);
-            const float r1 = bias - __half2float(b_hi);
-            const __half b_lo = __float2half_rn(r1);
-            const __half b_lo2 = __float2half_rn(r1 - __half2float(b_lo));
-            *reinterpret_cast<uint4*>(a_row + 256 * part) = reinterpret_cast<const uint4*>(hi)[0];
-            *reinterpret_cast<uint4*>(a_row + 256 * part + 128) =
-                make_uint4(sb | (sb << 16), sb | ((uint32_t)__half_as_ushort(b_hi) << 16),
-                           (uint32_t)__half_as_ushort(b_lo) | ((uint32_t)__half_as_ushort(b_lo2) << 16), sb | (sb << 16));
-          }
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> visible to the MMA
-        mbar_arrive(smem_u32(&sm.a_ready));
-
-        // A score is S = -2^e ||t - c||^2 / 2 but for rounding: the bias takes 2^e ||t||^2 / 2 off and adds what the rounding
-        // of the target costs at c = t.  Error bound, in the score's units: 2^-10 of itself for the rounding to a half
-        // (rounded or truncated; twice for two instructions, whose parts have one sign); for the rest of the rounding of the
-        // target r ||t - c|| <= 2^-10 |S| + 2^9 r^2 2^-e with r = ||2^e t - hi||; 2^-19 of the sum of magnitudes
-        // 2^e (||t|| ||c|| + h + ||t||^2) for the sum of products in binary32, rounded or truncated (twice the terms for
-        // groups of 16); 2^-24 where a half is subnormal, and the split of h and of the bias.  Twice that is the margin, the
-        // last terms with a factor 2 to spare: margin + kRelMargin |S|.
-        // How the tensor cores add and round is not documented: that a sum is formed to binary32 accuracy and is off by at
-        // most one unit of 2^-10 of itself per instruction as a half is an assumption.  What supports it are the tests, in
-        // which the codes are the same as those of binary64 distances.
-        const float margin = 2.0f * (517.0f * r2 / (in_range ? sc : 1.0f) +
-                                     (DG == 8 ? 3.814697265625e-6f /* 2^-18 */ : 7.62939453125e-6f) * sc *
-                                         (norm * cnmax + hmax + nt2) +
-                                     4.76837158203125e-7f /* 2^-21 */);
-        sm.margin[own] = in_range ? margin : -1.0f;
-        sm.seed[own] = in_range ? -0.5f * sc * prev * 1.0001f : kNegInf;  // (minus infinity without a stored code)
-      }
-      epi_sync();
-      const float margin = sm.margin[own];
+      if (alive) alive = wait_all(smem_u32(&sm.a_ready[par]), (unit_i >> 1) & 1);
+      __syncwarp();
+      const float margin = sm.margin[par][own], seed = sm.seed[par][own];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&sm.a_free[par]));
       const bool in_range = margin >= 0.0f;
+      uint32_t* const list = &sm.list[set ? 1 + par : 0][0][own];
       float best = kNegInf;
 
       // Each set takes the steps of one buffer.  The accumulators go to registers in one go, and the buffer back to its MMA
@@ -683,14 +756,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
       uint32_t list_cnt = 0, evicted = 0xffffffffu;
       // keys up to this one are remembered: at first those that may reach the score of the stored code.  (With no bound
       // to begin with, every thread remembers its first steps one after the other: 4096x4096 1x16 95 us instead of 90.)
-      const float seed = sm.seed[own];
       uint32_t lim = key_limit(seed - fmaf(kRelMargin, fabsf(seed), margin));
-      uint32_t cap = (lim + 1) * 0x10001u;  // (a key is a half with the sign bit: the limit is far below 0xffff)
+      // (a key is a half with the sign bit: the limit is far below 0xffff; nothing is below zero)
+      uint32_t cap = in_range ? (lim + 1) * 0x10001u : 0u;
       auto note = [&](uint32_t key, uint32_t sub) {
         if (key <= lim) {
           const uint32_t slot = list_cnt & (kTcListLen - 1);
-          if (list_cnt >= kTcListLen) evicted = min(evicted, sm.list[slot][tid]);
-          sm.list[slot][tid] = (key << 16) | sub;
+          if (list_cnt >= kTcListLen) evicted = min(evicted, list[slot * kTcTile]);
+          list[slot * kTcTile] = (key << 16) | sub;
           ++list_cnt;
           best = fmaxf(best, key_score(key));
           lim = min(lim, key_limit(best - fmaf(kRelMargin, fabsf(best), margin)));
@@ -698,14 +771,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
         }
       };
       for (uint32_t st = s_lo + ((it ^ set) & 1); st < s_hi && alive; st += 2, ++uses) {
-        // one lane polls (all threads polling one barrier slow every barrier operation of the CTA
-        // down); the warp-wide exchange orders the other lanes after its observation
-        if (!__all_sync(0xffffffffu, mbar_try_wait(full, uses & 1))) {
-          bool ok = true;
-          if (lane == 0) ok = mbar_wait(full, uses & 1, abort_flag, p.status, p.max_spins);
-          alive = __shfl_sync(0xffffffffu, ok, 0);
-          if (!alive) break;
-        }
+        alive = wait_all(full, uses & 1);
+        if (!alive) break;
         tc_fence_after();
         tmem_ld64(acc, v);
         tmem_ld64(acc + 64, w);
@@ -720,32 +787,35 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
       }
       it += s_hi - s_lo;
       if (set == 1) {
-        sm.odd_best[own] = best;
-        sm.odd_cnt[own] = list_cnt;
-        sm.odd_evicted[own] = evicted;
+        sm.odd_best[par][own] = best;
+        sm.odd_cnt[par][own] = list_cnt;
+        sm.odd_evicted[par][own] = evicted;
       }
-      epi_sync();
+      pair_sync();
 
       // leave the candidates of this (tile, slice) for the rescoring kernel (minimum convention: -S)
-      if (set == 0 && alive && have) {
+      if (set == 0 && alive && margin != kAbsent) {
         CandRecord rec;
         rec.w[0] = rec.w[1] = rec.w[2] = 0;
         if (in_range) {
-          const uint32_t other_cnt = sm.odd_cnt[own];
-          best = fmaxf(best, sm.odd_best[own]);
+          const uint32_t other_cnt = sm.odd_cnt[par][own];
+          best = fmaxf(best, sm.odd_best[par][own]);
           lim = min(lim, key_limit(best - fmaf(kRelMargin, fabsf(best), margin)));
           uint32_t cnt_out = 0;
-#pragma unroll
-          for (int q = 0; q < 2 * kTcListLen; ++q) {
-            const uint32_t entry = sm.list[q / 2][own + (q & 1) * kTcTile];
-            if ((uint32_t)(q / 2) < ((q & 1) ? other_cnt : list_cnt) && (entry >> 16) <= lim) {
-              if (cnt_out < (uint32_t)kCandMost) cand_add(rec, cnt_out, entry & 0xffffu);
-              ++cnt_out;
+          auto pick = [&](const uint32_t* from, uint32_t cnt) {  // (seldom more than two)
+            for (uint32_t q = 0; q < cnt && q < (uint32_t)kTcListLen; ++q) {
+              const uint32_t entry = from[q * kTcTile];
+              if ((entry >> 16) <= lim) {
+                if (cnt_out < (uint32_t)kCandMost) cand_add(rec, cnt_out, entry & 0xffffu);
+                ++cnt_out;
+              }
             }
-          }
+          };
+          pick(list, list_cnt);
+          pick(&sm.list[1 + par][0][own], other_cnt);
           rec.best = -best;
           // (an evicted entry stays above every key while nothing was evicted)
-          const bool all = cnt_out > (uint32_t)kCandMost || (min(evicted, sm.odd_evicted[own]) >> 16) <= lim;
+          const bool all = cnt_out > (uint32_t)kCandMost || (min(evicted, sm.odd_evicted[par][own]) >> 16) <= lim;
           rec.w[0] |= (all ? kCandOverflow : cnt_out) << 24;
         } else {
           rec.best = kNegInf;  // passes every limit: the whole slice is rescored exactly
@@ -761,7 +831,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
   tc_fence_before();
   __syncthreads();
   pdl_trigger();
-  if (warp == kTcEpiWarps + 1) {
+  if (warp == kTcMmaWarp) {
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);
   }
@@ -819,6 +889,7 @@ cudaError_t launch_encode_m1_tc(const pvt_layer& L, uint64_t G, const uint32_t* 
   p.K = (uint32_t)L.codebook_size;
   p.n_tiles = lay.n_tiles;
   p.n_slices = lay.n_slices;
+  p.slice_div = make_fast_div(lay.n_slices);
   p.tile = kTcTile;
   p.n_units = lay.n_steps;
   p.unit_cw = kTcStepCw;

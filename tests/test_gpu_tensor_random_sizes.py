@@ -34,3 +34,21 @@ def test_tensor_search_random_shapes(seed):
                 assert exact >= k - max(4, k // 500), (case, gd, K, rows, cols, k)
             else:
                 g16._encode_case(K, True, rows, cols, k, L=L, idx=idx)
+
+
+@pytest.mark.parametrize("gd,K,k", [
+    (8, 100, 114001),   # one step per unit, four units and a ragged tile per thread block: the odd read-out set has none
+    (8, 380, 76003),    # three steps, the sets take turns at the first
+    (8, 1152, 40001),   # nine steps: a stage of the codebook holds steps of two units
+    (16, 100, 60001),
+    (8, 40000, 700),    # many slices, one unit per thread block
+])
+def test_tensor_search_over_short_units(gd, K, k):
+    rows, cols = 1024, 128 * gd  # 131072 groups
+    L = synth.make_layer(rows, cols, cfg=340 + K % 7, codebook_size=K, codebook_fp16=True, group_dim=gd)
+    idx = np.sort(np.random.default_rng(k).permutation(L.num_groups)[:k]).astype(np.uint32)
+    with parity.search_engine("tensor"):
+        if gd == 8:
+            parity.check_encode(L, idx)
+        else:
+            g16._encode_case(K, True, rows, cols, k, L=L, idx=idx)
