@@ -326,17 +326,20 @@ __global__ void __launch_bounds__(kEncThreads + 32, 1) encode_m1_kernel(const En
 // ---- rescoring --------------------------------------------------------------------
 // Eight lanes per target, four targets per warp: the kernel is a chain of dependent memory round trips
 // ((index, global minimum, margin, records) -> (W, g, scale) -> codewords), so what counts is how many targets
-// are in flight per warp, not how fast one of them is evaluated.  (With every candidate evaluated in binary64, 1048576
-// targets took 368 us instead of 310.)
+// are in flight per warp, not how fast one of them is evaluated; four codewords of a lane are on their way at once, and
+// the registers are held to what five blocks per SM allow (16-byte codewords; three otherwise).  1048576 / 20971 targets
+// 259 / 14.6 us, 10485 of 16 weights 14.9; a codeword at a time 310 / 16.8 / 17.9; eight at once in four blocks 291 / 14.6.
+// With every candidate evaluated in binary64 the first took 368.  (Remembering 32 codewords where the tensor engine
+// remembers 64 takes 215 / 12.7 here and costs its search 108 / 2.5.)
 constexpr int kRsLanes = 8;
 constexpr int kRsPerWarp = 32 / kRsLanes;
 constexpr int kRsPerBlock = 8 * kRsPerWarp;  // 256 threads
+constexpr int kRsEach = 4;  // codewords of a lane on their way at once
 static_assert(kMaxSlices <= 2 * kRsLanes, "two records per lane must cover every slice");
 
-template <bool CB_F16, int DG>
-__global__ void __launch_bounds__(256) rescore_m1_kernel(const EncM1Params p) {
+template <bool CB_F16, int DG, int SUB>
+__global__ void __launch_bounds__(256, DG == 8 && CB_F16 ? 5 : 3) rescore_m1_kernel(const EncM1Params p) {
   constexpr uint32_t kFull = 0xffffffffu;
-  const uint32_t sub_cw = p.sub_cw;
   const int lane = threadIdx.x & 31, grp = lane / kRsLanes, l = lane % kRsLanes;
   const int gshift = grp * kRsLanes;
   const uint64_t n = ((uint64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * kRsPerWarp + grp;
@@ -371,13 +374,14 @@ __global__ void __launch_bounds__(256) rescore_m1_kernel(const EncM1Params p) {
     else
       form_target16(p, j, t);
   }
-  const uint32_t subs_per_unit = p.unit_cw / sub_cw;
+  const uint32_t subs_per_unit = p.unit_cw / SUB;
   double best_d = __longlong_as_double(0x7ff0000000000000ll);
   uint32_t best_code = 0xffffffffu;
 
-  auto score = [&](uint32_t kappa) {
+  using Raw = RawCodeword<CB_F16, DG>;
+  auto score = [&](uint32_t kappa, const Raw& raw) {
     float c[DG];
-    load_codeword<CB_F16, DG>(p.book, kappa, c);
+    widen_codeword<CB_F16, DG>(raw, c);
     double d = 0.0;
 #pragma unroll
     for (int i = 0; i < DG; ++i) {
@@ -395,9 +399,9 @@ __global__ void __launch_bounds__(256) rescore_m1_kernel(const EncM1Params p) {
   // equal), or the least is no number of the range, every candidate of the target is evaluated in binary64.
   float near1 = __uint_as_float(0x7f800000u), near2 = near1;
   uint32_t near_code = 0;
-  auto estimate = [&](uint32_t kappa) {
+  auto estimate = [&](uint32_t kappa, const Raw& raw) {
     float c[DG];
-    load_codeword<CB_F16, DG>(p.book, kappa, c);
+    widen_codeword<CB_F16, DG>(raw, c);
     float d = 0.0f;
 #pragma unroll
     for (int i = 0; i < DG; ++i) {
@@ -419,10 +423,20 @@ __global__ void __launch_bounds__(256) rescore_m1_kernel(const EncM1Params p) {
   const uint32_t slices = ((in0 >> gshift) & 0xffu) | (((in1 >> gshift) & 0xffu) << kRsLanes);
   auto sweep = [&](bool on, auto&& take) {
     auto visit = [&](uint32_t sub) {
-      for (uint32_t w = l; w < sub_cw; w += kRsLanes) {
-        const uint32_t kappa = sub * sub_cw + w;
-        if (kappa < p.K) take(kappa);
+#pragma unroll 1
+      for (uint32_t at = sub * SUB + l; at < (sub + 1) * SUB; at += kRsEach * kRsLanes) {
+        Raw raw[kRsEach];
+#pragma unroll
+        for (int q = 0; q < kRsEach; ++q) fetch_codeword<CB_F16, DG>(p.book, min(at + q * kRsLanes, p.K - 1), &raw[q]);
+#pragma unroll
+        for (int q = 0; q < kRsEach; ++q)
+          if (at + q * kRsLanes < p.K) take(at + q * kRsLanes, raw[q]);
       }
+    };
+    auto visit_one = [&](uint32_t kappa) {
+      Raw raw;
+      fetch_codeword<CB_F16, DG>(p.book, kappa, &raw);
+      take(kappa, raw);
     };
     uint32_t live = on ? slices : 0;
     while (__any_sync(kFull, live != 0)) {
@@ -458,7 +472,7 @@ __global__ void __launch_bounds__(256) rescore_m1_kernel(const EncM1Params p) {
         const uint32_t n = p.n_exc[b];
         for (uint32_t e = l; e < n && e < p.exc_per_block; e += kRsLanes) {
           const uint32_t kappa = p.exc_list[(size_t)b * p.exc_per_block + e];
-          if (kappa < p.K) take(kappa);
+          if (kappa < p.K) visit_one(kappa);
         }
       }
     }
@@ -470,7 +484,11 @@ __global__ void __launch_bounds__(256) rescore_m1_kernel(const EncM1Params p) {
   const float inside = fmaf(least, 3.814697265625e-6f /* 2^-18 */, least) + 1e-36f;
   const uint32_t again = __ballot_sync(kFull, active && (near2 <= inside || !(least < 1e38f)));
   const bool all = (again >> gshift) & 0xffu;
-  if (active && !all && near1 <= inside) score(near_code);
+  if (active && !all && near1 <= inside) {
+    Raw raw;
+    fetch_codeword<CB_F16, DG>(p.book, near_code, &raw);
+    score(near_code, raw);
+  }
   if (again) sweep(active && all, score);
   // lexicographic minimum of (distance, code) over the eight lanes of the target; distances are >= 0 so their
   // bits order like u64
@@ -533,7 +551,6 @@ cudaError_t launch_encode_m1(const pvt_layer& L, uint64_t G, const uint32_t* idx
   p.n2max_bits = reinterpret_cast<const uint32_t*>(base + lay.n2max_off);
   p.n_units = lay.n_chunks;
   p.unit_cw = kChunkCodewords;
-  p.sub_cw = kSubCodewords;
   p.rel_margin = 0.0f;
   p.any_exc = nullptr;
   p.exc_list = nullptr;
@@ -571,20 +588,18 @@ cudaError_t launch_encode_m1(const pvt_layer& L, uint64_t G, const uint32_t* idx
   if ((err = cudaGetLastError()) != cudaSuccess) return err;
   err = tt == 8 ? launch_tt<8>(p, lay.n_ctas, stream) : launch_tt<4>(p, lay.n_ctas, stream);
   if (err != cudaSuccess) return err;
-  return launch_rescore_m1(p, f16, stream);
+  return launch_rescore_m1(p, f16, false, stream);
 }
 
-cudaError_t launch_rescore_m1(const EncM1Params& p, bool codebook_f16, cudaStream_t stream) {
+cudaError_t launch_rescore_m1(const EncM1Params& p, bool codebook_f16, bool tensor_engine, cudaStream_t stream) {
   timing_begin(kKernEncodeRescore, stream);
   const unsigned blocks = (unsigned)((p.k + kRsPerBlock - 1) / kRsPerBlock);
+  auto run = [&](auto kernel) { return launch_dependent(kernel, blocks, 256, 0, stream, p); };
   cudaError_t err;
-  if (p.dg == 16) {  // groups of 16 weights come from the tensor engine only: fp16 codebooks
-    err = launch_dependent(rescore_m1_kernel<true, 16>, blocks, 256, 0, stream, p);
-  } else if (codebook_f16) {
-    err = launch_dependent(rescore_m1_kernel<true, 8>, blocks, 256, 0, stream, p);
-  } else {
-    err = launch_dependent(rescore_m1_kernel<false, 8>, blocks, 256, 0, stream, p);
-  }
+  if (tensor_engine)  // fp16 codebooks
+    err = p.dg == 16 ? run(rescore_m1_kernel<true, 16, kTcSubCodewords>) : run(rescore_m1_kernel<true, 8, kTcSubCodewords>);
+  else
+    err = codebook_f16 ? run(rescore_m1_kernel<true, 8, kSubCodewords>) : run(rescore_m1_kernel<false, 8, kSubCodewords>);
   count_launches(1);
   timing_end(kKernEncodeRescore, stream);
   return err;

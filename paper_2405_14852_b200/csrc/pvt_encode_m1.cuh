@@ -37,7 +37,6 @@ struct EncM1Params {
   uint32_t K, n_tiles, n_slices, tile;
   uint32_t n_units, unit_cw;  // the codebook is cut into n_units units of unit_cw codewords; a slice is a run of whole units
   FastDiv slice_div;          // n_slices as a divisor
-  uint32_t sub_cw;            // codewords per remembered sub-chunk (a multiple of 32 that divides unit_cw)
   // codewords the fast score cannot represent, always rescored: their number (may be null), and by block of codewords the
   // number and the places in the list
   const uint32_t *any_exc, *n_exc;
@@ -99,14 +98,24 @@ __device__ __forceinline__ void form_target16(const EncM1Params& p, uint32_t j, 
   }
 }
 
-// one codeword of DG elements, widened to binary32
+// one codeword of DG elements as it lies in memory, and widened to binary32
 template <bool CB_F16, int DG>
-__device__ __forceinline__ void load_codeword(const void* book, uint32_t kappa, float* c) {
+struct RawCodeword {
+  uint4 part[CB_F16 ? DG / 8 : DG / 4];
+};
+template <bool CB_F16, int DG>
+__device__ __forceinline__ void fetch_codeword(const void* book, uint32_t kappa, RawCodeword<CB_F16, DG>* raw) {
+  constexpr int kParts = CB_F16 ? DG / 8 : DG / 4;
+#pragma unroll
+  for (int part = 0; part < kParts; ++part)
+    raw->part[part] = reinterpret_cast<const uint4*>(book)[(size_t)kappa * kParts + part];
+}
+template <bool CB_F16, int DG>
+__device__ __forceinline__ void widen_codeword(const RawCodeword<CB_F16, DG>& raw, float* c) {
   if (CB_F16) {
 #pragma unroll
     for (int part = 0; part < DG / 8; ++part) {
-      const uint4 raw = reinterpret_cast<const uint4*>(book)[(size_t)kappa * (DG / 8) + part];
-      const __half2* h = reinterpret_cast<const __half2*>(&raw);
+      const __half2* h = reinterpret_cast<const __half2*>(&raw.part[part]);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const float2 f = __half22float2(h[i]);
@@ -115,13 +124,20 @@ __device__ __forceinline__ void load_codeword(const void* book, uint32_t kappa, 
       }
     }
   } else {
-    const float4* q = reinterpret_cast<const float4*>(book) + (size_t)kappa * (DG / 4);
 #pragma unroll
     for (int part = 0; part < DG / 4; ++part) {
-      const float4 a = q[part];
-      c[4 * part] = a.x; c[4 * part + 1] = a.y; c[4 * part + 2] = a.z; c[4 * part + 3] = a.w;
+      c[4 * part] = __uint_as_float(raw.part[part].x);
+      c[4 * part + 1] = __uint_as_float(raw.part[part].y);
+      c[4 * part + 2] = __uint_as_float(raw.part[part].z);
+      c[4 * part + 3] = __uint_as_float(raw.part[part].w);
     }
   }
+}
+template <bool CB_F16, int DG>
+__device__ __forceinline__ void load_codeword(const void* book, uint32_t kappa, float* c) {
+  RawCodeword<CB_F16, DG> raw;
+  fetch_codeword<CB_F16, DG>(book, kappa, &raw);
+  widen_codeword<CB_F16, DG>(raw, c);
 }
 
 // ---- PTX helpers ---------------------------------------------------------------
@@ -188,6 +204,6 @@ __device__ __forceinline__ void slice_units(const EncM1Params& p, uint32_t sl, u
 }  // namespace m1
 
 // exact rescoring + code write after either search kernel (defined with the FP32 search)
-cudaError_t launch_rescore_m1(const m1::EncM1Params& p, bool codebook_f16, cudaStream_t stream);
+cudaError_t launch_rescore_m1(const m1::EncM1Params& p, bool codebook_f16, bool tensor_engine, cudaStream_t stream);
 
 }  // namespace pvt

@@ -75,7 +75,6 @@ struct TcDim {
 };
 constexpr int kTcStepBytes = TcDim<8>::kStepBytes;
 constexpr int kTcListLen = 8;           // remembered near-maximum sub-chunks per target
-constexpr int kTcSubCw = 64;            // tracking granularity of the running maximum
 constexpr int kTcGroupSteps = 8;        // steps per codebook stage: the MMA warps wait for the codebook once per eight steps
 constexpr int kTcStages = 2;            // codebook stages (eight steps each: 32 KB, or 64 KB for groups of 16)
 constexpr int kTcEpiThreads = 512;      // two sets of 256, one thread per target each: even and odd steps
@@ -893,7 +892,6 @@ cudaError_t launch_encode_m1_tc(const pvt_layer& L, uint64_t G, const uint32_t* 
   p.tile = kTcTile;
   p.n_units = lay.n_steps;
   p.unit_cw = kTcStepCw;
-  p.sub_cw = kTcSubCw;
   p.rel_margin = rel_margin(L.group_dim);
   p.any_exc = &stats->any_exc;
   p.n_exc = stats->n_exc;
@@ -915,7 +913,7 @@ cudaError_t launch_encode_m1_tc(const pvt_layer& L, uint64_t G, const uint32_t* 
   const cudaError_t err =
       L.group_dim == 16 ? launch_tc<16>(L, p, lay, base, stats, stream) : launch_tc<8>(L, p, lay, base, stats, stream);
   if (err != cudaSuccess) return err;
-  return launch_rescore_m1(p, true, stream);
+  return launch_rescore_m1(p, true, true, stream);
 }
 
 }  // namespace pvt

@@ -48,6 +48,7 @@ SelectLayout select_layout(uint64_t G);
 constexpr int kEncThreads = 256;     // compute threads per CTA (8 warps) + 1 producer warp
 constexpr int kChunkCodewords = 256; // codewords per staged chunk (one bulk copy)
 constexpr int kSubCodewords = 32;    // tracking granularity of the running minimum
+constexpr int kTcSubCodewords = 64;  // the same on the tensor engine
 constexpr int kChunkBytes = kChunkCodewords * (kGroupDim * 4 + 4);  // 9216: pairs interleaved + half norms
 constexpr int kEncStages = 4;
 constexpr int kListLen = 4;          // near-minimum sub-chunks per (target, slice) that the FP32 engine remembers
