@@ -234,6 +234,13 @@ __device__ __forceinline__ bool fetch_image(void* dst, const void* src, uint32_t
   return __syncthreads_and(ok) != 0;
 }
 
+// Where codeword k stands among the columns of the tiles: the 32 codewords of a cell are what one thread sees of a
+// residual, columns 2 q and 2 q + 1 of sixteen tiles (q = lane % 4).
+__device__ __forceinline__ int stage_column(int k) {
+  const int cell = k >> 5, i = k & 31;
+  return 8 * (16 * (cell & 1) + (i >> 1)) + 2 * (cell >> 1) + (i & 1);
+}
+
 // ---- the codebook image: one block, one codeword of every codebook per thread (K <= 256 = block size) ----
 template <int M, bool TC>
 __global__ void __launch_bounds__(kBsThreads) beam_image_kernel(const BeamParams p, BeamImage<M, TC>* img) {
@@ -263,16 +270,18 @@ __global__ void __launch_bounds__(kBsThreads) beam_image_kernel(const BeamParams
     } else {
       StageImage<TC>& st = sm.st[m - 1];
       if constexpr (TC) {
+        const int at = stage_column(tid);
 #pragma unroll
         for (int qq = 0; qq < 4; ++qq) {
           const __half2 v = __floats2half2_rn(c[2 * qq], c[2 * qq + 1]);  // exact: the codebook is fp16
-          st.b[tid >> 3][4 * (tid & 7) + qq] = *reinterpret_cast<const uint32_t*>(&v);
+          st.b[at >> 3][4 * (at & 7) + qq] = *reinterpret_cast<const uint32_t*>(&v);
         }
+        st.h[at] = h;
       } else {
 #pragma unroll
         for (int i = 0; i < 8; ++i) st.x[tid >> 1][2 * i + (tid & 1)] = c[i];
+        st.h[tid] = h;
       }
-      st.h[tid] = h;
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) n2 = fmaxf(n2, __shfl_xor_sync(0xffffffffu, n2, o));
@@ -334,7 +343,7 @@ __device__ __forceinline__ void team_min_exact(double& d, uint32_t& key) {
 }
 
 // One further stage's fast scores for the lane's residual (target my_q, kept tuple my_b; rho = ||r||^2/2): the minimum
-// of every 32 codewords.  The residuals of all lanes are in w.r.  Returns what the tensor path adds to the margin.
+// of each of eight cells of 32 codewords.  The residuals of all lanes are in w.r.  Returns what the tensor path adds to the margin.
 template <bool TC>
 __device__ __forceinline__ float stage_minima(const StageImage<TC>& st, BeamScratch& w, const float (&r)[8], float rho,
                                               bool active, float smax, float (&sub_min)[8]) {
@@ -366,33 +375,32 @@ __device__ __forceinline__ float stage_minima(const StageImage<TC>& st, BeamScra
       a[r4 >> 1][r4 & 1] = *reinterpret_cast<const uint32_t*>(&hi);
       a[r4 >> 1][2 + (r4 & 1)] = *reinterpret_cast<const uint32_t*>(&lo);
     }
-#pragma unroll 2
-    for (int sub = 0; sub < 8; ++sub) {
-      float m[4] = {kInf, kInf, kInf, kInf};
+    // a cell is what one thread sees of a residual in half the tiles: no exchange between the threads (with cells of 32
+    // adjacent columns, two exchanges per cell and row: 11008x4096 k = 56360 two codebooks 1.8 us more, three 4.8 us)
+    float m[4][2];
 #pragma unroll
-      for (int n4 = 0; n4 < 4; ++n4) {
-        const int nt = 4 * sub + n4;
+    for (int half = 0; half < 2; ++half) {
+      float x[4] = {kInf, kInf, kInf, kInf};
+#pragma unroll 4
+      for (int n = 0; n < 16; ++n) {
+        const int nt = 16 * half + n;
         const uint32_t b = st.b[nt][lane];
         const float2 hh = *reinterpret_cast<const float2*>(&st.h[8 * nt + 2 * qd]);
         const float hx = hh.x * sc, hy = hh.y * sc;
         float d0[4], d1[4];
         mma_16x8x16(d0, a[0], b, b, hx, hy);
         mma_16x8x16(d1, a[1], b, b, hx, hy);
-        m[0] = min3(m[0], d0[0], d0[1]);
-        m[1] = min3(m[1], d0[2], d0[3]);
-        m[2] = min3(m[2], d1[0], d1[1]);
-        m[3] = min3(m[3], d1[2], d1[3]);
+        x[0] = min3(x[0], d0[0], d0[1]);
+        x[1] = min3(x[1], d0[2], d0[3]);
+        x[2] = min3(x[2], d1[0], d1[1]);
+        x[3] = min3(x[3], d1[2], d1[3]);
       }
 #pragma unroll
-      for (int r4 = 0; r4 < 4; ++r4) {
-        m[r4] = fminf(m[r4], __shfl_xor_sync(0xffffffffu, m[r4], 1));
-        m[r4] = fminf(m[r4], __shfl_xor_sync(0xffffffffu, m[r4], 2));
-      }
-      if (qd == 0) {
-#pragma unroll
-        for (int r4 = 0; r4 < 4; ++r4) w.wmin[16 * (r4 >> 1) + 8 * (r4 & 1) + g8][sub] = m[r4];
-      }
+      for (int r4 = 0; r4 < 4; ++r4) m[r4][half] = x[r4];
     }
+#pragma unroll
+    for (int r4 = 0; r4 < 4; ++r4)
+      *reinterpret_cast<float2*>(&w.wmin[16 * (r4 >> 1) + 8 * (r4 & 1) + g8][2 * qd]) = make_float2(m[r4][0], m[r4][1]);
     __syncwarp();
     const float4 ma = *reinterpret_cast<const float4*>(&w.wmin[lane][0]);
     const float4 mb = *reinterpret_cast<const float4*>(&w.wmin[lane][4]);
@@ -431,7 +439,7 @@ __device__ __forceinline__ float stage_minima(const StageImage<TC>& st, BeamScra
   }
 }
 
-// The target's 64 (kept tuple, sub-chunk) flags from its lanes' eight: byte b belongs to kept tuple b.
+// The target's 64 (kept tuple, cell) flags from its lanes' eight: byte b belongs to kept tuple b.
 __device__ __forceinline__ uint64_t team_flags(uint32_t mine, uint32_t my_b) {
   uint32_t lo = my_b < 4 ? mine << (8 * my_b) : 0u, hi = my_b >= 4 ? mine << (8 * (my_b - 4)) : 0u;
 #pragma unroll
@@ -714,7 +722,7 @@ __global__ void __launch_bounds__(kBsThreads, kBsCtasPerSm) encode_beam_kernel(c
             const float4 ca = *reinterpret_cast<const float4*>(&sm.c[m][k2][0]);
             const float4 cb = *reinterpret_cast<const float4*>(&sm.c[m][k2][4]);
             const float cv[8] = {ca.x, ca.y, ca.z, ca.w, cb.x, cb.y, cb.z, cb.w};
-            float s2 = __fadd_rn(st.h[k2], srho);
+            float s2 = __fadd_rn(st.h[TC ? stage_column(k2) : k2], srho);
 #pragma unroll
             for (int i = 0; i < 8; ++i) s2 = __fmaf_rn(-sr[i], cv[i], s2);
             const bool in = work && s2 <= limit && k2 < p.K;
