@@ -8,9 +8,10 @@
 //   the result is the smallest member of the last stage's extensions and the previous tuple.
 //
 // A warp handles four targets at a time; the codebooks live in shared memory; three CTAs (24 warps) share an SM.
-//   stage 1 (per target, the whole warp): lane l owns codewords l, l+32, ..., l+224 of codebook 1:
-//            score1 = ||c1||^2/2 - <t, c1> for 256 codewords (8 per lane, packed f32x2); the `beam` smallest are
-//            extracted with warp-wide integer minimum reductions on (score bits | code) keys.
+//   stage 1 (four targets side by side): fast scores ||c1||^2/2 - <t, c1>, on the tensor pipe for fp16 codebooks (mma.sync,
+//            the codewords as rows); a thread keeps the minima of cells of four codewords, 64 per target, and goes on as a
+//            stage in the middle.  Binary32 codebooks: one target after the other, 256 scores on the FP32 pipe, 8 per lane,
+//            of which the `beam` smallest are extracted with warp-wide minima on (score bits | code) keys.
 //   further stages (four targets x eight kept tuples = 32 residuals, one per lane): fast scores
 //            ||r||^2/2 + ||c||^2/2 - <r, c> of all residuals against all codewords, on the tensor pipe for fp16
 //            codebooks (mma.sync, the residuals as rows), on the FP32 pipe otherwise; only the minimum of each
@@ -23,12 +24,13 @@
 // Fast scores are binary32.  Every decision they cannot settle within twice their rounding-error bound (membership of
 // the beam, the final argmin) is taken on binary64 distances accumulated in index order (the residual carried through
 // the codebooks in order), so the result is the argmin of (distance, tuple) over the pool exactly as defined.
-// What bounds it: no unit by itself.  With two / three codebooks 740 / 1470 warp instructions per target fill 64 / 60 % of
-// the issue slots and shared memory is busy 66 / 76 % of the time; the rest are the dependences of one target's chain
-// (sort, warp minima, acceptance), which six warps per scheduler do not hide.  56 360 targets of an 11008 x 4096 layer,
-// two / three / four fp16 codebooks of 256: 72 / 152 / 258 us; three binary32 codebooks 220 us.  (A warp per target, with
-// two passes over all extensions in every stage and every decision in binary64: 415 / 522 us for three / four, 992 us for
-// three binary32 codebooks.)
+// What bounds it: no unit by itself; issue slots and shared memory are busy two thirds of the time, the rest are the
+// dependences of one target's chain (sort, minima over eight lanes, acceptance), which six warps per scheduler do not hide.
+// A step of an 11008 x 4096 layer, k = 56 360, two / three fp16 codebooks of 256: 160.5 / 233.4 us, of which the search is
+// 63 / 139 (four codebooks 230 by itself).  With stage 1 of fp16 codebooks one target after the other on the FP32
+// pipe 169.3 / 236.1; with the binary64 decisions of choose_exact inlined 160.4 / 238.2 (spills).  Before all that, a warp
+// per target, with two passes over all extensions in every stage and every decision in binary64: 415 / 522 us for three /
+// four codebooks by themselves, 992 us for three of binary32.
 #include <cuda_fp16.h>
 
 #include "pvt_internal.h"
@@ -68,6 +70,21 @@ struct BeamParams {
 // Everything the kernel derives from the codebooks, in the byte order it has in shared memory.  One small kernel writes
 // it once per call into the workspace; every CTA of the search fetches it with a single bulk copy (cp.async.bulk,
 // completion on an mbarrier; no multicast).
+// The first codebook.  A cell of stage 1 is four adjacent codewords, what one thread sees of a target in two tiles; cell
+// 8 g + c, codeword x of it (0..3) is row g + 8 (x % 2) of tile 2 c + x / 2.
+template <bool TC>
+struct FirstImage;
+template <>
+struct FirstImage<true> {  // tensor pipe: A fragments, [tile][lane] = halves (c[row][2 (lane%4)], [.. + 1]) of rows lane/4, + 8
+  uint2 a[kBsK / 16][32];
+  float2 h2[kBsK / 16][8];  // ||c||^2/2 of rows g, g + 8
+  float h[kBsK];            // the same by codeword
+};
+template <>
+struct FirstImage<false> {  // FP32 pipe
+  uint64_t p1[4][8][32];  // (c1[l+64q][i], c1[l+64q+32][i])
+  uint64_t h1[4][32];     // (||c1||^2/2) pairs in the same order
+};
 template <bool TC>
 struct StageImage;
 template <>
@@ -83,8 +100,7 @@ struct StageImage<false> {  // FP32 pipe
 template <int M, bool TC>
 struct BeamImage {
   alignas(16) float c[M][kBsK][8];
-  alignas(16) uint64_t p1[4][8][32];  // stage-1 operands: (c1[l+64q][i], c1[l+64q+32][i])
-  uint64_t h1[4][32];                 // (||c1||^2/2) pairs in the same order
+  alignas(16) FirstImage<TC> first;
   StageImage<TC> st[M - 1];
   float smax[4];                      // largest norm per codebook
 };
@@ -97,6 +113,7 @@ struct BeamScratch {  // per warp
   };
   alignas(16) float t[kBsGroup][8];            // the targets of the group
   alignas(16) uint32_t kept[kBsGroup][8];      // their kept tuples: code of codebook q in bits [31 - 8 q : 24 - 8 q]
+  uint8_t cells[kBsGroup][64];                 // stage 1: a target's cells within the margin
 };
 template <int M, bool TC>
 struct BeamSmem {
@@ -127,6 +144,13 @@ __device__ __forceinline__ void mma_16x8x16(float (&d)[4], const uint32_t (&a)[4
       "{%10, %11, %10, %11};"
       : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(c0), "f"(c1));
+}
+// the same with the roles exchanged, rows = codewords, columns = targets: both K halves of A are the codeword
+__device__ __forceinline__ void mma_codeword_rows(float (&d)[4], uint2 a, uint32_t b0, uint32_t b1, float c_lo, float c_hi) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %4, %5}, {%6, %7}, "
+      "{%8, %8, %9, %9};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a.x), "r"(a.y), "r"(b0), "r"(b1), "f"(c_lo), "f"(c_hi));
 }
 __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
   return (uint64_t)__float_as_uint(lo) | ((uint64_t)__float_as_uint(hi) << 32);
@@ -261,12 +285,23 @@ __global__ void __launch_bounds__(kBsThreads) beam_image_kernel(const BeamParams
     }
     const float h = real ? 0.5f * n2 : kPadHalfNorm;
     if (m == 0) {
-      // codeword tid = l + 32*jj, jj = 2q + half
-      const int jj = tid >> 5, q = jj >> 1, half = jj & 1;
-      float* p1f = reinterpret_cast<float*>(&sm.p1[0][0][0]);
+      if constexpr (TC) {
+        const int cell = tid >> 2, x = tid & 3, row = cell >> 3, tile = 2 * (cell & 7) + (x >> 1), lower = x & 1;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) p1f[(((q * 8 + i) * 32) + lane) * 2 + half] = c[i];
-      reinterpret_cast<float*>(&sm.h1[0][0])[(q * 32 + lane) * 2 + half] = h;
+        for (int qq = 0; qq < 4; ++qq) {
+          const __half2 v = __floats2half2_rn(c[2 * qq], c[2 * qq + 1]);  // exact: the codebook is fp16
+          reinterpret_cast<uint32_t*>(&sm.first.a[tile][4 * row + qq])[lower] = *reinterpret_cast<const uint32_t*>(&v);
+        }
+        reinterpret_cast<float*>(&sm.first.h2[tile][row])[lower] = h;
+        sm.first.h[tid] = h;
+      } else {
+        // codeword tid = l + 32*jj, jj = 2q + half
+        const int jj = tid >> 5, q = jj >> 1, half = jj & 1;
+        float* p1f = reinterpret_cast<float*>(&sm.first.p1[0][0][0]);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) p1f[(((q * 8 + i) * 32) + lane) * 2 + half] = c[i];
+        reinterpret_cast<float*>(&sm.first.h1[0][0])[(q * 32 + lane) * 2 + half] = h;
+      }
     } else {
       StageImage<TC>& st = sm.st[m - 1];
       if constexpr (TC) {
@@ -315,11 +350,24 @@ __device__ __forceinline__ void sort4(uint32_t (&key)[4]) {
   PVT_CE(0, 1) PVT_CE(2, 3) PVT_CE(0, 2) PVT_CE(1, 3) PVT_CE(1, 2)
 }
 #undef PVT_CE
-// minimum over the eight lanes of a target
+// The eight lanes of a target: adjacent ones (S = 1, lane = 8 target + member), or every fourth (S = 4, lane = target +
+// 4 member: as the tensor pipe leaves stage 1).  Minimum over them:
+template <int S = 1>
 __device__ __forceinline__ uint32_t team_min(uint32_t v) {
 #pragma unroll
-  for (int o = 1; o < 8; o <<= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
+  for (int o = S; o < 8 * S; o <<= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
+}
+// of a warp-wide ballot, the target's bits; and those of its members before this one
+template <int S>
+__device__ __forceinline__ uint32_t team_bits(uint32_t ballot) {
+  const uint32_t lane = threadIdx.x & 31;
+  return S == 1 ? (ballot >> (lane & 24u)) & 0xffu : (ballot >> (lane & 3u)) & 0x11111111u;
+}
+template <int S>
+__device__ __forceinline__ uint32_t bits_before(uint32_t bits) {
+  const uint32_t lane = threadIdx.x & 31;
+  return bits & ((1u << (S == 1 ? lane & 7u : lane & 28u)) - 1u);
 }
 // drops the head of the sorted list if it is `head` (keys are distinct where they matter)
 template <int N>
@@ -330,9 +378,10 @@ __device__ __forceinline__ void pop_if(uint32_t (&key)[N], uint32_t head) {
   key[N - 1] = own ? 0xffffffffu : key[N - 1];
 }
 // lexicographic minimum of (distance, tuple) over the eight lanes of a target
+template <int S = 1>
 __device__ __forceinline__ void team_min_exact(double& d, uint32_t& key) {
 #pragma unroll
-  for (int o = 1; o < 8; o <<= 1) {
+  for (int o = S; o < 8 * S; o <<= 1) {
     const double od = __shfl_xor_sync(0xffffffffu, d, o);
     const uint32_t ok = __shfl_xor_sync(0xffffffffu, key, o);
     if (od < d || (od == d && ok < key)) {
@@ -340,6 +389,144 @@ __device__ __forceinline__ void team_min_exact(double& d, uint32_t& key) {
       key = ok;
     }
   }
+}
+
+// The power of two that brings the largest element (of non-negative bit pattern rbits) to [1/2, 1), and its inverse
+__device__ __forceinline__ void unit_scale(uint32_t rbits, float& sc, float& inv) {
+  int e = 126 - (int)((rbits >> 23) & 0xffu);
+  e = e > 15 ? 15 : (e < -100 ? -100 : e);
+  sc = __uint_as_float((uint32_t)(e + 127) << 23);
+  inv = __uint_as_float((uint32_t)(127 - e) << 23);
+}
+// x, y as the sum of two pairs of halves
+__device__ __forceinline__ void split_halves(float x, float y, uint32_t& hi_bits, uint32_t& lo_bits) {
+  const __half2 hi = __floats2half2_rn(x, y);
+  const float2 back = __half22float2(hi);
+  const __half2 lo = __floats2half2_rn(x - back.x, y - back.y);
+  hi_bits = *reinterpret_cast<const uint32_t*>(&hi);
+  lo_bits = *reinterpret_cast<const uint32_t*>(&lo);
+}
+
+// The `keep` smallest of a target's extensions under (binary64 distance, tuple), the one of member `b`: of the n_list listed
+// ones (unsure), or of all (more than the list holds).  Seldom needed: not inlined.
+template <int S>
+__device__ __noinline__ uint32_t choose_exact(const uint2* list, uint32_t n_list, uint32_t b, uint32_t keep, bool unsure, bool all,
+                                              const float* t, const float (*books)[kBsK][8], int codes,
+                                              const uint32_t* kept, uint32_t before, uint32_t K) {
+  constexpr uint32_t kFull = 0xffffffffu;
+  uint32_t next = 0;
+  if (__any_sync(kFull, unsure)) {
+    double ed[4];
+    uint32_t ek[4];
+#pragma unroll 1
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t at = 8 * i + b;
+      ek[i] = at < n_list ? list[at].y : kFull;
+      ed[i] = unsure && ek[i] != kFull ? exact_partial(t, books, ek[i], codes) : __longlong_as_double(kInfBits);
+    }
+    for (uint32_t r = 0; r < keep; ++r) {
+      double d = ed[0];
+      uint32_t k = ek[0];
+      for (int i = 1; i < 4; ++i)
+        if (ed[i] < d || (ed[i] == d && ek[i] < k)) d = ed[i], k = ek[i];
+      team_min_exact<S>(d, k);
+      if (unsure && b == r) next = k;
+      for (int i = 0; i < 4; ++i)
+        if (ek[i] == k) ed[i] = __longlong_as_double(kInfBits), ek[i] = kFull;
+    }
+  }
+  if (__any_sync(kFull, all)) {
+    double ld = -1.0;  // the (distance, tuple) taken last
+    uint32_t lk = 0;
+    for (uint32_t r = 0; r < keep; ++r) {
+      double d = __longlong_as_double(kInfBits);
+      uint32_t k = kFull;
+      for (uint32_t e = b; e < before * K; e += 8) {
+        if (!all) break;
+        const uint32_t key2 = (codes > 1 ? kept[e / K] : 0u) | ((e % K) << (32 - 8 * codes));
+        const double x = exact_partial(t, books, key2, codes);
+        const bool later = x > ld || (x == ld && (key2 > lk || r == 0));
+        if (later && (x < d || (x == d && key2 < k))) d = x, k = key2;
+      }
+      __syncwarp();
+      team_min_exact<S>(d, k);
+      if (all && b == r) next = k;
+      ld = d;
+      lk = k;
+    }
+  }
+  return next;
+}
+// The `keep` smallest of a target's listed extensions under (score, tuple), n_list of them (more than kBsList: the list is
+// not complete): the one of member `b`.  Scores decide where exactly `keep` lie within the margin, otherwise binary64.
+// `before` tuples were kept before the stage; with its codeword a tuple has `codes` codes.
+template <int S>
+__device__ __forceinline__ uint32_t choose_kept(const uint2* list, uint32_t n_list, uint32_t b, uint32_t keep, float margin,
+                                                bool target, const float* t, const float (*books)[kBsK][8], int codes,
+                                                const uint32_t* kept, uint32_t before, uint32_t K) {
+  constexpr uint32_t kFull = 0xffffffffu;
+  // eight lanes per target, up to four entries each
+  float es[4];
+  uint32_t key[4];
+  const bool all = n_list > (uint32_t)kBsList;  // many equal extensions: every one of them gets its distance
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t at = 8 * i + b;
+    const bool have = at < n_list && !all;
+    es[i] = have ? __uint_as_float(list[at].x) : kInf;
+    key[i] = have ? (ord(es[i]) & ~31u) | at : kFull;
+  }
+  sort4(key);
+  uint32_t pick = kFull, last = 0;  // the list entry that becomes kept tuple b
+  for (uint32_t r = 0; r < keep; ++r) {
+    last = team_min<S>(key[0]);
+    if (b == r) pick = last & 31u;
+    pop_if(key, last);
+  }
+  // exactly `keep` entries up to the last one's bucket plus the margin: provably the exact ones
+  const float sure = unord(last | 31u) + margin;
+  uint32_t near = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) near += es[i] <= sure && 8 * i + b < n_list;
+#pragma unroll
+  for (int o = S; o < 8 * S; o <<= 1) near += __shfl_xor_sync(kFull, near, o);
+  uint32_t next = b < keep && pick < n_list ? list[pick].y : 0u;
+  const bool unsure = target && !all && near != keep;
+  if (__any_sync(kFull, unsure || (target && all))) {
+    const uint32_t exact = choose_exact<S>(list, n_list, b, keep, unsure, target && all, t, books, codes, kept, before, K);
+    if (unsure || (target && all)) next = exact;
+  }
+  return next;
+}
+// A limit that the list of more extensions than it holds (one target in fifty) is collected again with: the keep-th
+// smallest of those it holds, plus the margin.  Equal scores in that number are left to choose_kept.
+template <int S>
+__device__ __forceinline__ float lower_limit(const uint2* list, bool over, uint32_t b, uint32_t keep, float margin) {
+  uint32_t key[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) key[i] = over ? (ord(__uint_as_float(list[8 * i + b].x)) & ~31u) | (8 * i + b) : 0xffffffffu;
+  sort4(key);
+  uint32_t last = 0;
+  for (uint32_t r = 0; r < keep; ++r) {
+    last = team_min<S>(key[0]);
+    pop_if(key, last);
+  }
+  return unord(last | 31u) + margin;
+}
+// The limit up to which fast scores matter: the keep-th smallest of a target's 64 cell minima (keep different extensions
+// score no more than that), plus the margin; without a limit if there are fewer cells, or padding among them
+template <int S>
+__device__ __forceinline__ float kept_limit(const float (&cell_min)[8], uint32_t b, uint32_t keep, float margin) {
+  uint32_t key[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) key[c] = (ord(cell_min[c]) & ~63u) | (b * 8 + c);
+  sort8(key);
+  uint32_t last = 0;
+  for (uint32_t r = 0; r < keep; ++r) {
+    last = team_min<S>(key[0]);
+    pop_if(key, last);
+  }
+  return last >= ord(1.0e38f) ? kInf : unord(last | 63u) + margin;
 }
 
 // One further stage's fast scores for the lane's residual (target my_q, kept tuple my_b; rho = ||r||^2/2): the minimum
@@ -362,19 +549,11 @@ __device__ __forceinline__ float stage_minima(const StageImage<TC>& st, BeamScra
       rmax = fmaxf(rmax, fmaxf(fabsf(nr[r4].x), fabsf(nr[r4].y)));
     }
     const uint32_t rbits = __reduce_max_sync(0xffffffffu, __float_as_uint(rmax));  // non-negative floats order as u32
-    int e = 126 - (int)((rbits >> 23) & 0xffu);
-    e = e > 15 ? 15 : (e < -100 ? -100 : e);
-    const float sc = __uint_as_float((uint32_t)(e + 127) << 23), inv = __uint_as_float((uint32_t)(127 - e) << 23);
+    float sc, inv;
+    unit_scale(rbits, sc, inv);
     uint32_t a[2][4];
 #pragma unroll
-    for (int r4 = 0; r4 < 4; ++r4) {
-      const float x = nr[r4].x * -sc, y = nr[r4].y * -sc;
-      const __half2 hi = __floats2half2_rn(x, y);
-      const float2 back = __half22float2(hi);
-      const __half2 lo = __floats2half2_rn(x - back.x, y - back.y);
-      a[r4 >> 1][r4 & 1] = *reinterpret_cast<const uint32_t*>(&hi);
-      a[r4 >> 1][2 + (r4 & 1)] = *reinterpret_cast<const uint32_t*>(&lo);
-    }
+    for (int r4 = 0; r4 < 4; ++r4) split_halves(nr[r4].x * -sc, nr[r4].y * -sc, a[r4 >> 1][r4 & 1], a[r4 >> 1][2 + (r4 & 1)]);
     // a cell is what one thread sees of a residual in half the tiles: no exchange between the threads (with cells of 32
     // adjacent columns, two exchanges per cell and row: 11008x4096 k = 56360 two codebooks 1.8 us more, three 4.8 us)
     float m[4][2];
@@ -500,122 +679,217 @@ __global__ void __launch_bounds__(kBsThreads, kBsCtasPerSm) encode_beam_kernel(c
     }
     __syncwarp();
 
-    // ---- stage 1, one target after the other, the whole warp on each
-#pragma unroll 1
-    for (uint32_t q = 0; q < (uint32_t)kBsGroup; ++q) {
+    if constexpr (TC) {
+      // ---- stage 1 on the tensor pipe, the four targets side by side: lane = target q + 4 part.  The columns of B are the
+      // targets (every other column: a thread then has one target's scores), split in two halves like the residuals below.
+      const uint32_t q = (uint32_t)lane & 3u, part = (uint32_t)lane >> 2;
       const uint64_t n = gi * kBsGroup + q;
-      if (n >= p.k) break;
       const uint32_t j = __shfl_sync(kFull, lane_j, 8 * q);
-      const uint32_t prev = __shfl_sync(kFull, lane_prev, 8 * q);
-      if (j >= p.G) {
-        if (lane == 0) atomicOr(p.status, PVT_DEV_BAD_INDEX);
-        continue;
-      }
-      float t[8];
+      const bool target = j < p.G;
+      if (n < p.k && !target && part == 0) atomicOr(p.status, PVT_DEV_BAD_INDEX);
+      const float* tq = &w.t[q][0];
+      float sr[8], tnorm;
       {
-        const float4 ta = *reinterpret_cast<const float4*>(&w.t[q][0]);
-        const float4 tb = *reinterpret_cast<const float4*>(&w.t[q][4]);
-        t[0] = ta.x, t[1] = ta.y, t[2] = ta.z, t[3] = ta.w, t[4] = tb.x, t[5] = tb.y, t[6] = tb.z, t[7] = tb.w;
-      }
-      float nt2 = 0.0f;
+        const float4 ta = *reinterpret_cast<const float4*>(tq), tb = *reinterpret_cast<const float4*>(tq + 4);
+        sr[0] = ta.x, sr[1] = ta.y, sr[2] = ta.z, sr[3] = ta.w, sr[4] = tb.x, sr[5] = tb.y, sr[6] = tb.z, sr[7] = tb.w;
+        float nt2 = 0.0f;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) nt2 = fmaf(t[i], t[i], nt2);
-      const float tnorm = sqrtf(nt2);
-      // twice the rounding-error bound of the fast score (factor >= 2 to spare), u = 2^-24:
-      //   |score1_fl - score1| <= 16.1 u (||c1||^2/2 + ||t|| ||c1||)
-      const float margin1 = 3.8146973e-6f /* 2^-18 */ * (0.5f * s1max * s1max + tnorm * s1max) + 1e-30f;
-
-      // 256 scores, 8 per lane
-      float f[8];
+        for (int i = 0; i < 8; ++i) nt2 = fmaf(sr[i], sr[i], nt2);
+        tnorm = sqrtf(nt2);
+      }
+      my_j = lane_j < p.G ? lane_j : kFull;
+      my_prev = lane_prev;
+      my_sall = __shfl_sync(kFull, tnorm, my_q) + sall_books;
+      float sc, inv, cell_min[8];
       {
-        uint64_t acc[4];
+        float2 x = make_float2(0.0f, 0.0f);
+        if (!(part & 1u)) x = *reinterpret_cast<const float2*>(&w.t[part >> 1][2 * q]);
+        unit_scale(__reduce_max_sync(kFull, __float_as_uint(fmaxf(fabsf(x.x), fabsf(x.y)))), sc, inv);
+        uint32_t b0, b1;
+        split_halves(x.x * -sc, x.y * -sc, b0, b1);
 #pragma unroll
-        for (int qq = 0; qq < 4; ++qq) acc[qq] = sm.h1[qq][lane];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const uint64_t ntd = pack2(-t[i], -t[i]);
-#pragma unroll
-          for (int qq = 0; qq < 4; ++qq) acc[qq] = fma2(ntd, sm.p1[qq][i][lane], acc[qq]);
-        }
-#pragma unroll
-        for (int qq = 0; qq < 4; ++qq) {
-          f[2 * qq] = lo_of(acc[qq]);
-          f[2 * qq + 1] = hi_of(acc[qq]);
-        }
-      }
-      // extract the B smallest (score truncated to 24 bits | code): a first guess of the beam.  Every lane sorts
-      // its eight keys once; a round is then one warp minimum of the lanes' heads and a shift of the winning lane's list.
-      uint32_t key[8];
-#pragma unroll
-      for (int jj = 0; jj < 8; ++jj) key[jj] = (ord(f[jj]) & 0xffffff00u) | (uint32_t)(lane + 32 * jj);
-      sort8(key);
-      uint32_t beam_code[8];
-      uint32_t last = 0;  // the key extracted last
-#pragma unroll
-      for (int b = 0; b < 8; ++b) {
-        beam_code[b] = 0;
-        if ((uint32_t)b < B) {
-          last = __reduce_min_sync(kFull, key[0]);
-          beam_code[b] = last & 0xffu;
-          pop_if(key, last);  // keys are distinct: they end in the code
+        for (int c = 0; c < 8; ++c) {
+          float d0[4], d1[4];
+          const float2 h0 = sm.first.h2[2 * c][part], h1 = sm.first.h2[2 * c + 1][part];
+          mma_codeword_rows(d0, sm.first.a[2 * c][lane], b0, b1, h0.x * sc, h0.y * sc);
+          mma_codeword_rows(d1, sm.first.a[2 * c + 1][lane], b0, b1, h1.x * sc, h1.y * sc);
+          const float least = min3(fminf(d0[0], d0[2]), d1[0], d1[2]);
+          cell_min[c] = target ? least * inv : kInf;
         }
       }
-      // is that guess provably the exact beam?  theta = an upper bound of the scores in the guess (the top of the
-      // truncation bucket of the key extracted last); every member of the exact beam scores <= theta + margin1; if
-      // exactly B codewords do, they are the guess and the exact beam at once.
-      {
-        uint32_t cnt = 0;
-        const float theta = unord(last | 0xffu);
-        const float limit1 = theta + margin1;
-        uint32_t member = 0;
+      // as below: twice the rounding-error bound of a fast score with a factor 2 to spare, and what the halves add
+      const float reach = tnorm + s1max;
+      const float margin = (7.6293945e-6f /* 2^-17 */ * reach) * reach + 4.76837158203125e-7f /* 2^-21 */ * inv * s1max + 1e-30f;
+      float limit = kept_limit<4>(cell_min, part, B, margin);
+      uint32_t n_list = 0;  // the same in the target's eight lanes
+#pragma unroll 1
+      for (int pass = 0;; ++pass) {
+        // the cells within the limit, eight at a time, one per lane, four codewords each
+        uint32_t hits = 0;
 #pragma unroll
-        for (int jj = 0; jj < 8; ++jj) {
-          const bool in = f[jj] <= limit1 && (uint32_t)(lane + 32 * jj) < p.K;
-          member |= in ? (1u << jj) : 0u;
-          cnt += in;
+        for (int c = 0; c < 8; ++c) hits |= target && cell_min[c] <= limit ? 1u << c : 0u;
+        uint32_t at = __popc(hits), total;
+        {
+          const uint32_t mine = at;
+#pragma unroll
+          for (int o = 4; o < 32; o <<= 1) {
+            const uint32_t up = __shfl_up_sync(kFull, at, o);
+            if (lane >= o) at += up;
+          }
+          total = __shfl_sync(kFull, at, 28 + q);
+          at -= mine;
         }
-        cnt = __reduce_add_sync(kFull, cnt);
-        if (cnt != B) {
-          // undecided: order the shortlisted codewords by (binary64 distance, code)
-          for (uint32_t b = 0; b < B; ++b) {
-            double ld = __longlong_as_double(kInfBits);
-            uint32_t lk = kFull;
+        for (uint32_t m = hits; m; m &= m - 1) w.cells[q][at++] = (uint8_t)(8 * part + __ffs(m) - 1);
+        __syncwarp();
+        n_list = 0;
+        for (uint32_t base = 0; __any_sync(kFull, base < total); base += 8) {
+          const bool work = base + part < total;
+          const uint32_t cell = work ? w.cells[q][base + part] : 0u;
 #pragma unroll
-            for (int jj = 0; jj < 8; ++jj) {
-              if (member & (1u << jj)) {
-                const uint32_t kap = lane + 32 * jj;
-                const double d = exact1(t, sm.c[0][kap]);
-                if (d < ld || (d == ld && kap < lk)) {
-                  ld = d;
-                  lk = kap;
-                }
-              }
-            }
-            // warp-wide lexicographic minimum of (ld, lk); distances are >= 0 so their bits order like u64
-            const uint64_t bits = (uint64_t)__double_as_longlong(ld);
-            const uint32_t hi = (uint32_t)(bits >> 32), lo = (uint32_t)bits;
-            const uint32_t mhi = __reduce_min_sync(kFull, hi);
-            const uint32_t mlo = __reduce_min_sync(kFull, hi == mhi ? lo : kFull);
-            const uint32_t mk = __reduce_min_sync(kFull, (hi == mhi && lo == mlo) ? lk : kFull);
-            const uint32_t chosen = mk < (uint32_t)kBsK ? mk : 0u;
+          for (uint32_t c = 0; c < 4; ++c) {
+            const uint32_t k1 = 4 * cell + ((c + part) & 3u);  // (the lanes begin at different ones: fewer bank conflicts)
+            const float4 ca = *reinterpret_cast<const float4*>(&sm.c[0][k1][0]);
+            const float4 cb = *reinterpret_cast<const float4*>(&sm.c[0][k1][4]);
+            const float cv[8] = {ca.x, ca.y, ca.z, ca.w, cb.x, cb.y, cb.z, cb.w};
+            float s1 = sm.first.h[k1];
 #pragma unroll
-            for (int bb = 0; bb < 8; ++bb)
-              if ((uint32_t)bb == b) beam_code[bb] = chosen;
-            if ((chosen & 31u) == (uint32_t)lane) member &= ~(1u << (chosen >> 5));
+            for (int i = 0; i < 8; ++i) s1 = __fmaf_rn(-sr[i], cv[i], s1);
+            const bool in = work && s1 <= limit && k1 < p.K;
+            const uint32_t who = team_bits<4>(__ballot_sync(kFull, in));
+            const uint32_t to = n_list + __popc(bits_before<4>(who));
+            if (in && to < (uint32_t)kBsList) w.list[q][to] = make_uint2(__float_as_uint(s1), k1 << 24);
+            n_list += __popc(who);
           }
         }
+        __syncwarp();
+        const bool over = n_list > (uint32_t)kBsList;
+        if (pass == 3 || !__any_sync(kFull, over)) break;
+        const float lower = lower_limit<4>(w.list[q], over, part, B, margin);
+        const bool again = over && lower < limit;
+        if (!__any_sync(kFull, again)) break;
+        if (again) limit = lower;
+        __syncwarp();
       }
-      // hand the beam to the lanes of the further stages
-      if (lane == 0) {
-        *reinterpret_cast<uint4*>(&w.kept[q][0]) =
-            make_uint4(beam_code[0] << 24, beam_code[1] << 24, beam_code[2] << 24, beam_code[3] << 24);
-        *reinterpret_cast<uint4*>(&w.kept[q][4]) =
-            make_uint4(beam_code[4] << 24, beam_code[5] << 24, beam_code[6] << 24, beam_code[7] << 24);
-      }
-      if (my_q == q) {
-        my_j = j;
-        my_prev = prev;
-        my_sall = tnorm + sall_books;
+      const uint32_t next = choose_kept<4>(w.list[q], n_list, part, B, margin, target, tq, sm.c, 1, nullptr, 1, p.K);
+      if (target) w.kept[q][part] = next;
+    } else {
+      // ---- stage 1, one target after the other, the whole warp on each
+#pragma unroll 1
+      for (uint32_t q = 0; q < (uint32_t)kBsGroup; ++q) {
+        const uint64_t n = gi * kBsGroup + q;
+        if (n >= p.k) break;
+        const uint32_t j = __shfl_sync(kFull, lane_j, 8 * q);
+        const uint32_t prev = __shfl_sync(kFull, lane_prev, 8 * q);
+        if (j >= p.G) {
+          if (lane == 0) atomicOr(p.status, PVT_DEV_BAD_INDEX);
+          continue;
+        }
+        float t[8];
+        {
+          const float4 ta = *reinterpret_cast<const float4*>(&w.t[q][0]);
+          const float4 tb = *reinterpret_cast<const float4*>(&w.t[q][4]);
+          t[0] = ta.x, t[1] = ta.y, t[2] = ta.z, t[3] = ta.w, t[4] = tb.x, t[5] = tb.y, t[6] = tb.z, t[7] = tb.w;
+        }
+        float nt2 = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) nt2 = fmaf(t[i], t[i], nt2);
+        const float tnorm = sqrtf(nt2);
+        // twice the rounding-error bound of the fast score (factor >= 2 to spare), u = 2^-24:
+        //   |score1_fl - score1| <= 16.1 u (||c1||^2/2 + ||t|| ||c1||)
+        const float margin1 = 3.8146973e-6f /* 2^-18 */ * (0.5f * s1max * s1max + tnorm * s1max) + 1e-30f;
+
+        // 256 scores, 8 per lane
+        float f[8];
+        {
+          uint64_t acc[4];
+#pragma unroll
+          for (int qq = 0; qq < 4; ++qq) acc[qq] = sm.first.h1[qq][lane];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const uint64_t ntd = pack2(-t[i], -t[i]);
+#pragma unroll
+            for (int qq = 0; qq < 4; ++qq) acc[qq] = fma2(ntd, sm.first.p1[qq][i][lane], acc[qq]);
+          }
+#pragma unroll
+          for (int qq = 0; qq < 4; ++qq) {
+            f[2 * qq] = lo_of(acc[qq]);
+            f[2 * qq + 1] = hi_of(acc[qq]);
+          }
+        }
+        // extract the B smallest (score truncated to 24 bits | code): a first guess of the beam.  Every lane sorts
+        // its eight keys once; a round is then one warp minimum of the lanes' heads and a shift of the winning lane's list.
+        uint32_t key[8];
+#pragma unroll
+        for (int jj = 0; jj < 8; ++jj) key[jj] = (ord(f[jj]) & 0xffffff00u) | (uint32_t)(lane + 32 * jj);
+        sort8(key);
+        uint32_t beam_code[8];
+        uint32_t last = 0;  // the key extracted last
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+          beam_code[b] = 0;
+          if ((uint32_t)b < B) {
+            last = __reduce_min_sync(kFull, key[0]);
+            beam_code[b] = last & 0xffu;
+            pop_if(key, last);  // keys are distinct: they end in the code
+          }
+        }
+        // is that guess provably the exact beam?  theta = an upper bound of the scores in the guess (the top of the
+        // truncation bucket of the key extracted last); every member of the exact beam scores <= theta + margin1; if
+        // exactly B codewords do, they are the guess and the exact beam at once.
+        {
+          uint32_t cnt = 0;
+          const float theta = unord(last | 0xffu);
+          const float limit1 = theta + margin1;
+          uint32_t member = 0;
+#pragma unroll
+          for (int jj = 0; jj < 8; ++jj) {
+            const bool in = f[jj] <= limit1 && (uint32_t)(lane + 32 * jj) < p.K;
+            member |= in ? (1u << jj) : 0u;
+            cnt += in;
+          }
+          cnt = __reduce_add_sync(kFull, cnt);
+          if (cnt != B) {
+            // undecided: order the shortlisted codewords by (binary64 distance, code)
+            for (uint32_t b = 0; b < B; ++b) {
+              double ld = __longlong_as_double(kInfBits);
+              uint32_t lk = kFull;
+#pragma unroll
+              for (int jj = 0; jj < 8; ++jj) {
+                if (member & (1u << jj)) {
+                  const uint32_t kap = lane + 32 * jj;
+                  const double d = exact1(t, sm.c[0][kap]);
+                  if (d < ld || (d == ld && kap < lk)) {
+                    ld = d;
+                    lk = kap;
+                  }
+                }
+              }
+              // warp-wide lexicographic minimum of (ld, lk); distances are >= 0 so their bits order like u64
+              const uint64_t bits = (uint64_t)__double_as_longlong(ld);
+              const uint32_t hi = (uint32_t)(bits >> 32), lo = (uint32_t)bits;
+              const uint32_t mhi = __reduce_min_sync(kFull, hi);
+              const uint32_t mlo = __reduce_min_sync(kFull, hi == mhi ? lo : kFull);
+              const uint32_t mk = __reduce_min_sync(kFull, (hi == mhi && lo == mlo) ? lk : kFull);
+              const uint32_t chosen = mk < (uint32_t)kBsK ? mk : 0u;
+#pragma unroll
+              for (int bb = 0; bb < 8; ++bb)
+                if ((uint32_t)bb == b) beam_code[bb] = chosen;
+              if ((chosen & 31u) == (uint32_t)lane) member &= ~(1u << (chosen >> 5));
+            }
+          }
+        }
+        // hand the beam to the lanes of the further stages
+        if (lane == 0) {
+          *reinterpret_cast<uint4*>(&w.kept[q][0]) =
+              make_uint4(beam_code[0] << 24, beam_code[1] << 24, beam_code[2] << 24, beam_code[3] << 24);
+          *reinterpret_cast<uint4*>(&w.kept[q][4]) =
+              make_uint4(beam_code[4] << 24, beam_code[5] << 24, beam_code[6] << 24, beam_code[7] << 24);
+        }
+        if (my_q == q) {
+          my_j = j;
+          my_prev = prev;
+          my_sall = tnorm + sall_books;
+        }
       }
     }
     __syncwarp();
@@ -674,17 +948,7 @@ __global__ void __launch_bounds__(kBsThreads, kBsCtasPerSm) encode_beam_kernel(c
         for (int o = 1; o < 8; o <<= 1) gmin = fminf(gmin, __shfl_xor_sync(kFull, gmin, o));
         limit = gmin + margin;
       } else {
-        uint32_t key[8];
-#pragma unroll
-        for (int sub = 0; sub < 8; ++sub) key[sub] = (ord(sub_min[sub]) & ~63u) | (my_b * 8 + sub);
-        sort8(key);
-        uint32_t last = 0;
-        for (uint32_t b = 0; b < keep; ++b) {
-          last = team_min(key[0]);
-          pop_if(key, last);
-        }
-        // fewer cells than `keep` (or padding among them): no limit
-        limit = last >= ord(1.0e38f) ? kInf : unord(last | 63u) + margin;
+        limit = kept_limit<1>(sub_min, my_b, keep, margin);
       }
       auto flag_cells = [&]() {
         uint32_t hits = 0;
@@ -736,29 +1000,18 @@ __global__ void __launch_bounds__(kBsThreads, kBsCtasPerSm) encode_beam_kernel(c
                 }
               }
             } else {
-              const uint32_t who = (__ballot_sync(kFull, in) >> (8 * my_q)) & 0xffu;
-              const uint32_t at = n_list + __popc(who & ((1u << my_b) - 1u));
+              const uint32_t who = team_bits<1>(__ballot_sync(kFull, in));
+              const uint32_t at = n_list + __popc(bits_before<1>(who));
               if (in && at < (uint32_t)kBsList) w.list[my_q][at] = make_uint2(__float_as_uint(s2), key);
               n_list += __popc(who);
             }
           }
         }
         if (m == M - 1) break;
-        // More extensions within the limit than the list holds (one target in fifty): the keep-th smallest of those it
-        // holds is a lower limit.  Equal scores in that number are left to the exact path below.
         const bool over = n_list > (uint32_t)kBsList;
         if (pass == 3 || !__any_sync(kFull, over)) break;
         __syncwarp();
-        uint32_t key[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) key[i] = over ? (ord(__uint_as_float(w.list[my_q][8 * i + my_b].x)) & ~31u) | (8 * i + my_b) : kFull;
-        sort4(key);
-        uint32_t last = 0;
-        for (uint32_t b = 0; b < keep; ++b) {
-          last = team_min(key[0]);
-          pop_if(key, last);
-        }
-        const float lower = unord(last | 31u) + margin;
+        const float lower = lower_limit<1>(w.list[my_q], over, my_b, keep, margin);
         const bool again = over && lower < limit;
         if (!__any_sync(kFull, again)) break;
         if (again) {
@@ -770,76 +1023,10 @@ __global__ void __launch_bounds__(kBsThreads, kBsCtasPerSm) encode_beam_kernel(c
         __syncwarp();
       }
       if (m < M - 1) {
-        // the `keep` smallest of the list: eight lanes per target, up to four entries each
         __syncwarp();
-        float es[4];
-        uint32_t ek[4], key[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const uint32_t at = 8 * i + my_b;
-          const bool have = at < n_list && n_list <= (uint32_t)kBsList;
-          const uint2 entry = have ? w.list[my_q][at] : make_uint2(0x7f800000u, kFull);
-          es[i] = __uint_as_float(entry.x);
-          ek[i] = entry.y;
-          key[i] = have ? (ord(es[i]) & ~31u) | at : kFull;
-        }
-        sort4(key);
-        uint32_t pick = kFull, last = 0;  // the list entry that becomes kept tuple my_b
-        for (uint32_t b = 0; b < keep; ++b) {
-          last = team_min(key[0]);
-          if (my_b == b) pick = last & 31u;
-          pop_if(key, last);
-        }
-        // exactly `keep` entries up to the last one's bucket plus the margin: provably the exact ones
-        const float sure = unord(last | 31u) + margin;
-        uint32_t near = 0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) near += ek[i] != kFull && es[i] <= sure;
-#pragma unroll
-        for (int o = 1; o < 8; o <<= 1) near += __shfl_xor_sync(kFull, near, o);
-        uint32_t next = my_b < keep && pick < n_list ? w.list[my_q][pick].y : 0u;
         const bool target = my_j != kFull;
-        const bool all = n_list > (uint32_t)kBsList;  // many equal extensions: every one of them gets its distance
-        const bool unsure = target && !all && near != keep;
-        auto partial = [&](uint32_t tuple) { return exact_partial(w.t[my_q], sm.c, tuple, m + 1); };
-        if (__any_sync(kFull, unsure)) {
-          double ed[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            ed[i] = unsure && ek[i] != kFull ? partial(ek[i]) : __longlong_as_double(kInfBits);
-          for (uint32_t b = 0; b < keep; ++b) {
-            double d = ed[0];
-            uint32_t k = ek[0];
-#pragma unroll
-            for (int i = 1; i < 4; ++i)
-              if (ed[i] < d || (ed[i] == d && ek[i] < k)) d = ed[i], k = ek[i];
-            team_min_exact(d, k);
-            if (unsure && my_b == b) next = k;
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-              if (ek[i] == k) ed[i] = __longlong_as_double(kInfBits), ek[i] = kFull;
-          }
-        }
-        if (__any_sync(kFull, target && all)) {
-          double ld = -1.0;  // the (distance, tuple) taken last
-          uint32_t lk = 0;
-          for (uint32_t b = 0; b < keep; ++b) {
-            double d = __longlong_as_double(kInfBits);
-            uint32_t k = kFull;
-            for (uint32_t e = my_b; e < B * p.K; e += 8) {
-              if (!(target && all)) break;
-              const uint32_t key2 = w.kept[my_q][e / p.K] | ((e % p.K) << (24 - 8 * m));
-              const double x = partial(key2);
-              const bool later = x > ld || (x == ld && (key2 > lk || b == 0));
-              if (later && (x < d || (x == d && key2 < k))) d = x, k = key2;
-            }
-            __syncwarp();
-            team_min_exact(d, k);
-            if (target && all && my_b == b) next = k;
-            ld = d;
-            lk = k;
-          }
-        }
+        const uint32_t next = choose_kept<1>(w.list[my_q], n_list, my_b, keep, margin, target, w.t[my_q], sm.c, m + 1,
+                                             w.kept[my_q], B, p.K);
         __syncwarp();  // everybody has read the tuples that are replaced now
         if (target) w.kept[my_q][my_b] = next;
         B = keep;

@@ -51,3 +51,26 @@ def test_a_target_that_is_not_finite_is_reported_and_keeps_its_codes(M, f16, val
     rest = np.setdiff1d(idx, odd)
     decisive = (want.d_second - want.d_best)[rest] > 1e-6 * want.d_second[rest]
     assert np.array_equal(got[rest][decisive], want.codes[rest][decisive])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,K,beam,f16", [
+    (2, 2, 8, True), (2, 3, 8, True), (2, 8, 8, True), (2, 9, 8, True), (2, 33, 8, True), (2, 251, 5, True), (2, 256, 1, True),
+    (2, 9, 8, False), (2, 251, 5, False),
+])
+def test_small_and_ragged_first_codebook(M, K, beam, f16):
+    L = synth.make_layer(16, 264, cfg=330 + M, num_codebooks=M, codebook_size=K, codebook_fp16=f16, beam=beam,
+                         nearest=oracle_nearest)
+    check_encode(L, np.arange(2, L.num_groups, 3, dtype=np.uint32))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M", [2, 3])
+@pytest.mark.parametrize("copies,jitter", [(16, 1e-3), (40, 1e-3), (16, 0.0), (40, 0.0), (32, 1e-6), (5, 0.0)])
+def test_clustered_first_codebook(M, copies, jitter):
+    """more codewords at the limit of stage 1 than its list holds, apart, nearly equal and equal"""
+    L = synth.make_layer(16, 256, cfg=340 + M, num_codebooks=M, codebook_size=256, codebook_fp16=True, nearest=oracle_nearest)
+    rng = np.random.default_rng(copies)
+    base = L.codebooks[0].astype(np.float32)[np.arange(256) // copies]
+    L.codebooks[0] = (base + rng.normal(0.0, jitter, size=base.shape)).astype(L.codebooks.dtype)
+    check_encode(L, np.arange(L.num_groups, dtype=np.uint32))
