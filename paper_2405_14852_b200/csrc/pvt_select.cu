@@ -12,13 +12,15 @@
 //   2. bin:    every CTA finds the threshold bin and writes two bits per group, above it and inside it; the members of
 //              the bin are counted by their lower 18 bits, in a table of all 2^18 of them (few members: few atomics) and
 //              in one of the upper nine of these bits
-//   3. write:  every CTA reads the threshold from those two tables, looks up the keys inside the bin, counts what it
-//              takes, waits for the counts of the CTAs before it and writes its part of the list by ballots:
+//   3. write:  the last warp of every CTA reads the threshold from those two tables, while the others ask for the masks and
+//              the keys of the first members of the bin; then it counts what it takes, waits for the counts of the CTAs
+//              before it and writes its part of the list by ballots:
 //              position = (#greater before) + min(#equal before, ties to take)
-// Measured as graph replays, 4096 x 4096 / 11008 x 4096 / 28672 x 8192: 32 / 53 / 245 us.  Of the first, by its counters,
-// pass 1 takes 16 us (4.2 TB/s of g from cold; 5.4 for the second), the others 4.5, 10 and 12.  Five passes with one bin
-// per eighth of an octave took 45 / 74 / 344 us.  One cooperative kernel with the keys in shared memory takes 33 us, and
-// about 10 us more to launch.
+// Measured as calls one after the other, 4096 x 4096 / 11008 x 4096: 27.7 / 52.2 us (29.7 / 54.5 with nothing asked for
+// ahead, one CTA per SM and polls without a pause).  By counters of the kernels by themselves pass 1 takes 16 us of the
+// first (4.2 TB/s of g from cold; 5.4 for the second), the others 4.5, 10 and 12; 28672 x 8192: 245 us.  Five passes with
+// one bin per eighth of an octave took 45 / 74 / 344 us.  One cooperative kernel with the keys in shared memory takes
+// 33 us, and about 10 us more to launch.  Clearing the large tables in pass 1, and contiguous shares there: no gain.
 #include "pvt_internal.h"
 
 namespace pvt {
@@ -337,11 +339,22 @@ __global__ void __launch_bounds__(kSelThreads) select_write_kernel(const SelPara
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   pdl_trigger();
   pdl_wait();
-  if (tid == 32) {
-    ticket = atomicAdd(&p.state[2], 1u);
-    sum_gt = sum_eq = all_gt = all_eq = 0;
-  }
-  if (warp == 0) {
+  constexpr uint32_t kReaders = kSelThreads - 32;  // the last warp finds the threshold
+  const uint64_t n_words = (p.G + 31) / 32;
+  uint2 early = make_uint2(0, 0);  // of the first trip: this thread's masks, the key of its first member of the bin
+  uint32_t early_key = 0;
+  if (tid < kReaders) {
+    if (tid == 0) {
+      ticket = atomicAdd(&p.state[2], 1u);
+      sum_gt = sum_eq = all_gt = all_eq = 0;
+    }
+    asm volatile("bar.sync 1, %0;" ::"n"(kReaders) : "memory");
+    const uint64_t w = (uint64_t)ticket * p.words + tid;
+    if (tid < p.words && w < n_words) {
+      early = __ldcg(p.masks + w);
+      if (early.y) early_key = __ldcg(p.keys + w * 32 + (uint32_t)__ffs(early.y) - 1);
+    }
+  } else {
     const uint32_t bin = __ldcg(p.state), in_bin = __ldcg(p.state + 1);
     uint32_t d1, d2, left;
     find_digit_warp(p.hist1, in_bin, &d1, &left);
@@ -353,16 +366,17 @@ __global__ void __launch_bounds__(kSelThreads) select_write_kernel(const SelPara
   }
   __syncthreads();
   const uint32_t cta = ticket, threshold = sh_threshold, need_eq = sh_need;
-  const uint64_t w_lo = (uint64_t)cta * p.words, n_words = (p.G + 31) / 32;
+  const uint64_t w_lo = (uint64_t)cta * p.words;
   const uint64_t w_hi = w_lo + p.words < n_words ? w_lo + p.words : n_words;
 
   // one word of 32 groups per thread and trip; the members of the threshold bin (few) are looked up
   auto resolve = [&](uint64_t w) {
-    uint2 m = __ldcg(p.masks + w);
+    const bool known = w == w_lo + tid && tid < kReaders;
+    const uint2 m = known ? early : __ldcg(p.masks + w);
     uint32_t gt = m.x, eq = 0;
     for (uint32_t in = m.y; in; in &= in - 1) {
       const uint32_t b = (uint32_t)__ffs(in) - 1;
-      const uint32_t key = __ldcg(p.keys + w * 32 + b);
+      const uint32_t key = known && in == m.y ? early_key : __ldcg(p.keys + w * 32 + b);
       gt |= key > threshold ? 1u << b : 0u;
       eq |= key == threshold ? 1u << b : 0u;
     }
@@ -392,8 +406,10 @@ __global__ void __launch_bounds__(kSelThreads) select_write_kernel(const SelPara
   uint32_t prev_gt = 0, prev_eq = 0;
   for (uint32_t b = tid; b < cta; b += kSelThreads) {
     uint64_t c = 0;
-    for (uint32_t i = 0; i < kSelMaxPolls && !(c >> 63); ++i)
+    for (uint32_t i = 0; i < kSelMaxPolls && !(c >> 63); ++i) {
+      if (i) __nanosleep(40);
       asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(c) : "l"(p.counts + b) : "memory");
+    }
     ok &= (c >> 63) != 0;
     prev_gt += (uint32_t)c & 0x7fffffffu;
     prev_eq += (uint32_t)(c >> 31) & 0x7fffffffu;
@@ -522,7 +538,15 @@ cudaError_t launch_select_keyed(const pvt_layer& L, uint64_t G, uint64_t k, uint
       err = L.group_dim == 16 ? launch_group<16>(key_mode, p, sm_count, stream)
                               : launch_group<8>(key_mode, p, sm_count, stream);
     if (err == cudaSuccess) err = launch_dependent(select_bin_kernel, (unsigned)n_cta, kSelThreads, 0, stream, p);
-    if (err == cudaSuccess) err = launch_dependent(select_write_kernel, (unsigned)n_cta, kSelThreads, 0, stream, p);
+    // the last pass: one trip of words per CTA (of those that ask early), for which two CTAs of an SM may be needed
+    // (11008 x 4096: 1 us less than two trips of one CTA)
+    const uint64_t words = (G + 31) / 32, trip = kSelThreads - 32;
+    uint64_t w_cta = n_cta;
+    if (p.words > trip) w_cta = (words + trip - 1) / trip;
+    if (w_cta > 2 * most) w_cta = 2 * most;
+    if (w_cta > kSelMaxCtas) w_cta = kSelMaxCtas;
+    p.words = (uint32_t)((words + w_cta - 1) / w_cta);
+    if (err == cudaSuccess) err = launch_dependent(select_write_kernel, (unsigned)w_cta, kSelThreads, 0, stream, p);
     count_launches(3);
   }
   count_launches(1);

@@ -34,3 +34,15 @@ def test_selection_edges(rows, cols, k, offset, levels):
         B.pvt_vstep_select(desc, k, idx, ws)
     assert B.pvt_status(ws) == 0
     assert np.array_equal(idx.cpu().numpy().astype(np.uint32), np.asarray(want, dtype=np.uint32))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("rows,cols,k,offset,levels", [
+    (4096, 9184, 47001, 0, 0),     # 148 CTAs of 993 words: the first size with more CTAs than SMs in the last pass
+    (16003, 2440, 48809, 0, 0),    # more words than threads per SM: two CTAs of an SM
+    (16003, 2440, 1000000, 0, 2),  # the same with ties in every word
+    (20003, 3928, 98214, 0, 0),    # and several trips of those
+    (1031, 32, 900, 0, 1),         # one norm only
+])
+def test_selection_edges_of_the_last_pass(rows, cols, k, offset, levels):
+    test_selection_edges(rows, cols, k, offset, levels)
