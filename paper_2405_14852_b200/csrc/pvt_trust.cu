@@ -13,14 +13,14 @@
 //                  codes; counts of the first digit
 //   4 x radix pass stable LSD sort of the pairs by descending key: positions ascend, so equal norms keep the
 //                  lowest index first
-//   sq_norm        ||W_hat||^2 of the whole matrix in binary64 (fixed summation tree)
+//   sq_norm        ||W_hat||^2 of the whole matrix in binary64 (fixed summation tree), beside the radix passes
 //   search         the library's own encode kernels on the ascending list
 //   change         squared change of each group's dequantised weights, summed along the rank order block by block
 //   cut            running sum of the blocks, first position that breaks the bound
 //   restore        previous codes for every position from the cut on
 // Bound by the latency of these short dependent kernels: each is launched while the one before it runs, and up to
-// kSortDirect blocks a radix pass is one kernel.  (Three plain launches per pass: step of 4096x4096, k = 20971, 306 us;
-// now 209.)
+// kSortDirect blocks a radix pass is one kernel, with a quarter of the norm beside it.  (Three plain launches per pass: step
+// of 4096x4096, k = 20971, 306 us; one kernel per pass 209; now, with a faster selection and search, 170.)
 #include <cuda_fp16.h>
 
 #include "pvt_internal.h"
@@ -179,16 +179,18 @@ __global__ void __launch_bounds__(kScanThreads) sort_scan_kernel(uint32_t* count
 
 // stable scatter: within a block the pairs are visited in position order (round, then thread); a pair's slot is
 // the block's start for its digit + the number of earlier pairs of the block with the same digit
+struct ScatterSmem {
+  uint32_t seen[kSortBins];             // pairs of earlier rounds, per digit, plus the block's start
+  uint32_t cnt[kSortWarps][kSortBins];  // this round: per warp and digit
+  uint32_t warp_total[kSortWarps];
+};
 template <bool DIRECT>
-__global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const uint64_t* in, uint64_t* out, const RankParams p,
-                                                                    int pass) {
-  __shared__ uint32_t seen[kSortBins];               // pairs of earlier rounds, per digit, plus the block's start
-  __shared__ uint32_t cnt[kSortWarps][kSortBins];    // this round: per warp and digit
-  __shared__ uint32_t warp_total[kSortWarps];
+__device__ __forceinline__ void sort_scatter(const uint64_t* in, uint64_t* out, const RankParams& p, int pass, ScatterSmem& sm) {
+  auto& seen = sm.seen;
+  auto& cnt = sm.cnt;
+  auto& warp_total = sm.warp_total;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint64_t k = p.k;
-  pdl_trigger();
-  pdl_wait();
   if (DIRECT) {
     // thread = digit: pairs of the digit in earlier blocks and in all, then all pairs of smaller digits
     const uint4* row = reinterpret_cast<const uint4*>(p.counts + ((size_t)pass * kSortBins + threadIdx.x) * p.stride);
@@ -251,6 +253,13 @@ __global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const uint64
     }
     __syncthreads();
   }
+}
+__global__ void __launch_bounds__(kSortThreads) sort_scatter_kernel(const uint64_t* in, uint64_t* out, const RankParams p,
+                                                                    int pass) {
+  __shared__ ScatterSmem sm;
+  pdl_trigger();
+  pdl_wait();
+  sort_scatter<false>(in, out, p, pass, sm);
 }
 
 // ---- codes and dequantised values ------------------------------------------------------------------------------
@@ -342,17 +351,21 @@ struct TrustParams {
 // block to finish adds the block sums in a fixed tree -- the same binary64 result on every run.
 // Four groups are in flight per thread, since each is a chain code -> codeword.  (One at a time, and the last block's sums
 // added by one thread: 32 us for 4096x4096 1x16.)
+struct NormSmem {
+  double sh[kNormThreads];
+  bool last;
+};
+// share `part` of `parts`, one after the other: a share is a run of the trips that all blocks make side by side
 template <bool CB_F16, bool CODE_U16, int DG>
-__global__ void __launch_bounds__(kNormThreads) sq_norm_kernel(const TrustParams p) {
+__device__ __forceinline__ void sq_norm(const TrustParams& p, uint32_t block, uint32_t blocks, uint32_t part, uint32_t parts,
+                                        NormSmem& sm) {
   constexpr int kFlight = DG == 8 ? 4 : 2;
-  __shared__ double sh[kNormThreads];
-  __shared__ bool last;
+  auto& sh = sm.sh;
   double acc = 0.0;
   bool bad = false;
-  pdl_trigger();
-  pdl_wait();
-  const uint64_t stride = (uint64_t)gridDim.x * kNormThreads;
-  for (uint64_t j0 = (uint64_t)blockIdx.x * kNormThreads + threadIdx.x; j0 < p.G; j0 += kFlight * stride) {
+  const uint64_t stride = (uint64_t)blocks * kNormThreads, trip = kFlight * stride, trips = (p.G + trip - 1) / trip;
+  for (uint64_t t = trips * part / parts; t < trips * (part + 1) / parts; ++t) {
+    const uint64_t j0 = t * trip + (uint64_t)block * kNormThreads + threadIdx.x;
     uint32_t packed[kFlight];
     float s[kFlight], w[kFlight][DG];
 #pragma unroll
@@ -384,21 +397,46 @@ __global__ void __launch_bounds__(kNormThreads) sq_norm_kernel(const TrustParams
   };
   const double mine = block_sum(acc);
   if (threadIdx.x == 0) {
-    p.partial[blockIdx.x] = mine;
+    p.partial[block] = part ? p.partial[block] + mine : mine;
     __threadfence();
-    last = atomicAdd(p.ticket, 1u) == gridDim.x - 1;
+    sm.last = part == parts - 1 && atomicAdd(p.ticket, 1u) == blocks - 1;
   }
   __syncthreads();
-  if (last) {
+  if (sm.last) {
     __threadfence();
-    double part = 0.0;
-    for (unsigned b = threadIdx.x; b < gridDim.x; b += kNormThreads) part += __ldcg(p.partial + b);
-    const double total = block_sum(part);
+    double some = 0.0;
+    for (unsigned b = threadIdx.x; b < blocks; b += kNormThreads) some += __ldcg(p.partial + b);
+    const double total = block_sum(some);
     if (threadIdx.x == 0) {
       p.stats[0] = total;
       *p.ticket = 0;
     }
   }
+}
+template <bool CB_F16, bool CODE_U16, int DG>
+__global__ void __launch_bounds__(kNormThreads) sq_norm_kernel(const TrustParams p) {
+  __shared__ NormSmem sm;
+  pdl_trigger();
+  pdl_wait();
+  sq_norm<CB_F16, CODE_U16, DG>(p, blockIdx.x, gridDim.x, 0, 1, sm);
+}
+
+// One pass of the sort, and beside it a quarter of the norm, which needs nothing of it: the few blocks of the sort leave
+// the chip to a chain of dependent trips to memory.  (One after the other: 4096x4096 1x16, k = 20971, 175.8 us for 169.7.)
+static_assert(kSortThreads == kNormThreads, "blocks of both kinds in one launch");
+template <bool CB_F16, bool CODE_U16, int DG>
+__global__ void __launch_bounds__(kSortThreads) sort_norm_kernel(const uint64_t* in, uint64_t* out, const RankParams p, int pass,
+                                                                 const TrustParams norm, uint32_t norm_blocks) {
+  __shared__ union {
+    ScatterSmem sort;
+    NormSmem norm;
+  } sm;
+  pdl_trigger();
+  pdl_wait();
+  if (blockIdx.x < p.n_blocks)
+    sort_scatter<true>(in, out, p, pass, sm.sort);
+  else
+    sq_norm<CB_F16, CODE_U16, DG>(norm, blockIdx.x - p.n_blocks, norm_blocks, pass, 4, sm.norm);
 }
 
 // inclusive sums of a block's values in thread order (a fixed tree), by all of its threads; BLOCK / 32 warps
@@ -554,55 +592,6 @@ TrustLayout trust_layout(uint64_t G, uint64_t k, size_t encode_bytes, int sm_cou
   return t;
 }
 
-cudaError_t launch_trust_rank(const pvt_layer& L, uint64_t G, uint64_t k, void* ws, const TrustLayout& t,
-                              cudaStream_t stream) {
-  char* base = static_cast<char*>(ws);
-  uint32_t* status = reinterpret_cast<uint32_t*>(base);
-  const uint32_t* idx = reinterpret_cast<const uint32_t*>(base + t.idx_off);
-  RankParams p;
-  p.g = L.g;
-  p.G = G;
-  p.k = k;
-  p.eta = L.eta;
-  p.idx = idx;
-  p.pairs = reinterpret_cast<uint64_t*>(base + t.pairs_a_off);
-  p.other = reinterpret_cast<uint64_t*>(base + t.pairs_b_off);
-  p.counts = reinterpret_cast<uint32_t*>(base + t.counts_off);
-  p.n_blocks = t.sort_blocks;
-  p.stride = t.sort_stride;
-  p.rounds = t.sort_rounds;
-  p.codes = L.codes;
-  p.M = L.num_codebooks;
-  p.code_u16 = L.code_dtype == PVT_U16;
-  p.saved = reinterpret_cast<uint32_t*>(base + t.saved_off);
-  p.status = status;
-  p.clear_a = reinterpret_cast<uint32_t*>(base + t.stats_off);
-  p.n_clear_a = 64 / 4;
-  p.clear_b = reinterpret_cast<uint32_t*>(base + t.encode_off);
-  p.n_clear_b = kWsHeaderBytes / 4;
-  cudaError_t e = launch_dependent(L.group_dim == 16 ? rank_init_kernel<16> : rank_init_kernel<8>, t.sort_blocks,
-                                   kSortThreads, 0, stream, p, t.sort_direct);
-  count_launches(1);
-  uint64_t *a = p.pairs, *b = p.other;
-  for (int pass = 0; pass < 4 && e == cudaSuccess; ++pass) {
-    if (t.sort_direct) {
-      e = launch_dependent(sort_scatter_kernel<true>, t.sort_blocks, kSortThreads, 0, stream, a, b, p, pass);
-      count_launches(1);
-    } else {
-      if (pass > 0) e = launch_dependent(sort_count_kernel, t.sort_blocks, kSortThreads, 0, stream, a, p, pass);
-      if (e == cudaSuccess)
-        e = launch_dependent(sort_scan_kernel, 1, kScanThreads, 0, stream, p.counts, kSortBins * t.sort_blocks);
-      if (e == cudaSuccess)
-        e = launch_dependent(sort_scatter_kernel<false>, t.sort_blocks, kSortThreads, 0, stream, a, b, p, pass);
-      count_launches(pass > 0 ? 3 : 2);
-    }
-    uint64_t* tmp = a;
-    a = b;
-    b = tmp;
-  }
-  return e;
-}
-
 namespace {
 
 TrustParams make_params(const pvt_layer& L, uint64_t G, uint64_t k, float ratio, uint32_t* idx_out, uint64_t* n_out,
@@ -634,6 +623,71 @@ TrustParams make_params(const pvt_layer& L, uint64_t G, uint64_t k, float ratio,
   return p;
 }
 
+// a pass of the sort with a quarter of the norm
+template <bool CB_F16, bool CODE_U16>
+cudaError_t launch_sort_norm(const uint64_t* in, uint64_t* out, const RankParams& p, int pass, const TrustParams& norm, int dg,
+                             uint32_t norm_blocks, cudaStream_t stream) {
+  return launch_dependent(dg == 16 ? sort_norm_kernel<CB_F16, CODE_U16, 16> : sort_norm_kernel<CB_F16, CODE_U16, 8>,
+                          p.n_blocks + norm_blocks, kSortThreads, 0, stream, in, out, p, pass, norm, norm_blocks);
+}
+
+}  // namespace
+
+cudaError_t launch_trust_rank(const pvt_layer& L, uint64_t G, uint64_t k, void* ws, const TrustLayout& t,
+                              cudaStream_t stream) {
+  char* base = static_cast<char*>(ws);
+  uint32_t* status = reinterpret_cast<uint32_t*>(base);
+  const uint32_t* idx = reinterpret_cast<const uint32_t*>(base + t.idx_off);
+  RankParams p;
+  p.g = L.g;
+  p.G = G;
+  p.k = k;
+  p.eta = L.eta;
+  p.idx = idx;
+  p.pairs = reinterpret_cast<uint64_t*>(base + t.pairs_a_off);
+  p.other = reinterpret_cast<uint64_t*>(base + t.pairs_b_off);
+  p.counts = reinterpret_cast<uint32_t*>(base + t.counts_off);
+  p.n_blocks = t.sort_blocks;
+  p.stride = t.sort_stride;
+  p.rounds = t.sort_rounds;
+  p.codes = L.codes;
+  p.M = L.num_codebooks;
+  p.code_u16 = L.code_dtype == PVT_U16;
+  p.saved = reinterpret_cast<uint32_t*>(base + t.saved_off);
+  p.status = status;
+  p.clear_a = reinterpret_cast<uint32_t*>(base + t.stats_off);
+  p.n_clear_a = 64 / 4;
+  p.clear_b = reinterpret_cast<uint32_t*>(base + t.encode_off);
+  p.n_clear_b = kWsHeaderBytes / 4;
+  cudaError_t e = launch_dependent(L.group_dim == 16 ? rank_init_kernel<16> : rank_init_kernel<8>, t.sort_blocks,
+                                   kSortThreads, 0, stream, p, t.sort_direct);
+  count_launches(1);
+  const TrustParams norm = make_params(L, G, k, 0.0f, nullptr, nullptr, ws, t);
+  uint64_t *a = p.pairs, *b = p.other;
+  for (int pass = 0; pass < 4 && e == cudaSuccess; ++pass) {
+    if (t.sort_direct) {
+      const bool f16 = L.codebook_dtype == PVT_F16, u16 = L.code_dtype == PVT_U16;
+      const auto launch = f16 ? (u16 ? launch_sort_norm<true, true> : launch_sort_norm<true, false>)
+                              : (u16 ? launch_sort_norm<false, true> : launch_sort_norm<false, false>);
+      e = launch(a, b, p, pass, norm, L.group_dim, t.norm_blocks, stream);
+      count_launches(1);
+    } else {
+      if (pass > 0) e = launch_dependent(sort_count_kernel, t.sort_blocks, kSortThreads, 0, stream, a, p, pass);
+      if (e == cudaSuccess)
+        e = launch_dependent(sort_scan_kernel, 1, kScanThreads, 0, stream, p.counts, kSortBins * t.sort_blocks);
+      if (e == cudaSuccess)
+        e = launch_dependent(sort_scatter_kernel, t.sort_blocks, kSortThreads, 0, stream, a, b, p, pass);
+      count_launches(pass > 0 ? 3 : 2);
+    }
+    uint64_t* tmp = a;
+    a = b;
+    b = tmp;
+  }
+  return e;
+}
+
+namespace {
+
 template <bool CB_F16, bool CODE_U16>
 cudaError_t before_search(const TrustParams& p, int dg, unsigned norm_blocks, cudaStream_t stream) {
   count_launches(1);
@@ -656,6 +710,7 @@ cudaError_t after_search(const TrustParams& p, int dg, cudaStream_t stream) {
 
 cudaError_t launch_trust_before_search(const pvt_layer& L, uint64_t G, uint64_t k, void* ws, const TrustLayout& t,
                                        cudaStream_t stream) {
+  if (t.sort_direct) return cudaSuccess;  // the norm went along with the sort
   const TrustParams p = make_params(L, G, k, 0.0f, nullptr, nullptr, ws, t);
   const bool f16 = L.codebook_dtype == PVT_F16, u16 = L.code_dtype == PVT_U16;
   const int dg = L.group_dim;

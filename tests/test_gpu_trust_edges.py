@@ -17,3 +17,12 @@ def test_trust_step_at_the_sort_edges(k_max, ratio):
     L = settle(synth.make_layer(rows, cols, cfg=197, codebook_size=16, codebook_fp16=False))
     L.g = np.round(L.g, 3)  # few distinct values: equal norms
     run_case(L, k_max, ratio)
+
+
+@pytest.mark.parametrize("rows,cols,k_max", [
+    (16, 264, 100),        # one trip of the norm: three of its four shares are empty
+    (2048, 2400, 3000),    # two trips
+    (4096, 6080, 3000),    # six: shares of one and two
+])
+def test_trust_step_with_uneven_shares_of_the_norm(rows, cols, k_max):
+    run_case(settle(synth.make_layer(rows, cols, cfg=198, codebook_size=16, codebook_fp16=True)), k_max, 0.02)
