@@ -3,13 +3,16 @@
 // codebooks.  A move replaces one code of the group's tuple by the value that lowers ||t - sum_m C_m[b_m]||^2
 // most (the neighbour that is smallest under (error, tuple)), and is taken only if the error strictly drops.
 //
-// One warp per target, one to four codebooks.  Every error that decides is the binary64 sum the final decision of the
-// search kernels uses (residual through the codebooks in order, terms added in element order), so the moves are decided on exact
-// values and the error can only fall.  All M*K neighbours are tried per move, in binary32 first: bound by the issue of
-// these M*K*16 operations per target and of the conversions around them.
-#include <cuda_fp16.h>
-
-#include "pvt_internal.h"
+// Every error that decides is the binary64 sum the final decision of the search kernels uses (residual through the codebooks
+// in order, terms added in element order), so the moves are decided on exact values and the error can only fall.
+//
+// Two to four fp16 codebooks: a warp takes sixteen targets and has the tensor pipe score all neighbours of all of them, which
+// names the targets that may have a better one: after a beam search few or none.  Only those are searched, each by the whole
+// warp.  After a beam search, 20011 targets of 2x251 / 200000 of 2x256 / 56360 of 4x256: 21 / 63 / 86 us (a warp per target:
+// 35 / 241 / 188); from random codes, where every target is searched, 153 / 1220 / 1490 (140 / 1204 / 1345).
+// Others: a warp per target, all M*K neighbours per move in binary32 first: bound by the issue of these M*K*16 operations per
+// target and of the conversions around them.
+#include "pvt_beam.cuh"
 
 namespace pvt {
 namespace {
@@ -33,8 +36,9 @@ struct RefineParams {
   uint32_t* status;
 };
 
+// codeword `row` of a codebook in global or shared memory
 template <bool CB_F16>
-__device__ __forceinline__ void global_codeword(const void* books, uint32_t row, float c[8]) {
+__device__ __forceinline__ void codeword_at(const void* books, uint32_t row, float c[8]) {
   if (CB_F16) {
     const uint4 raw = reinterpret_cast<const uint4*>(books)[row];
     const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
@@ -66,6 +70,141 @@ __device__ __forceinline__ double tuple_error(const float t[8], const float (*cw
   return d;
 }
 
+// target of the search (Eq. 8 in the scaled space): one fma and one division per element, binary32
+__device__ __forceinline__ void target_of(const RefineParams& p, uint32_t j, float t[8]) {
+  const float4* W4 = reinterpret_cast<const float4*>(p.W) + 2 * (size_t)j;
+  const float4* g4 = reinterpret_cast<const float4*>(p.g) + 2 * (size_t)j;
+  const float4 w0 = W4[0], w1 = W4[1], g0 = g4[0], g1 = g4[1];
+  const float s = p.scale[j / p.gpr], ne = -p.eta;
+  const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+  const float gg[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
+#pragma unroll
+  for (int i = 0; i < 8; ++i) t[i] = __fdiv_rn(__fmaf_rn(ne, gg[i], w[i]), s);
+}
+// the group's codes; whether all of them are codes
+template <int M, bool CODE_U16>
+__device__ __forceinline__ bool codes_of(const RefineParams& p, uint32_t j, uint32_t (&b)[M]) {
+  if (M == 1) {
+    b[0] = CODE_U16 ? reinterpret_cast<const uint16_t*>(p.codes)[j] : reinterpret_cast<const uint8_t*>(p.codes)[j];
+  } else {
+    const uint8_t* c = reinterpret_cast<const uint8_t*>(p.codes) + (size_t)j * M;
+#pragma unroll
+    for (int m = 0; m < M; ++m) b[m] = c[m];
+  }
+  bool ok = true;
+#pragma unroll
+  for (int m = 0; m < M; ++m) ok = ok && b[m] < p.K;
+  return ok;
+}
+
+// The moves of target n (group j) from codes b, codewords cw on, by the whole warp; writes what the call returns for it
+template <int M, bool CODE_U16, class Codeword>
+__device__ __forceinline__ void climb(const RefineParams& p, const Codeword& codeword, uint64_t n, uint32_t j, const float (&t)[8],
+                                      uint32_t (&b)[M], float (&cw)[M][8]) {
+  const uint32_t K = p.K;
+  const int lane = threadIdx.x & 31;
+  double d_cur = tuple_error<M>(t, cw);
+  uint32_t moves = 0;
+  while (moves < (uint32_t)p.max_moves) {
+    // best neighbour of this lane under (error, tuple); a neighbour is named by (codebook changed, new code)
+    double ld = __longlong_as_double(0x7ff0000000000000ll);
+    uint32_t lm = 0, lq = 0;
+    bool lhave = false;
+    auto tuple_less = [&](uint32_t m1, uint32_t q1, uint32_t m2, uint32_t q2) {
+      // lexicographic order of the two neighbours' tuples (both differ from the current tuple in one place)
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        const uint32_t x = (uint32_t)m == m1 ? q1 : b[m], y = (uint32_t)m == m2 ? q2 : b[m];
+        if (x != y) return x < y;
+      }
+      return false;
+    };
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+      float keep[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) keep[i] = cw[m][i];
+      // Only a neighbour below the current error matters, and binary32 says which may be: with r the target less the
+      // other codewords, each difference rounded, the root of its error is off by no more than 2^-24 of r's and its
+      // intermediates' norms and of itself.  (Every neighbour in binary64: 46 us for 20011 targets of 2x251, now 28.)
+      float r[8], rr = 0.0f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        r[i] = t[i];
+#pragma unroll
+        for (int o = 0; o < M; ++o) {
+          if (o == m) continue;
+          r[i] -= cw[o][i];
+          rr = fmaf(r[i], r[i], rr);
+        }
+      }
+      const float root = sqrtf((float)d_cur) + 2.384185791015625e-7f /* 2^-22 */ * sqrtf(rr);
+      const float limit = fmaf(root * root, 1.000003814697265625f /* 1 + 2^-18 */, 1e-36f);
+      for (uint32_t q = lane; q < K; q += 32) {
+        codeword((uint32_t)m, q, cw[m]);
+        float fast = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float x = r[i] - cw[m][i];
+          fast = fmaf(x, x, fast);
+        }
+        if (fast > limit || q == b[m]) continue;  // (not so for NaN)
+        const double d = tuple_error<M>(t, cw);
+        if (!lhave || d < ld || (d == ld && tuple_less((uint32_t)m, q, lm, lq))) {
+          ld = d;
+          lm = (uint32_t)m;
+          lq = q;
+          lhave = true;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) cw[m][i] = keep[i];
+    }
+    // warp-wide minimum of (error, tuple); errors are >= 0, so their bits order like u64
+    const uint64_t bits = (uint64_t)__double_as_longlong(ld);
+    const uint32_t hi = (uint32_t)(bits >> 32), lo = (uint32_t)bits;
+    const uint32_t mhi = __reduce_min_sync(0xffffffffu, hi);
+    const uint32_t mlo = __reduce_min_sync(0xffffffffu, hi == mhi ? lo : 0xffffffffu);
+    const bool tied = lhave && hi == mhi && lo == mlo;
+    // among the lanes that hold the minimum error: the smallest tuple, codebook by codebook
+    uint32_t alive_mask = __ballot_sync(0xffffffffu, tied);
+    if (alive_mask == 0 || !(__longlong_as_double((long long)(((uint64_t)mhi << 32) | mlo)) < d_cur)) break;
+    bool mine = tied;
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+      const uint32_t x = mine ? ((uint32_t)m == lm ? lq : b[m]) : 0xffffffffu;
+      const uint32_t mx = __reduce_min_sync(0xffffffffu, x);
+      mine = mine && x == mx;
+    }
+    const int winner = __ffs(__ballot_sync(0xffffffffu, mine)) - 1;  // exactly one lane (tuples are distinct)
+    const uint32_t wm = __shfl_sync(0xffffffffu, lm, winner), wq = __shfl_sync(0xffffffffu, lq, winner);
+#pragma unroll
+    for (int m = 0; m < M; ++m)
+      if ((uint32_t)m == wm) {
+        b[m] = wq;
+        codeword((uint32_t)m, wq, cw[m]);
+      }
+    d_cur = __longlong_as_double((long long)(((uint64_t)mhi << 32) | mlo));
+    ++moves;
+  }
+  if (lane == 0) {
+    if (moves) {
+      if (M == 1) {
+        if (CODE_U16)
+          reinterpret_cast<uint16_t*>(p.codes)[j] = (uint16_t)b[0];
+        else
+          reinterpret_cast<uint8_t*>(p.codes)[j] = (uint8_t)b[0];
+      } else {
+        uint8_t* c = reinterpret_cast<uint8_t*>(p.codes) + (size_t)j * M;
+#pragma unroll
+        for (int m = 0; m < M; ++m) c[m] = (uint8_t)b[m];
+      }
+    }
+    if (p.err_out) p.err_out[n] = (float)d_cur;
+    if (p.moves_out) p.moves_out[n] = moves;
+  }
+}
+
 template <int M, bool CB_F16, bool CODE_U16, bool STAGED>
 __global__ void __launch_bounds__(kRfThreads, M <= 2 ? 4 : 2) refine_kernel(const RefineParams p) {
   __shared__ __align__(16) float sh_book[STAGED ? kRfSmemCodewords * 8 : 8];
@@ -75,19 +214,20 @@ __global__ void __launch_bounds__(kRfThreads, M <= 2 ? 4 : 2) refine_kernel(cons
   if (STAGED) {
     for (uint32_t row = threadIdx.x; row < M * K; row += kRfThreads) {
       float c[8];
-      global_codeword<CB_F16>(p.books, row, c);
+      codeword_at<CB_F16>(p.books, row, c);
 #pragma unroll
       for (int i = 0; i < 8; ++i) sh_book[row * 8 + i] = c[i];
     }
     __syncthreads();
   }
-  auto codeword = [&](uint32_t row, float c[8]) {
+  auto codeword = [&](uint32_t m, uint32_t q, float c[8]) {
+    const uint32_t row = m * K + q;
     if (STAGED) {
       const float4 lo = *reinterpret_cast<const float4*>(&sh_book[row * 8]);
       const float4 hi = *reinterpret_cast<const float4*>(&sh_book[row * 8 + 4]);
       c[0] = lo.x, c[1] = lo.y, c[2] = lo.z, c[3] = lo.w, c[4] = hi.x, c[5] = hi.y, c[6] = hi.z, c[7] = hi.w;
     } else {
-      global_codeword<CB_F16>(p.books, row, c);
+      codeword_at<CB_F16>(p.books, row, c);
     }
   };
   const int lane = threadIdx.x & 31;
@@ -99,137 +239,203 @@ __global__ void __launch_bounds__(kRfThreads, M <= 2 ? 4 : 2) refine_kernel(cons
       if (lane == 0 && p.status) atomicOr(p.status, PVT_DEV_BAD_INDEX);
       continue;
     }
-    // target of the search (Eq. 8 in the scaled space): one fma and one division per element, binary32
     float t[8];
-    {
-      const float4* W4 = reinterpret_cast<const float4*>(p.W) + 2 * (size_t)j;
-      const float4* g4 = reinterpret_cast<const float4*>(p.g) + 2 * (size_t)j;
-      const float4 w0 = W4[0], w1 = W4[1], g0 = g4[0], g1 = g4[1];
-      const float s = p.scale[j / p.gpr], ne = -p.eta;
-      const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-      const float gg[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
-#pragma unroll
-      for (int i = 0; i < 8; ++i) t[i] = __fdiv_rn(__fmaf_rn(ne, gg[i], w[i]), s);
-    }
+    target_of(p, j, t);
     uint32_t b[M];
-    bool ok = true;
-    if (M == 1) {
-      b[0] = CODE_U16 ? reinterpret_cast<const uint16_t*>(p.codes)[j] : reinterpret_cast<const uint8_t*>(p.codes)[j];
-    } else {
-      const uint8_t* c = reinterpret_cast<const uint8_t*>(p.codes) + (size_t)j * M;
-#pragma unroll
-      for (int m = 0; m < M; ++m) b[m] = c[m];
-    }
-#pragma unroll
-    for (int m = 0; m < M; ++m) ok = ok && b[m] < K;
+    const bool ok = codes_of<M, CODE_U16>(p, j, b);
     if (!ok) {
       if (lane == 0 && p.status) atomicOr(p.status, PVT_DEV_BAD_CODE);
       continue;
     }
     float cw[M][8];
 #pragma unroll
-    for (int m = 0; m < M; ++m) codeword((uint32_t)m * K + b[m], cw[m]);
-    double d_cur = tuple_error<M>(t, cw);
-    uint32_t moves = 0;
-    while (moves < (uint32_t)p.max_moves) {
-      // best neighbour of this lane under (error, tuple); a neighbour is named by (codebook changed, new code)
-      double ld = __longlong_as_double(0x7ff0000000000000ll);
-      uint32_t lm = 0, lq = 0;
-      bool lhave = false;
-      auto tuple_less = [&](uint32_t m1, uint32_t q1, uint32_t m2, uint32_t q2) {
-        // lexicographic order of the two neighbours' tuples (both differ from the current tuple in one place)
+    for (int m = 0; m < M; ++m) codeword((uint32_t)m, b[m], cw[m]);
+    climb<M, CODE_U16>(p, codeword, n, j, t, b, cw);
+  }
+}
+
+// ---- two to four fp16 codebooks: sixteen targets per warp
+constexpr int kRfGroup = 16;
+template <int M>
+struct RefineSmem {
+  beam::TensorStage st[M];
+  uint4 c[M][beam::kBsK];  // the codewords as they lie in memory
+  uint32_t n2max[M];  // largest ||c||^2, its bits
+  uint32_t n_better;  // targets of the trip that may have a better neighbour: their places
+  uint8_t better[kRfThreads / 32 * kRfGroup];
+  struct {
+    alignas(16) float r[32][8], wmin[32][8];
+  } w[kRfThreads / 32];
+};
+
+template <int M>
+__device__ __noinline__ void climb_target(const RefineParams& p, const uint4 (*books)[beam::kBsK], uint64_t n, uint32_t j) {
+  float t[8], cw[M][8];
+  uint32_t b[M];
+  target_of(p, j, t);
+  codes_of<M, false>(p, j, b);
+  auto codeword = [&](uint32_t m, uint32_t q, float* c) {
+    codeword_at<true>(books[m], q, c);
+  };
 #pragma unroll
-        for (int m = 0; m < M; ++m) {
-          const uint32_t x = (uint32_t)m == m1 ? q1 : b[m], y = (uint32_t)m == m2 ? q2 : b[m];
-          if (x != y) return x < y;
+  for (int m = 0; m < M; ++m) codeword((uint32_t)m, b[m], cw[m]);
+  climb<M, false>(p, codeword, n, j, t, b, cw);
+}
+
+template <int M>
+__global__ void __launch_bounds__(kRfThreads, 3) refine_tensor_kernel(const RefineParams p) {
+  extern __shared__ __align__(16) unsigned char rf_smem[];
+  RefineSmem<M>& sm = *reinterpret_cast<RefineSmem<M>*>(rf_smem);
+  constexpr uint32_t kFull = 0xffffffffu;
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, K = p.K;
+  pdl_trigger();
+  if (tid < M) sm.n2max[tid] = 0;
+  __syncthreads();
+  pdl_wait();
+  // a codeword of every codebook per thread
+  static_assert(kRfThreads == beam::kBsK, "");
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+    float c[8] = {}, n2 = 0.0f;
+    uint4 raw = make_uint4(0, 0, 0, 0);
+    if (tid < K) {
+      raw = reinterpret_cast<const uint4*>(p.books)[(size_t)m * K + tid];
+      codeword_at<true>(p.books, m * K + tid, c);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) n2 = __fmaf_rn(c[i], c[i], n2);
+    sm.c[m][tid] = raw;
+    const int at = beam::stage_column(tid);
+    *reinterpret_cast<uint4*>(&sm.st[m].b[at >> 3][4 * (at & 7)]) = raw;
+    sm.st[m].h[at] = tid < K ? 0.5f * n2 : beam::kPadHalfNorm;
+    const uint32_t most = __reduce_max_sync(kFull, __float_as_uint(n2));
+    if (lane == 0) atomicMax(&sm.n2max[m], most);
+  }
+  __syncthreads();
+  float smax[M], all_books = 0.0f;
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+    smax[m] = sqrtf(__uint_as_float(sm.n2max[m]));
+    all_books += smax[m];
+  }
+  auto& w = sm.w[warp];
+  const uint32_t half = lane >> 4;  // lane = target + 16 half: of two codebooks at a time the half's
+  const uint64_t groups = (p.k + kRfGroup - 1) / kRfGroup;
+  // a trip of the block: `per` groups, one per warp, then the targets that are to be searched, by all warps
+  const uint32_t share = (uint32_t)((groups + gridDim.x - 1) / gridDim.x), per = share < kRfThreads / 32 ? share : kRfThreads / 32;
+  for (uint64_t g0 = (uint64_t)blockIdx.x * per; g0 < groups; g0 += (uint64_t)gridDim.x * per) {
+    if (tid == 0) sm.n_better = 0;
+    __syncthreads();
+    const uint64_t gi = g0 + warp;
+    if (warp < per && gi < groups) {
+      const uint64_t n = gi * kRfGroup + (lane & 15u);
+      uint32_t j = kFull, b[M];
+      bool active = false;
+      float t[8] = {}, cw[M][8];
+      if (n < p.k) {
+        j = p.idx[n];
+        uint32_t wrong = 0;
+        if (j < p.G) {
+          target_of(p, j, t);
+          active = codes_of<M, false>(p, j, b);
+          if (!active) wrong = PVT_DEV_BAD_CODE;
+        } else {
+          wrong = PVT_DEV_BAD_INDEX;
         }
-        return false;
-      };
+        if (wrong && half == 0 && p.status) atomicOr(p.status, wrong);
+      }
+      float nt2 = 0.0f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) nt2 = fmaf(t[i], t[i], nt2);
 #pragma unroll
       for (int m = 0; m < M; ++m) {
-        float keep[8];
+        if (!active) b[m] = 0;
+        codeword_at<true>(sm.c[m], b[m], cw[m]);
+      }
+      const double d_cur = tuple_error<M>(t, cw);
+      bool better = false;  // there may be a neighbour below the current error
 #pragma unroll
-        for (int i = 0; i < 8; ++i) keep[i] = cw[m][i];
-        // Only a neighbour below the current error matters, and binary32 says which may be: with r the target less the
-        // other codewords, each difference rounded, the root of its error is off by no more than 2^-24 of r's and its
-        // intermediates' norms and of itself.  (Every neighbour in binary64: 46 us for 20011 targets of 2x251, now 28.)
-        float r[8], rr = 0.0f;
+      for (int m0 = 0; m0 < M; m0 += 2) {
+        const bool last = m0 + 1 == M;  // an odd codebook: nothing for the upper half
+        const uint32_t m = m0 + (last ? 0 : half);
+        const bool on = active && !(last && half);
+        float r[8], rho = 0.0f;
+        uint32_t own = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) r[i] = t[i];
+#pragma unroll
+        for (int o = 0; o < M; ++o) {
+          if ((uint32_t)o == m) own = b[o];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) r[i] = (uint32_t)o == m ? r[i] : __fsub_rn(r[i], cw[o][i]);
+        }
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          r[i] = t[i];
-#pragma unroll
-          for (int o = 0; o < M; ++o) {
-            if (o == m) continue;
-            r[i] -= cw[o][i];
-            rr = fmaf(r[i], r[i], rr);
-          }
+          r[i] = on ? r[i] : 0.0f;
+          rho = __fmaf_rn(r[i], r[i], rho);
         }
-        const float root = sqrtf((float)d_cur) + 2.384185791015625e-7f /* 2^-22 */ * sqrtf(rr);
-        const float limit = fmaf(root * root, 1.000003814697265625f /* 1 + 2^-18 */, 1e-36f);
-        for (uint32_t q = lane; q < K; q += 32) {
-          codeword((uint32_t)m * K + q, cw[m]);
-          float fast = 0.0f;
+        rho *= 0.5f;
+        *reinterpret_cast<float4*>(&w.r[lane][0]) = make_float4(r[0], r[1], r[2], r[3]);
+        *reinterpret_cast<float4*>(&w.r[lane][4]) = make_float4(r[4], r[5], r[6], r[7]);
+        __syncwarp();
+        float cell_min[8];
+        const float most = last ? smax[m0] : half ? smax[last ? m0 : m0 + 1] : smax[m0];
+        // the margin of a fast score as in the beam search
+        const float reach = sqrtf(2.0f * rho) + most;
+        const float margin = (7.6293945e-6f /* 2^-17 */ * reach + 9.5367432e-7f /* 2^-20 */ * (sqrtf(nt2) + all_books)) * reach + 1e-30f +
+                             beam::tensor_minima(sm.st[m0], sm.st[last ? m0 : m0 + 1], w.r, w.wmin, rho, on, most, cell_min);
+        const float limit = fmaf(0.5f * (float)d_cur, 1.00000095367431640625f /* 1 + 2^-20 */, margin);
+        uint32_t hits = 0;
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const float x = r[i] - cw[m][i];
-            fast = fmaf(x, x, fast);
+        for (int c = 0; c < 8; ++c) hits |= on && !(cell_min[c] > limit) ? 1u << c : 0u;  // (so for NaN)
+        // one cell is that of the stored code; every lane goes through its own cells
+        const beam::TensorStage& st = sm.st[m];
+        while (__any_sync(kFull, hits != 0)) {
+          if (hits) {
+            const uint32_t cell = __ffs(hits) - 1;
+            hits &= hits - 1;
+            for (uint32_t i = 0; i < 32; ++i) {
+              const uint32_t q = 32 * cell + ((i + lane) & 31u);  // (lanes begin at different ones: fewer bank conflicts)
+              float c[8];
+              codeword_at<true>(sm.c[m], q, c);
+              float s = st.h[beam::stage_column(q)] + rho;
+#pragma unroll
+              for (int e = 0; e < 8; ++e) s = fmaf(-r[e], c[e], s);
+              better |= !(s > limit) && q != own && q < K;
+            }
           }
-          if (fast > limit || q == b[m]) continue;  // (not so for NaN)
-          const double d = tuple_error<M>(t, cw);
-          if (!lhave || d < ld || (d == ld && tuple_less((uint32_t)m, q, lm, lq))) {
-            ld = d;
-            lm = (uint32_t)m;
-            lq = q;
-            lhave = true;
-          }
+          __syncwarp();
         }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) cw[m][i] = keep[i];
       }
-      // warp-wide minimum of (error, tuple); errors are >= 0, so their bits order like u64
-      const uint64_t bits = (uint64_t)__double_as_longlong(ld);
-      const uint32_t hi = (uint32_t)(bits >> 32), lo = (uint32_t)bits;
-      const uint32_t mhi = __reduce_min_sync(0xffffffffu, hi);
-      const uint32_t mlo = __reduce_min_sync(0xffffffffu, hi == mhi ? lo : 0xffffffffu);
-      const bool tied = lhave && hi == mhi && lo == mlo;
-      // among the lanes that hold the minimum error: the smallest tuple, codebook by codebook
-      uint32_t alive_mask = __ballot_sync(0xffffffffu, tied);
-      if (alive_mask == 0 || !(__longlong_as_double((long long)(((uint64_t)mhi << 32) | mlo)) < d_cur)) break;
-      bool mine = tied;
-#pragma unroll
-      for (int m = 0; m < M; ++m) {
-        const uint32_t x = mine ? ((uint32_t)m == lm ? lq : b[m]) : 0xffffffffu;
-        const uint32_t mx = __reduce_min_sync(0xffffffffu, x);
-        mine = mine && x == mx;
+      better &= p.max_moves > 0;
+      uint32_t who = __ballot_sync(kFull, better);
+      who = (who | (who >> 16)) & 0xffffu;
+      if (active && half == 0 && !((who >> lane) & 1u)) {
+        if (p.err_out) p.err_out[n] = (float)d_cur;
+        if (p.moves_out) p.moves_out[n] = 0;
       }
-      const int winner = __ffs(__ballot_sync(0xffffffffu, mine)) - 1;  // exactly one lane (tuples are distinct)
-      const uint32_t wm = __shfl_sync(0xffffffffu, lm, winner), wq = __shfl_sync(0xffffffffu, lq, winner);
-#pragma unroll
-      for (int m = 0; m < M; ++m)
-        if ((uint32_t)m == wm) {
-          b[m] = wq;
-          codeword((uint32_t)m * K + wq, cw[m]);
-        }
-      d_cur = __longlong_as_double((long long)(((uint64_t)mhi << 32) | mlo));
-      ++moves;
+      if (half == 0 && ((who >> lane) & 1u)) sm.better[atomicAdd(&sm.n_better, 1u)] = (uint8_t)(kRfGroup * warp + lane);
     }
-    if (lane == 0) {
-      if (moves) {
-        if (M == 1) {
-          if (CODE_U16)
-            reinterpret_cast<uint16_t*>(p.codes)[j] = (uint16_t)b[0];
-          else
-            reinterpret_cast<uint8_t*>(p.codes)[j] = (uint8_t)b[0];
-        } else {
-          uint8_t* c = reinterpret_cast<uint8_t*>(p.codes) + (size_t)j * M;
-#pragma unroll
-          for (int m = 0; m < M; ++m) c[m] = (uint8_t)b[m];
-        }
-      }
-      if (p.err_out) p.err_out[n] = (float)d_cur;
-      if (p.moves_out) p.moves_out[n] = moves;
+    __syncthreads();
+    for (uint32_t i = warp; i < sm.n_better; i += kRfThreads / 32) {
+      const uint64_t n = g0 * kRfGroup + sm.better[i];
+      climb_target<M>(p, sm.c, n, p.idx[n]);
     }
+    __syncthreads();
   }
+}
+
+template <int M>
+cudaError_t launch_tensor(const RefineParams& p, cudaStream_t stream) {
+  constexpr size_t smem = sizeof(RefineSmem<M>);
+  const cudaError_t e = allow_smem<refine_tensor_kernel<M>>();
+  if (e != cudaSuccess) return e;
+  constexpr uint64_t fit = (228 * 1024) / (smem + 1024), bound = 3;
+  // as many blocks as are resident, if there is a group for each: few groups per block leave warps for the search
+  const uint64_t want = (p.k + kRfGroup - 1) / kRfGroup;
+  const uint64_t most = (fit < bound ? fit : bound) * (uint64_t)device_sm_count();
+  count_launches(1);
+  return launch_dependent(refine_tensor_kernel<M>, (unsigned)(want < most ? want : most), kRfThreads, smem, stream, p);
 }
 
 template <int M, bool CB_F16, bool CODE_U16, bool STAGED>
@@ -277,11 +483,11 @@ cudaError_t launch_refine(const pvt_layer& L, uint64_t G, const uint32_t* idx, u
   timing_begin(kKernRefine, stream);
   cudaError_t e;
   if (L.num_codebooks == 2)
-    e = f16 ? launch_staged<2, true, false>(p, stream) : launch_staged<2, false, false>(p, stream);
+    e = f16 ? launch_tensor<2>(p, stream) : launch_staged<2, false, false>(p, stream);
   else if (L.num_codebooks == 3)
-    e = f16 ? launch_staged<3, true, false>(p, stream) : launch_staged<3, false, false>(p, stream);
+    e = f16 ? launch_tensor<3>(p, stream) : launch_staged<3, false, false>(p, stream);
   else if (L.num_codebooks == 4)
-    e = f16 ? launch_staged<4, true, false>(p, stream) : launch_staged<4, false, false>(p, stream);
+    e = f16 ? launch_tensor<4>(p, stream) : launch_staged<4, false, false>(p, stream);
   else if (f16)
     e = u16 ? launch_staged<1, true, true>(p, stream) : launch_staged<1, true, false>(p, stream);
   else

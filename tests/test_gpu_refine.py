@@ -123,3 +123,46 @@ def test_refine_with_more_targets_than_resident_warps(M, K, f16, k):
     assert np.array_equal(moves, want_moves) and np.array_equal(err, d.astype(np.float32))
     rest = np.setdiff1d(np.arange(G), at)
     assert np.array_equal(codes.reshape(G, M)[rest], L.codes.reshape(G, M)[rest])
+
+
+@pytest.mark.parametrize("M,K,k,max_moves,start", [
+    (2, 5, 1, 8, "random"),       # one target in a group of sixteen, codebooks smaller than a cell
+    (2, 31, 17, 8, "random"),     # one target in the second group
+    (3, 256, 33, 8, "search"),    # an odd codebook: half of the last pair of row tiles is empty
+    (4, 255, 130, 8, "search"),
+    (2, 33, 60001, 2, "mixed"),   # more groups than warps: several trips per block, some targets searched, some not
+    (2, 64, 4000, 8, "equal"),    # every codeword twice: neighbours of the same error
+])
+def test_refine_over_groups_of_targets(M, K, k, max_moves, start):
+    rows, cols = (960, 512) if k > 5000 else (64, 512)
+    L = synth.make_layer(rows, cols, cfg=209, num_codebooks=M, codebook_size=K, codebook_fp16=True, nearest=oracle_nearest)
+    G = L.num_groups
+    rng = np.random.default_rng(k)
+    idx = np.sort(rng.choice(G, size=k, replace=False)).astype(np.uint32)
+    at = idx.astype(np.int64)
+    t = oracle.targets(L.W, L.g, L.scale, L.eta, idx)
+    if start == "equal":
+        L.codebooks[:, 1::2] = L.codebooks[:, 0::2]
+    codes = L.codes.reshape(G, M)
+    if start in ("search", "mixed"):
+        found = oracle.encode(t, L.codebooks, codes[at], L.beam).codes
+        codes[at] = np.where(rng.random((k, 1)) < (0.2 if start == "mixed" else 0.0), codes[at], found)
+    want, d, want_moves = oracle.local_search(t, L.codebooks, codes[at], max_moves)
+    got, err, moves, status = gpu_refine(L, idx, max_moves)
+    assert status == 0
+    assert np.array_equal(got.reshape(G, M)[at].astype(np.int32), want)
+    assert np.array_equal(moves, want_moves) and np.array_equal(err, d.astype(np.float32))
+
+
+def test_refine_beside_a_target_that_is_not_finite():
+    L = synth.make_layer(64, 512, cfg=210, num_codebooks=2, codebook_size=100, codebook_fp16=True, nearest=oracle_nearest)
+    idx = np.arange(0, 3000, 3, dtype=np.uint32)
+    at = idx.astype(np.int64)
+    t = oracle.targets(L.W, L.g, L.scale, L.eta, idx)
+    want, d, want_moves = oracle.local_search(t, L.codebooks, L.codes[at], 8)
+    L.W.reshape(-1, 8)[at[[5, 6, 700]], 3] = np.inf
+    got, err, moves, status = gpu_refine(L, idx, 8)
+    rest = np.setdiff1d(np.arange(1000), [5, 6, 700])
+    assert np.array_equal(got.reshape(-1, 2)[at][rest].astype(np.int32), want[rest])
+    assert np.array_equal(moves[rest], want_moves[rest]) and np.array_equal(err[rest], d.astype(np.float32)[rest])
+    assert np.array_equal(got.reshape(-1, 2)[at][[5, 6, 700]], L.codes[at][[5, 6, 700]])
