@@ -7,7 +7,7 @@
 //   after stages 1..M-1 the `beam` smallest extensions under (score, tuple) are kept;
 //   the result is the smallest member of the last stage's extensions and the previous tuple.
 //
-// A warp handles four targets at a time; the codebooks live in shared memory; three CTAs (24 warps) share an SM.
+// A warp handles four targets at a time; the codebooks live in shared memory; three or four CTAs (24 or 32 warps) share an SM.
 //   stage 1 (four targets side by side): fast scores ||c1||^2/2 - <t, c1>, on the tensor pipe for fp16 codebooks (mma.sync,
 //            the codewords as rows); a thread keeps the minima of cells of four codewords, 64 per target, and goes on as a
 //            stage in the middle.  Binary32 codebooks: one target after the other, 256 scores on the FP32 pipe, 8 per lane,
@@ -25,10 +25,10 @@
 // the beam, the final argmin) is taken on binary64 distances accumulated in index order (the residual carried through
 // the codebooks in order), so the result is the argmin of (distance, tuple) over the pool exactly as defined.
 // What bounds it: no unit by itself; issue slots and shared memory are busy two thirds of the time, the rest are the
-// dependences of one target's chain (sort, minima over eight lanes, acceptance), which six warps per scheduler do not hide.
-// A step of an 11008 x 4096 layer, k = 56 360, two / three fp16 codebooks of 256: 160.5 / 233.4 us, of which the search is
-// 63 / 139 (four codebooks 230 by itself).  With stage 1 of fp16 codebooks one target after the other on the FP32
-// pipe 169.3 / 236.1; with the binary64 decisions of choose_exact inlined 160.4 / 238.2 (spills).  Before all that, a warp
+// dependences of one target's chain (sort, minima over eight lanes, acceptance), which six to eight warps per scheduler do not hide.
+// A step of an 11008 x 4096 layer, k = 56 360, two / three fp16 codebooks of 256: 153 / 226 us, of which the search is
+// 63 / 140 (four codebooks 230 by itself).  When it was 160.5 / 233.4: with stage 1 of fp16 codebooks one target after the
+// other on the FP32 pipe 169.3 / 236.1; with the binary64 decisions of choose_exact inlined 160.4 / 238.2 (spills).  Before all that, a warp
 // per target, with two passes over all extensions in every stage and every decision in binary64: 415 / 522 us for three /
 // four codebooks by themselves, 992 us for three of binary32.
 #include "pvt_beam.cuh"
@@ -44,7 +44,10 @@ namespace {
 
 constexpr int kBsThreads = 256;
 constexpr int kBsWarps = kBsThreads / 32;
-constexpr int kBsCtasPerSm = 3;  // resident CTAs per SM the kernel is compiled for (registers) and launched as
+// Resident CTAs per SM the kernel is compiled for (registers) and launched as: four for two fp16 codebooks (56360 / 20011
+// targets 63.4 / 27.1 us, with three 64.2 / 29.1; two of binary32 106.9 and 105.4), three otherwise (three / four fp16
+// codebooks 140 / 230 us, with four 144 / 235: spills).
+constexpr int beam_ctas_per_sm(int M, bool tc) { return M == 2 && tc ? 4 : 3; }
 constexpr int kBsGroup = 4;      // targets per warp iteration: 4 targets x 8 kept tuples = 32 lanes
 constexpr int kBsList = 32;      // extensions per target that a middle stage's list holds
 constexpr long long kInfBits = 0x7ff0000000000000ll;
@@ -532,7 +535,7 @@ __device__ __forceinline__ uint64_t team_flags(uint32_t mine, uint32_t my_b) {
 }
 
 template <int M, bool TC>
-__global__ void __launch_bounds__(kBsThreads, kBsCtasPerSm) encode_beam_kernel(const BeamParams p,
+__global__ void __launch_bounds__(kBsThreads, beam_ctas_per_sm(M, TC)) encode_beam_kernel(const BeamParams p,
                                                                                const BeamImage<M, TC>* image) {
   extern __shared__ __align__(16) unsigned char beam_smem[];
   BeamSmem<M, TC>& smem = *reinterpret_cast<BeamSmem<M, TC>*>(beam_smem);
@@ -982,7 +985,7 @@ cudaError_t launch_beam(const BeamParams& p, unsigned char* image_at, int sm_cou
   timing_end(kKernEncodeAux, stream);
   if (err != cudaSuccess) return err;
   constexpr uint64_t fit = (228 * 1024) / (smem + 1024);
-  constexpr uint64_t per_sm = fit < kBsCtasPerSm ? fit : kBsCtasPerSm;  // persistent: the resident CTAs
+  constexpr uint64_t bound = beam_ctas_per_sm(M, TC), per_sm = fit < bound ? fit : bound;  // persistent: the resident CTAs
   const uint64_t groups = (p.k + kBsGroup - 1) / kBsGroup, want = (groups + kBsWarps - 1) / kBsWarps;
   const uint64_t most = per_sm * (uint64_t)sm_count;
   timing_begin(kKernEncodeMain, stream);
