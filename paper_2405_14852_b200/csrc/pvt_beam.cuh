@@ -13,8 +13,8 @@ constexpr int kBsK = 256;  // codebooks are padded to this many codewords
 constexpr float kPadHalfNorm = 3.0e38f;
 constexpr float kInf = __builtin_huge_valf();
 
-// A codebook: B fragments, word [tile][lane] = halves (c[column 8 tile + lane/4][2 (lane%4)], [.. + 1]); codeword k stands at
-// column stage_column(k)
+// A codebook: B fragments, word [tile][lane] = halves (c[column 8 tile + lane/4][2 (lane%4)], [.. + 1]); codeword k stands
+// at column stage_column(k)
 struct TensorStage {
   alignas(16) uint32_t b[kBsK / 8][32];
   alignas(8) float h[kBsK];  // ||c||^2/2 by column

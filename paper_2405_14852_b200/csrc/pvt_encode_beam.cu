@@ -7,7 +7,8 @@
 //   after stages 1..M-1 the `beam` smallest extensions under (score, tuple) are kept;
 //   the result is the smallest member of the last stage's extensions and the previous tuple.
 //
-// A warp handles four targets at a time; the codebooks live in shared memory; three or four CTAs (24 or 32 warps) share an SM.
+// A warp handles four targets at a time; the codebooks live in shared memory; three or four CTAs (24 or 32 warps) share an
+// SM.
 //   stage 1 (four targets side by side): fast scores ||c1||^2/2 - <t, c1>, on the tensor pipe for fp16 codebooks (mma.sync,
 //            the codewords as rows); a thread keeps the minima of cells of four codewords, 64 per target, and goes on as a
 //            stage in the middle.  Binary32 codebooks: one target after the other, 256 scores on the FP32 pipe, 8 per lane,
@@ -25,12 +26,12 @@
 // the beam, the final argmin) is taken on binary64 distances accumulated in index order (the residual carried through
 // the codebooks in order), so the result is the argmin of (distance, tuple) over the pool exactly as defined.
 // What bounds it: no unit by itself; issue slots and shared memory are busy two thirds of the time, the rest are the
-// dependences of one target's chain (sort, minima over eight lanes, acceptance), which six to eight warps per scheduler do not hide.
-// A step of an 11008 x 4096 layer, k = 56 360, two / three fp16 codebooks of 256: 153 / 226 us, of which the search is
-// 63 / 140 (four codebooks 230 by itself).  When it was 160.5 / 233.4: with stage 1 of fp16 codebooks one target after the
-// other on the FP32 pipe 169.3 / 236.1; with the binary64 decisions of choose_exact inlined 160.4 / 238.2 (spills).  Before all that, a warp
-// per target, with two passes over all extensions in every stage and every decision in binary64: 415 / 522 us for three /
-// four codebooks by themselves, 992 us for three of binary32.
+// dependences of one target's chain (sort, minima over eight lanes, acceptance), which six to eight warps per scheduler do
+// not hide.  A step of an 11008 x 4096 layer, k = 56 360, two / three fp16 codebooks of 256: 153 / 226 us, of which the
+// search is 63 / 140 (four codebooks 230 by itself).  When it was 160.5 / 233.4: with stage 1 of fp16 codebooks one target
+// after the other on the FP32 pipe 169.3 / 236.1; with the binary64 decisions of choose_exact inlined 160.4 / 238.2
+// (spills).  Before all that, a warp per target, with two passes over all extensions in every stage and every decision in
+// binary64: 415 / 522 us for three / four codebooks by themselves, 992 us for three of binary32.
 #include "pvt_beam.cuh"
 
 namespace pvt {
@@ -75,7 +76,7 @@ struct BeamParams {
 template <bool TC>
 struct FirstImage;
 template <>
-struct FirstImage<true> {  // tensor pipe: A fragments, [tile][lane] = halves (c[row][2 (lane%4)], [.. + 1]) of rows lane/4, + 8
+struct FirstImage<true> {  // tensor pipe: A fragments, [tile][lane] = halves (c[row][2 (lane%4)], [.. + 1]), rows lane/4, + 8
   uint2 a[kBsK / 16][32];
   float2 h2[kBsK / 16][8];  // ||c||^2/2 of rows g, g + 8
   float h[kBsK];            // the same by codeword
@@ -367,8 +368,8 @@ __device__ __forceinline__ void team_min_exact(double& d, uint32_t& key) {
 // The `keep` smallest of a target's extensions under (binary64 distance, tuple), the one of member `b`: of the n_list listed
 // ones (unsure), or of all (more than the list holds).  Seldom needed: not inlined.
 template <int S>
-__device__ __noinline__ uint32_t choose_exact(const uint2* list, uint32_t n_list, uint32_t b, uint32_t keep, bool unsure, bool all,
-                                              const float* t, const float (*books)[kBsK][8], int codes,
+__device__ __noinline__ uint32_t choose_exact(const uint2* list, uint32_t n_list, uint32_t b, uint32_t keep, bool unsure,
+                                              bool all, const float* t, const float (*books)[kBsK][8], int codes,
                                               const uint32_t* kept, uint32_t before, uint32_t K) {
   constexpr uint32_t kFull = 0xffffffffu;
   uint32_t next = 0;
@@ -487,7 +488,8 @@ __device__ __forceinline__ float kept_limit(const float (&cell_min)[8], uint32_t
 }
 
 // One further stage's fast scores for the lane's residual (target my_q, kept tuple my_b; rho = ||r||^2/2): the minimum
-// of each of eight cells of 32 codewords.  The residuals of all lanes are in w.r.  Returns what the tensor path adds to the margin.
+// of each of eight cells of 32 codewords.  The residuals of all lanes are in w.r.  Returns what the tensor path adds to the
+// margin.
 template <bool TC>
 __device__ __forceinline__ float stage_minima(const StageImage<TC>& st, BeamScratch& w, const float (&r)[8], float rho,
                                               bool active, float smax, float (&sub_min)[8]) {
@@ -624,7 +626,8 @@ __global__ void __launch_bounds__(kBsThreads, beam_ctas_per_sm(M, TC)) encode_be
       }
       // as below: twice the rounding-error bound of a fast score with a factor 2 to spare, and what the halves add
       const float reach = tnorm + s1max;
-      const float margin = (7.6293945e-6f /* 2^-17 */ * reach) * reach + 4.76837158203125e-7f /* 2^-21 */ * inv * s1max + 1e-30f;
+      const float margin =
+          (7.6293945e-6f /* 2^-17 */ * reach) * reach + 4.76837158203125e-7f /* 2^-21 */ * inv * s1max + 1e-30f;
       float limit = kept_limit<4>(cell_min, part, B, margin);
       uint32_t n_list = 0;  // the same in the target's eight lanes
 #pragma unroll 1

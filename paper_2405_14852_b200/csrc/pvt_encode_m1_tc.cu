@@ -17,8 +17,8 @@
 // the best is therefore small, and with it the rounding to fp16, which is relative; and what the rounding of t to one half
 // costs is (2^e t - hi) . (c - t), a small vector times the distance.  So one instruction of fp16 accuracy serves where
 // <t, c> - h needed t in two halves, two instructions and binary32 scores, and few sub-chunks come within the margin.
-// The codebook image is written once per call by a small kernel in exactly the shared-memory byte order, so every
-// 128-codeword step arrives with one 1-D bulk copy (4 KB); the A rows are written by threads of the CTA.
+// The codebook image is written once per call by a small kernel in exactly the shared-memory byte order, so eight steps of
+// 128 codewords arrive with one 1-D bulk copy (32 KB); the A rows are written by threads of the CTA.
 // e_n is chosen per target so that max_i |2^e t_i| lies in [1/2, 1), smaller if the best score would not be a half.
 //
 // CTA = 256 targets (two 128-row A blocks) x a slice of the codebook, one CTA per SM, persistent over (tile, slice) units.
@@ -37,9 +37,13 @@
 // the next unit's targets formed beside the search, units counted without 64-bit divisions: 2367 / 63.6.  (A unit used to
 // begin 7500 cycles after the end of the one before it.)
 // Tried and slower: two issuing warps (2800), the events of a step handled while the next one's columns are on their way
-// (2520: spills), the read-out warps issuing their own MMAs (a bare ring of this kind: 411 cycles for 250), 64-column
-// accumulators (344), mma.sync beside tcgen05 (they share a pipe), four or five codebook stages (no change).  Against
-// binary32 accumulators, two instructions per step and eight read-out warps: 4556.
+// (2520: spills), limits exchanged between the two sets (2450), the read-out warps issuing their own MMAs (a bare ring of
+// this kind: 411 cycles for 250), 64-column accumulators (344), mma.sync beside tcgen05 (they share a pipe), four or five
+// codebook stages (no change).  Against binary32 accumulators, two instructions per step and eight read-out warps: 4556.
+// Where the stored codes exclude nothing (random ones), events make it 2703 / 84.  With the slices of a tile one after the
+// other, each beginning with the best score so far, 20971 / 88473 such targets take 77 / 253 in place of 86 / 302, but a
+// step over the layers of a block whose codes are near 1823 in place of 1802, as the rows of all tiles are then gathered at
+// the same time; slices that run together and exchange their best scores after a few steps 78 / 278, and 1820.
 //
 // Codewords whose half squared norm exceeds the fp16 range get a sentinel row
 // that can never win and are listed as "exceptions": the rescoring kernel always
@@ -97,7 +101,9 @@ constexpr uint32_t kTmemCols = 512;
 constexpr float kMaxHalfNorm = 60000.0f;  // largest ||c||^2/2 the image represents
 constexpr float kNegInf = -__builtin_huge_valf();
 // share of a score that its error may take, doubled: see the kernel
-__host__ __device__ constexpr float rel_margin(int dg) { return 2.0f * 1.01f * (dg == 8 ? 2.0f : 3.0f) * 0.0009765625f /* 2^-10 */; }
+__host__ __device__ constexpr float rel_margin(int dg) {
+  return 2.0f * 1.01f * (dg == 8 ? 2.0f : 3.0f) * 0.0009765625f /* 2^-10 */;
+}
 
 }  // namespace
 
@@ -689,7 +695,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
       constexpr int kRounds = (kTcTile + kTcFormers - 1) / kTcFormers;
       uint32_t j[kRounds];
 #pragma unroll
-      for (int q = 0; q < kRounds; ++q) j[q] = first + q * kTcFormers < kTcTile ? target_index(tile, first + q * kTcFormers) : 0;
+      for (int q = 0; q < kRounds; ++q)
+        j[q] = first + q * kTcFormers < kTcTile ? target_index(tile, first + q * kTcFormers) : 0;
       alive = wait_asleep(smem_u32(&sm.a_free[par]), ((unit_i >> 1) & 1) ^ 1, 500);
       if (!alive) break;
 #pragma unroll 1

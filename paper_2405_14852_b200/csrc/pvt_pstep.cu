@@ -95,10 +95,12 @@ __device__ __forceinline__ void put_products(double* row, uint32_t lane, double 
 
 // The sums start at zero.  (Two fills by the driver instead, and the sums launched behind them the plain way: gradient, both
 // updates and dequantisation of 4096x4096 1x16 72.8 us for 65.3.)
-__global__ void __launch_bounds__(kPsThreads) pstep_clear_kernel(double* books, uint64_t n_books, double* scale, uint64_t n_scale) {
+__global__ void __launch_bounds__(kPsThreads) pstep_clear_kernel(double* books, uint64_t n_books, double* scale,
+                                                                 uint64_t n_scale) {
   pdl_trigger();
   pdl_wait();
-  for (uint64_t i = (uint64_t)blockIdx.x * kPsThreads + threadIdx.x; i < n_books + n_scale; i += (uint64_t)gridDim.x * kPsThreads) {
+  const uint64_t stride = (uint64_t)gridDim.x * kPsThreads;
+  for (uint64_t i = (uint64_t)blockIdx.x * kPsThreads + threadIdx.x; i < n_books + n_scale; i += stride) {
     if (i < n_books)
       books[i] = 0.0;
     else

@@ -6,10 +6,10 @@
 // Every error that decides is the binary64 sum the final decision of the search kernels uses (residual through the codebooks
 // in order, terms added in element order), so the moves are decided on exact values and the error can only fall.
 //
-// Two to four fp16 codebooks: a warp takes sixteen targets and has the tensor pipe score all neighbours of all of them, which
-// names the targets that may have a better one: after a beam search few or none.  Only those are searched, each by the whole
-// warp.  After a beam search, 20011 targets of 2x251 / 200000 of 2x256 / 56360 of 4x256: 21 / 63 / 86 us (a warp per target:
-// 35 / 241 / 188); from random codes, where every target is searched, 153 / 1220 / 1490 (140 / 1204 / 1345).
+// Two to four fp16 codebooks: a warp takes sixteen targets and has the tensor pipe score all neighbours of all of them,
+// which names the targets that may have a better one: after a beam search few or none.  Only those are searched, each by a
+// whole warp.  After a beam search, 20011 targets of 2x251 / 200000 of 2x256 / 56360 of 4x256: 21 / 63 / 86 us (a warp per
+// target: 35 / 241 / 188); from random codes, where every target is searched, 153 / 1220 / 1490 (140 / 1204 / 1345).
 // Others: a warp per target, all M*K neighbours per move in binary32 first: bound by the issue of these M*K*16 operations per
 // target and of the conversions around them.
 #include "pvt_beam.cuh"
@@ -322,7 +322,8 @@ __global__ void __launch_bounds__(kRfThreads, 3) refine_tensor_kernel(const Refi
   const uint32_t half = lane >> 4;  // lane = target + 16 half: of two codebooks at a time the half's
   const uint64_t groups = (p.k + kRfGroup - 1) / kRfGroup;
   // a trip of the block: `per` groups, one per warp, then the targets that are to be searched, by all warps
-  const uint32_t share = (uint32_t)((groups + gridDim.x - 1) / gridDim.x), per = share < kRfThreads / 32 ? share : kRfThreads / 32;
+  const uint32_t share = (uint32_t)((groups + gridDim.x - 1) / gridDim.x);
+  const uint32_t per = share < kRfThreads / 32 ? share : kRfThreads / 32;
   for (uint64_t g0 = (uint64_t)blockIdx.x * per; g0 < groups; g0 += (uint64_t)gridDim.x * per) {
     if (tid == 0) sm.n_better = 0;
     __syncthreads();
@@ -382,8 +383,9 @@ __global__ void __launch_bounds__(kRfThreads, 3) refine_tensor_kernel(const Refi
         const float most = last ? smax[m0] : half ? smax[last ? m0 : m0 + 1] : smax[m0];
         // the margin of a fast score as in the beam search
         const float reach = sqrtf(2.0f * rho) + most;
-        const float margin = (7.6293945e-6f /* 2^-17 */ * reach + 9.5367432e-7f /* 2^-20 */ * (sqrtf(nt2) + all_books)) * reach + 1e-30f +
-                             beam::tensor_minima(sm.st[m0], sm.st[last ? m0 : m0 + 1], w.r, w.wmin, rho, on, most, cell_min);
+        const float margin =
+            (7.6293945e-6f /* 2^-17 */ * reach + 9.5367432e-7f /* 2^-20 */ * (sqrtf(nt2) + all_books)) * reach + 1e-30f +
+            beam::tensor_minima(sm.st[m0], sm.st[last ? m0 : m0 + 1], w.r, w.wmin, rho, on, most, cell_min);
         const float limit = fmaf(0.5f * (float)d_cur, 1.00000095367431640625f /* 1 + 2^-20 */, margin);
         uint32_t hits = 0;
 #pragma unroll

@@ -185,7 +185,8 @@ struct ScatterSmem {
   uint32_t warp_total[kSortWarps];
 };
 template <bool DIRECT>
-__device__ __forceinline__ void sort_scatter(const uint64_t* in, uint64_t* out, const RankParams& p, int pass, ScatterSmem& sm) {
+__device__ __forceinline__ void sort_scatter(const uint64_t* in, uint64_t* out, const RankParams& p, int pass,
+                                             ScatterSmem& sm) {
   auto& seen = sm.seen;
   auto& cnt = sm.cnt;
   auto& warp_total = sm.warp_total;
