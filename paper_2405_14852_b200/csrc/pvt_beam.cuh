@@ -32,10 +32,12 @@ __device__ __forceinline__ void mma_16x8x16(float (&d)[4], const uint32_t (&a)[4
       : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(c0), "f"(c1));
 }
-// The power of two that brings the largest element (of non-negative bit pattern rbits) to [1/2, 1), and its inverse
+// The power of two that brings the largest element (of non-negative bit pattern rbits) to [1/2, 1), and its inverse.  Both
+// are normal numbers, and no finite element leaves the range of a half: those from 2^126 on, for which the power would not
+// be normal, come to [1, 4).
 __device__ __forceinline__ void unit_scale(uint32_t rbits, float& sc, float& inv) {
   int e = 126 - (int)((rbits >> 23) & 0xffu);
-  e = e > 15 ? 15 : (e < -100 ? -100 : e);
+  e = e > 15 ? 15 : (e < -126 ? -126 : e);
   sc = __uint_as_float((uint32_t)(e + 127) << 23);
   inv = __uint_as_float((uint32_t)(127 - e) << 23);
 }

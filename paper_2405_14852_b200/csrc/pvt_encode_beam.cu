@@ -596,12 +596,16 @@ __global__ void __launch_bounds__(kBsThreads, beam_ctas_per_sm(M, TC)) encode_be
       if (n < p.k && !target && part == 0) atomicOr(p.status, PVT_DEV_BAD_INDEX);
       const float* tq = &w.t[q][0];
       float sr[8], tnorm;
+      bool search = target;  // (no codeword is near a target that is not finite)
       {
         const float4 ta = *reinterpret_cast<const float4*>(tq), tb = *reinterpret_cast<const float4*>(tq + 4);
         sr[0] = ta.x, sr[1] = ta.y, sr[2] = ta.z, sr[3] = ta.w, sr[4] = tb.x, sr[5] = tb.y, sr[6] = tb.z, sr[7] = tb.w;
         float nt2 = 0.0f;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) nt2 = fmaf(sr[i], sr[i], nt2);
+        for (int i = 0; i < 8; ++i) {
+          nt2 = fmaf(sr[i], sr[i], nt2);
+          search = search && fabsf(sr[i]) < kInf;
+        }
         tnorm = sqrtf(nt2);
       }
       my_j = lane_j < p.G ? lane_j : kFull;
@@ -628,6 +632,8 @@ __global__ void __launch_bounds__(kBsThreads, beam_ctas_per_sm(M, TC)) encode_be
       const float reach = tnorm + s1max;
       const float margin =
           (7.6293945e-6f /* 2^-17 */ * reach) * reach + 4.76837158203125e-7f /* 2^-21 */ * inv * s1max + 1e-30f;
+      // Scores and margin of a target of large elements (from 2^64 on the margin) may be infinite and the limit then not a
+      // number: what is not above the limit is within it, so that binary64 decides between all codewords.
       float limit = kept_limit<4>(cell_min, part, B, margin);
       uint32_t n_list = 0;  // the same in the target's eight lanes
 #pragma unroll 1
@@ -635,7 +641,7 @@ __global__ void __launch_bounds__(kBsThreads, beam_ctas_per_sm(M, TC)) encode_be
         // the cells within the limit, eight at a time, one per lane, four codewords each
         uint32_t hits = 0;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) hits |= target && cell_min[c] <= limit ? 1u << c : 0u;
+        for (int c = 0; c < 8; ++c) hits |= search && !(cell_min[c] > limit) ? 1u << c : 0u;
         uint32_t at = __popc(hits), total;
         {
           const uint32_t mine = at;
@@ -662,7 +668,7 @@ __global__ void __launch_bounds__(kBsThreads, beam_ctas_per_sm(M, TC)) encode_be
             float s1 = sm.first.h[k1];
 #pragma unroll
             for (int i = 0; i < 8; ++i) s1 = __fmaf_rn(-sr[i], cv[i], s1);
-            const bool in = work && s1 <= limit && k1 < p.K;
+            const bool in = work && !(s1 > limit) && k1 < p.K;
             const uint32_t who = team_bits<4>(__ballot_sync(kFull, in));
             const uint32_t to = n_list + __popc(bits_before<4>(who));
             if (in && to < (uint32_t)kBsList) w.list[q][to] = make_uint2(__float_as_uint(s1), k1 << 24);

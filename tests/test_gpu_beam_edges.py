@@ -74,3 +74,33 @@ def test_clustered_first_codebook(M, copies, jitter):
     base = L.codebooks[0].astype(np.float32)[np.arange(256) // copies]
     L.codebooks[0] = (base + rng.normal(0.0, jitter, size=base.shape)).astype(L.codebooks.dtype)
     check_encode(L, np.arange(L.num_groups, dtype=np.uint32))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M", [2, 3, 4])
+@pytest.mark.parametrize("K,size", [(251, 2.0 ** 60), (251, 2.0 ** 66), (251, 2.0 ** 101), (251, 2.0 ** 117), (251, 2.0 ** 126.5),
+                                    (251, 2.0 ** 127.9), (20, 2.0 ** 117)])
+def test_a_target_of_large_elements_beside_ordinary_ones(M, K, size):
+    """Scores of such a target are not to be told apart in binary32, or not finite; its distances are finite in binary64 and
+    the same for all tuples (the elements of codewords are below half a unit of its own): the lowest tuple.  Half of the
+    large targets have no valid previous tuple, so that nothing stands in for what the search finds."""
+    L = synth.make_layer(16, 256, cfg=350 + M, num_codebooks=M, codebook_size=K, codebook_fp16=True, nearest=oracle_nearest)
+    large = np.arange(1, L.num_groups, 16)  # one of four targets, the others of its group of sixteen as they were
+    rng = np.random.default_rng(M)
+    elements = rng.choice([-1.0, 1.0], (large.size, 8)) * size * rng.uniform(0.5, 1.0, (large.size, 8))
+    L.W.reshape(-1, 8)[large] = elements * L.scale[large // (L.cols // 8), None]
+    idx = np.arange(L.num_groups, dtype=np.uint32)
+    t = oracle.targets(L.W, L.g, L.scale, L.eta, idx)
+    assert np.isfinite(t).all() and np.abs(t).max() > 0.5 * size
+    codes = L.codes.reshape(-1, M)
+    want = oracle.encode(t, L.codebooks, codes, L.beam)
+    assert not want.codes[large].any()
+    codes[large[::2], M - 1] = 255
+    got, _, status = run_encode(L, idx)
+    got = got.reshape(-1, M)
+    assert status == B.PVT_DEV_BAD_CODE  # reported for the places that hold no code
+    assert got.max() < K
+    assert not got[large].any()
+    rest = np.setdiff1d(idx, large)
+    decisive = (want.d_second - want.d_best)[rest] > 1e-6 * want.d_second[rest]
+    assert np.array_equal(got[rest][decisive], want.codes[rest][decisive])
