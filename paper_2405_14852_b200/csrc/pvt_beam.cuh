@@ -32,22 +32,29 @@ __device__ __forceinline__ void mma_16x8x16(float (&d)[4], const uint32_t (&a)[4
       : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(c0), "f"(c1));
 }
-// The power of two that brings the largest element (of non-negative bit pattern rbits) to [1/2, 1), and its inverse.  Both
-// are normal numbers, and no finite element leaves the range of a half: those from 2^126 on, for which the power would not
-// be normal, come to [1, 4).
-__device__ __forceinline__ void unit_scale(uint32_t rbits, float& sc, float& inv) {
-  int e = 126 - (int)((rbits >> 23) & 0xffu);
-  e = e > 15 ? 15 : (e < -126 ? -126 : e);
+// The power of two that brings the largest element (of non-negative bit pattern rbits) to [2^14, 2^15), and its inverse:
+// both are normal numbers for every finite element, and halves of up to 2^-30 of it are not subnormal.  Elements below 2^-15
+// get less (a score of 2^29 times a codeword's squared norm is finite).
+__device__ __forceinline__ void half_scale(uint32_t rbits, float& sc, float& inv) {
+  int e = 140 - (int)((rbits >> 23) & 0xffu);
+  e = e > 29 ? 29 : e;
   sc = __uint_as_float((uint32_t)(e + 127) << 23);
   inv = __uint_as_float((uint32_t)(127 - e) << 23);
 }
-// x, y as the sum of two pairs of halves
+// x, y as the sum of two pairs of halves (22 significant bits)
 __device__ __forceinline__ void split_halves(float x, float y, uint32_t& hi_bits, uint32_t& lo_bits) {
   const __half2 hi = __floats2half2_rn(x, y);
   const float2 back = __half22float2(hi);
   const __half2 lo = __floats2half2_rn(x - back.x, y - back.y);
   hi_bits = *reinterpret_cast<const uint32_t*>(&hi);
   lo_bits = *reinterpret_cast<const uint32_t*>(&lo);
+}
+// the same of three pairs: all bits
+__device__ __forceinline__ void split_three_halves(float x, float y, uint32_t& hi_bits, uint32_t& mid_bits, uint32_t& lo_bits) {
+  const __half2 hi = __floats2half2_rn(x, y);
+  const float2 back = __half22float2(hi);
+  hi_bits = *reinterpret_cast<const uint32_t*>(&hi);
+  split_halves(x - back.x, y - back.y, mid_bits, lo_bits);
 }
 
 // Where codeword k stands among the columns of the tiles: the 32 codewords of a cell are what one thread sees of a
@@ -60,13 +67,15 @@ __device__ __forceinline__ int stage_column(int k) {
 // The fast scores ||r - c||^2/2 of 32 residuals, the lane's in r[lane], those of lanes 0..15 against one codebook, of lanes
 // 16..31 against another (or the same): the lane's minimum of each of eight cells of 32 adjacent codewords (rho =
 // ||r||^2/2 of its residual; infinity where it is not active).  Returns what the halves add to the margin of a score.
+// The margins take a sum of the tensor pipe to be off by no more than 26 u (||r|| + ||c||)^2, u = 2^-24.  How the tensor cores
+// add is not documented, so that this is an assumption; the largest errors against binary64 were 3.5 to 7.1 u of ||c||^2/2 +
+// ||r|| ||c|| over 4 million scores each of vectors as the layers have them, 16 times larger and smaller, and of mixed sizes.
 __device__ __forceinline__ float tensor_minima(const TensorStage& st0, const TensorStage& st1, const float (*wr)[8],
                                                float (*wmin)[8], float rho, bool active, float smax, float (&sub_min)[8]) {
   const uint32_t lane = threadIdx.x & 31;
   // The 32 residuals are the rows of two 16-row A tiles, each row [ -hi(2^e r) | -lo(2^e r) ] in fp16 (hi + lo keeps 22
   // significant bits of r, or all bits above 2^-25 in scaled units); the columns of B are the codewords, [ c | c ]; C
-  // starts at 2^e ||c||^2/2.  e is common to the group: the largest residual element becomes [1/2, 1).  A thread
-  // holds elements 2 qd, 2 qd + 1 of rows g8, g8 + 8 of each tile.
+  // starts at 2^e ||c||^2/2.  e is common to the residuals: the largest element becomes [2^14, 2^15).  A thread holds elements 2 qd, 2 qd + 1 of rows g8, g8 + 8 of each tile.
   const uint32_t g8 = lane >> 2, qd = lane & 3u;
   float2 nr[4];
   float rmax = 0.0f;
@@ -77,7 +86,7 @@ __device__ __forceinline__ float tensor_minima(const TensorStage& st0, const Ten
   }
   const uint32_t rbits = __reduce_max_sync(0xffffffffu, __float_as_uint(rmax));  // non-negative floats order as u32
   float sc, inv;
-  unit_scale(rbits, sc, inv);
+  half_scale(rbits, sc, inv);
   uint32_t a[2][4];
 #pragma unroll
   for (int r4 = 0; r4 < 4; ++r4) split_halves(nr[r4].x * -sc, nr[r4].y * -sc, a[r4 >> 1][r4 & 1], a[r4 >> 1][2 + (r4 & 1)]);

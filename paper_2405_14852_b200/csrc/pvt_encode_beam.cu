@@ -27,11 +27,14 @@
 // the codebooks in order), so the result is the argmin of (distance, tuple) over the pool exactly as defined.
 // What bounds it: no unit by itself; issue slots and shared memory are busy two thirds of the time, the rest are the
 // dependences of one target's chain (sort, minima over eight lanes, acceptance), which six to eight warps per scheduler do
-// not hide.  A step of an 11008 x 4096 layer, k = 56 360, two / three fp16 codebooks of 256: 153 / 226 us, of which the
-// search is 63 / 140 (four codebooks 230 by itself).  When it was 160.5 / 233.4: with stage 1 of fp16 codebooks one target
-// after the other on the FP32 pipe 169.3 / 236.1; with the binary64 decisions of choose_exact inlined 160.4 / 238.2
-// (spills).  Before all that, a warp per target, with two passes over all extensions in every stage and every decision in
-// binary64: 415 / 522 us for three / four codebooks by themselves, 992 us for three of binary32.
+// not hide.  A step of an 11008 x 4096 layer, k = 56 360, two / three fp16 codebooks of 256: 151.5 / 228 us; calls of the
+// search alone, one after the other, 56 / 139 (four codebooks 222).  Stage 1 in two halves on one scale for the four targets,
+// with a margin for residuals, took 155 / 231 and 59 / 139 (231), and where one target in four is 1024 times larger than the
+// others 76 instead of 58, with 2^20 times 1811 instead of 787 (a stage 1 in binary32, one target after the other, 72 and
+// 802).  When a step was 160.5 / 233.4: with stage 1 of fp16 codebooks one target after the other on the FP32 pipe 169.3 /
+// 236.1; with the binary64 decisions of choose_exact inlined 160.4 / 238.2 (spills).  Before all that, a warp per target, with
+// two passes over all extensions in every stage and every decision in binary64: 415 / 522 us for three / four codebooks by
+// themselves, 992 us for three of binary32.
 #include "pvt_beam.cuh"
 
 namespace pvt {
@@ -130,12 +133,18 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
-// the same with the roles exchanged, rows = codewords, columns = targets: both K halves of A are the codeword
-__device__ __forceinline__ void mma_codeword_rows(float (&d)[4], uint2 a, uint32_t b0, uint32_t b1, float c_lo, float c_hi) {
+// the same with the roles exchanged, rows = codewords, columns = targets: both K halves of A are the codeword; C = 0
+__device__ __forceinline__ void mma_codeword_rows(float (&d)[4], uint2 a, uint32_t b0, uint32_t b1) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %4, %5}, {%6, %7}, "
-      "{%8, %8, %9, %9};"
+      "{%8, %8, %8, %8};"
       : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-      : "r"(a.x), "r"(a.y), "r"(b0), "r"(b1), "f"(c_lo), "f"(c_hi));
+      : "r"(a.x), "r"(a.y), "r"(b0), "r"(b1), "f"(0.0f));
+}
+// largest magnitude; not a number if one of them is not
+__device__ __forceinline__ float max_abs3(float a, float b, float c) {
+  float d;
+  asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
 }
 __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
   return (uint64_t)__float_as_uint(lo) | ((uint64_t)__float_as_uint(hi) << 32);
@@ -588,50 +597,63 @@ __global__ void __launch_bounds__(kBsThreads, beam_ctas_per_sm(M, TC)) encode_be
 
     if constexpr (TC) {
       // ---- stage 1 on the tensor pipe, the four targets side by side: lane = target q + 4 part.  The columns of B are the
-      // targets (every other column: a thread then has one target's scores), split in two halves like the residuals below.
+      // targets, split in three halves, which keep every bit: [ -hi | 0 ] in an even column, [ -mid | -lo ] in the next, each
+      // target on a scale of its own.  A thread gets both sums of one target and adds the codeword's half norm.
       const uint32_t q = (uint32_t)lane & 3u, part = (uint32_t)lane >> 2;
       const uint64_t n = gi * kBsGroup + q;
       const uint32_t j = __shfl_sync(kFull, lane_j, 8 * q);
       const bool target = j < p.G;
       if (n < p.k && !target && part == 0) atomicOr(p.status, PVT_DEV_BAD_INDEX);
       const float* tq = &w.t[q][0];
-      float sr[8], tnorm;
-      bool search = target;  // (no codeword is near a target that is not finite)
+      float sr[8], tnorm, top;
       {
         const float4 ta = *reinterpret_cast<const float4*>(tq), tb = *reinterpret_cast<const float4*>(tq + 4);
         sr[0] = ta.x, sr[1] = ta.y, sr[2] = ta.z, sr[3] = ta.w, sr[4] = tb.x, sr[5] = tb.y, sr[6] = tb.z, sr[7] = tb.w;
         float nt2 = 0.0f;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          nt2 = fmaf(sr[i], sr[i], nt2);
-          search = search && fabsf(sr[i]) < kInf;
-        }
+        for (int i = 0; i < 8; ++i) nt2 = fmaf(sr[i], sr[i], nt2);
         tnorm = sqrtf(nt2);
+        top = max_abs3(max_abs3(sr[0], sr[1], sr[2]), max_abs3(sr[3], sr[4], sr[5]), max_abs3(sr[6], sr[7], sr[7]));
       }
+      const bool search = target && top < kInf;  // (no codeword is near a target that is not finite)
       my_j = lane_j < p.G ? lane_j : kFull;
       my_prev = lane_prev;
       my_sall = __shfl_sync(kFull, tnorm, my_q) + sall_books;
       float sc, inv, cell_min[8];
+      half_scale(__float_as_uint(top), sc, inv);
       {
-        float2 x = make_float2(0.0f, 0.0f);
-        if (!(part & 1u)) x = *reinterpret_cast<const float2*>(&w.t[part >> 1][2 * q]);
-        unit_scale(__reduce_max_sync(kFull, __float_as_uint(fmaxf(fabsf(x.x), fabsf(x.y)))), sc, inv);
-        uint32_t b0, b1;
-        split_halves(x.x * -sc, x.y * -sc, b0, b1);
+        const uint32_t column = part >> 1;  // the target of this lane's column
+        const float2 x = *reinterpret_cast<const float2*>(&w.t[column][2 * q]);
+        const float neg = -__shfl_sync(kFull, sc, column);
+        uint32_t hi, mid, lo;
+        split_three_halves(x.x * neg, x.y * neg, hi, mid, lo);
+        const uint32_t b0 = part & 1u ? mid : hi, b1 = part & 1u ? lo : 0u;
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
           float d0[4], d1[4];
           const float2 h0 = sm.first.h2[2 * c][part], h1 = sm.first.h2[2 * c + 1][part];
-          mma_codeword_rows(d0, sm.first.a[2 * c][lane], b0, b1, h0.x * sc, h0.y * sc);
-          mma_codeword_rows(d1, sm.first.a[2 * c + 1][lane], b0, b1, h1.x * sc, h1.y * sc);
-          const float least = min3(fminf(d0[0], d0[2]), d1[0], d1[2]);
-          cell_min[c] = target ? least * inv : kInf;
+          mma_codeword_rows(d0, sm.first.a[2 * c][lane], b0, b1);
+          mma_codeword_rows(d1, sm.first.a[2 * c + 1][lane], b0, b1);
+          const float s0 = __fmaf_rn(d0[0], inv, __fmaf_rn(d0[1], inv, h0.x));
+          const float s1 = __fmaf_rn(d0[2], inv, __fmaf_rn(d0[3], inv, h0.y));
+          const float s2 = __fmaf_rn(d1[0], inv, __fmaf_rn(d1[1], inv, h1.x));
+          const float s3 = __fmaf_rn(d1[2], inv, __fmaf_rn(d1[3], inv, h1.y));
+          cell_min[c] = target ? min3(fminf(s0, s1), s2, s3) : kInf;
         }
       }
-      // as below: twice the rounding-error bound of a fast score with a factor 2 to spare, and what the halves add
+      // Twice the rounding-error bound of a fast score with a factor 2 to spare, as for binary32 below; then what binary64
+      // distances, which decide, are off (2^-53 of at most twelve terms of (||t|| + ||c||)^2; it counts for targets 2^18
+      // times larger than codewords), and what subnormal halves are.  How the tensor cores add is not documented: that these
+      // sums are off by no more than a chain of fused multiply-adds in binary32 (16.1 u (||c||^2/2 + ||t|| ||c||), u = 2^-24)
+      // is an assumption.  What supports it: over 4 million scores each of targets and codewords as the layers have them,
+      // targets 16 times larger and smaller, one of four 1024 times larger, targets next to codewords, elements and codewords
+      // of mixed sizes, the largest errors against binary64 were 2.5 to 5.1 u of that sum of magnitudes (the chain: 3.6 to
+      // 8.3), their root mean squares 0.30 to 0.94 u (0.31 to 1.32), the chain's larger in each.  (Two halves, on one
+      // scale for the four targets: up to 2000 u beside the larger one; 1.7 times the chain's root mean square for targets 16
+      // times larger.)
       const float reach = tnorm + s1max;
-      const float margin =
-          (7.6293945e-6f /* 2^-17 */ * reach) * reach + 4.76837158203125e-7f /* 2^-21 */ * inv * s1max + 1e-30f;
+      const float margin = 3.8146973e-6f /* 2^-18 */ * (0.5f * s1max * s1max + tnorm * s1max) +
+                           (3.5527137e-15f /* 2^-48 */ * reach) * reach + 4.76837158203125e-7f /* 2^-21 */ * inv * s1max + 1e-30f;
       // Scores and margin of a target of large elements (from 2^64 on the margin) may be infinite and the limit then not a
       // number: what is not above the limit is within it, so that binary64 decides between all codewords.
       float limit = kept_limit<4>(cell_min, part, B, margin);

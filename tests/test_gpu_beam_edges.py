@@ -104,3 +104,13 @@ def test_a_target_of_large_elements_beside_ordinary_ones(M, K, size):
     rest = np.setdiff1d(idx, large)
     decisive = (want.d_second - want.d_best)[rest] > 1e-6 * want.d_second[rest]
     assert np.array_equal(got[rest][decisive], want.codes[rest][decisive])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,K", [(2, 256), (3, 251), (4, 64)])
+@pytest.mark.parametrize("f16", [True, False])
+def test_targets_of_very_different_sizes_side_by_side(M, K, f16):
+    """the scores of a target owe nothing to the size of the other three of its group"""
+    L = synth.make_layer(16, 264, cfg=360 + M, num_codebooks=M, codebook_size=K, codebook_fp16=f16, nearest=oracle_nearest)
+    L.W.reshape(-1, 8)[:] *= np.exp2(np.random.default_rng(K).integers(-12, 13, (L.num_groups, 1))).astype(np.float32)
+    check_encode(L, np.arange(L.num_groups, dtype=np.uint32))
