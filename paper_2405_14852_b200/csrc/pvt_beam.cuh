@@ -75,7 +75,8 @@ __device__ __forceinline__ float tensor_minima(const TensorStage& st0, const Ten
   const uint32_t lane = threadIdx.x & 31;
   // The 32 residuals are the rows of two 16-row A tiles, each row [ -hi(2^e r) | -lo(2^e r) ] in fp16 (hi + lo keeps 22
   // significant bits of r, or all bits above 2^-25 in scaled units); the columns of B are the codewords, [ c | c ]; C
-  // starts at 2^e ||c||^2/2.  e is common to the residuals: the largest element becomes [2^14, 2^15).  A thread holds elements 2 qd, 2 qd + 1 of rows g8, g8 + 8 of each tile.
+  // starts at 2^e ||c||^2/2.  e is common to the residuals: the largest element becomes [2^14, 2^15).  A thread holds
+  // elements 2 qd, 2 qd + 1 of rows g8, g8 + 8 of each tile.
   const uint32_t g8 = lane >> 2, qd = lane & 3u;
   float2 nr[4];
   float rmax = 0.0f;

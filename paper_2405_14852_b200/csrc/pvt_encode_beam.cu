@@ -653,7 +653,8 @@ __global__ void __launch_bounds__(kBsThreads, beam_ctas_per_sm(M, TC)) encode_be
       // times larger.)
       const float reach = tnorm + s1max;
       const float margin = 3.8146973e-6f /* 2^-18 */ * (0.5f * s1max * s1max + tnorm * s1max) +
-                           (3.5527137e-15f /* 2^-48 */ * reach) * reach + 4.76837158203125e-7f /* 2^-21 */ * inv * s1max + 1e-30f;
+                           (3.5527137e-15f /* 2^-48 */ * reach) * reach +
+                           4.76837158203125e-7f /* 2^-21 */ * inv * s1max + 1e-30f;
       // Scores and margin of a target of large elements (from 2^64 on the margin) may be infinite and the limit then not a
       // number: what is not above the limit is within it, so that binary64 decides between all codewords.
       float limit = kept_limit<4>(cell_min, part, B, margin);
@@ -732,7 +733,10 @@ __global__ void __launch_bounds__(kBsThreads, beam_ctas_per_sm(M, TC)) encode_be
         const float tnorm = sqrtf(nt2);
         // twice the rounding-error bound of the fast score (factor >= 2 to spare), u = 2^-24:
         //   |score1_fl - score1| <= 16.1 u (||c1||^2/2 + ||t|| ||c1||)
-        const float margin1 = 3.8146973e-6f /* 2^-18 */ * (0.5f * s1max * s1max + tnorm * s1max) + 1e-30f;
+        // and what binary64 distances, which decide, are off
+        const float reach1 = tnorm + s1max;
+        const float margin1 = 3.8146973e-6f /* 2^-18 */ * (0.5f * s1max * s1max + tnorm * s1max) +
+                              (3.5527137e-15f /* 2^-48 */ * reach1) * reach1 + 1e-30f;
 
         // 256 scores, 8 per lane
         float f[8];

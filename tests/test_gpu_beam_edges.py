@@ -78,13 +78,15 @@ def test_clustered_first_codebook(M, copies, jitter):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("M", [2, 3, 4])
-@pytest.mark.parametrize("K,size", [(251, 2.0 ** 60), (251, 2.0 ** 66), (251, 2.0 ** 101), (251, 2.0 ** 117), (251, 2.0 ** 126.5),
-                                    (251, 2.0 ** 127.9), (20, 2.0 ** 117)])
-def test_a_target_of_large_elements_beside_ordinary_ones(M, K, size):
+@pytest.mark.parametrize("K,size,f16", [
+    (251, 2.0 ** 60, True), (251, 2.0 ** 66, True), (251, 2.0 ** 101, True), (251, 2.0 ** 117, True), (251, 2.0 ** 126.5, True),
+    (251, 2.0 ** 127.9, True), (20, 2.0 ** 117, True), (251, 2.0 ** 60, False), (251, 2.0 ** 117, False),
+])
+def test_a_target_of_large_elements_beside_ordinary_ones(M, K, size, f16):
     """Scores of such a target are not to be told apart in binary32, or not finite; its distances are finite in binary64 and
     the same for all tuples (the elements of codewords are below half a unit of its own): the lowest tuple.  Half of the
     large targets have no valid previous tuple, so that nothing stands in for what the search finds."""
-    L = synth.make_layer(16, 256, cfg=350 + M, num_codebooks=M, codebook_size=K, codebook_fp16=True, nearest=oracle_nearest)
+    L = synth.make_layer(16, 256, cfg=350 + M, num_codebooks=M, codebook_size=K, codebook_fp16=f16, nearest=oracle_nearest)
     large = np.arange(1, L.num_groups, 16)  # one of four targets, the others of its group of sixteen as they were
     rng = np.random.default_rng(M)
     elements = rng.choice([-1.0, 1.0], (large.size, 8)) * size * rng.uniform(0.5, 1.0, (large.size, 8))
