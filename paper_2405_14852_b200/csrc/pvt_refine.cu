@@ -6,13 +6,17 @@
 // Every error that decides is the binary64 sum the final decision of the search kernels uses (residual through the codebooks
 // in order, terms added in element order), so the moves are decided on exact values and the error can only fall.
 //
-// Two to four fp16 codebooks: a warp takes sixteen targets and has the tensor pipe score all neighbours of all of them,
-// which names the targets that may have a better one: after a beam search few or none.  Only those are searched, each by a
-// whole warp.  After a beam search, 20011 targets of 2x251 / 200000 of 2x256 / 56360 of 4x256: 21 / 63 / 86 us (a warp per
-// target: 35 / 241 / 188); from random codes, where every target is searched, 153 / 1220 / 1490 (140 / 1204 / 1345).
-// Others: a warp per target, all M*K neighbours per move in binary32 first: bound by the issue of these M*K*16 operations per
-// target and of the conversions around them.
-#include "pvt_beam.cuh"
+// Every neighbour is tried in binary32 first (M*K*16 operations per target), which says what may be below an error.
+// Two to four fp16 codebooks: a warp takes sixteen targets, a lane a target and a codebook, and finds which targets have a
+// neighbour within the limit at all: after a beam search few or none.  Only those are searched, each by a whole warp.  After a
+// beam search, 20011 targets of 2x251 / 200000 of 2x256 / 56360 of 4x256: 23 / 91 / 80 us, bound by the issue of packed
+// arithmetic (a warp per target: 35 / 241 / 188; with the filter on the tensor pipe, targets in two halves: 21 / 63 / 86, but
+// its scores were less exact than binary32 distances).  From random codes, where every target is searched, 130 / 1033 / 1627
+// (a warp per target 138 / 1203 / 1345); the filter ends once every target has a neighbour.
+// Others: a warp per target; bound by the issue of the binary32 operations and of the conversions around them.
+#include <cuda_fp16.h>
+
+#include "pvt_internal.h"
 
 namespace pvt {
 namespace {
@@ -97,15 +101,101 @@ __device__ __forceinline__ bool codes_of(const RefineParams& p, uint32_t j, uint
   return ok;
 }
 
+// Two binary32 values in one register pair (packed arithmetic rounds each as the scalar one does)
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  return (uint64_t)__float_as_uint(lo) | ((uint64_t)__float_as_uint(hi) << 32);
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+
+// Only a neighbour below a known error d matters, and binary32 says which may be: with r the target less the other codewords,
+// each difference rounded, the root of ||r - c||^2 is off by no more than 2^-24 of r's and its intermediates' norms (rr: the
+// sum of their squares) and of itself.  What is not above the limit of d's root may be below d (so for NaN).
+__device__ __forceinline__ float rounding_of(float rr) { return 2.384185791015625e-7f /* 2^-22 */ * sqrtf(rr); }
+__device__ __forceinline__ float limit_of(float root, float off) {
+  root += off;
+  return fmaf(root * root, 1.000003814697265625f /* 1 + 2^-18 */, 1e-36f);
+}
+
+// target less the codewords of all codebooks but m
+template <int M>
+__device__ __forceinline__ void residual_of(const float (&t)[8], const float (&cw)[M][8], uint32_t m, float (&r)[8],
+                                            float& rr) {
+  rr = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    r[i] = t[i];
+#pragma unroll
+    for (int o = 0; o < M; ++o) {
+      if ((uint32_t)o == m) continue;
+      r[i] -= cw[o][i];
+      rr = fmaf(r[i], r[i], rr);
+    }
+  }
+}
+
+// The codebooks as a search goes through them, kWide adjacent codewords per lane and step
+template <bool CB_F16>
+struct Plain {  // one, as it lies in global or shared memory
+  static constexpr int kWide = 1;
+  const void* books;
+  uint32_t K;
+  __device__ __forceinline__ void codeword(uint32_t m, uint32_t q, float c[8]) const {
+    codeword_at<CB_F16>(books, m * K + q, c);
+  }
+  __device__ __forceinline__ void distances(uint32_t m, uint32_t q, const float (&r)[8], float (&fast)[1]) const {
+    float c[8];
+    codeword(m, q, c);
+    fast[0] = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float x = r[i] - c[i];
+      fast[0] = fmaf(x, x, fast[0]);
+    }
+  }
+};
+constexpr int kRfPairs = 128;      // a codebook of up to 256 codewords
+constexpr int kRfPairFloats = 20;  // a pair's 16 values and a gap: eight lanes that read adjacent pairs meet no bank twice
+struct Pairs {  // two, in shared memory as binary32: codewords 2 p and 2 p + 1, element by element
+  static constexpr int kWide = 2;
+  const float (*pair)[kRfPairs][kRfPairFloats];
+  __device__ __forceinline__ void codeword(uint32_t m, uint32_t q, float c[8]) const {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) c[i] = pair[m][q >> 1][2 * i + (q & 1u)];
+  }
+  __device__ __forceinline__ void distances(uint32_t m, uint32_t q, const float (&r)[8], float (&fast)[2]) const {
+    const ulonglong2* at = reinterpret_cast<const ulonglong2*>(&pair[m][q >> 1][0]);
+    uint64_t sum = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const ulonglong2 c = at[i];
+      const uint64_t x = sub2(pack2(r[2 * i], r[2 * i]), c.x), y = sub2(pack2(r[2 * i + 1], r[2 * i + 1]), c.y);
+      sum = fma2(x, x, sum);
+      sum = fma2(y, y, sum);
+    }
+    fast[0] = __uint_as_float((uint32_t)sum);
+    fast[1] = __uint_as_float((uint32_t)(sum >> 32));
+  }
+};
+
 // The moves of target n (group j) from codes b, codewords cw on, by the whole warp; writes what the call returns for it
-template <int M, bool CODE_U16, class Codeword>
-__device__ __forceinline__ void climb(const RefineParams& p, const Codeword& codeword, uint64_t n, uint32_t j, const float (&t)[8],
+template <int M, bool CODE_U16, class Books>
+__device__ __forceinline__ void climb(const RefineParams& p, const Books& books, uint64_t n, uint32_t j, const float (&t)[8],
                                       uint32_t (&b)[M], float (&cw)[M][8]) {
   const uint32_t K = p.K;
   const int lane = threadIdx.x & 31;
   double d_cur = tuple_error<M>(t, cw);
   uint32_t moves = 0;
   while (moves < (uint32_t)p.max_moves) {
+    const float root = sqrtf((float)d_cur);  // no neighbour matters whose distance has a larger one
     // best neighbour of this lane under (error, tuple); a neighbour is named by (codebook changed, new code)
     double ld = __longlong_as_double(0x7ff0000000000000ll);
     uint32_t lm = 0, lq = 0;
@@ -124,37 +214,24 @@ __device__ __forceinline__ void climb(const RefineParams& p, const Codeword& cod
       float keep[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) keep[i] = cw[m][i];
-      // Only a neighbour below the current error matters, and binary32 says which may be: with r the target less the
-      // other codewords, each difference rounded, the root of its error is off by no more than 2^-24 of r's and its
-      // intermediates' norms and of itself.  (Every neighbour in binary64: 46 us for 20011 targets of 2x251, now 28.)
-      float r[8], rr = 0.0f;
+      float r[8], rr;
+      residual_of<M>(t, cw, m, r, rr);
+      const float limit = limit_of(root, rounding_of(rr));
+      for (uint32_t q0 = Books::kWide * lane; q0 < K; q0 += 32 * Books::kWide) {
+        float fast[Books::kWide];
+        books.distances((uint32_t)m, q0, r, fast);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        r[i] = t[i];
-#pragma unroll
-        for (int o = 0; o < M; ++o) {
-          if (o == m) continue;
-          r[i] -= cw[o][i];
-          rr = fmaf(r[i], r[i], rr);
-        }
-      }
-      const float root = sqrtf((float)d_cur) + 2.384185791015625e-7f /* 2^-22 */ * sqrtf(rr);
-      const float limit = fmaf(root * root, 1.000003814697265625f /* 1 + 2^-18 */, 1e-36f);
-      for (uint32_t q = lane; q < K; q += 32) {
-        codeword((uint32_t)m, q, cw[m]);
-        float fast = 0.0f;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float x = r[i] - cw[m][i];
-          fast = fmaf(x, x, fast);
-        }
-        if (fast > limit || q == b[m]) continue;  // (not so for NaN)
-        const double d = tuple_error<M>(t, cw);
-        if (!lhave || d < ld || (d == ld && tuple_less((uint32_t)m, q, lm, lq))) {
-          ld = d;
-          lm = (uint32_t)m;
-          lq = q;
-          lhave = true;
+        for (int w = 0; w < Books::kWide; ++w) {
+          const uint32_t q = q0 + w;
+          if (fast[w] > limit || q == b[m] || q >= K) continue;  // (not so for NaN)
+          books.codeword((uint32_t)m, q, cw[m]);
+          const double d = tuple_error<M>(t, cw);
+          if (!lhave || d < ld || (d == ld && tuple_less((uint32_t)m, q, lm, lq))) {
+            ld = d;
+            lm = (uint32_t)m;
+            lq = q;
+            lhave = true;
+          }
         }
       }
 #pragma unroll
@@ -182,7 +259,7 @@ __device__ __forceinline__ void climb(const RefineParams& p, const Codeword& cod
     for (int m = 0; m < M; ++m)
       if ((uint32_t)m == wm) {
         b[m] = wq;
-        codeword((uint32_t)m, wq, cw[m]);
+        books.codeword((uint32_t)m, wq, cw[m]);
       }
     d_cur = __longlong_as_double((long long)(((uint64_t)mhi << 32) | mlo));
     ++moves;
@@ -220,16 +297,7 @@ __global__ void __launch_bounds__(kRfThreads, M <= 2 ? 4 : 2) refine_kernel(cons
     }
     __syncthreads();
   }
-  auto codeword = [&](uint32_t m, uint32_t q, float c[8]) {
-    const uint32_t row = m * K + q;
-    if (STAGED) {
-      const float4 lo = *reinterpret_cast<const float4*>(&sh_book[row * 8]);
-      const float4 hi = *reinterpret_cast<const float4*>(&sh_book[row * 8 + 4]);
-      c[0] = lo.x, c[1] = lo.y, c[2] = lo.z, c[3] = lo.w, c[4] = hi.x, c[5] = hi.y, c[6] = hi.z, c[7] = hi.w;
-    } else {
-      codeword_at<CB_F16>(p.books, row, c);
-    }
-  };
+  const Plain<!STAGED && CB_F16> books{STAGED ? (const void*)sh_book : p.books, K};
   const int lane = threadIdx.x & 31;
   // persistent blocks: the codebooks are staged once per block, not once per eight targets
   for (uint64_t n = (uint64_t)blockIdx.x * (kRfThreads / 32) + (threadIdx.x >> 5); n < p.k;
@@ -249,8 +317,8 @@ __global__ void __launch_bounds__(kRfThreads, M <= 2 ? 4 : 2) refine_kernel(cons
     }
     float cw[M][8];
 #pragma unroll
-    for (int m = 0; m < M; ++m) codeword((uint32_t)m, b[m], cw[m]);
-    climb<M, CODE_U16>(p, codeword, n, j, t, b, cw);
+    for (int m = 0; m < M; ++m) books.codeword((uint32_t)m, b[m], cw[m]);
+    climb<M, CODE_U16>(p, books, n, j, t, b, cw);
   }
 }
 
@@ -258,80 +326,55 @@ __global__ void __launch_bounds__(kRfThreads, M <= 2 ? 4 : 2) refine_kernel(cons
 constexpr int kRfGroup = 16;
 template <int M>
 struct RefineSmem {
-  beam::TensorStage st[M];
-  uint4 c[M][beam::kBsK];  // the codewords as they lie in memory
-  uint32_t n2max[M];  // largest ||c||^2, its bits
-  uint32_t n_better;  // targets of the trip that may have a better neighbour: their places
+  alignas(16) float pair[M][kRfPairs][kRfPairFloats];
+  uint32_t n_better, next;  // targets of the trip that have a neighbour to be looked at: their places; the next one to search
   uint8_t better[kRfThreads / 32 * kRfGroup];
-  struct {
-    alignas(16) float r[32][8], wmin[32][8];
-  } w[kRfThreads / 32];
 };
 
 template <int M>
-__device__ __noinline__ void climb_target(const RefineParams& p, const uint4 (*books)[beam::kBsK], uint64_t n, uint32_t j) {
+__device__ __forceinline__ void climb_target(const RefineParams& p, const Pairs books, uint64_t n, uint32_t j) {
   float t[8], cw[M][8];
   uint32_t b[M];
   target_of(p, j, t);
   codes_of<M, false>(p, j, b);
-  auto codeword = [&](uint32_t m, uint32_t q, float* c) {
-    codeword_at<true>(books[m], q, c);
-  };
 #pragma unroll
-  for (int m = 0; m < M; ++m) codeword((uint32_t)m, b[m], cw[m]);
-  climb<M, false>(p, codeword, n, j, t, b, cw);
+  for (int m = 0; m < M; ++m) books.codeword((uint32_t)m, b[m], cw[m]);
+  climb<M, false>(p, books, n, j, t, b, cw);
 }
 
 template <int M>
-__global__ void __launch_bounds__(kRfThreads, 3) refine_tensor_kernel(const RefineParams p) {
-  extern __shared__ __align__(16) unsigned char rf_smem[];
-  RefineSmem<M>& sm = *reinterpret_cast<RefineSmem<M>*>(rf_smem);
+__global__ void __launch_bounds__(kRfThreads, 3) refine_group_kernel(const RefineParams p) {
+  __shared__ RefineSmem<M> sm;
   constexpr uint32_t kFull = 0xffffffffu;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, K = p.K;
   pdl_trigger();
-  if (tid < M) sm.n2max[tid] = 0;
-  __syncthreads();
   pdl_wait();
   // a codeword of every codebook per thread
-  static_assert(kRfThreads == beam::kBsK, "");
+  static_assert(kRfThreads == 2 * kRfPairs, "");
 #pragma unroll
   for (int m = 0; m < M; ++m) {
-    float c[8] = {}, n2 = 0.0f;
-    uint4 raw = make_uint4(0, 0, 0, 0);
-    if (tid < K) {
-      raw = reinterpret_cast<const uint4*>(p.books)[(size_t)m * K + tid];
-      codeword_at<true>(p.books, m * K + tid, c);
-    }
+    float c[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) n2 = __fmaf_rn(c[i], c[i], n2);
-    sm.c[m][tid] = raw;
-    const int at = beam::stage_column(tid);
-    *reinterpret_cast<uint4*>(&sm.st[m].b[at >> 3][4 * (at & 7)]) = raw;
-    sm.st[m].h[at] = tid < K ? 0.5f * n2 : beam::kPadHalfNorm;
-    const uint32_t most = __reduce_max_sync(kFull, __float_as_uint(n2));
-    if (lane == 0) atomicMax(&sm.n2max[m], most);
-  }
-  __syncthreads();
-  float smax[M], all_books = 0.0f;
+    for (int i = 0; i < 8; ++i) c[i] = 1.0e30f;  // (beyond the codebook: at no distance that counts)
+    if (tid < K) codeword_at<true>(p.books, m * K + tid, c);
 #pragma unroll
-  for (int m = 0; m < M; ++m) {
-    smax[m] = sqrtf(__uint_as_float(sm.n2max[m]));
-    all_books += smax[m];
+    for (int i = 0; i < 8; ++i) sm.pair[m][tid >> 1][2 * i + (tid & 1u)] = c[i];
   }
-  auto& w = sm.w[warp];
+  const Pairs books{sm.pair};
   const uint32_t half = lane >> 4;  // lane = target + 16 half: of two codebooks at a time the half's
   const uint64_t groups = (p.k + kRfGroup - 1) / kRfGroup;
   // a trip of the block: `per` groups, one per warp, then the targets that are to be searched, by all warps
   const uint32_t share = (uint32_t)((groups + gridDim.x - 1) / gridDim.x);
   const uint32_t per = share < kRfThreads / 32 ? share : kRfThreads / 32;
   for (uint64_t g0 = (uint64_t)blockIdx.x * per; g0 < groups; g0 += (uint64_t)gridDim.x * per) {
-    if (tid == 0) sm.n_better = 0;
+    if (tid == 0) sm.n_better = sm.next = 0;
     __syncthreads();
-    const uint64_t gi = g0 + warp;
+    const uint64_t gi = g0 + warp, n = gi * kRfGroup + (lane & 15u);
+    uint32_t who = 0;  // the group's targets that are to be searched
+    bool active = false;
+    double d_cur = 0.0;
     if (warp < per && gi < groups) {
-      const uint64_t n = gi * kRfGroup + (lane & 15u);
       uint32_t j = kFull, b[M];
-      bool active = false;
       float t[8] = {}, cw[M][8];
       if (n < p.k) {
         j = p.idx[n];
@@ -345,99 +388,73 @@ __global__ void __launch_bounds__(kRfThreads, 3) refine_tensor_kernel(const Refi
         }
         if (wrong && half == 0 && p.status) atomicOr(p.status, wrong);
       }
-      float nt2 = 0.0f;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) nt2 = fmaf(t[i], t[i], nt2);
 #pragma unroll
       for (int m = 0; m < M; ++m) {
         if (!active) b[m] = 0;
-        codeword_at<true>(sm.c[m], b[m], cw[m]);
+        books.codeword((uint32_t)m, b[m], cw[m]);
       }
-      const double d_cur = tuple_error<M>(t, cw);
-      bool better = false;  // there may be a neighbour below the current error
+      d_cur = tuple_error<M>(t, cw);
+      // The search's own test of every neighbour, the operations in the same order: a target of which no code but the stored
+      // ones is within the limit stays as it is.
+      uint32_t done = __ballot_sync(kFull, !active || p.max_moves == 0);  // targets that are decided
 #pragma unroll
       for (int m0 = 0; m0 < M; m0 += 2) {
         const bool last = m0 + 1 == M;  // an odd codebook: nothing for the upper half
         const uint32_t m = m0 + (last ? 0 : half);
-        const bool on = active && !(last && half);
-        float r[8], rho = 0.0f;
+        float r[8], rr;
         uint32_t own = 0;
+        residual_of<M>(t, cw, m, r, rr);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) r[i] = t[i];
+        for (int o = 0; o < M; ++o) own = (uint32_t)o == m ? b[o] : own;
+        const float limit = active && !(last && half) ? limit_of(sqrtf((float)d_cur), rounding_of(rr)) : -1.0f;
+        float fast[2];
+        books.distances(m, own & ~1u, r, fast);
+        // codes within the limit, not counting the stored one
+        int within = (own & 1u ? fast[1] : fast[0]) > limit ? 0 : -1;
+        for (uint32_t q0 = 0; q0 < K && done != kFull; q0 += 16) {
 #pragma unroll
-        for (int o = 0; o < M; ++o) {
-          if ((uint32_t)o == m) own = b[o];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) r[i] = (uint32_t)o == m ? r[i] : __fsub_rn(r[i], cw[o][i]);
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          r[i] = on ? r[i] : 0.0f;
-          rho = __fmaf_rn(r[i], r[i], rho);
-        }
-        rho *= 0.5f;
-        *reinterpret_cast<float4*>(&w.r[lane][0]) = make_float4(r[0], r[1], r[2], r[3]);
-        *reinterpret_cast<float4*>(&w.r[lane][4]) = make_float4(r[4], r[5], r[6], r[7]);
-        __syncwarp();
-        float cell_min[8];
-        const float most = last ? smax[m0] : half ? smax[last ? m0 : m0 + 1] : smax[m0];
-        // the margin of a fast score as in the beam search
-        const float reach = sqrtf(2.0f * rho) + most;
-        const float margin =
-            (7.6293945e-6f /* 2^-17 */ * reach + 9.5367432e-7f /* 2^-20 */ * (sqrtf(nt2) + all_books)) * reach + 1e-30f +
-            beam::tensor_minima(sm.st[m0], sm.st[last ? m0 : m0 + 1], w.r, w.wmin, rho, on, most, cell_min);
-        const float limit = fmaf(0.5f * (float)d_cur, 1.00000095367431640625f /* 1 + 2^-20 */, margin);
-        uint32_t hits = 0;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) hits |= on && !(cell_min[c] > limit) ? 1u << c : 0u;  // (so for NaN)
-        // one cell is that of the stored code; every lane goes through its own cells
-        const beam::TensorStage& st = sm.st[m];
-        while (__any_sync(kFull, hits != 0)) {
-          if (hits) {
-            const uint32_t cell = __ffs(hits) - 1;
-            hits &= hits - 1;
-            for (uint32_t i = 0; i < 32; ++i) {
-              const uint32_t q = 32 * cell + ((i + lane) & 31u);  // (lanes begin at different ones: fewer bank conflicts)
-              float c[8];
-              codeword_at<true>(sm.c[m], q, c);
-              float s = st.h[beam::stage_column(q)] + rho;
-#pragma unroll
-              for (int e = 0; e < 8; ++e) s = fmaf(-r[e], c[e], s);
-              better |= !(s > limit) && q != own && q < K;
-            }
+          for (uint32_t i = 0; i < 16; i += 2) {
+            books.distances(m, q0 + i, r, fast);
+            within += fast[0] > limit ? 0 : 1;
+            within += fast[1] > limit ? 0 : 1;
           }
-          __syncwarp();
+          const uint32_t found = __ballot_sync(kFull, within > 0);
+          who |= found | found >> 16 | found << 16;
+          done |= who;
         }
       }
-      better &= p.max_moves > 0;
-      uint32_t who = __ballot_sync(kFull, better);
-      who = (who | (who >> 16)) & 0xffffu;
-      if (active && half == 0 && !((who >> lane) & 1u)) {
+    }
+    if (active && half == 0) {
+      if ((who >> lane) & 1u) {
+        sm.better[atomicAdd(&sm.n_better, 1u)] = (uint8_t)(kRfGroup * warp + lane);
+      } else {
         if (p.err_out) p.err_out[n] = (float)d_cur;
         if (p.moves_out) p.moves_out[n] = 0;
       }
-      if (half == 0 && ((who >> lane) & 1u)) sm.better[atomicAdd(&sm.n_better, 1u)] = (uint8_t)(kRfGroup * warp + lane);
     }
     __syncthreads();
-    for (uint32_t i = warp; i < sm.n_better; i += kRfThreads / 32) {
+    while (true) {
+      uint32_t i = 0;
+      if (lane == 0) i = atomicAdd(&sm.next, 1u);
+      i = __shfl_sync(kFull, i, 0);
+      if (i >= sm.n_better) break;
       const uint64_t n = g0 * kRfGroup + sm.better[i];
-      climb_target<M>(p, sm.c, n, p.idx[n]);
+      climb_target<M>(p, books, n, p.idx[n]);
     }
     __syncthreads();
   }
 }
 
 template <int M>
-cudaError_t launch_tensor(const RefineParams& p, cudaStream_t stream) {
-  constexpr size_t smem = sizeof(RefineSmem<M>);
-  const cudaError_t e = allow_smem<refine_tensor_kernel<M>>();
+cudaError_t launch_groups(const RefineParams& p, cudaStream_t stream) {
+  constexpr auto kernel = refine_group_kernel<M>;
+  uint64_t most = 0;
+  const cudaError_t e = resident_blocks<kernel>(kRfThreads, device_sm_count(), &most);
   if (e != cudaSuccess) return e;
-  constexpr uint64_t fit = (228 * 1024) / (smem + 1024), bound = 3;
   // as many blocks as are resident, if there is a group for each: few groups per block leave warps for the search
   const uint64_t want = (p.k + kRfGroup - 1) / kRfGroup;
-  const uint64_t most = (fit < bound ? fit : bound) * (uint64_t)device_sm_count();
   count_launches(1);
-  return launch_dependent(refine_tensor_kernel<M>, (unsigned)(want < most ? want : most), kRfThreads, smem, stream, p);
+  return launch_dependent(kernel, (unsigned)(want < most ? want : most), kRfThreads, 0, stream, p);
 }
 
 template <int M, bool CB_F16, bool CODE_U16, bool STAGED>
@@ -485,11 +502,11 @@ cudaError_t launch_refine(const pvt_layer& L, uint64_t G, const uint32_t* idx, u
   timing_begin(kKernRefine, stream);
   cudaError_t e;
   if (L.num_codebooks == 2)
-    e = f16 ? launch_tensor<2>(p, stream) : launch_staged<2, false, false>(p, stream);
+    e = f16 ? launch_groups<2>(p, stream) : launch_staged<2, false, false>(p, stream);
   else if (L.num_codebooks == 3)
-    e = f16 ? launch_tensor<3>(p, stream) : launch_staged<3, false, false>(p, stream);
+    e = f16 ? launch_groups<3>(p, stream) : launch_staged<3, false, false>(p, stream);
   else if (L.num_codebooks == 4)
-    e = f16 ? launch_tensor<4>(p, stream) : launch_staged<4, false, false>(p, stream);
+    e = f16 ? launch_groups<4>(p, stream) : launch_staged<4, false, false>(p, stream);
   else if (f16)
     e = u16 ? launch_staged<1, true, true>(p, stream) : launch_staged<1, true, false>(p, stream);
   else

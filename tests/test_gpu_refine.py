@@ -132,6 +132,9 @@ def test_refine_with_more_targets_than_resident_warps(M, K, f16, k):
     (4, 255, 130, 8, "search"),
     (2, 33, 60001, 2, "mixed"),   # more groups than warps: several trips per block, some targets searched, some not
     (2, 64, 4000, 8, "equal"),    # every codeword twice: neighbours of the same error
+    (2, 2, 40, 8, "random"),      # a pair of codewords per codebook
+    (3, 17, 500, 16, "mixed"),    # one codeword in the second round of sixteen, and one beyond the codebook beside it
+    (4, 16, 500, 16, "mixed"),
 ])
 def test_refine_over_groups_of_targets(M, K, k, max_moves, start):
     rows, cols = (960, 512) if k > 5000 else (64, 512)
@@ -166,3 +169,22 @@ def test_refine_beside_a_target_that_is_not_finite():
     assert np.array_equal(got.reshape(-1, 2)[at][rest].astype(np.int32), want[rest])
     assert np.array_equal(moves[rest], want_moves[rest]) and np.array_equal(err[rest], d.astype(np.float32)[rest])
     assert np.array_equal(got.reshape(-1, 2)[at][[5, 6, 700]], L.codes[at][[5, 6, 700]])
+
+
+@pytest.mark.parametrize("M,K", [(2, 251), (3, 64), (4, 33)])
+@pytest.mark.parametrize("size", [2.0 ** 20, 2.0 ** 60, 2.0 ** 66, 2.0 ** 117])
+def test_refine_beside_targets_of_large_elements(M, K, size):
+    """distances that binary32 cannot tell apart, or that leave its range: binary64 decides between all neighbours"""
+    L = synth.make_layer(64, 512, cfg=211, num_codebooks=M, codebook_size=K, codebook_fp16=True, nearest=oracle_nearest)
+    rng = np.random.default_rng(K)
+    large = np.arange(1, L.num_groups, 16)
+    L.W.reshape(-1, 8)[large] = rng.choice([-1.0, 1.0], (large.size, 8)) * size * L.scale[large // (L.cols // 8), None]
+    idx = np.arange(L.num_groups, dtype=np.uint32)
+    t = oracle.targets(L.W, L.g, L.scale, L.eta, idx)
+    assert np.isfinite(t).all()
+    want, d, want_moves = oracle.local_search(t, L.codebooks, L.codes.reshape(-1, M), 8)
+    got, err, moves, status = gpu_refine(L, idx, 8)
+    assert status == 0
+    assert np.array_equal(got.reshape(-1, M).astype(np.int32), want)
+    with np.errstate(over="ignore"):
+        assert np.array_equal(moves, want_moves) and np.array_equal(err, d.astype(np.float32))
