@@ -11,8 +11,9 @@
 // neighbour within the limit at all: after a beam search few or none.  Only those are searched, each by a whole warp.  After a
 // beam search, 20011 targets of 2x251 / 200000 of 2x256 / 56360 of 4x256: 23 / 91 / 80 us, bound by the issue of packed
 // arithmetic (a warp per target: 35 / 241 / 188; with the filter on the tensor pipe, targets in two halves: 21 / 63 / 86, but
-// its scores were less exact than binary32 distances).  From random codes, where every target is searched, 130 / 1033 / 1627
-// (a warp per target 138 / 1203 / 1345); the filter ends once every target has a neighbour.
+// its scores were less exact than binary32 distances).  From random codes, where every target is searched, 86 / 681 / 638
+// (a warp per target 138 / 1203 / 1345): the filter ends once every target has a neighbour, and the search evaluates in
+// binary64 only what may be as near as the nearest neighbour.  Three blocks per SM: two 87 / 654 / 773, four 101 / 692 / 787.
 // Others: a warp per target; bound by the issue of the binary32 operations and of the conversions around them.
 #include <cuda_fp16.h>
 
@@ -195,7 +196,32 @@ __device__ __forceinline__ void climb(const RefineParams& p, const Books& books,
   double d_cur = tuple_error<M>(t, cw);
   uint32_t moves = 0;
   while (moves < (uint32_t)p.max_moves) {
-    const float root = sqrtf((float)d_cur);  // no neighbour matters whose distance has a larger one
+    float root = sqrtf((float)d_cur);  // no neighbour matters whose distance has a larger one
+    float least[M], off[M];            // of the lane's neighbours by codebook
+    if constexpr (Books::kWide > 1) {
+      // No more is to be evaluated than what may be as near as the nearest neighbour of all: a pass over the codebooks finds
+      // that one's binary32 distance.  (Everything below the current error: from random codes 1033 us for 200000 targets of
+      // 2x256, two thirds of it the conversions to binary64; now 681.)
+      float nearest = __int_as_float(0x7f800000), off_most = 0.0f;
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        float r[8], rr;
+        residual_of<M>(t, cw, m, r, rr);
+        off[m] = rounding_of(rr);
+        least[m] = __int_as_float(0x7f800000);
+        for (uint32_t q0 = Books::kWide * lane; q0 < K; q0 += 32 * Books::kWide) {
+          float fast[Books::kWide];
+          books.distances((uint32_t)m, q0, r, fast);
+#pragma unroll
+          for (int w = 0; w < Books::kWide; ++w) least[m] = q0 + w == b[m] ? least[m] : fminf(least[m], fast[w]);
+        }
+        nearest = fminf(nearest, least[m]);
+        off_most = fmaxf(off_most, off[m]);
+      }
+      if (!__any_sync(0xffffffffu, !(nearest > limit_of(root, off_most)))) break;
+      nearest = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(nearest)));  // non-negative: ordered like u32
+      root = fminf(root, (sqrtf(nearest) + off_most) * 1.0000019073486328125f /* 1 + 2^-19 */);
+    }
     // best neighbour of this lane under (error, tuple); a neighbour is named by (codebook changed, new code)
     double ld = __longlong_as_double(0x7ff0000000000000ll);
     uint32_t lm = 0, lq = 0;
@@ -211,6 +237,7 @@ __device__ __forceinline__ void climb(const RefineParams& p, const Books& books,
     };
 #pragma unroll
     for (int m = 0; m < M; ++m) {
+      if (Books::kWide > 1 && !__any_sync(0xffffffffu, !(least[m] > limit_of(root, off[m])))) continue;
       float keep[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) keep[i] = cw[m][i];
