@@ -11,7 +11,7 @@
 // neighbour within the limit at all: after a beam search few or none.  Only those are searched, each by a whole warp.  After a
 // beam search, 20011 targets of 2x251 / 200000 of 2x256 / 56360 of 4x256: 23 / 91 / 80 us, bound by the issue of packed
 // arithmetic (a warp per target: 35 / 241 / 188; with the filter on the tensor pipe, targets in two halves: 21 / 63 / 86, but
-// its scores were less exact than binary32 distances).  From random codes, where every target is searched, 86 / 681 / 638
+// its scores were less exact than binary32 distances).  From random codes, where every target is searched, 86 / 674 / 640
 // (a warp per target 138 / 1203 / 1345): the filter ends once every target has a neighbour, and the search evaluates in
 // binary64 only what may be as near as the nearest neighbour.  Three blocks per SM: two 87 / 654 / 773, four 101 / 692 / 787.
 // Others: a warp per target; bound by the issue of the binary32 operations and of the conversions around them.
@@ -201,7 +201,7 @@ __device__ __forceinline__ void climb(const RefineParams& p, const Books& books,
     if constexpr (Books::kWide > 1) {
       // No more is to be evaluated than what may be as near as the nearest neighbour of all: a pass over the codebooks finds
       // that one's binary32 distance.  (Everything below the current error: from random codes 1033 us for 200000 targets of
-      // 2x256, two thirds of it the conversions to binary64; now 681.)
+      // 2x256, two thirds of it the conversions to binary64; now 674.)
       float nearest = __int_as_float(0x7f800000), off_most = 0.0f;
 #pragma unroll
       for (int m = 0; m < M; ++m) {
@@ -356,6 +356,7 @@ struct RefineSmem {
   alignas(16) float pair[M][kRfPairs][kRfPairFloats];
   uint32_t n_better, next;  // targets of the trip that have a neighbour to be looked at: their places; the next one to search
   uint8_t better[kRfThreads / 32 * kRfGroup];
+  uint32_t found[kRfThreads / 32];  // those of a group that several warps share
 };
 
 template <int M>
@@ -390,17 +391,21 @@ __global__ void __launch_bounds__(kRfThreads, 3) refine_group_kernel(const Refin
   const Pairs books{sm.pair};
   const uint32_t half = lane >> 4;  // lane = target + 16 half: of two codebooks at a time the half's
   const uint64_t groups = (p.k + kRfGroup - 1) / kRfGroup;
-  // a trip of the block: `per` groups, one per warp, then the targets that are to be searched, by all warps
+  // A trip of the block: `per` groups, each by `parts` warps that share the codewords, then the targets that are to be
+  // searched, by all warps.  (One warp per group: 3000 targets of 2x256 after a beam search 12.5 us, now 10.5.)
   const uint32_t share = (uint32_t)((groups + gridDim.x - 1) / gridDim.x);
   const uint32_t per = share < kRfThreads / 32 ? share : kRfThreads / 32;
+  const uint32_t parts = per > 4 ? 1 : per > 2 ? 2 : per > 1 ? 4 : 8, own_group = warp / parts, part = warp % parts;
+  const uint32_t steps = (K + 15) / 16, q_lo = 16 * (steps * part / parts), q_hi = 16 * (steps * (part + 1) / parts);
   for (uint64_t g0 = (uint64_t)blockIdx.x * per; g0 < groups; g0 += (uint64_t)gridDim.x * per) {
     if (tid == 0) sm.n_better = sm.next = 0;
+    if (tid < kRfThreads / 32) sm.found[tid] = 0;
     __syncthreads();
-    const uint64_t gi = g0 + warp, n = gi * kRfGroup + (lane & 15u);
+    const uint64_t gi = g0 + own_group, n = gi * kRfGroup + (lane & 15u);
     uint32_t who = 0;  // the group's targets that are to be searched
     bool active = false;
     double d_cur = 0.0;
-    if (warp < per && gi < groups) {
+    if (own_group < per && gi < groups) {
       uint32_t j = kFull, b[M];
       float t[8] = {}, cw[M][8];
       if (n < p.k) {
@@ -413,7 +418,7 @@ __global__ void __launch_bounds__(kRfThreads, 3) refine_group_kernel(const Refin
         } else {
           wrong = PVT_DEV_BAD_INDEX;
         }
-        if (wrong && half == 0 && p.status) atomicOr(p.status, wrong);
+        if (wrong && half == 0 && part == 0 && p.status) atomicOr(p.status, wrong);
       }
 #pragma unroll
       for (int m = 0; m < M; ++m) {
@@ -437,8 +442,8 @@ __global__ void __launch_bounds__(kRfThreads, 3) refine_group_kernel(const Refin
         float fast[2];
         books.distances(m, own & ~1u, r, fast);
         // codes within the limit, not counting the stored one
-        int within = (own & 1u ? fast[1] : fast[0]) > limit ? 0 : -1;
-        for (uint32_t q0 = 0; q0 < K && done != kFull; q0 += 16) {
+        int within = own < q_lo || own >= q_hi || (own & 1u ? fast[1] : fast[0]) > limit ? 0 : -1;
+        for (uint32_t q0 = q_lo; q0 < q_hi && done != kFull; q0 += 16) {
 #pragma unroll
           for (uint32_t i = 0; i < 16; i += 2) {
             books.distances(m, q0 + i, r, fast);
@@ -451,9 +456,14 @@ __global__ void __launch_bounds__(kRfThreads, 3) refine_group_kernel(const Refin
         }
       }
     }
-    if (active && half == 0) {
+    if (parts > 1) {
+      if (lane == 0 && who) atomicOr(&sm.found[own_group], who);
+      __syncthreads();
+      who = sm.found[own_group];
+    }
+    if (active && part == 0 && half == 0) {
       if ((who >> lane) & 1u) {
-        sm.better[atomicAdd(&sm.n_better, 1u)] = (uint8_t)(kRfGroup * warp + lane);
+        sm.better[atomicAdd(&sm.n_better, 1u)] = (uint8_t)(kRfGroup * own_group + lane);
       } else {
         if (p.err_out) p.err_out[n] = (float)d_cur;
         if (p.moves_out) p.moves_out[n] = 0;
