@@ -25,16 +25,15 @@
 // Fast scores are binary32.  Every decision they cannot settle within twice their rounding-error bound (membership of
 // the beam, the final argmin) is taken on binary64 distances accumulated in index order (the residual carried through
 // the codebooks in order), so the result is the argmin of (distance, tuple) over the pool exactly as defined.
-// What bounds it: no unit by itself; issue slots and shared memory are busy two thirds of the time, the rest are the
-// dependences of one target's chain (sort, minima over eight lanes, acceptance), which six to eight warps per scheduler do
-// not hide.  A step of an 11008 x 4096 layer, k = 56 360, two / three fp16 codebooks of 256: 151.5 / 228 us; calls of the
-// search alone, one after the other, 56 / 139 (four codebooks 222).  Stage 1 in two halves on one scale for the four targets,
-// with a margin for residuals, took 155 / 231 and 59 / 139 (231), and where one target in four is 1024 times larger than the
-// others 76 instead of 58, with 2^20 times 1811 instead of 787 (a stage 1 in binary32, one target after the other, 72 and
-// 802).  When a step was 160.5 / 233.4: with stage 1 of fp16 codebooks one target after the other on the FP32 pipe 169.3 /
-// 236.1; with the binary64 decisions of choose_exact inlined 160.4 / 238.2 (spills).  Before all that, a warp per target, with
-// two passes over all extensions in every stage and every decision in binary64: 415 / 522 us for three / four codebooks by
-// themselves, 992 us for three of binary32.
+// What bounds it: issue slots and shared memory, busy two thirds of the time, and between them the dependences of one target's
+// chain (sort, minima over eight lanes, acceptance), which six to eight warps per scheduler do not hide.  A step of an
+// 11008 x 4096 layer, k = 56 360, two / three fp16 codebooks of 256: 151 / 227 us, of which the search is 58 / 140 (four
+// codebooks 223 by itself).  Stage 1 in two halves on one scale for the four targets, with a margin for residuals: 155 / 229
+// and 62 / 140 (232); where one target in four is 1024 times larger than the others 76 instead of 58, with 2^20 times 1811
+// instead of 787 (a stage 1 in binary32, one target after the other, 72 and 802).  When a step was 160.5 / 233.4: with stage 1
+// of fp16 codebooks one target after the other on the FP32 pipe 169.3 / 236.1; with the binary64 decisions of choose_exact
+// inlined 160.4 / 238.2 (spills).  Before all that, a warp per target, with two passes over all extensions in every stage and
+// every decision in binary64: 415 / 522 us for three / four codebooks by themselves, 992 us for three of binary32.
 #include <cuda_fp16.h>
 
 #include "pvt_internal.h"
@@ -51,9 +50,9 @@ constexpr int kBsK = 256;  // codebooks are padded to this many codewords
 constexpr float kPadHalfNorm = 3.0e38f;
 constexpr float kInf = __builtin_huge_valf();
 constexpr int kBsWarps = kBsThreads / 32;
-// Resident CTAs per SM the kernel is compiled for (registers) and launched as: four for two fp16 codebooks (56360 / 20011
-// targets 63.4 / 27.1 us, with three 64.2 / 29.1; two of binary32 106.9 and 105.4), three otherwise (three / four fp16
-// codebooks 140 / 230 us, with four 144 / 235: spills).
+// Resident CTAs per SM the kernel is compiled for (registers) and launched as: four for two fp16 codebooks (563609 / 56360 /
+// 32768 targets 469 / 58.1 / 42.1 us, with three 487 / 59.8 / 43.3; 20011, where a warp has one group or two, 31.0 and 29.1;
+// two of binary32 106 and 105), three otherwise (three / four fp16 codebooks 140 / 223 us, with four 142 / 234: spills).
 constexpr int beam_ctas_per_sm(int M, bool tc) { return M == 2 && tc ? 4 : 3; }
 constexpr int kBsGroup = 4;      // targets per warp iteration: 4 targets x 8 kept tuples = 32 lanes
 constexpr int kBsList = 32;      // extensions per target that a middle stage's list holds

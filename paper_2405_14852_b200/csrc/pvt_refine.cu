@@ -501,9 +501,9 @@ cudaError_t launch_resident(const RefineParams& p, cudaStream_t stream) {
   uint64_t most = 0;
   const cudaError_t e = resident_blocks<kernel>(kRfThreads, device_sm_count(), &most);
   if (e != cudaSuccess) return e;
-  // Staged codebooks: the resident blocks and no more, since each further wave stages them again (20011 targets of 2x251
-  // 27.7 us, with twice as many blocks 29.3).  Nothing staged: a second wave evens out the first (56360 targets of
-  // 1x4096 309 us, without it 324).
+  // Staged codebooks: the resident blocks and no more, since each further wave stages them again (20011 targets of 2x251 in
+  // binary32 33.2 us, with twice as many blocks 35.2).  Nothing staged: a second wave evens out the first (56360 targets of
+  // 1x4096 310 us, without it 327).
   if (!STAGED) most *= 2;
   count_launches(1);
   return launch_dependent(kernel, (unsigned)(want < most ? want : most), kRfThreads, 0, stream, p);

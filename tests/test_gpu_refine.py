@@ -37,7 +37,7 @@ def gpu_refine(L, idx_np, max_moves, encode_first=False):
     (2, 200, False, 33, 72, 297),      # every group, ragged sizes
     (1, 256, False, 64, 256, 900),
     (3, 64, True, 64, 256, 600),
-    (4, 256, True, 32, 512, 300),      # codebooks read through L2 (1024 codewords)
+    (4, 256, True, 32, 512, 300),      # the largest codebooks in shared memory
     (4, 16, False, 32, 128, 512),
     (1, 2048, True, 64, 512, 333),     # two-byte codes; codebook read through L2 instead of shared memory
 ])
@@ -105,8 +105,8 @@ def test_refine_rejects_bad_arguments():
 
 
 @pytest.mark.parametrize("M,K,f16,k", [
-    (2, 100, True, 9473),    # staged: more targets than twice the resident warps, one in the last trip
-    (3, 64, False, 5000),    # two resident blocks per SM
+    (2, 100, True, 9473),    # one target in the last group of sixteen
+    (3, 64, False, 5000),    # staged, two resident blocks per SM: more targets than twice the resident warps
     (1, 600, True, 19001),   # nothing staged: more than the doubled grid takes at once
     (4, 200, True, 9500),
 ])
