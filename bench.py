@@ -388,8 +388,8 @@ def search_roofline(engine, pairs_per_step, enc_ms, enc_n, steps, peaks, traffic
              "peak_is": f"{peaks['sm_count']} SMs x 128 FP32 lanes x 2 flop x {peaks['sm_max_mhz_used']:.0f} MHz "
                         f"(derived; no measured FP32 peak)"}
         if engine == "beam":
-            r["note"] = ("issue slots and shared memory about two thirds, a target's dependences between them; all stages on the tensor pipe for "
-                         "fp16 codebooks; "
+            r["note"] = ("issue slots and shared memory about two thirds, a target's dependences between them; all stages "
+                         "on the tensor pipe for fp16 codebooks; "
                          "the search as written needs 16 (K1 + K2) + 2 B K2 flop per group (B.K2 cross terms reuse "
                          "<t, c2>), the 16 flop per pair of the metric count every pair as a full dot product")
     r.update(common)
