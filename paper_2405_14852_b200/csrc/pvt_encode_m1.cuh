@@ -22,11 +22,19 @@ struct WaitTestHook {
 WaitTestHook wait_test_hook();
 void set_wait_test_hook(uint32_t max_spins, uint32_t withhold_copy);
 
+struct StepLists {
+  const uint16_t* steps;     // rows of step numbers
+  const uint32_t* counts;    // steps of each row; null: `most`
+  const uint16_t* rows;      // row of each tile; null: its own
+  uint32_t stride, most;
+};
+
 struct EncM1Params {
   const float* W;
   const float* g;
   const float* scale;
   const uint32_t* idx;
+  const uint32_t* place;  // position in the caller's list of each of them (null: its own)
   uint64_t k, G;
   uint32_t gpr;
   FastDiv gpr_div;  // the same as a divisor
@@ -51,6 +59,12 @@ struct EncM1Params {
   int code_u16;
   float* err_out;
   uint32_t* status;
+  // the search over codewords and targets in spatial order (null elsewhere): the codebook in the order of the image, the
+  // codeword at each of its positions, the steps of a tile
+  const void* sorted_book;
+  const uint32_t* order;
+  StepLists lists;
+  uint32_t record, records;  // the record that a launch writes, of so many per target
   uint32_t max_spins;      // poll limit of every wait on an on-chip barrier
   uint32_t withhold_copy;  // kNoWithhold; otherwise the producer skips its copy of this sequence number (test hook)
 };
@@ -65,21 +79,29 @@ __device__ __forceinline__ float unord(uint32_t o) {
 }
 
 // t = (W - eta g) / s of group j in binary32: one fma, one division per element
-__device__ __forceinline__ void form_target(const EncM1Params& p, uint32_t j, float* t) {
+struct TargetIn {
+  float4 w0, w1, g0, g1;
+  float sc;
+};
+__device__ __forceinline__ TargetIn load_target(const EncM1Params& p, uint32_t j) {
   const float4* W4 = reinterpret_cast<const float4*>(p.W);
   const float4* g4 = reinterpret_cast<const float4*>(p.g);
-  const float4 w0 = W4[2 * (size_t)j], w1 = W4[2 * (size_t)j + 1];
-  const float4 g0 = g4[2 * (size_t)j], g1 = g4[2 * (size_t)j + 1];
-  const float sc = p.scale[fast_div(j, p.gpr_div)];
-  const float neg_eta = -p.eta;
-  t[0] = __fdiv_rn(__fmaf_rn(neg_eta, g0.x, w0.x), sc);
-  t[1] = __fdiv_rn(__fmaf_rn(neg_eta, g0.y, w0.y), sc);
-  t[2] = __fdiv_rn(__fmaf_rn(neg_eta, g0.z, w0.z), sc);
-  t[3] = __fdiv_rn(__fmaf_rn(neg_eta, g0.w, w0.w), sc);
-  t[4] = __fdiv_rn(__fmaf_rn(neg_eta, g1.x, w1.x), sc);
-  t[5] = __fdiv_rn(__fmaf_rn(neg_eta, g1.y, w1.y), sc);
-  t[6] = __fdiv_rn(__fmaf_rn(neg_eta, g1.z, w1.z), sc);
-  t[7] = __fdiv_rn(__fmaf_rn(neg_eta, g1.w, w1.w), sc);
+  return TargetIn{W4[2 * (size_t)j], W4[2 * (size_t)j + 1], g4[2 * (size_t)j], g4[2 * (size_t)j + 1],
+                  p.scale[fast_div(j, p.gpr_div)]};
+}
+__device__ __forceinline__ void form_target(const TargetIn& in, float eta, float* t) {
+  const float neg_eta = -eta;
+  t[0] = __fdiv_rn(__fmaf_rn(neg_eta, in.g0.x, in.w0.x), in.sc);
+  t[1] = __fdiv_rn(__fmaf_rn(neg_eta, in.g0.y, in.w0.y), in.sc);
+  t[2] = __fdiv_rn(__fmaf_rn(neg_eta, in.g0.z, in.w0.z), in.sc);
+  t[3] = __fdiv_rn(__fmaf_rn(neg_eta, in.g0.w, in.w0.w), in.sc);
+  t[4] = __fdiv_rn(__fmaf_rn(neg_eta, in.g1.x, in.w1.x), in.sc);
+  t[5] = __fdiv_rn(__fmaf_rn(neg_eta, in.g1.y, in.w1.y), in.sc);
+  t[6] = __fdiv_rn(__fmaf_rn(neg_eta, in.g1.z, in.w1.z), in.sc);
+  t[7] = __fdiv_rn(__fmaf_rn(neg_eta, in.g1.w, in.w1.w), in.sc);
+}
+__device__ __forceinline__ void form_target(const EncM1Params& p, uint32_t j, float* t) {
+  form_target(load_target(p, j), p.eta, t);
 }
 
 // the same for a group of 16 weights
@@ -138,6 +160,30 @@ __device__ __forceinline__ void load_codeword(const void* book, uint32_t kappa, 
   RawCodeword<CB_F16, DG> raw;
   fetch_codeword<CB_F16, DG>(book, kappa, &raw);
   widen_codeword<CB_F16, DG>(raw, c);
+}
+
+// largest ||c||^2 / 2 that the operand image of the tensor engine represents
+constexpr float kMaxHalfNorm = 60000.0f;
+
+// The power of two that a target of largest element m and squared norm nt2 is scaled by for the tensor engine (zero if it
+// is outside the range served); cnmin: the smallest norm of a codeword.
+struct TargetScale {
+  bool in_range;
+  float scale;
+};
+__device__ __forceinline__ TargetScale target_scale(float m, float nt2, float cnmin) {
+  bool in_range = (m < 256.0f) && (nt2 == nt2);  // also false for Inf / NaN
+  int e = 0;
+  if (in_range && m > 0.0f) {
+    e = -ilogbf(m) - 1;
+    e = e > 15 ? 15 : e;
+  }
+  // the best score, at least -2^e (||t|| + min ||c||)^2 / 2, has to be a half
+  // (and above that of the padding rows, -327520 2^e)
+  const float far = sqrtf(nt2) + cnmin, low = 0.5f * far * far;
+  in_range = in_range && low < 150000.0f;
+  if (in_range && low > 1.0f) e = min(e, 14 - ilogbf(low));
+  return TargetScale{in_range, in_range ? scalbnf(1.0f, e) : 0.0f};
 }
 
 // ---- PTX helpers ---------------------------------------------------------------

@@ -44,6 +44,8 @@
 // other, each beginning with the best score so far, 20971 / 88473 such targets take 77 / 253 in place of 86 / 302, but a
 // step over the layers of a block whose codes are near 1823 in place of 1802, as the rows of all tiles are then gathered at
 // the same time; slices that run together and exchange their best scores after a few steps 78 / 278, and 1820.
+// In spatial order (pvt_encode_m1_sorted.cu: many targets) a unit is a tile and goes over a list of steps in place of a slice:
+// a copy for each step, the list in shared memory with the rows, 29360128 targets 66 -> 32 ms in two launches.
 //
 // Codewords whose half squared norm exceeds the fp16 range get a sentinel row
 // that can never win and are listed as "exceptions": the rescoring kernel always
@@ -55,6 +57,7 @@
 #include <atomic>
 
 #include "pvt_encode_m1.cuh"
+#include "pvt_encode_m1_sorted.cuh"
 
 namespace pvt {
 
@@ -98,7 +101,6 @@ struct TcStats {
   uint2 norms[65536 / kTcPrepCw];     // bit pattern of the largest ||c||^2; 0x7f800000 - that of the smallest (zero: none)
 };
 constexpr uint32_t kTmemCols = 512;
-constexpr float kMaxHalfNorm = 60000.0f;  // largest ||c||^2/2 the image represents
 constexpr float kNegInf = -__builtin_huge_valf();
 // share of a score that its error may take, doubled: see the kernel
 __host__ __device__ constexpr float rel_margin(int dg) {
@@ -134,6 +136,38 @@ bool encode_m1_use_tc(const pvt_layer& L, uint64_t k) {
   return L.codebook_size >= kM1TensorCodebook;
 }
 
+namespace {
+// the scratch of the search in spatial order, from `base` on; returns its size
+size_t sorted_scratch(char* base, void* records, uint32_t K, uint64_t k, uint32_t n_tiles, uint32_t n_steps,
+                      m1::SortedScratch* s) {
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    char* p = base ? base + at : nullptr;
+    at += align_up(bytes, kWsAlign);
+    return p;
+  };
+  m1::SortedScratch out;
+  out.dims = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * m1::kSortedLevels));
+  out.tree = reinterpret_cast<float*>(take(sizeof(float) << m1::kSortedLevels));
+  out.order = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) << m1::kSortedLevels));
+  out.order2 = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) << m1::kSortedLevels));
+  out.book = reinterpret_cast<uint4*>(take(sizeof(uint4) * (size_t)K));
+  out.boxes = reinterpret_cast<float*>(take(sizeof(float) * 16 * m1::kSortedSteps));
+  out.packed = reinterpret_cast<uint4*>(take(32 * (size_t)(m1::kSortedSteps + m1::kSortedSteps / 8)));
+  out.near = reinterpret_cast<uint16_t*>(take(sizeof(uint16_t) * m1::kSortedSteps * m1::kSortedNear));
+  out.cells = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) << m1::kSortedLevels));
+  out.starts = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) << m1::kSortedLevels));
+  out.sidx = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * k));
+  out.place = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * k));
+  out.tile_step = reinterpret_cast<uint16_t*>(take(sizeof(uint16_t) * n_tiles));
+  out.lists = reinterpret_cast<uint16_t*>(take(sizeof(uint16_t) * n_tiles * (size_t)m1::list_stride(n_steps)));
+  out.counts = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * n_tiles));
+  out.keys = reinterpret_cast<uint2*>(records);  // (8 bytes per target, done with before the first record of 32)
+  if (s) *s = out;
+  return at;
+}
+}  // namespace
+
 EncodeM1TcLayout encode_m1_tc_layout(uint32_t K, uint64_t k, int sm_count, int group_dim) {
   EncodeM1TcLayout e;
   e.n_steps = (K + kTcStepCw - 1) / kTcStepCw;
@@ -155,6 +189,8 @@ EncodeM1TcLayout encode_m1_tc_layout(uint32_t K, uint64_t k, int sm_count, int g
   }
   e.n_slices = best_s;
   const uint64_t units = (uint64_t)e.n_tiles * e.n_slices;
+  e.sorted = group_dim == kGroupDim && m1_sorted(K, k);
+  if (e.sorted) e.n_slices = 2;  // two rounds, a record each
   e.n_ctas = (uint32_t)(units < (uint64_t)sm_count ? units : (uint64_t)sm_count);
   e.bimg_off = kWsHeaderBytes;
   e.stats_off = align_up(e.bimg_off + (size_t)e.n_steps * (group_dim == 16 ? TcDim<16>::kStepBytes : kTcStepBytes),
@@ -164,16 +200,22 @@ EncodeM1TcLayout encode_m1_tc_layout(uint32_t K, uint64_t k, int sm_count, int g
   e.margin_off = align_up(e.gbest_off + sizeof(uint32_t) * k, kWsAlign);
   e.rec_off = align_up(e.margin_off + sizeof(float) * k, kWsAlign);
   e.bytes = align_up(e.rec_off + (size_t)e.n_tiles * e.n_slices * kTcTile * sizeof(CandRecord), kWsAlign);
+  if (e.sorted) {
+    e.sorted_off = e.bytes;
+    e.bytes = sorted_scratch(nullptr, nullptr, K, k, e.n_tiles, e.n_steps, nullptr) + e.bytes;
+  }
   return e;
 }
 
 namespace {
 
 // ---- codebook image ------------------------------------------------------------
-template <int DG>
+// SORTED: codewords in the order of `order`, of which a copy is left as well.
+template <int DG, bool SORTED>
 __global__ void __launch_bounds__(kTcPrepCw) tc_prep_kernel(const uint4* book, uint32_t K, uint32_t n_steps,
                                                        unsigned char* bimg, TcStats* stats, uint32_t* exc_list,
-                                                       uint32_t* gbest, uint64_t k) {
+                                                       uint32_t* gbest, uint64_t k, const uint32_t* order,
+                                                       uint4* sorted_book) {
   using D = TcDim<DG>;
   __shared__ uint32_t sh_exc, sh_max, sh_inv;
   if (threadIdx.x == 0) sh_exc = sh_max = sh_inv = 0;
@@ -182,10 +224,11 @@ __global__ void __launch_bounds__(kTcPrepCw) tc_prep_kernel(const uint4* book, u
   __syncthreads();
   for (uint64_t n = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; n < k; n += (uint64_t)gridDim.x * blockDim.x)
     gbest[n] = 0xffffffffu;
-  const uint32_t kappa = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t pos = blockIdx.x * blockDim.x + threadIdx.x;
   uint32_t n2bits = 0, n2inv = 0;
-  if (kappa < n_steps * kTcStepCw) {
-    const bool real = kappa < K;
+  if (pos < n_steps * kTcStepCw) {
+    const bool real = pos < K;
+    const uint32_t kappa = SORTED && real ? order[pos] : pos;
     uint4 raw[D::kPart];
     float n2 = 0.0f, part2[D::kPart];
 #pragma unroll
@@ -194,6 +237,7 @@ __global__ void __launch_bounds__(kTcPrepCw) tc_prep_kernel(const uint4* book, u
       part2[part] = 0.0f;
       if (real) {
         raw[part] = book[(size_t)kappa * D::kPart + part];
+        if (SORTED) sorted_book[(size_t)pos * D::kPart + part] = raw[part];
         const __half2* h = reinterpret_cast<const __half2*>(&raw[part]);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -212,7 +256,7 @@ __global__ void __launch_bounds__(kTcPrepCw) tc_prep_kernel(const uint4* book, u
       n2bits = __float_as_uint(n2);
       n2inv = 0x7f800000u - n2bits;
     }
-    const uint32_t step = kappa / kTcStepCw, r = kappa % kTcStepCw;
+    const uint32_t step = pos / kTcStepCw, r = pos % kTcStepCw;
     unsigned char* row = bimg + (size_t)step * D::kStepBytes + (r >> 3) * D::kBGroupBytes + (r & 7) * 16;
 #pragma unroll
     for (int part = 0; part < D::kPart; ++part) {
@@ -364,7 +408,7 @@ __device__ __forceinline__ uint32_t key_limit(float score) {
 
 // ---- shared memory -----------------------------------------------------------------
 constexpr float kOutOfRange = -1.0f, kAbsent = -2.0f;  // in place of a margin
-template <int DG>
+template <int DG, bool SORTED>
 struct TcSmem {
   alignas(128) unsigned char a[2][2][TcDim<DG>::kABlockBytes];  // of this unit and the next: two A blocks of 128 targets
   alignas(128) unsigned char b[kTcStages][kTcGroupSteps][TcDim<DG>::kStepBytes];
@@ -381,18 +425,23 @@ struct TcSmem {
   float seed[2][kTcTile];     // score of the stored code
   float odd_best[2][kTcTile];  // what the odd set leaves for the even one
   uint32_t odd_cnt[2][kTcTile], odd_evicted[2][kTcTile];
+  // in spatial order: the steps of the units being formed and searched, and those the copying warp is at or will be next
+  alignas(16) uint16_t steps[SORTED ? 4 : 1][SORTED ? kSortedSteps : 1];
+  alignas(16) uint16_t ahead[SORTED ? 2 : 1][SORTED ? kSortedSteps : 1];
+  uint32_t n_steps[4];
   uint32_t tmem_base;
   uint32_t abort_flag;
   uint32_t n2max_bits, n2min_inv, n_exc;  // over all codewords
 };
 
-template <int DG>
+// SORTED: a unit is a tile, and its steps are those of a list (pvt_encode_m1_sorted.cu) in place of a slice of the codebook.
+template <int DG, bool SORTED>
 __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1Params p,
                                                                       const unsigned char* bimg, TcStats* stats) {
   using D = TcDim<DG>;
   constexpr int kStepBytes = D::kStepBytes;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  TcSmem<DG>& sm = *reinterpret_cast<TcSmem<DG>*>(smem_raw);
+  TcSmem<DG, SORTED>& sm = *reinterpret_cast<TcSmem<DG, SORTED>*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   volatile uint32_t* abort_flag = &sm.abort_flag;
 
@@ -431,13 +480,28 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
   const uint32_t units = p.n_tiles * p.n_slices;
   // (in 32 bits: at most 2^24 tiles of one slice, fewer of more; a 64-bit division takes a warp a thousand cycles)
   auto unit_steps = [&](uint32_t u, uint32_t* lo, uint32_t* hi) {
+    if (SORTED) {  // places in the tile's list
+      *lo = 0;
+      *hi = p.lists.counts ? p.lists.counts[u] : p.lists.most;
+      return u;
+    }
     const uint32_t tile = fast_div(u, p.slice_div);
     slice_units(p, u - tile * p.n_slices, lo, hi);
     return tile;
   };
+  auto step_list = [&](uint32_t tile) {
+    return p.lists.steps + (size_t)(p.lists.rows ? p.lists.rows[tile] : tile) * p.lists.stride;
+  };
   auto total_steps = [&] {  // of this CTA
     uint32_t total = 0;
-    if (p.n_slices == 1) {
+    if (SORTED) {  // (called by whole warps)
+      for (uint32_t u = blockIdx.x + lane * gridDim.x; u < units; u += 32 * gridDim.x) {
+        uint32_t lo, hi;
+        unit_steps(u, &lo, &hi);
+        total += hi;
+      }
+      total = __reduce_add_sync(0xffffffffu, total);
+    } else if (p.n_slices == 1) {
       total = ((units - 1 - blockIdx.x) / gridDim.x + 1) * p.n_units;
     } else {
       for (uint32_t u = blockIdx.x; u < units; u += gridDim.x) {
@@ -476,8 +540,28 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
     const uint64_t n = (uint64_t)tile * kTcTile + own;
     return n < p.k ? p.idx[n] : 0xffffffffu;
   };
+  // brings a tile's list to shared memory, `threads` threads of number `first` (16 bytes each; the last ones may be padding)
+  auto bring_list = [&](uint32_t tile, uint16_t* to, uint32_t n, uint32_t first, uint32_t threads) {
+    const uint4* from = reinterpret_cast<const uint4*>(step_list(tile));
+    for (uint32_t i = first; i < (n + 7) / 8; i += threads) reinterpret_cast<uint4*>(to)[i] = from[i];
+  };
+  // What a target is formed from (index j): in spatial order, where it is farther away, asked for ahead of its use.
+  struct RowIn {
+    TargetIn in;
+    uint32_t code;
+    uint32_t best;  // in the second round: of the first
+  };
+  auto load_row = [&](uint32_t j, uint32_t tile, uint32_t own) {
+    RowIn row = {};
+    if (SORTED && j < p.G) {
+      row.code = p.code_u16 ? reinterpret_cast<const uint16_t*>(p.codes)[j] : reinterpret_cast<const uint8_t*>(p.codes)[j];
+      row.in = load_target(p, j);
+      if (p.record > 0) row.best = p.gbest[(uint64_t)tile * kTcTile + own];
+    }
+    return row;
+  };
   // Forms target `own` of a unit: the group's index j -> its A row, margin and seed.
-  auto form_row = [&](uint32_t j, uint32_t own, uint32_t par) {
+  auto form_row = [&](uint32_t j, const RowIn& row, uint32_t own, uint32_t par) {
     const uint32_t rb = own >> 7, r = own & 127u;
     unsigned char* a_row = &sm.a[par][rb][(r >> 3) * D::kAGroupBytes + (r & 7) * 16];
     const float n2max = __uint_as_float(sm.n2max_bits);
@@ -491,15 +575,22 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
     const bool have = j < p.G;  // an index out of range is reported by the rescoring kernel
     if (have) {
       // the distance to the stored code: only what comes near it has to be remembered
-      const uint32_t code = p.code_u16 ? reinterpret_cast<const uint16_t*>(p.codes)[j]
-                                       : reinterpret_cast<const uint8_t*>(p.codes)[j];
-      if (DG == 8)
-        form_target(p, j, t);
-      else
-        form_target16(p, j, t);
+      uint32_t code = row.code;
+      float c[DG];
+      if (SORTED) {
+        RawCodeword<true, DG> stored;
+        fetch_codeword<true, DG>(p.book, code < p.K ? code : 0u, &stored);
+        form_target(row.in, p.eta, t);
+        widen_codeword<true, DG>(stored, c);
+      } else {
+        code = p.code_u16 ? reinterpret_cast<const uint16_t*>(p.codes)[j] : reinterpret_cast<const uint8_t*>(p.codes)[j];
+        if (DG == 8)
+          form_target(p, j, t);
+        else
+          form_target16(p, j, t);
+        if (code < p.K) load_codeword<true, DG>(p.book, code, c);
+      }
       if (code < p.K) {
-        float c[DG];
-        load_codeword<true, DG>(p.book, code, c);
         float d = 0.0f;
 #pragma unroll
         for (int i = 0; i < DG; ++i) d = fmaf(t[i] - c[i], t[i] - c[i], d);
@@ -512,19 +603,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
       m = fmaxf(m, fabsf(t[i]));
       nt2 = fmaf(t[i], t[i], nt2);
     }
-    bool in_range = (m < 256.0f) && (nt2 == nt2);  // also false for Inf / NaN
     const float norm = sqrtf(nt2);
-    int e = 0;
-    if (in_range && m > 0.0f) {
-      e = -ilogbf(m) - 1;
-      e = e > 15 ? 15 : e;
-    }
-    // the best score, at least -2^e (||t|| + min ||c||)^2 / 2, has to be a half
-    // (and above that of the padding rows, -327520 2^e)
-    const float far = norm + cnmin, low = 0.5f * far * far;
-    in_range = in_range && low < 150000.0f;
-    if (in_range && low > 1.0f) e = min(e, 14 - ilogbf(low));
-    const float sc = in_range ? scalbnf(1.0f, e) : 0.0f;
+    const TargetScale ts = target_scale(m, nt2, cnmin);
+    const bool in_range = ts.in_range;
+    const float sc = ts.scale;
     float r2 = 0.0f;  // ||2^e t - hi||^2
     {
       const uint32_t sb = __half_as_ushort(__float2half_rn(sc));
@@ -568,7 +650,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
                                      (norm * cnmax + hmax + nt2) +
                                  4.76837158203125e-7f /* 2^-21 */);
     sm.margin[par][own] = !have ? kAbsent : in_range ? margin : kOutOfRange;
-    sm.seed[par][own] = in_range ? -0.5f * sc * prev * 1.0001f : kNegInf;  // (minus infinity without a stored code)
+    float seed = in_range ? -0.5f * sc * prev * 1.0001f : kNegInf;  // (minus infinity without a stored code)
+    // the second round goes on from what the first one found
+    if (SORTED && have && in_range && p.record > 0) seed = fmaxf(seed, -unord(row.best));
+    sm.seed[par][own] = seed;
   };
 
   if (warp == kTcCopyWarp) {
@@ -579,9 +664,25 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
       const uint32_t total = total_steps();
       uint32_t it = 0;
       bool alive = true;
-      for (uint32_t u = blockIdx.x; u < units && alive; u += gridDim.x) {
-        uint32_t s_lo, s_hi;
-        unit_steps(u, &s_lo, &s_hi);
+      // in spatial order: steps of the next unit, whose list is brought near while this one's is gone through
+      uint32_t next_n = 0, place = 0;
+      if (SORTED && blockIdx.x < units) {
+        uint32_t lo;
+        unit_steps(blockIdx.x, &lo, &next_n);
+        bring_list(blockIdx.x, sm.ahead[0], next_n, lane, 32);
+      }
+      for (uint32_t u = blockIdx.x; u < units && alive; u += gridDim.x, place ^= 1) {
+        uint32_t s_lo = 0, s_hi = next_n;
+        if (!SORTED) {
+          unit_steps(u, &s_lo, &s_hi);
+        } else {
+          __syncwarp();  // (all lanes are done with the list before)
+          if (u + gridDim.x < units) {
+            uint32_t lo;
+            unit_steps(u + gridDim.x, &lo, &next_n);
+            bring_list(u + gridDim.x, sm.ahead[place ^ 1], next_n, lane, 32);
+          }
+        }
         for (uint32_t st = s_lo; st < s_hi && alive;) {
           const uint32_t grp = it / kTcGroupSteps, sub = it % kTcGroupSteps, s = grp % kTcStages;
           const uint32_t fb = smem_u32(&sm.full_bar[s]);
@@ -600,7 +701,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
           const uint32_t room = kTcGroupSteps - sub, n = s_hi - st < room ? s_hi - st : room;
           // test hook: a step that is never copied leaves its stage's barrier incomplete, so the MMA warps' wait
           // for that stage runs out
-          if (lane == 0 && p.withhold_copy - it >= n)
+          if (SORTED) {  // the steps of a list: a copy each
+            if ((uint32_t)lane < n && p.withhold_copy != it + lane)
+              bulk_g2s(smem_u32(&sm.b[s][sub + lane][0]), bimg + (size_t)sm.ahead[place][st + lane] * kStepBytes, kStepBytes, fb);
+          } else if (lane == 0 && p.withhold_copy - it >= n)
             bulk_g2s(smem_u32(&sm.b[s][sub][0]), bimg + (size_t)st * kStepBytes, n * kStepBytes, fb);
           st += n;
           it += n;
@@ -649,12 +753,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
           const uint32_t it = base + 2 * j + buf;
           if (it < total && alive) {
             while (it >= unit_end && alive) {  // the next unit begins: its A rows must be in place
-              uint32_t s_lo, s_hi;
-              unit_steps(u, &s_lo, &s_hi);
-              unit_end += s_hi - s_lo;
-              u += gridDim.x;
+              if (!SORTED) {
+                uint32_t s_lo, s_hi;
+                unit_steps(u, &s_lo, &s_hi);
+                unit_end += s_hi - s_lo;
+                u += gridDim.x;
+              }
               if (unit_i > 0) umma_commit(smem_u32(&sm.a_free[(unit_i - 1) & 1]));  // the unit before is behind this warp
               alive = wait_all(smem_u32(&sm.a_ready[unit_i & 1]), (unit_i >> 1) & 1);
+              if (SORTED && alive) unit_end += *reinterpret_cast<volatile uint32_t*>(&sm.n_steps[unit_i & 3]);
 #pragma unroll
               for (int m = 0; m < D::kMmas; ++m) a_desc[m] = (unit_i & 1) ? a_desc[m] + kAUnit : a_desc[m] - kAUnit;
               ++unit_i;
@@ -696,14 +803,24 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
       uint32_t j[kRounds];
 #pragma unroll
       for (int q = 0; q < kRounds; ++q)
-        j[q] = first + q * kTcFormers < kTcTile ? target_index(tile, first + q * kTcFormers) : 0;
+        j[q] = first + q * kTcFormers < kTcTile ? target_index(tile, first + q * kTcFormers) : 0xffffffffu;
+      RowIn row = load_row(j[0], tile, first);
+      uint32_t lo, n = 0;
+      if (SORTED) unit_steps(u, &lo, &n);
       alive = wait_asleep(smem_u32(&sm.a_free[par]), ((unit_i >> 1) & 1) ^ 1, 500);
       if (!alive) break;
+      if (SORTED) {  // (four places: whoever still reads the list of three units ago has not let this unit's rows be formed)
+        bring_list(u, sm.steps[unit_i & 3], n, first, kTcFormers);
+        if (first == 0) sm.n_steps[unit_i & 3] = n;
+      }
 #pragma unroll 1
       for (int q = 0; q < kRounds; ++q) {
-        if (first + q * kTcFormers < kTcTile) form_row(j[0], first + q * kTcFormers, par);
+        const uint32_t mine = j[0];
 #pragma unroll
         for (int i = 0; i + 1 < kRounds; ++i) j[i] = j[i + 1];
+        const RowIn next = load_row(q + 1 < kRounds ? j[0] : 0xffffffffu, tile, first + (q + 1) * kTcFormers);
+        if (first + q * kTcFormers < kTcTile) form_row(mine, row, first + q * kTcFormers, par);
+        row = next;
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> visible to the MMA
       mbar_arrive(smem_u32(&sm.a_ready[par]));
@@ -731,7 +848,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
       }
       asm volatile("bar.sync 9, %0;" ::"n"(kTcTile) : "memory");
       if (blockIdx.x == 0 && own == 0) stats->any_exc = sm.n_exc;
-      form_row(j, own, 0);
+      form_row(j, load_row(j, fast_div(blockIdx.x, p.slice_div), own), own, 0);
+      if (SORTED) {
+        uint32_t lo, n;
+        unit_steps(blockIdx.x, &lo, &n);
+        bring_list(blockIdx.x, sm.steps[0], n, own, kTcTile);
+        if (own == 0) sm.n_steps[0] = n;
+      }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> visible to the MMA
       mbar_arrive(smem_u32(&sm.a_first));
     }
@@ -741,11 +864,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
     bool alive = true;  // after a wait that ran out the set only keeps its turn at the barrier of each unit
 
     for (uint32_t u = blockIdx.x; u < units; u += gridDim.x, ++unit_i) {
-      uint32_t s_lo, s_hi;
-      const uint32_t tile = unit_steps(u, &s_lo, &s_hi), sl = u - tile * p.n_slices, par = unit_i & 1;
+      uint32_t s_lo = 0, s_hi = 0, tile = u;
+      if (!SORTED) tile = unit_steps(u, &s_lo, &s_hi);
+      const uint32_t sl = u - tile * p.n_slices, par = unit_i & 1;
       const uint64_t n = (uint64_t)tile * kTcTile + own;
       if (alive) alive = wait_all(smem_u32(&sm.a_ready[par]), (unit_i >> 1) & 1);
       __syncwarp();
+      if (SORTED && alive) s_hi = *reinterpret_cast<volatile uint32_t*>(&sm.n_steps[unit_i & 3]);
       const float margin = sm.margin[par][own], seed = sm.seed[par][own];
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&sm.a_free[par]));
@@ -812,7 +937,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
             for (uint32_t q = 0; q < cnt && q < (uint32_t)kTcListLen; ++q) {
               const uint32_t entry = from[q * kTcTile];
               if ((entry >> 16) <= lim) {
-                if (cnt_out < (uint32_t)kCandMost) cand_add(rec, cnt_out, entry & 0xffffu);
+                uint32_t sub = entry & 0xffffu;
+                if (SORTED) sub = 2u * sm.steps[unit_i & 3][sub >> 1] + (sub & 1u);
+                if (cnt_out < (uint32_t)kCandMost) cand_add(rec, cnt_out, sub);
                 ++cnt_out;
               }
             }
@@ -824,12 +951,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
           const bool all = cnt_out > (uint32_t)kCandMost || (min(evicted, sm.odd_evicted[par][own]) >> 16) <= lim;
           rec.w[0] |= (all ? kCandOverflow : cnt_out) << 24;
         } else {
-          rec.best = kNegInf;  // passes every limit: the whole slice is rescored exactly
+          // passes every limit: the whole slice (in spatial order the whole codebook, on account of the first record) is
+          // rescored exactly
+          rec.best = SORTED && p.record > 0 ? -kNegInf : kNegInf;
           rec.w[0] = kCandOverflow << 24;
         }
-        cand_write(&p.rec[((size_t)tile * p.n_slices + sl) * kTcTile + own], rec);
+        if (SORTED)
+          cand_write(&p.rec[((size_t)tile * p.records + p.record) * kTcTile + own], rec);
+        else
+          cand_write(&p.rec[((size_t)tile * p.n_slices + sl) * kTcTile + own], rec);
         atomicMin(&p.gbest[n], ord(rec.best));
-        if (sl == 0) p.margin[n] = in_range ? margin : 0.0f;
+        if (sl == 0 && !(SORTED && p.record > 0)) p.margin[n] = in_range ? margin : 0.0f;
       }
     }
   }
@@ -847,28 +979,79 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
 
 namespace {
 
-template <int DG>
-cudaError_t launch_tc(const pvt_layer& L, const EncM1Params& p, const EncodeM1TcLayout& lay, char* base, TcStats* stats,
-                      cudaStream_t stream) {
-  timing_begin(kKernEncodeAux, stream);
+template <int DG, bool SORTED>
+cudaError_t launch_image(const pvt_layer& L, const EncM1Params& p, const EncodeM1TcLayout& lay, char* base, TcStats* stats,
+                         const uint32_t* order, uint4* sorted_book, cudaStream_t stream) {
   const uint32_t n_cw = lay.n_steps * kTcStepCw;
   // enough threads for one codeword each, and for no more than four of the initial minima each until the chip is full
   const uint64_t fill = (p.k + 1023) / 1024 < 592 ? (p.k + 1023) / 1024 : 592;
   const uint32_t image = (n_cw + kTcPrepCw - 1) / kTcPrepCw;
-  cudaError_t err = launch_dependent(tc_prep_kernel<DG>, fill > image ? (unsigned)fill : image, kTcPrepCw, 0, stream,
-                                     reinterpret_cast<const uint4*>(L.codebooks), p.K, lay.n_steps,
-                                     reinterpret_cast<unsigned char*>(base + lay.bimg_off), stats,
-                                     reinterpret_cast<uint32_t*>(base + lay.exc_off), p.gbest, p.k);
   count_launches(1);
+  return launch_dependent(tc_prep_kernel<DG, SORTED>, fill > image ? (unsigned)fill : image, kTcPrepCw, 0, stream,
+                          reinterpret_cast<const uint4*>(L.codebooks), p.K, lay.n_steps,
+                          reinterpret_cast<unsigned char*>(base + lay.bimg_off), stats,
+                          reinterpret_cast<uint32_t*>(base + lay.exc_off), p.gbest, p.k, order, sorted_book);
+}
+
+template <int DG, bool SORTED>
+cudaError_t launch_search(const EncM1Params& p, const EncodeM1TcLayout& lay, char* base, TcStats* stats,
+                          cudaStream_t stream) {
+  const cudaError_t err = allow_smem<encode_m1_tc_kernel<DG, SORTED>>();
+  if (err != cudaSuccess) return err;
+  count_launches(1);
+  return launch_dependent(encode_m1_tc_kernel<DG, SORTED>, lay.n_ctas, kTcThreads, sizeof(TcSmem<DG, SORTED>), stream, p,
+                          reinterpret_cast<const unsigned char*>(base + lay.bimg_off), stats);
+}
+
+template <int DG>
+cudaError_t launch_tc(const pvt_layer& L, const EncM1Params& p, const EncodeM1TcLayout& lay, char* base, TcStats* stats,
+                      cudaStream_t stream) {
+  timing_begin(kKernEncodeAux, stream);
+  cudaError_t err = launch_image<DG, false>(L, p, lay, base, stats, nullptr, nullptr, stream);
   timing_end(kKernEncodeAux, stream);
   if (err != cudaSuccess) return err;
-  const size_t smem = sizeof(TcSmem<DG>);
-  if ((err = allow_smem<encode_m1_tc_kernel<DG>>()) != cudaSuccess) return err;
   timing_begin(kKernEncodeMain, stream);
-  err = launch_dependent(encode_m1_tc_kernel<DG>, lay.n_ctas, kTcThreads, smem, stream, p,
-                         reinterpret_cast<const unsigned char*>(base + lay.bimg_off), stats);
+  err = launch_search<DG, false>(p, lay, base, stats, stream);
   timing_end(kKernEncodeMain, stream);
-  count_launches(1);
+  return err;
+}
+
+// the same with codewords and targets in spatial order; leaves in p what the rescoring kernel needs
+cudaError_t launch_tc_sorted(const pvt_layer& L, EncM1Params& p, const EncodeM1TcLayout& lay, char* base, TcStats* stats,
+                             int sm_count, cudaStream_t stream) {
+  SortedScratch s;
+  sorted_scratch(base + lay.sorted_off, p.rec, p.K, p.k, lay.n_tiles, lay.n_steps, &s);
+  const uint32_t* idx = p.idx;
+  const TcNorms norms{stats->norms, p.exc_blocks};
+  p.n_slices = 1;
+  p.slice_div = make_fast_div(1);
+  p.sorted_book = s.book;
+  p.order = s.order;
+  timing_begin(kKernEncodeAux, stream);
+  cudaError_t err = launch_sorted_codebook(p.book, p.K, s, stream);
+  if (err == cudaSuccess) err = launch_image<8, true>(L, p, lay, base, stats, s.order, s.book, stream);
+  if (err == cudaSuccess) err = launch_sorted_targets(p, idx, norms, s, sm_count, stream);
+  timing_end(kKernEncodeAux, stream);
+  if (err != cudaSuccess) return err;
+  p.idx = s.sidx;
+  p.place = s.place;
+  p.records = 2;
+  p.record = 0;
+  p.lists = StepLists{s.near, nullptr, s.tile_step, kSortedNear, kSortedNear};
+  timing_begin(kKernEncodeMain, stream);
+  err = launch_search<8, true>(p, lay, base, stats, stream);
+  timing_end(kKernEncodeMain, stream);
+  if (err != cudaSuccess) return err;
+  timing_begin(kKernEncodeAux, stream);
+  err = launch_sorted_reach(p, norms, s, sm_count, stream);
+  timing_end(kKernEncodeAux, stream);
+  if (err != cudaSuccess) return err;
+  p.record = 1;
+  p.lists = StepLists{s.lists, s.counts, nullptr, list_stride(lay.n_steps), 0};
+  timing_begin(kKernEncodeMain, stream);
+  err = launch_search<8, true>(p, lay, base, stats, stream);
+  timing_end(kKernEncodeMain, stream);
+  p.n_slices = p.records;
   return err;
 }
 
@@ -879,7 +1062,7 @@ cudaError_t launch_encode_m1_tc(const pvt_layer& L, uint64_t G, const uint32_t* 
   const EncodeM1TcLayout lay = encode_m1_tc_layout((uint32_t)L.codebook_size, k, sm_count, L.group_dim);
   char* base = static_cast<char*>(ws);
   TcStats* stats = reinterpret_cast<TcStats*>(base + lay.stats_off);
-  EncM1Params p;
+  EncM1Params p = {};
   p.W = L.W;
   p.g = L.g;
   p.scale = L.scale;
@@ -917,8 +1100,9 @@ cudaError_t launch_encode_m1_tc(const pvt_layer& L, uint64_t G, const uint32_t* 
   p.max_spins = hook.max_spins;
   p.withhold_copy = hook.withhold_copy;
 
-  const cudaError_t err =
-      L.group_dim == 16 ? launch_tc<16>(L, p, lay, base, stats, stream) : launch_tc<8>(L, p, lay, base, stats, stream);
+  const cudaError_t err = L.group_dim == 16 ? launch_tc<16>(L, p, lay, base, stats, stream)
+                          : lay.sorted      ? launch_tc_sorted(L, p, lay, base, stats, sm_count, stream)
+                                            : launch_tc<8>(L, p, lay, base, stats, stream);
   if (err != cudaSuccess) return err;
   return launch_rescore_m1(p, true, true, stream);
 }

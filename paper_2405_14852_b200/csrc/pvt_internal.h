@@ -85,7 +85,9 @@ struct EncodeM1TcLayout {
   size_t stats_off;   // TcStats: exceptions and extreme norms by block of codewords
   size_t exc_off;     // u32 [K]: codewords the image cannot represent, by block
   size_t gbest_off, margin_off, rec_off;
+  size_t sorted_off;  // scratch of the search in spatial order
   size_t bytes;
+  bool sorted;
   uint32_t n_steps;   // 128-codeword steps
   uint32_t n_tiles;   // tiles of 256 targets
   uint32_t n_slices;
@@ -95,6 +97,15 @@ bool encode_m1_use_tc(const pvt_layer& L, uint64_t k);
 // fp16 codebooks from here on: the tensor engine (the line that pvt.h states).  20971 / 500000 targets, 512 codewords:
 // small-codebook kernel 17 / 173 us, tensor engine 18 / 210; 768: 27 / 237 and 19 / 218; 1024: 29 / 299 and 19 / 224.
 constexpr int kM1TensorCodebook = 1024;
+// The tensor engine takes codewords and targets in spatial order if both are many: what that leaves out grows with either,
+// and its making costs 0.2 ms and some passes over the targets.  Step over 500000 / 700000 / 1000000 / 2000000 / 4000000
+// targets in ms, 65536 codewords: every codeword 1.40 / 1.97 / 2.72 / 5.16 / 10.1, in spatial order 1.46 / 1.88 / 2.43 /
+// 4.11 / 7.19; 50000: 1.14 / 1.60 / 2.21 / 4.16 / 8.10 and 1.28 / 1.69 / 2.14 / 3.59 / 6.43; 40000: 0.98 / 1.37 / 1.87 /
+// 3.51 / 6.79 and 1.16 / 1.52 / 1.97 / 3.32 / 5.89; 33000: 0.87 / 1.21 / 1.64 / 3.05 / 5.88 and 1.09 / 1.42 / 1.82 / 3.02 /
+// 5.41.  The two meet where targets times the square of the codewords is 2.2e15 to 2.8e15.
+inline bool m1_sorted(uint32_t K, uint64_t k) {
+  return K > 32768 && k >= 3000000000000000ull / ((uint64_t)K * K);
+}
 // Without the tensor engine: codebooks up to here stay in shared memory (both sides measured at the kernel).
 constexpr uint32_t kM1SmallCodebook = 1024;
 constexpr size_t kM1SmallWorkspace = kWsHeaderBytes + kWsAlign;

@@ -1,0 +1,135 @@
+"""The tensor search over codewords and targets in spatial order (many targets, a codebook of more than 32768 codewords)
+against the FP32 engine, which tries every codeword of every target: codes and errors are the same to the bit."""
+import numpy as np
+import pytest
+import torch
+
+import test_gpu_parity as parity
+from paper_2405_14852_b200.vstep import VStepLayer
+
+pytestmark = pytest.mark.gpu
+
+
+def enough(K):
+    """targets from which on the order is worth its making"""
+    return -(-3 * 10 ** 15 // (K * K))
+
+
+def layer(rows, cols, K, seed, change=None):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    W = torch.randn(rows, cols, generator=gen, device="cuda").mul_(0.02)
+    g = torch.randn(rows, cols, generator=gen, device="cuda").mul_(1e-3)
+    scale = W.abs().amax(1)
+    G = W.numel() // 8
+    pick = torch.randperm(G, generator=gen, device="cuda")[:K]
+    books = (W.view(-1, 8)[pick] / scale[pick // (cols // 8), None]).half()[None].contiguous()
+    codes = torch.randint(0, K, (G, 1), generator=gen, device="cuda").to(torch.int16)
+    if change:
+        change(W, g, scale, books[0], codes)
+    return W, g, scale, books, codes
+
+
+def check(parts, idx, again=False, other="fp32"):
+    """other: the engine to compare with, on the targets in portions too small for the order"""
+    W, g, scale, books, codes = parts
+    rows, cols = W.shape
+    got = []
+    for engine, portion in (("tensor", idx.numel()), (other, enough(65536) // 2)):
+        own = codes.clone()
+        err = torch.full((idx.numel(),), -1.0, device="cuda")
+        with parity.search_engine(engine):
+            L = VStepLayer(rows, cols, W, g, scale, books, own, max_k=portion)
+            for _ in range(1 + again):
+                for at in range(0, idx.numel(), portion):
+                    L.encode(idx[at:at + portion].contiguous(), err[at:at + portion])
+            torch.cuda.synchronize()
+            assert L.status() == 0
+        got.append((own, err))
+    assert torch.equal(got[0][0], got[1][0])
+    assert torch.equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("K,more", [
+    (65536, 0), (65536, 513), (65535, 300001), (50048, 1), (40000, 255),  # a last step that is full, and one that is not
+    (32769, 77),  # the smallest: the last step has one codeword
+])
+def test_same_codes_as_the_exhaustive_search(K, more):
+    k = enough(K) + more
+    parts = layer(4096, 8192, K, K + k)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(k)
+    idx = torch.randperm(4096 * 1024, generator=gen, device="cuda")[:k].int()
+    check(parts, idx)
+    check(parts, idx.sort().values, again=True)  # from stored codes that are the nearest
+
+
+def equal_codewords(W, g, scale, book, codes):
+    book[1000:30000] = book[31000:60000]
+
+
+def few_values(W, g, scale, book, codes):
+    book.copy_((book * 4).round() / 4)  # most codewords many times over
+
+
+def one_dimension(W, g, scale, book, codes):
+    book[:, 1:] = 0
+
+
+def one_codeword(W, g, scale, book, codes):
+    book.copy_(book[:1].expand_as(book))
+
+
+def outliers(W, g, scale, book, codes):
+    book[::97] *= 400.0     # beyond the scaled range of most boxes
+    book[5::5003] = 300.0   # not in the operand image
+    book[7::9001] = -60000.0
+    book[11, 3] = float("inf")
+    book[13, 2] = float("nan")
+    book[17, 2] = float("-inf")
+    book[19] = -book[13]
+
+
+def far_targets(W, g, scale, book, codes):
+    scale[3] = 1e-4    # elements up to 256 and beyond
+    scale[4] = 1e-3
+    scale[5] = 1e6     # next to zero
+    scale[6] *= 0.1
+
+
+def small_codewords(W, g, scale, book, codes):
+    book.mul_(2.0 ** -10)
+
+
+def large_codewords(W, g, scale, book, codes):
+    book.mul_(64.0)
+
+
+def bad_codes(W, g, scale, book, codes):
+    codes.fill_(-1)  # stored codes beyond the codebook: no bound to begin with
+
+
+def spread_dimensions(W, g, scale, book, codes):
+    f = torch.tensor([1, 0.5, 0.25, 0.1, 4, 0.01, 1, 2], device="cuda")
+    W.view(-1, 8).mul_(f)
+    g.view(-1, 8).mul_(f)
+    book.mul_(f.half())
+
+
+@pytest.mark.parametrize("change", [equal_codewords, few_values, one_dimension, one_codeword, outliers, far_targets,
+                                    small_codewords, large_codewords, bad_codes, spread_dimensions])
+def test_unusual_inputs(change):
+    K = 60000
+    parts = layer(4096, 2048, K, 7, change)
+    idx = torch.arange(enough(K), dtype=torch.int32, device="cuda")
+    check(parts, idx, other="tensor")  # (which takes codewords that are no numbers)
+
+
+def test_an_index_out_of_range_is_reported():
+    W, g, scale, books, codes = layer(4096, 2048, 65536, 3)
+    idx = torch.arange(enough(65536), dtype=torch.int32, device="cuda")
+    idx[12345] = 4096 * 256
+    L = VStepLayer(4096, 2048, W, g, scale, books, codes, max_k=idx.numel())
+    L.encode(idx)
+    torch.cuda.synchronize()
+    assert L.status() == 1
