@@ -350,6 +350,35 @@ size_t pvt_block_workspace_bytes(const pvt_layer* layers, const uint64_t* k, int
   return need;
 }
 
+namespace {
+bool overlap(const void* a, size_t n, const void* b, size_t m) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return a && b && x < y + m && y < x + n;
+}
+
+// Whether a step of a (checked) layer is one kernel: every group, one small codebook, and nothing that is written shares
+// memory with anything else, since a group's results are written while other groups are still to be read.
+bool one_kernel(const pvt_layer& L, uint64_t k, const uint32_t* idx_out, const void* W_hat, int32_t out_dtype,
+                const void* ws) {
+  const uint64_t n = (uint64_t)L.rows * L.cols, G = n / L.group_dim;
+  if (k != G || L.group_dim != kGroupDim || L.num_codebooks != 1 || encode_m1_use_tc(L, k) ||
+      (uint32_t)L.codebook_size > kM1SmallCodebook)
+    return false;
+  if (!ws || (reinterpret_cast<uintptr_t>(ws) & (kWsAlign - 1))) return false;  // (which the selection reports)
+  const size_t cw = kGroupDim * (L.codebook_dtype == PVT_F16 ? 2 : 4);
+  const struct { const void* p; size_t n; } out[] = {{W_hat, n * (out_dtype == PVT_F16 ? 2 : 4)}, {idx_out, 4 * G},
+                                                     {L.codes, G * (L.code_dtype == PVT_U16 ? 2 : 1)}},
+      in[] = {{L.W, 4 * n}, {L.g, 4 * n}, {L.scale, 4 * (size_t)L.rows}, {L.codebooks, L.codebook_size * cw}, {ws, kM1SmallWorkspace}};
+  for (const auto& o : out) {
+    for (const auto& i : in)
+      if (overlap(o.p, o.n, i.p, i.n)) return false;
+    for (const auto& other : out)
+      if (&o != &other && overlap(o.p, o.n, other.p, other.n)) return false;
+  }
+  return true;
+}
+}  // namespace
+
 int pvt_vstep_block(const pvt_layer* layers, const uint64_t* k, int32_t n_layers, uint32_t* const* idx_out,
                     void* const* W_hat, int32_t out_dtype, void* ws, size_t ws_bytes, void* cuda_stream) {
   if (!layers || !k || !idx_out || n_layers < 1) return PVT_EINVAL;
@@ -377,6 +406,14 @@ int pvt_vstep_block(const pvt_layer* layers, const uint64_t* k, int32_t n_layers
   }
   if (W_hat && out_dtype != PVT_F32 && out_dtype != PVT_F16) return PVT_EINVAL;
   for (int32_t i = 0; i < n_layers; ++i) {
+    if (one_kernel(layers[i], k[i], idx_out[i], W_hat ? W_hat[i] : nullptr, out_dtype, ws)) {
+      uint64_t G = 0;
+      check_layer(&layers[i], &G);
+      const cudaError_t e = launch_step_m1_small(layers[i], G, idx_out[i], W_hat ? W_hat[i] : nullptr, out_dtype, ws, sm_count(),
+                                                 static_cast<cudaStream_t>(cuda_stream));
+      if (e != cudaSuccess) return fail_cuda(e);
+      continue;
+    }
     int rc = pvt_vstep_select(&layers[i], k[i], idx_out[i], ws, ws_bytes, cuda_stream);
     if (rc == PVT_OK) rc = pvt_vstep_encode(&layers[i], idx_out[i], k[i], nullptr, ws, ws_bytes, cuda_stream);
     if (rc == PVT_OK && W_hat && W_hat[i]) rc = pvt_dequant(&layers[i], W_hat[i], out_dtype, nullptr, cuda_stream);

@@ -123,6 +123,9 @@ cudaError_t launch_encode_m1(const pvt_layer& L, uint64_t G, const uint32_t* idx
                              void* ws, int sm_count, cudaStream_t stream);
 cudaError_t launch_encode_m1_small(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
                                    void* ws, int sm_count, cudaStream_t stream);
+// selection of all groups, their search and dequantisation (W_hat may be null) in one kernel
+cudaError_t launch_step_m1_small(const pvt_layer& L, uint64_t G, uint32_t* idx_out, void* W_hat, int32_t out_dtype, void* ws,
+                                 int sm_count, cudaStream_t stream);
 cudaError_t launch_encode_m1_tc(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
                                 void* ws, int sm_count, cudaStream_t stream);
 cudaError_t launch_encode_beam(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
