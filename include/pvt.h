@@ -302,7 +302,8 @@ int pvt_dequant(const pvt_layer* layer, void* W_hat, int32_t out_dtype, uint32_t
  * independent): for i = 0 .. n_layers-1, in order, on the one stream,
  *     pvt_vstep_select(layers[i], k[i]) -> idx_out[i];  pvt_vstep_encode(layers[i], idx_out[i], k[i]);
  *     pvt_dequant(layers[i]) -> W_hat[i]   (skipped when W_hat or W_hat[i] is NULL).
- * A convenience that adds no arithmetic of its own.  layers, k, idx_out, W_hat: HOST arrays of n_layers
+ * A convenience that adds no arithmetic of its own; a layer's W_hat is scratch until the call's work on it is done (it may
+ * be filled from the codes before the step, and the chosen groups again after the search).  layers, k, idx_out, W_hat: HOST arrays of n_layers
  * entries (descriptors, subspace sizes, device pointers to k[i] uint32, device pointers to rows x cols of
  * out_dtype).  ws: one device workspace shared by all layers, at least pvt_block_workspace_bytes (the largest
  * per-layer need), header cleared by pvt_workspace_init; status bits of all layers accumulate in it.

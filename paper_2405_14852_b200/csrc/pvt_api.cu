@@ -237,8 +237,10 @@ int pvt_vstep_sample(const pvt_layer* layer, uint64_t k, int32_t rule, uint64_t 
   return e == cudaSuccess ? PVT_OK : fail_cuda(e);
 }
 
-int pvt_vstep_encode(const pvt_layer* layer, const uint32_t* idx, uint64_t k, float* err_out, void* ws,
-                     size_t ws_bytes, void* cuda_stream) {
+namespace {
+// the search; with `out` the weights of the groups in idx are written as well
+int encode(const pvt_layer* layer, const uint32_t* idx, uint64_t k, float* err_out, void* ws, size_t ws_bytes, WeightsOut out,
+           void* cuda_stream) {
   uint64_t G = 0;
   int rc = check_layer(layer, &G);
   if (rc != PVT_OK) return rc;
@@ -250,29 +252,39 @@ int pvt_vstep_encode(const pvt_layer* layer, const uint32_t* idx, uint64_t k, fl
   if (reinterpret_cast<uintptr_t>(ws) & (kWsAlign - 1)) return PVT_EINVAL;
   const int sms = sm_count();
   cudaError_t e;
+  bool after = false;  // the weights by a kernel of their own
   if (layer->group_dim == 16 && !encode_m1_use_tc(*layer, k)) {
     if (ws_bytes < kWsHeaderBytes) return PVT_EWORKSPACE;
     e = launch_encode_g16(*layer, G, idx, k, err_out, ws, static_cast<cudaStream_t>(cuda_stream));
+    after = true;
   } else if (layer->group_dim == 16) {
     if (ws_bytes < encode_m1_tc_layout((uint32_t)layer->codebook_size, k, sms, 16).bytes) return PVT_EWORKSPACE;
-    e = launch_encode_m1_tc(*layer, G, idx, k, err_out, ws, sms, static_cast<cudaStream_t>(cuda_stream));
+    e = launch_encode_m1_tc(*layer, G, idx, k, err_out, out, ws, sms, static_cast<cudaStream_t>(cuda_stream));
   } else if (layer->num_codebooks == 1 && encode_m1_use_tc(*layer, k)) {
     if (ws_bytes < encode_m1_tc_layout((uint32_t)layer->codebook_size, k, sms).bytes) return PVT_EWORKSPACE;
-    e = launch_encode_m1_tc(*layer, G, idx, k, err_out, ws, sms, static_cast<cudaStream_t>(cuda_stream));
+    e = launch_encode_m1_tc(*layer, G, idx, k, err_out, out, ws, sms, static_cast<cudaStream_t>(cuda_stream));
   } else if (layer->num_codebooks == 1 && (uint32_t)layer->codebook_size <= kM1SmallCodebook) {
     if (ws_bytes < kM1SmallWorkspace) return PVT_EWORKSPACE;
-    e = launch_encode_m1_small(*layer, G, idx, k, err_out, ws, sms, static_cast<cudaStream_t>(cuda_stream));
+    e = launch_encode_m1_small(*layer, G, idx, k, err_out, out, ws, sms, static_cast<cudaStream_t>(cuda_stream));
   } else if (layer->num_codebooks == 1) {
     const EncodeM1Layout lay =
         encode_m1_layout((uint32_t)layer->codebook_size, k, sms, encode_m1_targets_per_thread(k, sms));
     if (ws_bytes < lay.bytes) return PVT_EWORKSPACE;
-    e = launch_encode_m1(*layer, G, idx, k, err_out, ws, sms, static_cast<cudaStream_t>(cuda_stream));
+    e = launch_encode_m1(*layer, G, idx, k, err_out, out, ws, sms, static_cast<cudaStream_t>(cuda_stream));
   } else {
     if ((rc = check_beam(layer)) != PVT_OK) return rc;
     if (ws_bytes < encode_beam_workspace_bytes()) return PVT_EWORKSPACE;
-    e = launch_encode_beam(*layer, G, idx, k, err_out, ws, sms, static_cast<cudaStream_t>(cuda_stream));
+    e = launch_encode_beam(*layer, G, idx, k, err_out, out, ws, sms, static_cast<cudaStream_t>(cuda_stream));
   }
+  if (e == cudaSuccess && after && out.W_hat)
+    e = launch_dequant_list(*layer, G, idx, k, out.W_hat, out.f16 ? PVT_F16 : PVT_F32, static_cast<cudaStream_t>(cuda_stream));
   return e == cudaSuccess ? PVT_OK : fail_cuda(e);
+}
+}  // namespace
+
+int pvt_vstep_encode(const pvt_layer* layer, const uint32_t* idx, uint64_t k, float* err_out, void* ws,
+                     size_t ws_bytes, void* cuda_stream) {
+  return encode(layer, idx, k, err_out, ws, ws_bytes, WeightsOut{}, cuda_stream);
 }
 
 int pvt_vstep_trust(const pvt_layer* layer, uint64_t k_max, float ratio, uint32_t* idx_out, uint64_t* n_out,
@@ -356,19 +368,15 @@ bool overlap(const void* a, size_t n, const void* b, size_t m) {
   return a && b && x < y + m && y < x + n;
 }
 
-// Whether a step of a (checked) layer is one kernel: every group, one small codebook, and nothing that is written shares
-// memory with anything else, since a group's results are written while other groups are still to be read.
-bool one_kernel(const pvt_layer& L, uint64_t k, const uint32_t* idx_out, const void* W_hat, int32_t out_dtype,
-                const void* ws) {
-  const uint64_t n = (uint64_t)L.rows * L.cols, G = n / L.group_dim;
-  if (k != G || L.group_dim != kGroupDim || L.num_codebooks != 1 || encode_m1_use_tc(L, k) ||
-      (uint32_t)L.codebook_size > kM1SmallCodebook)
-    return false;
-  if (!ws || (reinterpret_cast<uintptr_t>(ws) & (kWsAlign - 1))) return false;  // (which the selection reports)
-  const size_t cw = kGroupDim * (L.codebook_dtype == PVT_F16 ? 2 : 4);
-  const struct { const void* p; size_t n; } out[] = {{W_hat, n * (out_dtype == PVT_F16 ? 2 : 4)}, {idx_out, 4 * G},
-                                                     {L.codes, G * (L.code_dtype == PVT_U16 ? 2 : 1)}},
-      in[] = {{L.W, 4 * n}, {L.g, 4 * n}, {L.scale, 4 * (size_t)L.rows}, {L.codebooks, L.codebook_size * cw}, {ws, kM1SmallWorkspace}};
+// Whether what a step of a (checked) layer writes shares no memory with anything else.
+bool apart(const pvt_layer& L, uint64_t k, const uint32_t* idx_out, const void* W_hat, int32_t out_dtype, const void* ws,
+           size_t ws_bytes) {
+  const uint64_t n = (uint64_t)L.rows * L.cols, n_codes = n / L.group_dim * L.num_codebooks;
+  const size_t cw = L.group_dim * (L.codebook_dtype == PVT_F16 ? 2 : 4);
+  const struct { const void* p; size_t n; } out[] = {{W_hat, n * (out_dtype == PVT_F16 ? 2 : 4)}, {idx_out, 4 * k},
+                                                     {L.codes, n_codes * (L.code_dtype == PVT_U16 ? 2 : 1)}, {ws, ws_bytes}},
+      in[] = {{L.W, 4 * n}, {L.g, 4 * n}, {L.scale, 4 * (size_t)L.rows},
+              {L.codebooks, (size_t)L.num_codebooks * L.codebook_size * cw}};
   for (const auto& o : out) {
     for (const auto& i : in)
       if (overlap(o.p, o.n, i.p, i.n)) return false;
@@ -376,6 +384,20 @@ bool one_kernel(const pvt_layer& L, uint64_t k, const uint32_t* idx_out, const v
       if (&o != &other && overlap(o.p, o.n, other.p, other.n)) return false;
   }
   return true;
+}
+
+// Whether a step is one kernel: every group, one small codebook.  (A group's results are written while other groups are
+// still to be read.)
+bool one_kernel(const pvt_layer& L, uint64_t k, uint64_t G) {
+  return k == G && L.group_dim == kGroupDim && L.num_codebooks == 1 && !encode_m1_use_tc(L, k) &&
+         (uint32_t)L.codebook_size <= kM1SmallCodebook;
+}
+// Whether all groups are dequantised from their present codes beside the selection, and those chosen again after the search:
+// while they are few.
+// while they are few.  (Three and four codebooks: fp32 results need the whole SM, 28672 x 8192 4x8 636 us one after the
+// other, 699 side by side; fp16 results gain nothing in the smallest layers, 32768 groups 52.3 and 53.6 us.)
+bool dequant_first(const pvt_layer& L, uint64_t k, uint64_t G, int32_t out_dtype) {
+  return k <= G / 8 && (L.num_codebooks < 3 || (out_dtype == PVT_F16 && G >= 100000));
 }
 }  // namespace
 
@@ -406,12 +428,19 @@ int pvt_vstep_block(const pvt_layer* layers, const uint64_t* k, int32_t n_layers
   }
   if (W_hat && out_dtype != PVT_F32 && out_dtype != PVT_F16) return PVT_EINVAL;
   for (int32_t i = 0; i < n_layers; ++i) {
-    if (one_kernel(layers[i], k[i], idx_out[i], W_hat ? W_hat[i] : nullptr, out_dtype, ws)) {
-      uint64_t G = 0;
-      check_layer(&layers[i], &G);
-      const cudaError_t e = launch_step_m1_small(layers[i], G, idx_out[i], W_hat ? W_hat[i] : nullptr, out_dtype, ws, sm_count(),
-                                                 static_cast<cudaStream_t>(cuda_stream));
+    const pvt_layer& L = layers[i];
+    void* const out = W_hat ? W_hat[i] : nullptr;
+    const uint64_t G = (uint64_t)L.rows * (L.cols / L.group_dim);
+    cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+    const bool good_ws = ws && !(reinterpret_cast<uintptr_t>(ws) & (kWsAlign - 1));  // (which the selection reports)
+    const bool whole = one_kernel(L, k[i], G), first = out && dequant_first(L, k[i], G, out_dtype);
+    if (good_ws && (whole || first) && apart(L, k[i], idx_out[i], out, out_dtype, ws, ws_bytes)) {
+      cudaError_t e = whole ? launch_step_m1_small(L, G, idx_out[i], WeightsOut{out, out_dtype == PVT_F16}, ws, sm_count(), stream)
+                            : launch_select(L, G, k[i], idx_out[i], ws, sm_count(), stream, out, out_dtype);
       if (e != cudaSuccess) return fail_cuda(e);
+      if (whole) continue;
+      const int rc = encode(&L, idx_out[i], k[i], nullptr, ws, ws_bytes, WeightsOut{out, out_dtype == PVT_F16}, cuda_stream);
+      if (rc != PVT_OK) return rc;
       continue;
     }
     int rc = pvt_vstep_select(&layers[i], k[i], idx_out[i], ws, ws_bytes, cuda_stream);

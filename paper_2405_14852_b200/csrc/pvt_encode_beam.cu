@@ -182,6 +182,7 @@ struct BeamParams {
   const void* books;
   uint32_t K, beam;
   uint8_t* codes;  // M adjacent bytes per group
+  WeightsOut out;
   float* err_out;
   uint32_t* status;
 };
@@ -231,10 +232,11 @@ struct BeamScratch {  // per warp
   alignas(16) uint32_t kept[kBsGroup][8];      // their kept tuples: code of codebook q in bits [31 - 8 q : 24 - 8 q]
   uint8_t cells[kBsGroup][64];                 // stage 1: a target's cells within the margin
 };
-template <int M, bool TC>
+template <int M, bool TC, bool WRITE>
 struct BeamSmem {
   BeamImage<M, TC> img;
   BeamScratch w[kBsWarps];
+  float scale[WRITE ? kBsWarps : 1][kBsGroup];  // of the targets' rows
   alignas(8) uint64_t img_bar;  // completion of the image copy
 };
 
@@ -660,11 +662,12 @@ __device__ __forceinline__ uint64_t team_flags(uint32_t mine, uint32_t my_b) {
   return ((uint64_t)hi << 32) | lo;
 }
 
-template <int M, bool TC>
+// WRITE: the weights of the re-encoded groups are written as well.
+template <int M, bool TC, bool WRITE>
 __global__ void __launch_bounds__(kBsThreads, beam_ctas_per_sm(M, TC)) encode_beam_kernel(const BeamParams p,
                                                                                const BeamImage<M, TC>* image) {
   extern __shared__ __align__(16) unsigned char beam_smem[];
-  BeamSmem<M, TC>& smem = *reinterpret_cast<BeamSmem<M, TC>*>(beam_smem);
+  BeamSmem<M, TC, WRITE>& smem = *reinterpret_cast<BeamSmem<M, TC, WRITE>*>(beam_smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   pdl_trigger();
   pdl_wait();
@@ -705,6 +708,7 @@ __global__ void __launch_bounds__(kBsThreads, beam_ctas_per_sm(M, TC)) encode_be
           for (int m = 0; m < M; ++m) lane_prev |= (uint32_t)p.codes[(size_t)lane_j * M + m] << (24 - 8 * m);
         }
         tv = __fdiv_rn(__fmaf_rn(-p.eta, gv, wv), sc);
+        if (WRITE && my_b == 0) smem.scale[warp][my_q] = sc;
       }
       w.t[my_q][my_b] = tv;
     }
@@ -1104,6 +1108,17 @@ __global__ void __launch_bounds__(kBsThreads, beam_ctas_per_sm(M, TC)) encode_be
     }
     __syncwarp();
     team_min_exact(bd, bk);
+    // each lane an element of the group's weights, as dequantisation forms it
+    if (WRITE && my_j != kFull && bd < __longlong_as_double(kInfBits)) {
+      float v = sm.c[0][bk >> 24][my_b];
+#pragma unroll
+      for (int m = 1; m < M; ++m) v = __fadd_rn(v, sm.c[m][(bk >> (24 - 8 * m)) & 0xffu][my_b]);
+      const float x = __fmul_rn(smem.scale[warp][my_q], v);
+      if (p.out.f16)
+        reinterpret_cast<__half*>(p.out.W_hat)[(size_t)my_j * 8 + my_b] = __float2half_rn(x);
+      else
+        reinterpret_cast<float*>(p.out.W_hat)[(size_t)my_j * 8 + my_b] = x;
+    }
     if (my_b == 0 && my_j != kFull) {
       if (bd < __longlong_as_double(kInfBits)) {
         if (M == 2) {
@@ -1121,13 +1136,13 @@ __global__ void __launch_bounds__(kBsThreads, beam_ctas_per_sm(M, TC)) encode_be
   }
 }
 
-template <int M, bool TC>
+template <int M, bool TC, bool WRITE>
 cudaError_t launch_beam(const BeamParams& p, unsigned char* image_at, int sm_count, cudaStream_t stream) {
   using Image = BeamImage<M, TC>;
   static_assert(sizeof(Image) % 16 == 0, "the bulk copy moves multiples of 16 bytes");
   static_assert(sizeof(Image) <= 77824, "the workspace reserves 76 KiB for the image");
-  constexpr size_t smem = sizeof(BeamSmem<M, TC>);
-  cudaError_t err = allow_smem<encode_beam_kernel<M, TC>>();
+  constexpr size_t smem = sizeof(BeamSmem<M, TC, WRITE>);
+  cudaError_t err = allow_smem<encode_beam_kernel<M, TC, WRITE>>();
   if (err != cudaSuccess) return err;
   Image* image = reinterpret_cast<Image*>(image_at);
   timing_begin(kKernEncodeAux, stream);
@@ -1139,17 +1154,24 @@ cudaError_t launch_beam(const BeamParams& p, unsigned char* image_at, int sm_cou
   const uint64_t groups = (p.k + kBsGroup - 1) / kBsGroup, want = (groups + kBsWarps - 1) / kBsWarps;
   const uint64_t most = per_sm * (uint64_t)sm_count;
   timing_begin(kKernEncodeMain, stream);
-  err = launch_dependent(encode_beam_kernel<M, TC>, (unsigned)(want < most ? want : most), kBsThreads, smem, stream, p,
+  err = launch_dependent(encode_beam_kernel<M, TC, WRITE>, (unsigned)(want < most ? want : most), kBsThreads, smem, stream, p,
                          (const Image*)image);
   count_launches(2);
   timing_end(kKernEncodeMain, stream);
   return err;
 }
 
+template <int M>
+cudaError_t launch_type(const pvt_layer& L, const BeamParams& p, unsigned char* image, int sm_count, cudaStream_t stream) {
+  if (L.codebook_dtype == PVT_F16)
+    return p.out.W_hat ? launch_beam<M, true, true>(p, image, sm_count, stream) : launch_beam<M, true, false>(p, image, sm_count, stream);
+  return p.out.W_hat ? launch_beam<M, false, true>(p, image, sm_count, stream) : launch_beam<M, false, false>(p, image, sm_count, stream);
+}
+
 }  // namespace
 
-cudaError_t launch_encode_beam(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out, void* ws,
-                               int sm_count, cudaStream_t stream) {
+cudaError_t launch_encode_beam(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
+                             WeightsOut out, void* ws, int sm_count, cudaStream_t stream) {
   BeamParams p;
   p.W = L.W;
   p.g = L.g;
@@ -1163,14 +1185,14 @@ cudaError_t launch_encode_beam(const pvt_layer& L, uint64_t G, const uint32_t* i
   p.K = (uint32_t)L.codebook_size;
   p.beam = (uint32_t)L.beam;
   p.codes = static_cast<uint8_t*>(L.codes);
+  p.out = out;
   p.err_out = err_out;
   p.status = static_cast<uint32_t*>(ws);
   unsigned char* image = static_cast<unsigned char*>(ws) + kWsHeaderBytes;
-  const bool f16 = L.codebook_dtype == PVT_F16;
   switch (L.num_codebooks) {
-    case 2: return f16 ? launch_beam<2, true>(p, image, sm_count, stream) : launch_beam<2, false>(p, image, sm_count, stream);
-    case 3: return f16 ? launch_beam<3, true>(p, image, sm_count, stream) : launch_beam<3, false>(p, image, sm_count, stream);
-    default: return f16 ? launch_beam<4, true>(p, image, sm_count, stream) : launch_beam<4, false>(p, image, sm_count, stream);
+    case 2: return launch_type<2>(L, p, image, sm_count, stream);
+    case 3: return launch_type<3>(L, p, image, sm_count, stream);
+    default: return launch_type<4>(L, p, image, sm_count, stream);
   }
 }
 

@@ -32,6 +32,8 @@
 // that is nearest in exact arithmetic is always among those rescored.
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "pvt_encode_m1.cuh"
 
 namespace pvt {
@@ -337,8 +339,8 @@ constexpr int kRsPerBlock = 8 * kRsPerWarp;  // 256 threads
 constexpr int kRsEach = 4;  // codewords of a lane on their way at once
 static_assert(kMaxSlices <= 2 * kRsLanes, "two records per lane must cover every slice");
 
-// SORTED: the candidates are positions of the codebook in spatial order.
-template <bool CB_F16, int DG, int SUB, bool SORTED = false>
+// SORTED: the candidates are positions of the codebook in spatial order.  WRITE: the groups' weights are written as well.
+template <bool CB_F16, int DG, int SUB, bool SORTED, bool WRITE>
 __global__ void __launch_bounds__(256, DG == 8 && CB_F16 ? 5 : 3) rescore_m1_kernel(const EncM1Params p) {
   constexpr uint32_t kFull = 0xffffffffu;
   static_assert(!SORTED || (DG == 8 && CB_F16), "the order is that of fp16 codewords of eight elements");
@@ -524,6 +526,19 @@ __global__ void __launch_bounds__(256, DG == 8 && CB_F16 ? 5 : 3) rescore_m1_ker
       code = ocode;
     }
   }
+  if (WRITE && active && code < p.K) {  // each lane its element (two of sixteen), as dequantisation forms it
+    const float s = p.scale[fast_div(j, p.gpr_div)];
+#pragma unroll
+    for (int q = 0; q < DG / kRsLanes; ++q) {
+      const size_t from = (size_t)code * DG + l + q * kRsLanes, to = (size_t)j * DG + l + q * kRsLanes;
+      const float c = CB_F16 ? __half2float(reinterpret_cast<const __half*>(p.book)[from]) : reinterpret_cast<const float*>(p.book)[from];
+      const float w = __fmul_rn(s, c);
+      if (p.out.f16)
+        reinterpret_cast<__half*>(p.out.W_hat)[to] = __float2half_rn(w);
+      else
+        reinterpret_cast<float*>(p.out.W_hat)[to] = w;
+    }
+  }
   if (l == 0 && active) {
     if (code < p.K) {
       if (p.code_u16)
@@ -552,7 +567,7 @@ cudaError_t launch_tt(const EncM1Params& p, uint32_t n_ctas, cudaStream_t stream
 }  // namespace
 
 cudaError_t launch_encode_m1(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
-                             void* ws, int sm_count, cudaStream_t stream) {
+                             WeightsOut out, void* ws, int sm_count, cudaStream_t stream) {
   const int tt = encode_m1_targets_per_thread(k, sm_count);
   const EncodeM1Layout lay = encode_m1_layout((uint32_t)L.codebook_size, k, sm_count, tt);
   char* base = static_cast<char*>(ws);
@@ -585,6 +600,7 @@ cudaError_t launch_encode_m1(const pvt_layer& L, uint64_t G, const uint32_t* idx
   p.book = L.codebooks;
   p.codes = L.codes;
   p.code_u16 = L.code_dtype == PVT_U16;
+  p.out = out;
   p.err_out = err_out;
   p.status = reinterpret_cast<uint32_t*>(base);
   const WaitTestHook hook = wait_test_hook();
@@ -615,13 +631,17 @@ cudaError_t launch_rescore_m1(const EncM1Params& p, bool codebook_f16, bool tens
   timing_begin(kKernEncodeRescore, stream);
   const unsigned blocks = (unsigned)((p.k + kRsPerBlock - 1) / kRsPerBlock);
   auto run = [&](auto kernel) { return launch_dependent(kernel, blocks, 256, 0, stream, p); };
-  cudaError_t err;
-  if (tensor_engine)  // fp16 codebooks
-    err = p.dg == 16  ? run(rescore_m1_kernel<true, 16, kTcSubCodewords>)
-          : p.order ? run(rescore_m1_kernel<true, 8, kTcSubCodewords, true>)
-                    : run(rescore_m1_kernel<true, 8, kTcSubCodewords>);
-  else
-    err = codebook_f16 ? run(rescore_m1_kernel<true, 8, kSubCodewords>) : run(rescore_m1_kernel<false, 8, kSubCodewords>);
+  auto pick = [&](auto write) {
+    constexpr bool W = decltype(write)::value;
+    if (tensor_engine) {  // fp16 codebooks
+      if (p.dg == 16) return run(rescore_m1_kernel<true, 16, kTcSubCodewords, false, W>);
+      return p.order ? run(rescore_m1_kernel<true, 8, kTcSubCodewords, true, W>)
+                     : run(rescore_m1_kernel<true, 8, kTcSubCodewords, false, W>);
+    }
+    return codebook_f16 ? run(rescore_m1_kernel<true, 8, kSubCodewords, false, W>)
+                        : run(rescore_m1_kernel<false, 8, kSubCodewords, false, W>);
+  };
+  const cudaError_t err = p.out.W_hat ? pick(std::true_type{}) : pick(std::false_type{});
   count_launches(1);
   timing_end(kKernEncodeRescore, stream);
   return err;

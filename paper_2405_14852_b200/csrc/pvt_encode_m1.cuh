@@ -57,6 +57,7 @@ struct EncM1Params {
   const void* book;  // the caller's codebook [K][dg]
   void* codes;
   int code_u16;
+  WeightsOut out;
   float* err_out;
   uint32_t* status;
   // the search over codewords and targets in spatial order (null elsewhere): the codebook in the order of the image, the

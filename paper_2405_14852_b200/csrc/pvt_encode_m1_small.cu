@@ -42,18 +42,15 @@ __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
 __host__ __device__ constexpr uint32_t small_blocks(uint32_t K) { return (K + 15) / 16; }  // 16 codewords: a pair per lane
 __host__ __device__ constexpr size_t small_smem_bytes(uint32_t K) { return (size_t)small_blocks(K) * (512 + 64); }
 
-// What a step over every group leaves besides the codes: the list of them, and the weights.
-struct WholeOut {
-  uint32_t* idx;
-  void* W_hat;  // may be null
-  int out_f16;
-};
+// What a search leaves besides the codes: kCodes nothing, kWeights the groups' weights, kStep those (if anywhere) and the list
+// of groups, which are all.
+enum SmallOut { kCodes, kWeights, kStep };
 
-// WHOLE: every group is a target (no list to read), and the team that found a group's codeword writes its weights too, so
+// kStep: every group is a target (no list to read), and the team that found a group's codeword writes its weights too, so
 // that a step is one kernel in place of three.  256 x 256 weights, 256 fp32 codewords: 10.2 -> 7.0 us per step, the first on new
 // buffers 29 -> 24.
-template <bool CB_F16, int TT, bool WHOLE>
-__global__ void __launch_bounds__(kSmThreads, 4) encode_m1_small_kernel(const EncM1Params p, const WholeOut out) {
+template <bool CB_F16, int TT, SmallOut OUT>
+__global__ void __launch_bounds__(kSmThreads, 4) encode_m1_small_kernel(const EncM1Params p, uint32_t* idx_out) {
   // [block of 16 codewords][piece q of 4][lane of 8]: (c[2l][2q], c[2l+1][2q], c[2l][2q+1], c[2l+1][2q+1])
   extern __shared__ __align__(16) float sm_vals[];
   __shared__ uint32_t sm_n2max;
@@ -98,7 +95,7 @@ __global__ void __launch_bounds__(kSmThreads, 4) encode_m1_small_kernel(const En
 #pragma unroll
     for (int tt = 0; tt < TT; ++tt) {
       const uint64_t n = tile * per_cta + (uint64_t)tt * n_teams + team;
-      j[tt] = n < p.k ? (WHOLE ? (uint32_t)n : p.idx[n]) : kFull;
+      j[tt] = n < p.k ? (OUT == kStep ? (uint32_t)n : p.idx[n]) : kFull;
       mine[tt] = 0.0f;
     }
 #pragma unroll
@@ -200,9 +197,9 @@ __global__ void __launch_bounds__(kSmThreads, 4) encode_m1_small_kernel(const En
         } else {
           atomicOr(p.status, PVT_DEV_INTERNAL);  // non-finite target: no distance compares below infinity
         }
-        if (WHOLE) out.idx[n] = (uint32_t)n;
+        if (OUT == kStep) idx_out[n] = (uint32_t)n;
       }
-      if (WHOLE && out.W_hat && real) {  // element l, as dequantisation forms it
+      if (OUT != kCodes && p.out.W_hat && real) {  // element l, as dequantisation forms it
         uint32_t kappa = code;
         if (kappa >= K) {  // the stored code stays
           kappa = p.code_u16 ? reinterpret_cast<const uint16_t*>(p.codes)[j[tt]] : reinterpret_cast<const uint8_t*>(p.codes)[j[tt]];
@@ -210,35 +207,36 @@ __global__ void __launch_bounds__(kSmThreads, 4) encode_m1_small_kernel(const En
         }
         const float c = sm_vals[(kappa >> 4) * 128 + (l >> 1) * 32 + ((kappa >> 1) & 7u) * 4 + (l & 1u) * 2 + (kappa & 1u)];
         const float w = __fmul_rn(row_scale[tt], c);
-        if (out.out_f16)
-          reinterpret_cast<__half*>(out.W_hat)[(size_t)j[tt] * 8 + l] = __float2half_rn(w);
+        if (p.out.f16)
+          reinterpret_cast<__half*>(p.out.W_hat)[(size_t)j[tt] * 8 + l] = __float2half_rn(w);
         else
-          reinterpret_cast<float*>(out.W_hat)[(size_t)j[tt] * 8 + l] = w;
+          reinterpret_cast<float*>(p.out.W_hat)[(size_t)j[tt] * 8 + l] = w;
       }
     }
   }
 }
 
-template <bool CB_F16, int TT, bool WHOLE>
-cudaError_t launch_small(const EncM1Params& p, const WholeOut& out, int sm_count, cudaStream_t stream) {
+template <bool CB_F16, int TT, SmallOut OUT>
+cudaError_t launch_small(const EncM1Params& p, uint32_t* idx_out, int sm_count, cudaStream_t stream) {
   const size_t smem = small_smem_bytes(p.K);
-  const cudaError_t err = allow_smem<encode_m1_small_kernel<CB_F16, TT, WHOLE>>();
+  const cudaError_t err = allow_smem<encode_m1_small_kernel<CB_F16, TT, OUT>>();
   if (err != cudaSuccess) return err;
   const uint64_t per_cta = kSmThreads / 8 * TT, tiles = (p.k + per_cta - 1) / per_cta;
   constexpr uint64_t kMost = 1024 / kSmThreads;  // 64 registers a thread
   const uint64_t fit = (228 * 1024) / (smem + 2048), per_sm = fit < kMost ? fit : kMost;
   const uint64_t resident = per_sm * (uint64_t)sm_count;
   timing_begin(kKernEncodeMain, stream);
-  const cudaError_t e = launch_dependent(encode_m1_small_kernel<CB_F16, TT, WHOLE>,
-                                         (unsigned)(tiles < resident ? tiles : resident), kSmThreads, smem, stream, p, out);
+  const cudaError_t e = launch_dependent(encode_m1_small_kernel<CB_F16, TT, OUT>,
+                                         (unsigned)(tiles < resident ? tiles : resident), kSmThreads, smem, stream, p,
+                                         idx_out);
   timing_end(kKernEncodeMain, stream);
   count_launches(1);
   return e;
 }
 
-template <bool WHOLE>
+template <SmallOut OUT>
 cudaError_t launch_kind(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out, void* ws,
-                        const WholeOut& out, int sm_count, cudaStream_t stream) {
+                        WeightsOut out, uint32_t* idx_out, int sm_count, cudaStream_t stream) {
   EncM1Params p = {};
   p.W = L.W;
   p.g = L.g;
@@ -252,24 +250,26 @@ cudaError_t launch_kind(const pvt_layer& L, uint64_t G, const uint32_t* idx, uin
   p.book = L.codebooks;
   p.codes = L.codes;
   p.code_u16 = L.code_dtype == PVT_U16;
+  p.out = out;
   p.err_out = err_out;
   p.status = static_cast<uint32_t*>(ws);
   const bool two = k >= (uint64_t)sm_count * 256;  // otherwise one target per team keeps more SMs busy
   if (L.codebook_dtype == PVT_F16)
-    return two ? launch_small<true, 2, WHOLE>(p, out, sm_count, stream) : launch_small<true, 1, WHOLE>(p, out, sm_count, stream);
-  return two ? launch_small<false, 2, WHOLE>(p, out, sm_count, stream) : launch_small<false, 1, WHOLE>(p, out, sm_count, stream);
+    return two ? launch_small<true, 2, OUT>(p, idx_out, sm_count, stream) : launch_small<true, 1, OUT>(p, idx_out, sm_count, stream);
+  return two ? launch_small<false, 2, OUT>(p, idx_out, sm_count, stream) : launch_small<false, 1, OUT>(p, idx_out, sm_count, stream);
 }
 
 }  // namespace
 
 cudaError_t launch_encode_m1_small(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
-                                   void* ws, int sm_count, cudaStream_t stream) {
-  return launch_kind<false>(L, G, idx, k, err_out, ws, WholeOut{}, sm_count, stream);
+                                   WeightsOut out, void* ws, int sm_count, cudaStream_t stream) {
+  return out.W_hat ? launch_kind<kWeights>(L, G, idx, k, err_out, ws, out, nullptr, sm_count, stream)
+                   : launch_kind<kCodes>(L, G, idx, k, err_out, ws, out, nullptr, sm_count, stream);
 }
 
-cudaError_t launch_step_m1_small(const pvt_layer& L, uint64_t G, uint32_t* idx_out, void* W_hat, int32_t out_dtype, void* ws,
-                                 int sm_count, cudaStream_t stream) {
-  return launch_kind<true>(L, G, nullptr, G, nullptr, ws, WholeOut{idx_out, W_hat, out_dtype == PVT_F16}, sm_count, stream);
+cudaError_t launch_step_m1_small(const pvt_layer& L, uint64_t G, uint32_t* idx_out, WeightsOut out, void* ws, int sm_count,
+                                 cudaStream_t stream) {
+  return launch_kind<kStep>(L, G, nullptr, G, nullptr, ws, out, idx_out, sm_count, stream);
 }
 
 }  // namespace pvt

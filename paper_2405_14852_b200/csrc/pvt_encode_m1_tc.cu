@@ -1058,7 +1058,7 @@ cudaError_t launch_tc_sorted(const pvt_layer& L, EncM1Params& p, const EncodeM1T
 }  // namespace
 
 cudaError_t launch_encode_m1_tc(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
-                                void* ws, int sm_count, cudaStream_t stream) {
+                             WeightsOut out, void* ws, int sm_count, cudaStream_t stream) {
   const EncodeM1TcLayout lay = encode_m1_tc_layout((uint32_t)L.codebook_size, k, sm_count, L.group_dim);
   char* base = static_cast<char*>(ws);
   TcStats* stats = reinterpret_cast<TcStats*>(base + lay.stats_off);
@@ -1094,6 +1094,7 @@ cudaError_t launch_encode_m1_tc(const pvt_layer& L, uint64_t G, const uint32_t* 
   p.book = L.codebooks;
   p.codes = L.codes;
   p.code_u16 = L.code_dtype == PVT_U16;
+  p.out = out;
   p.err_out = err_out;
   p.status = reinterpret_cast<uint32_t*>(base);
   const WaitTestHook hook = wait_test_hook();

@@ -112,28 +112,40 @@ constexpr size_t kM1SmallWorkspace = kWsHeaderBytes + kWsAlign;
 void set_m1_search(int mode);
 EncodeM1TcLayout encode_m1_tc_layout(uint32_t K, uint64_t k, int sm_count, int group_dim = 8);
 
+// where a search writes the weights of the groups it re-encodes as well (null: nowhere)
+struct WeightsOut {
+  void* W_hat;
+  int f16;
+};
+
 // launchers (each returns a cudaError_t) --------------------------------------
+// (W_hat, k < G: dequantises all groups from their present codes beside the pass over g)
 cudaError_t launch_select(const pvt_layer& L, uint64_t G, uint64_t k, uint32_t* idx_out, void* ws, int sm_count,
-                          cudaStream_t stream);
+                          cudaStream_t stream, void* W_hat = nullptr, int32_t out_dtype = 0);
 // the same selection on other keys: 0 squared update norm, 1 the same while a straight-through buffer takes the
 // step, 2 uniformly random keys, 3 keys of a draw in proportion to the squared update norm (seeded)
 cudaError_t launch_select_keyed(const pvt_layer& L, uint64_t G, uint64_t k, uint32_t* idx_out, void* ws, int sm_count,
-                                cudaStream_t stream, int key_mode, float* buffer, uint64_t seed);
+                                cudaStream_t stream, int key_mode, float* buffer, uint64_t seed, void* W_hat = nullptr,
+                                int32_t out_dtype = 0);
 cudaError_t launch_encode_m1(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
-                             void* ws, int sm_count, cudaStream_t stream);
+                             WeightsOut out, void* ws, int sm_count, cudaStream_t stream);
 cudaError_t launch_encode_m1_small(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
-                                   void* ws, int sm_count, cudaStream_t stream);
-// selection of all groups, their search and dequantisation (W_hat may be null) in one kernel
-cudaError_t launch_step_m1_small(const pvt_layer& L, uint64_t G, uint32_t* idx_out, void* W_hat, int32_t out_dtype, void* ws,
-                                 int sm_count, cudaStream_t stream);
+                                   WeightsOut out, void* ws, int sm_count, cudaStream_t stream);
+// selection of all groups, their search and dequantisation (if there is anywhere to write) in one kernel
+cudaError_t launch_step_m1_small(const pvt_layer& L, uint64_t G, uint32_t* idx_out, WeightsOut out, void* ws, int sm_count,
+                                 cudaStream_t stream);
 cudaError_t launch_encode_m1_tc(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
-                                void* ws, int sm_count, cudaStream_t stream);
+                             WeightsOut out, void* ws, int sm_count, cudaStream_t stream);
 cudaError_t launch_encode_beam(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
-                               void* ws, int sm_count, cudaStream_t stream);
+                             WeightsOut out, void* ws, int sm_count, cudaStream_t stream);
 cudaError_t launch_encode_g16(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
                               void* ws, cudaStream_t stream);
 cudaError_t launch_dequant(const pvt_layer& L, uint64_t G, void* W_hat, int32_t out_dtype, uint32_t* status,
                            int sm_count, cudaStream_t stream);
+
+// the same for the groups of a list
+cudaError_t launch_dequant_list(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, void* W_hat, int32_t out_dtype,
+                                cudaStream_t stream);
 
 cudaError_t launch_pstep_grad(const pvt_layer& L, uint64_t G, double* grad_books, double* grad_scale, uint32_t* status,
                               int sm_count, cudaStream_t stream);
