@@ -16,14 +16,14 @@
 // What is left out is farther away than a codeword that is known, so codes are those of the exhaustive search, bit for bit.
 //
 // Normally distributed weights and 65536 codewords: with 1 / 8 / 29 million targets a tile keeps 0.53 / 0.42 / 0.38 of the
-// steps (a target by itself 0.06: what is lost is the union over 256).  Whole step of 28672 x 8192, every group: 72.7 -> 45.7
-// ms from near stored codes, 82.1 -> 48.2 from random ones; 8192 x 8192 20.8 -> 13.9, 8192 x 1024 2.65 -> 2.3.  Of 13.9 ms the
-// second round takes 7.1, the first 1.6 (finds: each of them is near its targets), the boxes 2.3 (issue slots: 7000
-// instructions per warp), rescoring 2.3, the codebook 0.2, the targets 0.4.  The tree is built by a block per node with the
+// steps (a target by itself 0.06: what is lost is the union over 256).  Whole step of 28672 x 8192, every group: 72.7 -> 43.7
+// ms from near stored codes, 82.1 -> 46.5 from random ones; 8192 x 8192 20.8 -> 13.3, 8192 x 1024 2.65 -> 2.2.  Of 13.3 ms the
+// second round takes 7.0, the first 1.6 (finds: each of its steps is near its targets), the boxes 2.0, rescoring 2.0, the
+// codebook 0.2, the targets 0.4.  The tree is built by a block per node with the
 // keys in shared memory (seven launches, 150 us) and by sorting nodes of 512 positions; with nodes of 4096 sorted and the
 // keys read again for every pass the codebook took 0.49 ms.  Tried for the boxes: bounds from the tree's planes alone (keeps
-// 0.03 more steps), the box of 32 targets in place of the targets (0.82 of the steps), words of steps that other warps have
-// marked left out (no change).
+// 0.03 more steps), the box of 32 targets in place of the targets (0.82 of the steps).  Tried for the search: each half of a
+// tile over the steps of its own (0.32 in place of 0.38 of them, but the issuing warps then look every step up: 7.1 -> 8.1).
 #include "pvt_encode_m1.cuh"
 #include "pvt_encode_m1_sorted.cuh"
 
@@ -282,8 +282,7 @@ __global__ void __launch_bounds__(128) sorted_box_kernel(const uint4* book, uint
 }
 
 // ---- boxes in half precision ------------------------------------------------------
-// Scaled by a power of two so that no element of a codeword exceeds 8, as centre and half width, the width rounded up so
-// that the box holds what it held; two boxes side by side.
+// Scaled by a power of two so that no element of a codeword exceeds 8, rounded outwards; two boxes side by side.
 __device__ __forceinline__ float box_scale(uint32_t n2max_bits) {
   const float c = sqrtf(__uint_as_float(n2max_bits));
   return c > 1e-15f ? scalbnf(1.0f, 2 - ilogbf(c)) : 1.0f;
@@ -291,14 +290,10 @@ __device__ __forceinline__ float box_scale(uint32_t n2max_bits) {
 __device__ void put_box(__half* to, uint32_t which, const float* lo, const float* hi, float scale) {
   const uint32_t pair = which >> 1, side = which & 1u;
   for (int i = 0; i < 8; ++i) {
-    __half c = __float2half_rn(0.0f), h = __float2half_rn(-65504.0f);  // empty: out of reach of everything
-    if (lo[i] <= hi[i]) {
-      const float l = lo[i] * scale, u = hi[i] * scale;
-      c = __float2half_rn(0.5f * (l + u));
-      h = __float2half_ru(fmaxf(__fsub_ru(u, __half2float(c)), __fsub_ru(__half2float(c), l)));
-    }
-    to[pair * 32 + 4 * i + side] = c;
-    to[pair * 32 + 4 * i + 2 + side] = h;
+    // (empty: out of reach of everything)
+    const bool some = lo[i] <= hi[i];
+    to[pair * 32 + 4 * i + side] = __float2half_rd(some ? lo[i] * scale : 65504.0f);
+    to[pair * 32 + 4 * i + 2 + side] = __float2half_ru(some ? hi[i] * scale : -65504.0f);
   }
 }
 
@@ -436,166 +431,178 @@ __global__ void __launch_bounds__(256) sorted_place_kernel(const uint32_t* idx, 
 }
 
 // ---- which steps a tile has to go over ----------------------------------------------
-// A block takes tiles of 256 sorted targets, a thread one target.  r is at least the distance to a codeword that is known:
+// A warp takes tiles of 256 sorted targets, a lane one of them at a time.  r is at least the distance to a codeword that is known:
 // the stored one, or the best of the first round (its score and the margin of that).  A step is left out for a target if
 // the distance to its box exceeds r for certain.  The distances are formed in half precision, two boxes per instruction,
 // first to the boxes of eight steps, whose steps are looked at if any target of the warp comes that near.
-// With elements scaled so that those of codewords are at most 8, the target rounded to half (2^-11 |t|), the difference
-// to the centre, the width taken off (2^-11 each): a gap is at least b (1 - 2^-11) - 2^-11 (2.01 |t_i| + 8.1), and the sum
-// of eight squares is off by less than 2^-7 of itself.  Hence the limit (r + 2^-11 (2.01 ||t|| + 23))^2 (1 + 2^-6) + 2^-14.
-__global__ void __launch_bounds__(256) sorted_reach_kernel(const EncM1Params p, const TcNorms norms, const uint4* packed,
-                                                           const uint16_t* near, const uint16_t* tile_step,
-                                                           uint16_t* lists, uint32_t* counts) {
+// The target is rounded to half (2^-11 |t_i|), the boxes outwards, and the nearest point of a box is a half, so that a gap is
+// at least b (1 - 2^-11) - 2^-11 |t_i| with b its value in half precision; the sum of the eight squares is off by less than
+// ten units of 2^-11 of itself, and by 2^-20 where halves are subnormal.  Hence the limit
+// (r + 1.01 2^-11 ||t||)^2 (1 + 2^-7) + 2^-14.  (Elements of codewords are scaled to at most 8.)
+// What bounds it: the pipes of half-precision arithmetic, about evenly: 44 instructions for two boxes.  A block with a tile,
+// every warp for itself: 2.34 ms for 8388608 targets; a warp with a tile, which leaves out what its earlier targets need,
+// 2.13; the nearest point by minimum and maximum in place of centre and width 2.02.
+constexpr int kReachThreads = 128, kReachBlocks = 10;
+__global__ void __launch_bounds__(kReachThreads, kReachBlocks) sorted_reach_kernel(
+    const EncM1Params p, const TcNorms norms, const uint4* packed, const uint16_t* near, const uint16_t* tile_step,
+    uint16_t* lists, uint32_t* counts) {
   __shared__ __align__(16) uint4 box[(kSortedSteps + kSortedSteps / 8) * 2];  // pairs of boxes, 64 bytes
-  __shared__ uint32_t bits[kSortedSteps / 32];
   __shared__ uint32_t n2max, n2min_inv;
+  constexpr uint32_t kFull = 0xffffffffu;
   const uint32_t tid = threadIdx.x, lane = tid & 31;
   if (tid == 0) n2max = n2min_inv = 0;
   pdl_trigger();
   pdl_wait();
   __syncthreads();
-  {
-    const uint2 part = tid < norms.blocks ? norms.norms[tid] : make_uint2(0, 0);
-    const uint32_t a = __reduce_max_sync(0xffffffffu, part.x), b = __reduce_max_sync(0xffffffffu, part.y);
+  for (uint32_t i = tid; i - lane < norms.blocks; i += kReachThreads) {
+    const uint2 part = i < norms.blocks ? norms.norms[i] : make_uint2(0, 0);
+    const uint32_t a = __reduce_max_sync(kFull, part.x), b = __reduce_max_sync(kFull, part.y);
     if (lane == 0) {
       atomicMax(&n2max, a);
       atomicMax(&n2min_inv, b);
     }
   }
-  for (uint32_t i = tid; i < (kSortedSteps + kSortedSteps / 8) * 2; i += 256) box[i] = packed[i];
+  for (uint32_t i = tid; i < (kSortedSteps + kSortedSteps / 8) * 2; i += kReachThreads) box[i] = packed[i];
   __syncthreads();
   const float scale = box_scale(n2max), cnmin = sqrtf(__uint_as_float(0x7f800000u - n2min_inv));
-  const uint32_t n_steps = p.n_units;
-  for (uint32_t tile = blockIdx.x; tile < p.n_tiles; tile += gridDim.x) {
-    if (tid < kSortedSteps / 32) bits[tid] = 0;
-    __syncthreads();
-    const uint64_t n = (uint64_t)tile * 256 + tid;
-    const uint32_t j = n < p.k ? p.idx[n] : 0xffffffffu;
-    __half2 x[8], lim;
+  const uint32_t n_steps = p.n_units, n_words = (n_steps + 31) / 32;
+  const uint4* groups = box + kSortedSteps * 2;
+  const uint32_t warps = gridDim.x * (kReachThreads / 32);
+  for (uint32_t tile = blockIdx.x * (kReachThreads / 32) + (tid >> 5); tile < p.n_tiles; tile += warps) {
+    // Lane w has word w of the steps that are needed; bit i: its step 2 i, bit 16 + i: step 2 i + 1.  What the first round has
+    // seen, and what earlier targets of the tile need, is not looked at again.
+    static_assert(kSortedNear == 32 && kSortedSteps == 512, "a step per lane, a word per lane of sixteen");
+    uint32_t seen = 0, marked = 0;
     {
-      float t[8], r2 = -1.0f, nt2 = 0.0f;  // (nothing to look for)
+      const uint32_t s = near[(uint32_t)tile_step[tile] * kSortedNear + lane];
+      const uint32_t bit = 1u << ((s >> 1 & 15) + 16 * (s & 1));
+#pragma unroll 1
+      for (uint32_t w = 0; w < n_words; ++w) {
+        const uint32_t word = __reduce_or_sync(kFull, (s >> 5) == w ? bit : 0u);
+        if (lane == w) seen = word;
+      }
+      marked = seen;
+    }
+    const uint64_t n0 = (uint64_t)tile * 256 + lane;
+    uint32_t j_next = n0 < p.k ? p.idx[n0] : kFull;
+#pragma unroll 1
+    for (uint32_t round = 0; round < 8; ++round) {
+      const uint64_t n = n0 + 32 * round;
+      const uint32_t j = j_next;
+      if (round < 7) j_next = n + 32 < p.k ? p.idx[n + 32] : kFull;
+      __half2 x[8], lim;
+      {
+        float t[8], r2 = -1.0f, nt2 = 0.0f;  // (nothing to look for)
 #pragma unroll
-      for (int i = 0; i < 8; ++i) t[i] = 0.0f;
-      if (j < p.G) {
-        form_target(p, j, t);
-        float m = 0.0f;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          m = fmaxf(m, fabsf(t[i]));
-          nt2 = fmaf(t[i], t[i], nt2);
-        }
-        const TargetScale ts = target_scale(m, nt2, cnmin);
-        if (ts.in_range) {  // (the others are rescored against the whole codebook)
-          const float score = unord(p.gbest[n]);  // 2^e d^2 / 2 of the best so far, but for rounding
-          r2 = 2.0f * (score + fmaf(p.rel_margin, fabsf(score), p.margin[n])) / ts.scale;
+        for (int i = 0; i < 8; ++i) t[i] = 0.0f;
+        if (j < p.G) {
           const uint32_t code = p.code_u16 ? reinterpret_cast<const uint16_t*>(p.codes)[j]
                                            : reinterpret_cast<const uint8_t*>(p.codes)[j];
-          if (code < p.K) {
-            float c[8];
-            load_codeword<true, 8>(p.book, code, c);
-            float d = 0.0f;
+          form_target(p, j, t);
+          float m = 0.0f;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) d = fmaf(t[i] - c[i], t[i] - c[i], d);
-            if (d < r2) r2 = d;
+          for (int i = 0; i < 8; ++i) {
+            m = fmaxf(m, fabsf(t[i]));
+            nt2 = fmaf(t[i], t[i], nt2);
           }
-          r2 = fmaxf(r2, 0.0f);
-        }
-      }
-      float limit = -1.0f;
-      if (r2 >= 0.0f) {
-        const float r = scale * sqrtf(r2) * 1.0001f + 4.8828125e-4f * fmaf(2.01f * scale, sqrtf(nt2), 23.0f);
-        limit = fmaf(r * r, 1.015625f, 6.103515625e-5f);
-      }
-      bool all = r2 != r2 || limit > 60000.0f;
+          const TargetScale ts = target_scale(m, nt2, cnmin);
+          if (ts.in_range) {  // (the others are rescored against the whole codebook)
+            const float score = unord(p.gbest[n]);  // 2^e d^2 / 2 of the best so far, but for rounding
+            r2 = 2.0f * (score + fmaf(p.rel_margin, fabsf(score), p.margin[n])) / ts.scale;
+            if (code < p.K) {
+              float c[8];
+              load_codeword<true, 8>(p.book, code, c);
+              float d = 0.0f;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float y = t[i] * scale;
-        all = all || (r2 >= 0.0f && !(fabsf(y) < 1000.0f));
-        x[i] = __float2half2_rn(y);
-      }
-      lim = __half2half2(__float2half_ru(limit));
-      if (all) {  // beyond what halves can tell: every step
-#pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = __float2half2_rn(0.0f);
-        lim = __half2half2(__ushort_as_half(0x7c00));
-      }
-    }
-    // whether the target may reach each of the two boxes at `at`: all bits of the low and of the high half
-    auto reached = [&](const uint4* at) -> uint32_t {
-      __half2 sum = __float2half2_rn(0.0f);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint4 raw = at[q];
-        const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const __half2 c = *reinterpret_cast<const __half2*>(&w[2 * i]), h = *reinterpret_cast<const __half2*>(&w[2 * i + 1]);
-          const __half2 gap = __hmax2(__hsub2(__habs2(__hsub2(x[2 * q + i], c)), h), __float2half2_rn(0.0f));
-          sum = __hfma2(gap, gap, sum);
-        }
-      }
-      return __hle2_mask(sum, lim);
-    };
-    const uint4* groups = box + kSortedSteps * 2;
-    const uint32_t n_words = (n_steps + 31) / 32;
-    volatile uint32_t* marked = bits;
-    // Bit i of a word: its step 2 i, bit 16 + i: step 2 i + 1.  The warps begin at different words, and what another warp has
-    // marked is not looked at again.
-#pragma unroll 1
-    for (uint32_t v = 0, w = (tid >> 5) * n_words / 8; v < n_words; ++v, w = w + 1 == n_words ? 0 : w + 1) {
-      const uint32_t known = marked[w];
-      uint32_t in = 0;
-#pragma unroll 1
-      for (uint32_t q = 0; q < 2; ++q) {
-        const uint32_t near8 = __reduce_or_sync(0xffffffffu, reached(groups + (2 * w + q) * 4));
-#pragma unroll
-        for (uint32_t side = 0; side < 2; ++side) {
-          const uint32_t at = 8 * q + 4 * side;  // four pairs of steps
-          if (near8 >> (16 * side) & 1u) {
-#pragma unroll
-            for (uint32_t i = 0; i < 4; ++i)
-              if (~known & (0x00010001u << (at + i)))
-                in |= reached(box + (16 * w + at + i) * 4) & (0x00010001u << (at + i));
+              for (int i = 0; i < 8; ++i) d = fmaf(t[i] - c[i], t[i] - c[i], d);
+              if (d < r2) r2 = d;
+            }
+            r2 = fmaxf(r2, 0.0f);
           }
         }
-      }
-      in = __reduce_or_sync(0xffffffffu, in);
-      if (lane == 0 && (in & ~known)) atomicOr(&bits[w], in);
-    }
-    __syncthreads();
-    if (tid < 32) {  // the list, without what the first round has seen
-      const uint16_t* seen = near + (uint32_t)tile_step[tile] * kSortedNear;
-      static_assert(kSortedNear == 32, "one per lane");
-      const uint32_t s = seen[lane];
-      atomicAnd(&bits[s >> 5], ~(1u << ((s >> 1 & 15) + 16 * (s & 1))));
-      __syncwarp();
-      uint32_t b = lane < kSortedSteps / 32 ? bits[lane] : 0u;
-      {  // in the order of the steps: the halves of the word interleaved
-        uint32_t x = b & 0xffffu, y = b >> 16;
-        x = (x | (x << 8)) & 0x00ff00ffu, y = (y | (y << 8)) & 0x00ff00ffu;
-        x = (x | (x << 4)) & 0x0f0f0f0fu, y = (y | (y << 4)) & 0x0f0f0f0fu;
-        x = (x | (x << 2)) & 0x33333333u, y = (y | (y << 2)) & 0x33333333u;
-        x = (x | (x << 1)) & 0x55555555u, y = (y | (y << 1)) & 0x55555555u;
-        b = x | (y << 1);
-      }
-      if (32 * lane + 32 > n_steps) b &= 32 * lane < n_steps ? (1u << (n_steps & 31)) - 1u : 0u;  // (steps that are there)
-      // (a search needs a step: one more than needed does no harm)
-      if (!__any_sync(0xffffffffu, b != 0) && lane == 0) b = 1u;
-      const uint32_t c = __popc(b);
-      uint32_t incl = c;
+        float limit = -1.0f;
+        if (r2 >= 0.0f) {
+          const float r = scale * fmaf(4.94e-4f, sqrtf(nt2), sqrtf(r2) * 1.0001f);
+          limit = fmaf(r * r, 1.0078125f, 6.103515625e-5f);
+        }
+        bool all = r2 != r2 || limit > 60000.0f;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t up = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= (uint32_t)o) incl += up;
+        for (int i = 0; i < 8; ++i) {
+          const float y = t[i] * scale;
+          all = all || (r2 >= 0.0f && !(fabsf(y) < 1000.0f));
+          x[i] = __float2half2_rn(y);
+        }
+        lim = __half2half2(__float2half_ru(limit));
+        if (all) {  // beyond what halves can tell: every step
+#pragma unroll
+          for (int i = 0; i < 8; ++i) x[i] = __float2half2_rn(0.0f);
+          lim = __half2half2(__ushort_as_half(0x7c00));
+        }
       }
-      uint16_t* to = lists + (size_t)tile * list_stride(n_steps) + incl - c;
-      while (b) {
-        *to++ = (uint16_t)(32 * lane + __ffs(b) - 1);
-        b &= b - 1;
+      // whether the target may reach each of the two boxes at `at`: all bits of the low and of the high half
+      auto reached = [&](const uint4* at) -> uint32_t {
+        __half2 sum = __float2half2_rn(0.0f);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint4 raw = at[q];
+          const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const __half2 lo = *reinterpret_cast<const __half2*>(&w[2 * i]), hi = *reinterpret_cast<const __half2*>(&w[2 * i + 1]);
+            const __half2 gap = __hsub2(x[2 * q + i], __hmin2(__hmax2(x[2 * q + i], lo), hi));
+            sum = __hfma2(gap, gap, sum);
+          }
+        }
+        return __hle2_mask(sum, lim);
+      };
+#pragma unroll 1
+      for (uint32_t w = 0; w < n_words; ++w) {
+        const uint32_t open = ~__shfl_sync(kFull, marked, w);
+        uint32_t in = 0;
+#pragma unroll 1
+        for (uint32_t q = 0; q < 2; ++q) {
+          if (!(open & (0x00ff00ffu << (8 * q)))) continue;
+          const uint32_t near8 = __reduce_or_sync(kFull, reached(groups + (2 * w + q) * 4));
+#pragma unroll
+          for (uint32_t side = 0; side < 2; ++side) {
+            const uint32_t at = 8 * q + 4 * side;  // four pairs of steps
+            if (near8 >> (16 * side) & 1u) {
+#pragma unroll
+              for (uint32_t i = 0; i < 4; ++i)
+                if (open & (0x00010001u << (at + i))) in |= reached(box + (16 * w + at + i) * 4) & (0x00010001u << (at + i));
+            }
+          }
+        }
+        in = __reduce_or_sync(kFull, in);
+        if (lane == w) marked |= in;
       }
-      if (lane == 31) counts[tile] = incl;
     }
-    __syncthreads();
+    // the list, without what the first round has seen
+    uint32_t b = marked & ~seen;
+    {  // in the order of the steps: the halves of the word interleaved
+      uint32_t x = b & 0xffffu, y = b >> 16;
+      x = (x | (x << 8)) & 0x00ff00ffu, y = (y | (y << 8)) & 0x00ff00ffu;
+      x = (x | (x << 4)) & 0x0f0f0f0fu, y = (y | (y << 4)) & 0x0f0f0f0fu;
+      x = (x | (x << 2)) & 0x33333333u, y = (y | (y << 2)) & 0x33333333u;
+      x = (x | (x << 1)) & 0x55555555u, y = (y | (y << 1)) & 0x55555555u;
+      b = x | (y << 1);
+    }
+    if (32 * lane + 32 > n_steps) b &= 32 * lane < n_steps ? (1u << (n_steps & 31)) - 1u : 0u;  // (steps that are there)
+    // (a search needs a step: one more than needed does no harm)
+    if (!__any_sync(kFull, b != 0) && lane == 0) b = 1u;
+    const uint32_t c = __popc(b);
+    uint32_t incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t up = __shfl_up_sync(kFull, incl, o);
+      if (lane >= (uint32_t)o) incl += up;
+    }
+    uint16_t* to = lists + (size_t)tile * list_stride(n_steps) + incl - c;
+    while (b) {
+      *to++ = (uint16_t)(32 * lane + __ffs(b) - 1);
+      b &= b - 1;
+    }
+    if (lane == 31) counts[tile] = incl;
   }
 }
 
@@ -643,11 +650,12 @@ cudaError_t launch_sorted_targets(const EncM1Params& p, const uint32_t* idx, con
 cudaError_t launch_sorted_reach(const EncM1Params& p, const TcNorms& norms, const SortedScratch& s, int sm_count,
                                 cudaStream_t stream) {
   uint64_t blocks;
-  cudaError_t e = resident_blocks<sorted_reach_kernel>(256, sm_count, &blocks);
+  cudaError_t e = resident_blocks<sorted_reach_kernel>(kReachThreads, sm_count, &blocks);
   if (e != cudaSuccess) return e;
-  if (blocks > p.n_tiles) blocks = p.n_tiles;
+  const uint64_t want = (p.n_tiles + kReachThreads / 32 - 1) / (kReachThreads / 32);
+  if (blocks > want) blocks = want;
   count_launches(1);
-  return launch_dependent(sorted_reach_kernel, (unsigned)blocks, 256, 0, stream, p, norms, (const uint4*)s.packed,
+  return launch_dependent(sorted_reach_kernel, (unsigned)blocks, kReachThreads, 0, stream, p, norms, (const uint4*)s.packed,
                           (const uint16_t*)s.near, (const uint16_t*)s.tile_step, s.lists, s.counts);
 }
 
