@@ -435,11 +435,12 @@ int pvt_vstep_block(const pvt_layer* layers, const uint64_t* k, int32_t n_layers
     const bool good_ws = ws && !(reinterpret_cast<uintptr_t>(ws) & (kWsAlign - 1));  // (which the selection reports)
     const bool whole = one_kernel(L, k[i], G), first = out && dequant_first(L, k[i], G, out_dtype);
     if (good_ws && (whole || first) && apart(L, k[i], idx_out[i], out, out_dtype, ws, ws_bytes)) {
-      cudaError_t e = whole ? launch_step_m1_small(L, G, idx_out[i], WeightsOut{out, out_dtype == PVT_F16}, ws, sm_count(), stream)
+      const WeightsOut weights{out, out_dtype == PVT_F16};
+      cudaError_t e = whole ? launch_step_m1_small(L, G, idx_out[i], weights, ws, sm_count(), stream)
                             : launch_select(L, G, k[i], idx_out[i], ws, sm_count(), stream, out, out_dtype);
       if (e != cudaSuccess) return fail_cuda(e);
       if (whole) continue;
-      const int rc = encode(&L, idx_out[i], k[i], nullptr, ws, ws_bytes, WeightsOut{out, out_dtype == PVT_F16}, cuda_stream);
+      const int rc = encode(&L, idx_out[i], k[i], nullptr, ws, ws_bytes, weights, cuda_stream);
       if (rc != PVT_OK) return rc;
       continue;
     }

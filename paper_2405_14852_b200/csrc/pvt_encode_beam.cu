@@ -1164,8 +1164,10 @@ cudaError_t launch_beam(const BeamParams& p, unsigned char* image_at, int sm_cou
 template <int M>
 cudaError_t launch_type(const pvt_layer& L, const BeamParams& p, unsigned char* image, int sm_count, cudaStream_t stream) {
   if (L.codebook_dtype == PVT_F16)
-    return p.out.W_hat ? launch_beam<M, true, true>(p, image, sm_count, stream) : launch_beam<M, true, false>(p, image, sm_count, stream);
-  return p.out.W_hat ? launch_beam<M, false, true>(p, image, sm_count, stream) : launch_beam<M, false, false>(p, image, sm_count, stream);
+    return p.out.W_hat ? launch_beam<M, true, true>(p, image, sm_count, stream)
+                       : launch_beam<M, true, false>(p, image, sm_count, stream);
+  return p.out.W_hat ? launch_beam<M, false, true>(p, image, sm_count, stream)
+                     : launch_beam<M, false, false>(p, image, sm_count, stream);
 }
 
 }  // namespace

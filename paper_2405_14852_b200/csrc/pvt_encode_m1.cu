@@ -505,33 +505,46 @@ __global__ void __launch_bounds__(256, DG == 8 && CB_F16 ? 5 : 3) rescore_m1_ker
   const float inside = fmaf(least, 3.814697265625e-6f /* 2^-18 */, least) + 1e-36f;
   const uint32_t again = __ballot_sync(kFull, active && (near2 <= inside || !(least < 1e38f)));
   const bool all = (again >> gshift) & 0xffu;
-  if (active && !all && near1 <= inside) {
-    Raw raw;
-    const bool position = SORTED && !(near_code & kNamed);
-    fetch_codeword<CB_F16, DG>(position ? p.sorted_book : p.book, near_code & ~kNamed, &raw);
-    score(near_code, raw);
+  // One codeword of one lane that near: it is the nearest, and binary64 would only say how far it is.
+  const uint32_t close = (__ballot_sync(kFull, active && near1 <= inside) >> gshift) & 0xffu;
+  const bool decided = !p.err_out && !all && __popc(close) == 1;
+  uint32_t hi = 0, lo = 0, code;
+  {
+    const uint32_t named = !SORTED ? near_code : (near_code & kNamed) ? near_code & ~kNamed : p.order[min(near_code, p.K - 1)];
+    code = __shfl_sync(kFull, named, gshift + (close ? __ffs(close) - 1 : 0));
   }
-  if (again) sweep(active && all, score);
-  // lexicographic minimum of (distance, code) over the eight lanes of the target; distances are >= 0 so their
-  // bits order like u64
-  const uint64_t bits = (uint64_t)__double_as_longlong(best_d);
-  uint32_t hi = (uint32_t)(bits >> 32), lo = (uint32_t)bits, code = best_code;
-#pragma unroll
-  for (int off = kRsLanes / 2; off > 0; off >>= 1) {
-    const uint32_t ohi = __shfl_xor_sync(kFull, hi, off), olo = __shfl_xor_sync(kFull, lo, off);
-    const uint32_t ocode = __shfl_xor_sync(kFull, code, off);
-    if (ohi < hi || (ohi == hi && (olo < lo || (olo == lo && ocode < code)))) {
-      hi = ohi;
-      lo = olo;
-      code = ocode;
+  if (__any_sync(kFull, active && !decided)) {
+    if (active && !all && !decided && near1 <= inside) {
+      Raw raw;
+      const bool position = SORTED && !(near_code & kNamed);
+      fetch_codeword<CB_F16, DG>(position ? p.sorted_book : p.book, near_code & ~kNamed, &raw);
+      score(near_code, raw);
     }
+    if (again) sweep(active && all, score);
+    // lexicographic minimum of (distance, code) over the eight lanes of the target; distances are >= 0 so their
+    // bits order like u64
+    const uint64_t bits = (uint64_t)__double_as_longlong(best_d);
+    uint32_t best = best_code;
+    hi = (uint32_t)(bits >> 32), lo = (uint32_t)bits;
+#pragma unroll
+    for (int off = kRsLanes / 2; off > 0; off >>= 1) {
+      const uint32_t ohi = __shfl_xor_sync(kFull, hi, off), olo = __shfl_xor_sync(kFull, lo, off);
+      const uint32_t ocode = __shfl_xor_sync(kFull, best, off);
+      if (ohi < hi || (ohi == hi && (olo < lo || (olo == lo && ocode < best)))) {
+        hi = ohi;
+        lo = olo;
+        best = ocode;
+      }
+    }
+    if (!decided) code = best;
   }
   if (WRITE && active && code < p.K) {  // each lane its element (two of sixteen), as dequantisation forms it
     const float s = p.scale[fast_div(j, p.gpr_div)];
 #pragma unroll
     for (int q = 0; q < DG / kRsLanes; ++q) {
       const size_t from = (size_t)code * DG + l + q * kRsLanes, to = (size_t)j * DG + l + q * kRsLanes;
-      const float c = CB_F16 ? __half2float(reinterpret_cast<const __half*>(p.book)[from]) : reinterpret_cast<const float*>(p.book)[from];
+      const float c = CB_F16 ? __half2float(reinterpret_cast<const __half*>(p.book)[from])
+                             : reinterpret_cast<const float*>(p.book)[from];
       const float w = __fmul_rn(s, c);
       if (p.out.f16)
         reinterpret_cast<__half*>(p.out.W_hat)[to] = __float2half_rn(w);

@@ -47,8 +47,8 @@ __host__ __device__ constexpr size_t small_smem_bytes(uint32_t K) { return (size
 enum SmallOut { kCodes, kWeights, kStep };
 
 // kStep: every group is a target (no list to read), and the team that found a group's codeword writes its weights too, so
-// that a step is one kernel in place of three.  256 x 256 weights, 256 fp32 codewords: 10.2 -> 7.0 us per step, the first on new
-// buffers 29 -> 24.
+// that a step is one kernel in place of three.  256 x 256 weights, 256 fp32 codewords: 10.2 -> 7.0 us per step, the first
+// on new buffers 29 -> 24.
 template <bool CB_F16, int TT, SmallOut OUT>
 __global__ void __launch_bounds__(kSmThreads, 4) encode_m1_small_kernel(const EncM1Params p, uint32_t* idx_out) {
   // [block of 16 codewords][piece q of 4][lane of 8]: (c[2l][2q], c[2l+1][2q], c[2l][2q+1], c[2l+1][2q+1])
@@ -202,7 +202,8 @@ __global__ void __launch_bounds__(kSmThreads, 4) encode_m1_small_kernel(const En
       if (OUT != kCodes && p.out.W_hat && real) {  // element l, as dequantisation forms it
         uint32_t kappa = code;
         if (kappa >= K) {  // the stored code stays
-          kappa = p.code_u16 ? reinterpret_cast<const uint16_t*>(p.codes)[j[tt]] : reinterpret_cast<const uint8_t*>(p.codes)[j[tt]];
+          kappa = p.code_u16 ? reinterpret_cast<const uint16_t*>(p.codes)[j[tt]]
+                             : reinterpret_cast<const uint8_t*>(p.codes)[j[tt]];
           if (kappa >= K) kappa = 0;
         }
         const float c = sm_vals[(kappa >> 4) * 128 + (l >> 1) * 32 + ((kappa >> 1) & 7u) * 4 + (l & 1u) * 2 + (kappa & 1u)];
@@ -255,8 +256,10 @@ cudaError_t launch_kind(const pvt_layer& L, uint64_t G, const uint32_t* idx, uin
   p.status = static_cast<uint32_t*>(ws);
   const bool two = k >= (uint64_t)sm_count * 256;  // otherwise one target per team keeps more SMs busy
   if (L.codebook_dtype == PVT_F16)
-    return two ? launch_small<true, 2, OUT>(p, idx_out, sm_count, stream) : launch_small<true, 1, OUT>(p, idx_out, sm_count, stream);
-  return two ? launch_small<false, 2, OUT>(p, idx_out, sm_count, stream) : launch_small<false, 1, OUT>(p, idx_out, sm_count, stream);
+    return two ? launch_small<true, 2, OUT>(p, idx_out, sm_count, stream)
+               : launch_small<true, 1, OUT>(p, idx_out, sm_count, stream);
+  return two ? launch_small<false, 2, OUT>(p, idx_out, sm_count, stream)
+             : launch_small<false, 1, OUT>(p, idx_out, sm_count, stream);
 }
 
 }  // namespace

@@ -18,7 +18,7 @@
 // Normally distributed weights and 65536 codewords: with 1 / 8 / 29 million targets a tile keeps 0.53 / 0.42 / 0.38 of the
 // steps (a target by itself 0.06: what is lost is the union over 256).  Whole step of 28672 x 8192, every group: 72.7 -> 43.7
 // ms from near stored codes, 82.1 -> 46.5 from random ones; 8192 x 8192 20.8 -> 13.3, 8192 x 1024 2.65 -> 2.2.  Of 13.3 ms the
-// second round takes 7.0, the first 1.6 (finds: each of its steps is near its targets), the boxes 2.0, rescoring 2.0, the
+// second sweep takes 7.0, the first 1.6 (finds: each of its steps is near its targets), the boxes 2.0, rescoring 2.0, the
 // codebook 0.2, the targets 0.4.  The tree is built by a block per node with the
 // keys in shared memory (seven launches, 150 us) and by sorting nodes of 512 positions; with nodes of 4096 sorted and the
 // keys read again for every pass the codebook took 0.49 ms.  Tried for the boxes: bounds from the tree's planes alone (keeps
@@ -61,7 +61,8 @@ __global__ void __launch_bounds__(kSplitThreads) sorted_dims_kernel(const uint4*
   pdl_wait();
   const uint32_t tid = threadIdx.x;
   if (blockIdx.x > 0) {
-    for (uint32_t i = (blockIdx.x - 1) * kSplitThreads + tid; i < kPositions; i += (gridDim.x - 1) * kSplitThreads) cells[i] = 0;
+    for (uint32_t i = (blockIdx.x - 1) * kSplitThreads + tid; i < kPositions; i += (gridDim.x - 1) * kSplitThreads)
+      cells[i] = 0;
     return;
   }
   __shared__ float part[kSplitThreads / 32][16];
@@ -431,8 +432,8 @@ __global__ void __launch_bounds__(256) sorted_place_kernel(const uint32_t* idx, 
 }
 
 // ---- which steps a tile has to go over ----------------------------------------------
-// A warp takes tiles of 256 sorted targets, a lane one of them at a time.  r is at least the distance to a codeword that is known:
-// the stored one, or the best of the first round (its score and the margin of that).  A step is left out for a target if
+// A warp takes tiles of 256 sorted targets, a lane one of them at a time.  r is at least the distance to a codeword that is
+// known: the stored one, or the best of the first sweep (its score and the margin of that).  A step is left out for a target if
 // the distance to its box exceeds r for certain.  The distances are formed in half precision, two boxes per instruction,
 // first to the boxes of eight steps, whose steps are looked at if any target of the warp comes that near.
 // The target is rounded to half (2^-11 |t_i|), the boxes outwards, and the nearest point of a box is a half, so that a gap is
@@ -469,7 +470,7 @@ __global__ void __launch_bounds__(kReachThreads, kReachBlocks) sorted_reach_kern
   const uint4* groups = box + kSortedSteps * 2;
   const uint32_t warps = gridDim.x * (kReachThreads / 32);
   for (uint32_t tile = blockIdx.x * (kReachThreads / 32) + (tid >> 5); tile < p.n_tiles; tile += warps) {
-    // Lane w has word w of the steps that are needed; bit i: its step 2 i, bit 16 + i: step 2 i + 1.  What the first round has
+    // Lane w has word w of the steps that are needed; bit i: its step 2 i, bit 16 + i: step 2 i + 1.  What the first sweep has
     // seen, and what earlier targets of the tile need, is not looked at again.
     static_assert(kSortedNear == 32 && kSortedSteps == 512, "a step per lane, a word per lane of sixteen");
     uint32_t seen = 0, marked = 0;
@@ -486,10 +487,10 @@ __global__ void __launch_bounds__(kReachThreads, kReachBlocks) sorted_reach_kern
     const uint64_t n0 = (uint64_t)tile * 256 + lane;
     uint32_t j_next = n0 < p.k ? p.idx[n0] : kFull;
 #pragma unroll 1
-    for (uint32_t round = 0; round < 8; ++round) {
-      const uint64_t n = n0 + 32 * round;
+    for (uint32_t turn = 0; turn < 8; ++turn) {
+      const uint64_t n = n0 + 32 * turn;
       const uint32_t j = j_next;
-      if (round < 7) j_next = n + 32 < p.k ? p.idx[n + 32] : kFull;
+      if (turn < 7) j_next = n + 32 < p.k ? p.idx[n + 32] : kFull;
       __half2 x[8], lim;
       {
         float t[8], r2 = -1.0f, nt2 = 0.0f;  // (nothing to look for)
@@ -548,7 +549,8 @@ __global__ void __launch_bounds__(kReachThreads, kReachBlocks) sorted_reach_kern
           const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
           for (int i = 0; i < 2; ++i) {
-            const __half2 lo = *reinterpret_cast<const __half2*>(&w[2 * i]), hi = *reinterpret_cast<const __half2*>(&w[2 * i + 1]);
+            const __half2 lo = *reinterpret_cast<const __half2*>(&w[2 * i]);
+            const __half2 hi = *reinterpret_cast<const __half2*>(&w[2 * i + 1]);
             const __half2 gap = __hsub2(x[2 * q + i], __hmin2(__hmax2(x[2 * q + i], lo), hi));
             sum = __hfma2(gap, gap, sum);
           }
@@ -577,7 +579,7 @@ __global__ void __launch_bounds__(kReachThreads, kReachBlocks) sorted_reach_kern
         if (lane == w) marked |= in;
       }
     }
-    // the list, without what the first round has seen
+    // the list, without what the first sweep has seen
     uint32_t b = marked & ~seen;
     {  // in the order of the steps: the halves of the word interleaved
       uint32_t x = b & 0xffffu, y = b >> 16;
@@ -619,8 +621,9 @@ cudaError_t launch_sorted_codebook(const void* book, uint32_t K, const SortedScr
   if ((e = allow_smem<sorted_split_kernel>()) != cudaSuccess) return e;
   for (int level = 0; (kPositions >> level) > kTailPositions; ++level, ++launches) {
     uint32_t* to = (level & 1) ? s.order : s.order2;  // (seven levels)
-    if ((e = launch_dependent(sorted_split_kernel, 1u << level, kSplitThreads, sizeof(uint16_t) * (kPositions >> level), stream, raw, K, (const uint32_t*)s.dims, level,
-                              from, to, s.tree)) != cudaSuccess)
+    const size_t keys = sizeof(uint16_t) * (kPositions >> level);
+    if ((e = launch_dependent(sorted_split_kernel, 1u << level, kSplitThreads, keys, stream, raw, K, (const uint32_t*)s.dims,
+                              level, from, to, s.tree)) != cudaSuccess)
       return e;
     from = to;
   }
@@ -640,7 +643,9 @@ cudaError_t launch_sorted_targets(const EncM1Params& p, const uint32_t* idx, con
   if ((e = launch_dependent(sorted_key_kernel, (unsigned)sm_count * 8, 256, 0, stream, p, idx, (const uint32_t*)s.dims,
                             (const float*)s.tree, s.cells, s.keys)) != cudaSuccess)
     return e;
-  if ((e = launch_dependent(sorted_scan_kernel, kPositions / 1024, 1024, 0, stream, (const uint32_t*)s.cells, s.starts)) != cudaSuccess) return e;
+  if ((e = launch_dependent(sorted_scan_kernel, kPositions / 1024, 1024, 0, stream, (const uint32_t*)s.cells, s.starts)) !=
+      cudaSuccess)
+    return e;
   e = launch_dependent(sorted_place_kernel, (unsigned)sm_count * 8, 256, 0, stream, idx, p.k, (const uint32_t*)s.starts,
                        (const uint2*)s.keys, p.n_units, s.sidx, s.place, s.tile_step);
   count_launches(5);

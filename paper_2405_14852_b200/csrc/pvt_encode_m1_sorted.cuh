@@ -8,7 +8,7 @@ namespace m1 {
 
 constexpr int kSortedLevels = 16;            // of the tree: 65536 positions, those behind the last codeword empty
 constexpr uint32_t kSortedSteps = 512;       // of 128 positions
-constexpr uint32_t kSortedNear = 32;         // steps of the first round
+constexpr uint32_t kSortedNear = 32;         // steps of the first sweep
 
 // rows of the tiles' lists begin at 16-byte boundaries
 __host__ __device__ constexpr uint32_t list_stride(uint32_t n_steps) { return (n_steps + 7) / 8 * 8; }

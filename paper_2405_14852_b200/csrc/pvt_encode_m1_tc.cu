@@ -190,7 +190,7 @@ EncodeM1TcLayout encode_m1_tc_layout(uint32_t K, uint64_t k, int sm_count, int g
   e.n_slices = best_s;
   const uint64_t units = (uint64_t)e.n_tiles * e.n_slices;
   e.sorted = group_dim == kGroupDim && m1_sorted(K, k);
-  if (e.sorted) e.n_slices = 2;  // two rounds, a record each
+  if (e.sorted) e.n_slices = 2;  // two sweeps, a record each
   e.n_ctas = (uint32_t)(units < (uint64_t)sm_count ? units : (uint64_t)sm_count);
   e.bimg_off = kWsHeaderBytes;
   e.stats_off = align_up(e.bimg_off + (size_t)e.n_steps * (group_dim == 16 ? TcDim<16>::kStepBytes : kTcStepBytes),
@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
   struct RowIn {
     TargetIn in;
     uint32_t code;
-    uint32_t best;  // in the second round: of the first
+    uint32_t best;  // in the second sweep: of the first
   };
   auto load_row = [&](uint32_t j, uint32_t tile, uint32_t own) {
     RowIn row = {};
@@ -651,7 +651,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
                                  4.76837158203125e-7f /* 2^-21 */);
     sm.margin[par][own] = !have ? kAbsent : in_range ? margin : kOutOfRange;
     float seed = in_range ? -0.5f * sc * prev * 1.0001f : kNegInf;  // (minus infinity without a stored code)
-    // the second round goes on from what the first one found
+    // the second sweep goes on from what the first one found
     if (SORTED && have && in_range && p.record > 0) seed = fmaxf(seed, -unord(row.best));
     sm.seed[par][own] = seed;
   };
@@ -703,7 +703,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
           // for that stage runs out
           if (SORTED) {  // the steps of a list: a copy each
             if ((uint32_t)lane < n && p.withhold_copy != it + lane)
-              bulk_g2s(smem_u32(&sm.b[s][sub + lane][0]), bimg + (size_t)sm.ahead[place][st + lane] * kStepBytes, kStepBytes, fb);
+              bulk_g2s(smem_u32(&sm.b[s][sub + lane][0]), bimg + (size_t)sm.ahead[place][st + lane] * kStepBytes, kStepBytes,
+                       fb);
           } else if (lane == 0 && p.withhold_copy - it >= n)
             bulk_g2s(smem_u32(&sm.b[s][sub][0]), bimg + (size_t)st * kStepBytes, n * kStepBytes, fb);
           st += n;
