@@ -31,7 +31,8 @@ constexpr int kSelBins1 = 512;        // key bits [17:9]
 constexpr int kSelBins2 = 512;        // key bits [8:0]
 constexpr uint32_t kSelMaxCtas = 1024;
 // counts per CTA, state, the histograms
-constexpr uint32_t kSelScratchWords = 2 * kSelMaxCtas + 16 + kSelBins0 + kSelBins1 + kSelBins1 * kSelBins2;
+constexpr uint32_t kSelCountStride = 4;  // a count (u64) per 32 bytes: all later CTAs poll it
+constexpr uint32_t kSelScratchWords = 2 * kSelCountStride * kSelMaxCtas + 16 + kSelBins0 + kSelBins1 + kSelBins1 * kSelBins2;
 
 struct SelectLayout {
   size_t scratch_off;  // u32 [kSelScratchWords]

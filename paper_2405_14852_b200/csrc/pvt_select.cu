@@ -20,7 +20,9 @@
 // ahead, one CTA per SM and polls without a pause).  By counters of the kernels by themselves pass 1 takes 16 us of the
 // first (4.2 TB/s of g from cold; 5.4 for the second), the others 4.5, 10 and 12; 28672 x 8192: 245 us.  Five passes with
 // one bin per eighth of an octave took 45 / 74 / 344 us.  One cooperative kernel with the keys in shared memory takes
-// 33 us, and about 10 us more to launch.  Clearing the large tables in pass 1, and contiguous shares there: no gain.
+// 33 us, and about 10 us more to launch.  Clearing the large tables in pass 1, and contiguous shares there: no gain.  The
+// counts that pass 3 waits for side by side, sixteen to a line: 27.1 / 49.0 us; each in a sector of its own: 24.8 / 48.0 (the
+// pass 7.5 us after the one before it, 10.5 where its line was slow to reach: those that poll kept the counts from arriving).
 #include "pvt_select.cuh"
 
 namespace pvt {
@@ -266,7 +268,7 @@ __global__ void __launch_bounds__(kSelThreads) select_write_kernel(const SelPara
   __syncthreads();
   if (tid == 0) {
     const uint64_t mine = (1ull << 63) | ((uint64_t)all_eq << 31) | all_gt;  // a CTA has fewer than 2^31 groups
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p.counts + cta), "l"(mine) : "memory");
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p.counts + kSelCountStride * cta), "l"(mine) : "memory");
   }
   bool ok = true;
   uint32_t prev_gt = 0, prev_eq = 0;
@@ -274,7 +276,7 @@ __global__ void __launch_bounds__(kSelThreads) select_write_kernel(const SelPara
     uint64_t c = 0;
     for (uint32_t i = 0; i < kSelMaxPolls && !(c >> 63); ++i) {
       if (i) __nanosleep(40);
-      asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(c) : "l"(p.counts + b) : "memory");
+      asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(c) : "l"(p.counts + kSelCountStride * b) : "memory");
     }
     ok &= (c >> 63) != 0;
     prev_gt += (uint32_t)c & 0x7fffffffu;
@@ -389,7 +391,7 @@ cudaError_t launch_select_keyed(const pvt_layer& L, uint64_t G, uint64_t k, uint
     p.masks = reinterpret_cast<uint2*>(base + lay.masks_off);
     uint32_t* scratch = reinterpret_cast<uint32_t*>(base + lay.scratch_off);
     p.counts = reinterpret_cast<uint64_t*>(scratch);
-    p.state = scratch + 2 * kSelMaxCtas;
+    p.state = scratch + 2 * kSelCountStride * kSelMaxCtas;
     p.hist0 = p.state + 16;
     p.hist1 = p.hist0 + kSelBins0;
     p.fine = p.hist1 + kSelBins1;
