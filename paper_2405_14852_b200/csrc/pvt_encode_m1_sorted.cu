@@ -16,14 +16,17 @@
 // What is left out is farther away than a codeword that is known, so codes are those of the exhaustive search, bit for bit.
 //
 // Normally distributed weights and 65536 codewords: with 1 / 8 / 29 million targets a tile keeps 0.53 / 0.42 / 0.38 of the
-// steps (a target by itself 0.06: what is lost is the union over 256).  Whole step of 28672 x 8192, every group: 72.7 -> 43.7
-// ms from near stored codes, 82.1 -> 46.5 from random ones; 8192 x 8192 20.8 -> 13.3, 8192 x 1024 2.65 -> 2.2.  Of 13.3 ms the
-// second sweep takes 7.0, the first 1.6 (finds: each of its steps is near its targets), the boxes 2.0, rescoring 2.0, the
-// codebook 0.2, the targets 0.4.  The tree is built by a block per node with the
-// keys in shared memory (seven launches, 150 us) and by sorting nodes of 512 positions; with nodes of 4096 sorted and the
-// keys read again for every pass the codebook took 0.49 ms.  Tried for the boxes: bounds from the tree's planes alone (keeps
-// 0.03 more steps), the box of 32 targets in place of the targets (0.82 of the steps).  Tried for the search: each half of a
-// tile over the steps of its own (0.32 in place of 0.38 of them, but the issuing warps then look every step up: 7.1 -> 8.1).
+// steps (a target by itself 0.06: what is lost is the union over 256).  Whole step of 28672 x 8192, every group: 73.5 -> 43.0
+// ms from near stored codes, 82.0 -> 45.4 from random ones; 8192 x 8192 20.8 -> 13.1, 8192 x 1024 2.65 -> 2.2.  Of 13.1 ms the
+// second sweep takes 7.0, the first 1.6 (finds: each of its steps is near its targets), the boxes 2.0, rescoring 1.8, the
+// codebook 0.2, the targets 0.4.  What it gives depends on the weights.  Search of 8388608 targets in ms, every codeword / in
+// spatial order: normal 20.7 / 12.9, uniform 20.7 / 8.8, correlated elements 22.1 / 6.4, Laplace 20.8 / 16.4, groups of unlike
+// size 20.8 / 15.2, a codebook ten times smaller than the targets 22.8 / 22.8.
+// The tree is built by a block per node with the keys in shared memory (seven launches, 150 us) and by sorting nodes of 512
+// positions; with nodes of 4096 sorted and the keys read again for every pass the codebook took 0.49 ms.  Tried for the boxes:
+// bounds from the tree's planes alone (keeps 0.03 more steps), the box of 32 targets in place of the targets (0.82 of the
+// steps).  Tried for the search: each half of a tile over the steps of its own (0.32 in place of 0.38 of them, but the issuing
+// warps then look every step up: 7.1 -> 8.1).
 #include "pvt_encode_m1.cuh"
 #include "pvt_encode_m1_sorted.cuh"
 

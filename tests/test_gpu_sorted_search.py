@@ -1,10 +1,10 @@
 """The tensor search over codewords and targets in spatial order (many targets, a codebook of more than 32768 codewords)
 against the FP32 engine, which tries every codeword of every target: codes and errors are the same to the bit."""
-import numpy as np
 import pytest
 import torch
 
 import test_gpu_parity as parity
+from paper_2405_14852_b200 import binding as B
 from paper_2405_14852_b200.vstep import VStepLayer
 
 pytestmark = pytest.mark.gpu
@@ -133,3 +133,32 @@ def test_an_index_out_of_range_is_reported():
     L.encode(idx)
     torch.cuda.synchronize()
     assert L.status() == 1
+
+
+@pytest.mark.parametrize("withhold", [0, 11])
+def test_a_wait_that_runs_out_is_reported_and_the_next_call_is_correct(withhold):
+    """The bounded waits (test_gpu_wait_limit.py) where a unit is a tile and a copy a step of its list."""
+    K = 65536
+    W, g, scale, books, codes = layer(4096, 2048, K, 4)
+    idx = torch.arange(enough(K), dtype=torch.int32, device="cuda")
+    own = codes.clone()
+    L = VStepLayer(4096, 2048, W, g, scale, books, own, max_k=idx.numel())
+    B.pvt_test_wait_limit(20000, withhold)
+    try:
+        L.encode(idx)
+        torch.cuda.synchronize()
+        status = L.status()
+    finally:
+        B.pvt_test_wait_limit(0, -1)
+    assert status & B.PVT_DEV_WAIT_EXPIRED
+    own.copy_(codes)
+    L.encode(idx)
+    torch.cuda.synchronize()
+    assert L.status() == 0
+    other = codes.clone()
+    portion = enough(K) // 2
+    M = VStepLayer(4096, 2048, W, g, scale, books, other, max_k=portion)
+    for at in range(0, idx.numel(), portion):
+        M.encode(idx[at:at + portion].contiguous())
+    torch.cuda.synchronize()
+    assert torch.equal(own, other)
