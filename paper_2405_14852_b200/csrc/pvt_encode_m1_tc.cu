@@ -45,7 +45,8 @@
 // step over the layers of a block whose codes are near 1823 in place of 1802, as the rows of all tiles are then gathered at
 // the same time; slices that run together and exchange their best scores after a few steps 78 / 278, and 1820.
 // In spatial order (pvt_encode_m1_sorted.cu: many targets) a unit is a tile and goes over a list of steps in place of a slice:
-// a copy for each step, the list in shared memory with the rows, 29360128 targets from random codes 74.5 -> 29.5 ms in two launches.
+// a copy for each step, the list in shared memory with the rows; 29360128 targets from random codes 74.5 -> 29.5 ms in two
+// launches.
 //
 // Codewords whose half squared norm exceeds the fp16 range get a sentinel row
 // that can never win and are listed as "exceptions": the rescoring kernel always

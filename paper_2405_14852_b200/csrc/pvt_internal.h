@@ -99,11 +99,11 @@ bool encode_m1_use_tc(const pvt_layer& L, uint64_t k);
 // small-codebook kernel 17 / 173 us, tensor engine 18 / 210; 768: 27 / 237 and 19 / 218; 1024: 29 / 299 and 19 / 224.
 constexpr int kM1TensorCodebook = 1024;
 // The tensor engine takes codewords and targets in spatial order if both are many: what that leaves out grows with either,
-// and its making costs 0.2 ms and some passes over the targets.  Step over 500000 / 700000 / 1000000 / 2000000 / 4000000
-// targets in ms, 65536 codewords: every codeword 1.40 / 1.97 / 2.72 / 5.16 / 10.1, in spatial order 1.46 / 1.88 / 2.43 /
-// 4.11 / 7.19; 50000: 1.14 / 1.60 / 2.21 / 4.16 / 8.10 and 1.28 / 1.69 / 2.14 / 3.59 / 6.43; 40000: 0.98 / 1.37 / 1.87 /
-// 3.51 / 6.79 and 1.16 / 1.52 / 1.97 / 3.32 / 5.89; 33000: 0.87 / 1.21 / 1.64 / 3.05 / 5.88 and 1.09 / 1.42 / 1.82 / 3.02 /
-// 5.41.  The two meet where targets times the square of the codewords is 2.2e15 to 2.8e15.
+// and its making costs 0.2 ms and some passes over the targets.  Step over 500000 / 700000 / 1000000 / 2000000 targets from
+// near stored codes in ms, 65536 codewords: every codeword 1.47 / 1.97 / 2.71 / 5.15, in spatial order 1.51 / 1.84 / 2.36 /
+// 3.94; 50000: 1.21 / 1.60 / 2.20 / 4.14 and 1.35 / 1.65 / 2.11 / 3.43; 40000: 1.05 / 1.37 / 1.87 / 3.49 and 1.24 / 1.50 /
+// 1.94 / 3.17; 33000: 0.92 / 1.20 / 1.63 / 3.04 and 1.17 / 1.41 / 1.79 / 2.95.  The two meet where targets times the square of
+// the codewords is 1.7e15 to 2.6e15 (normally distributed weights; where less can be left out they meet later).
 inline bool m1_sorted(uint32_t K, uint64_t k) {
   return K > 32768 && k >= 3000000000000000ull / ((uint64_t)K * K);
 }
