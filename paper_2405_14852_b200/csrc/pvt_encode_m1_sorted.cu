@@ -327,8 +327,7 @@ __global__ void __launch_bounds__(kSortedSteps) sorted_near_kernel(const float* 
       }
     }
   }
-  // (the number of the step in the last bits makes the distances different)
-  const uint32_t key = tid == s ? 0u : (__float_as_uint(d) & ~(kSortedSteps - 1)) | tid;
+  const uint32_t key = near_key(__float_as_uint(d), tid, s);
   dist[tid] = key;
   __syncthreads();
   if (s < n_steps && tid < n_steps) {

@@ -541,10 +541,16 @@ __global__ void __launch_bounds__(kTcThreads, 1) encode_m1_tc_kernel(const EncM1
     const uint64_t n = (uint64_t)tile * kTcTile + own;
     return n < p.k ? p.idx[n] : 0xffffffffu;
   };
-  // brings a tile's list to shared memory, `threads` threads of number `first` (16 bytes each; the last ones may be padding)
+  // brings a tile's list to shared memory, `threads` threads of number `first` (16 bytes each; the last ones may be padding);
+  // no number goes beyond the last step, whatever the list holds, so that none of them leads past the image
   auto bring_list = [&](uint32_t tile, uint16_t* to, uint32_t n, uint32_t first, uint32_t threads) {
     const uint4* from = reinterpret_cast<const uint4*>(step_list(tile));
-    for (uint32_t i = first; i < (n + 7) / 8; i += threads) reinterpret_cast<uint4*>(to)[i] = from[i];
+    const uint32_t last = (p.n_units - 1) * 0x10001u;
+    for (uint32_t i = first; i < (n + 7) / 8; i += threads) {
+      const uint4 eight = from[i];
+      reinterpret_cast<uint4*>(to)[i] =
+          make_uint4(__vminu2(eight.x, last), __vminu2(eight.y, last), __vminu2(eight.z, last), __vminu2(eight.w, last));
+    }
   };
   // What a target is formed from (index j): in spatial order, where it is farther away, asked for ahead of its use.
   struct RowIn {

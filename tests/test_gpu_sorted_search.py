@@ -30,8 +30,9 @@ def layer(rows, cols, K, seed, change=None):
     return W, g, scale, books, codes
 
 
-def check(parts, idx, again=False, other="fp32"):
-    """other: the engine to compare with, on the targets in portions too small for the order"""
+def check(parts, idx, again=False, other="fp32", fill=None):
+    """other: the engine to compare with, on the targets in portions too small for the order; fill: what every 16 bits of the
+    workspace behind its header hold before the call"""
     W, g, scale, books, codes = parts
     rows, cols = W.shape
     got = []
@@ -40,6 +41,8 @@ def check(parts, idx, again=False, other="fp32"):
         err = torch.full((idx.numel(),), -1.0, device="cuda")
         with parity.search_engine(engine):
             L = VStepLayer(rows, cols, W, g, scale, books, own, max_k=portion)
+            if fill is not None:
+                L.reserve(portion)[256:].view(torch.int16).fill_(fill)
             for _ in range(1 + again):
                 for at in range(0, idx.numel(), portion):
                     L.encode(idx[at:at + portion].contiguous(), err[at:at + portion])
@@ -123,6 +126,25 @@ def test_unusual_inputs(change):
     parts = layer(4096, 2048, K, 7, change)
     idx = torch.arange(enough(K), dtype=torch.int32, device="cuda")
     check(parts, idx, other="tensor")  # (which takes codewords that are no numbers)
+
+
+def repeated_codewords(W, g, scale, book, codes):
+    book[256:] = book[:256].repeat(-(-book.shape[0] // 256), 1)[256:book.shape[0]]
+
+
+def dead_codewords(W, g, scale, book, codes):
+    book.abs_()
+    book[torch.arange(book.shape[0], device="cuda") % 50 < 27] = 0
+
+
+@pytest.mark.parametrize("fill", [5, 300])  # numbers of steps that exist
+@pytest.mark.parametrize("K", [60000, 65536])
+@pytest.mark.parametrize("change", [one_codeword, repeated_codewords, dead_codewords])
+def test_equal_codewords_whatever_the_workspace_holds(change, K, fill):
+    """Steps whose boxes have the same centre: every place of the list of near ones is written (test_sorted_near_steps.py)."""
+    parts = layer(4096, 2048, K, 8, change)
+    idx = torch.arange(enough(K), dtype=torch.int32, device="cuda")
+    check(parts, idx, other="tensor", fill=fill)
 
 
 def test_an_index_out_of_range_is_reported():
