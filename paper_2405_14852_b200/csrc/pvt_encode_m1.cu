@@ -468,14 +468,21 @@ __global__ void __launch_bounds__(256, DG == 8 && CB_F16 ? 5 : 3) rescore_m1_ker
       uint32_t ids[3] = {upper ? y1 : y0, upper ? z1 : z0, upper ? w1 : w0};
       const uint32_t cnt = ids[0] >> 24;
       if (cnt == kCandOverflow) {
-        uint32_t u_lo, u_hi;
-        if (SORTED) {  // all of it: the list that was gone over is gone
-          u_lo = 0;
-          u_hi = p.n_units;
-        } else {
-          slice_units(p, (uint32_t)sl, &u_lo, &u_hi);
+        if (SORTED && limit > -__builtin_huge_valf()) {
+          // the steps that the record stands for; no step is in both lists of a tile
+          const StepLists& from = sl ? p.lists : p.near_lists;
+          const uint32_t tile = (uint32_t)(n / p.tile), row = from.rows ? from.rows[tile] : tile;
+          const uint16_t* steps = from.steps + (size_t)row * from.stride;
+          const uint32_t many = from.counts ? from.counts[tile] : from.most;
+          for (uint32_t i = 0; i < many; ++i) {
+            const uint32_t step = min((uint32_t)steps[i], p.n_units - 1);
+            for (uint32_t q = 0; q < subs_per_unit; ++q) visit(step * subs_per_unit + q);
+          }
+        } else {  // (in spatial order: a target that the tensor cores cannot serve, against the whole codebook)
+          uint32_t u_lo = 0, u_hi = p.n_units;
+          if (!SORTED) slice_units(p, (uint32_t)sl, &u_lo, &u_hi);
+          for (uint32_t sub = u_lo * subs_per_unit; sub < u_hi * subs_per_unit; ++sub) visit(sub);
         }
-        for (uint32_t sub = u_lo * subs_per_unit; sub < u_hi * subs_per_unit; ++sub) visit(sub);
       } else {
         for (uint32_t q = 0; q < cnt; ++q) {
           visit(ids[0] & 0xfffu);

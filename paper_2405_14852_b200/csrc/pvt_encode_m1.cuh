@@ -64,7 +64,8 @@ struct EncM1Params {
   // codeword at each of its positions, the steps of a tile
   const void* sorted_book;
   const uint32_t* order;
-  StepLists lists;
+  StepLists lists;       // of the sweep at hand, for the rescoring of the second
+  StepLists near_lists;  // for the rescoring: of the first
   uint32_t record, records;  // the record that a launch writes, of so many per target
   uint32_t max_spins;      // poll limit of every wait on an on-chip barrier
   uint32_t withhold_copy;  // kNoWithhold; otherwise the producer skips its copy of this sequence number (test hook)

@@ -582,18 +582,22 @@ __global__ void __launch_bounds__(kReachThreads, kReachBlocks) sorted_reach_kern
       }
     }
     // the list, without what the first sweep has seen
-    uint32_t b = marked & ~seen;
-    {  // in the order of the steps: the halves of the word interleaved
-      uint32_t x = b & 0xffffu, y = b >> 16;
+    auto in_order = [](uint32_t word) {  // of the steps: the halves of the word interleaved
+      uint32_t x = word & 0xffffu, y = word >> 16;
       x = (x | (x << 8)) & 0x00ff00ffu, y = (y | (y << 8)) & 0x00ff00ffu;
       x = (x | (x << 4)) & 0x0f0f0f0fu, y = (y | (y << 4)) & 0x0f0f0f0fu;
       x = (x | (x << 2)) & 0x33333333u, y = (y | (y << 2)) & 0x33333333u;
       x = (x | (x << 1)) & 0x55555555u, y = (y | (y << 1)) & 0x55555555u;
-      b = x | (y << 1);
-    }
+      return x | (y << 1);
+    };
+    uint32_t b = in_order(marked & ~seen);
     if (32 * lane + 32 > n_steps) b &= 32 * lane < n_steps ? (1u << (n_steps & 31)) - 1u : 0u;  // (steps that are there)
-    // (a search needs a step: one more than needed does no harm)
-    if (!__any_sync(kFull, b != 0) && lane == 0) b = 1u;
+    // A search needs a step.  One more than needed does no harm, if the first sweep has not gone over it either: the first such
+    // (there are far more steps than that sweep takes).
+    if (!__any_sync(kFull, b != 0)) {
+      const uint32_t open = ~in_order(seen);
+      if ((int)lane == __ffs(__ballot_sync(kFull, open != 0)) - 1) b = open & (0u - open);
+    }
     const uint32_t c = __popc(b);
     uint32_t incl = c;
 #pragma unroll

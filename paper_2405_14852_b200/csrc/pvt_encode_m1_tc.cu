@@ -1045,7 +1045,7 @@ cudaError_t launch_tc_sorted(const pvt_layer& L, EncM1Params& p, const EncodeM1T
   p.place = s.place;
   p.records = 2;
   p.record = 0;
-  p.lists = StepLists{s.near, nullptr, s.tile_step, kSortedNear, kSortedNear};
+  p.lists = p.near_lists = StepLists{s.near, nullptr, s.tile_step, kSortedNear, kSortedNear};
   timing_begin(kKernEncodeMain, stream);
   err = launch_search<8, true>(p, lay, base, stats, stream);
   timing_end(kKernEncodeMain, stream);

@@ -147,6 +147,42 @@ def test_equal_codewords_whatever_the_workspace_holds(change, K, fill):
     check(parts, idx, other="tensor", fill=fill)
 
 
+def unlike_groups(W, g, scale, book, codes):
+    """groups of unlike size: beside the largest of a row most are next to zero, and so are most codewords"""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(2)
+    W.view(-1, 8).mul_(torch.exp(torch.randn(codes.shape[0], 1, generator=gen, device="cuda")))
+    scale.copy_(W.abs().amax(1))
+    pick = torch.randperm(codes.shape[0], generator=gen, device="cuda")[:book.shape[0]]
+    book.copy_((W.view(-1, 8)[pick] / scale[pick // (W.shape[1] // 8), None]).half())
+
+
+@pytest.mark.parametrize("change", [one_codeword, unlike_groups])
+def test_codewords_too_many_to_remember_are_gone_over_once(change):
+    """Where more codewords are near than a record holds, all that it stands for are evaluated, and none twice: the search in
+    spatial order takes no longer than the one of every codeword (1.7 times as long when it visited them all for each record)."""
+    K = 60000
+    W, g, scale, books, codes = layer(4096, 2048, K, 9, change)
+    every = torch.arange(enough(K), dtype=torch.int32, device="cuda")
+    times = []
+    for portion in (every.numel(), -(-every.numel() // 2)):
+        own = codes.clone()
+        L = VStepLayer(4096, 2048, W, g, scale, books, own, max_k=portion)
+        parts = [p.contiguous() for p in every.split(portion)]
+        took = []
+        for _ in range(4):
+            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            start.record()
+            for p in parts:
+                L.encode(p)
+            end.record()
+            torch.cuda.synchronize()
+            took.append(start.elapsed_time(end))
+        times.append((min(took), own))
+    assert torch.equal(times[0][1], times[1][1])
+    assert times[0][0] < 1.25 * times[1][0]
+
+
 def test_an_index_out_of_range_is_reported():
     W, g, scale, books, codes = layer(4096, 2048, 65536, 3)
     idx = torch.arange(enough(65536), dtype=torch.int32, device="cuda")
