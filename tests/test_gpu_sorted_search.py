@@ -79,6 +79,24 @@ def one_dimension(W, g, scale, book, codes):
     book[:, 1:] = 0
 
 
+def timed(parts, idx):
+    """least time of a search over the lists, one after the other, and the codes that it leaves"""
+    W, g, scale, books, codes = parts
+    own = codes.clone()
+    L = VStepLayer(*W.shape, W, g, scale, books, own, max_k=max(i.numel() for i in idx))
+    idx = [i.contiguous() for i in idx]
+    took = []
+    for _ in range(4):
+        start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        start.record()
+        for i in idx:
+            L.encode(i)
+        end.record()
+        torch.cuda.synchronize()
+        took.append(start.elapsed_time(end))
+    return min(took), own
+
+
 def one_codeword(W, g, scale, book, codes):
     book.copy_(book[:1].expand_as(book))
 
@@ -162,25 +180,25 @@ def test_codewords_too_many_to_remember_are_gone_over_once(change):
     """Where more codewords are near than a record holds, all that it stands for are evaluated, and none twice: the search in
     spatial order takes no longer than the one of every codeword (1.7 times as long when it visited them all for each record)."""
     K = 60000
-    W, g, scale, books, codes = layer(4096, 2048, K, 9, change)
+    parts = layer(4096, 2048, K, 9, change)
     every = torch.arange(enough(K), dtype=torch.int32, device="cuda")
-    times = []
-    for portion in (every.numel(), -(-every.numel() // 2)):
-        own = codes.clone()
-        L = VStepLayer(4096, 2048, W, g, scale, books, own, max_k=portion)
-        parts = [p.contiguous() for p in every.split(portion)]
-        took = []
-        for _ in range(4):
-            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            start.record()
-            for p in parts:
-                L.encode(p)
-            end.record()
-            torch.cuda.synchronize()
-            took.append(start.elapsed_time(end))
-        times.append((min(took), own))
-    assert torch.equal(times[0][1], times[1][1])
-    assert times[0][0] < 1.25 * times[1][0]
+    whole, portions = timed(parts, [every]), timed(parts, every.chunk(2))
+    assert torch.equal(whole[1], portions[1])
+    assert whole[0] < 1.25 * portions[0]
+
+
+def pruned(W, g, scale, book, codes):
+    zero = torch.arange(codes.shape[0], device="cuda") % 10 != 0
+    W.view(-1, 8)[zero] = 0
+    g.view(-1, 8)[zero] = 0
+
+
+def test_many_equal_targets_do_not_queue():
+    """Nine of ten groups are zero: they all fall into one cell of the tree.  (Counted one by one they took 1.6 times as long as
+    targets that are spread.)"""
+    idx = torch.arange(4096 * 1024, dtype=torch.int32, device="cuda")
+    spread, equal = [timed(layer(4096, 8192, 65536, 10, change), [idx])[0] for change in (None, pruned)]
+    assert equal < 1.25 * spread
 
 
 def test_an_index_out_of_range_is_reported():
