@@ -392,13 +392,6 @@ bool one_kernel(const pvt_layer& L, uint64_t k, uint64_t G) {
   return k == G && L.group_dim == kGroupDim && L.num_codebooks == 1 && !encode_m1_use_tc(L, k) &&
          (uint32_t)L.codebook_size <= kM1SmallCodebook;
 }
-// Whether all groups are dequantised from their present codes beside the selection, and those chosen again after the search:
-// while they are few.
-// while they are few.  (Three and four codebooks: fp32 results need the whole SM, 28672 x 8192 4x8 636 us one after the
-// other, 699 side by side; fp16 results gain nothing in the smallest layers, 32768 groups 52.3 and 53.6 us.)
-bool dequant_first(const pvt_layer& L, uint64_t k, uint64_t G, int32_t out_dtype) {
-  return k <= G / 8 && (L.num_codebooks < 3 || (out_dtype == PVT_F16 && G >= 100000));
-}
 }  // namespace
 
 int pvt_vstep_block(const pvt_layer* layers, const uint64_t* k, int32_t n_layers, uint32_t* const* idx_out,
@@ -433,7 +426,7 @@ int pvt_vstep_block(const pvt_layer* layers, const uint64_t* k, int32_t n_layers
     const uint64_t G = (uint64_t)L.rows * (L.cols / L.group_dim);
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const bool good_ws = ws && !(reinterpret_cast<uintptr_t>(ws) & (kWsAlign - 1));  // (which the selection reports)
-    const bool whole = one_kernel(L, k[i], G), first = out && dequant_first(L, k[i], G, out_dtype);
+    const bool whole = one_kernel(L, k[i], G), first = out && step_dequant_first(L, k[i], G, out_dtype);
     if (good_ws && (whole || first) && apart(L, k[i], idx_out[i], out, out_dtype, ws, ws_bytes)) {
       const WeightsOut weights{out, out_dtype == PVT_F16};
       cudaError_t e = whole ? launch_step_m1_small(L, G, idx_out[i], weights, ws, sm_count(), stream)

@@ -113,6 +113,25 @@ constexpr size_t kM1SmallWorkspace = kWsHeaderBytes + kWsAlign;
 void set_m1_search(int mode);
 EncodeM1TcLayout encode_m1_tc_layout(uint32_t K, uint64_t k, int sm_count, int group_dim = 8);
 
+// Whether a step dequantises all groups from their present codes beside the selection, and those chosen again from the search:
+// while these are few.  It saves the latency of a kernel and, where one alone does not fill HBM, some of its time (2 to 15 us,
+// more in the largest layers and from fp32 codebooks to fp16 results); it costs a second write of the chosen groups, in pieces.
+// us one after the other less us side by side, at an 8th / 12th / 16th / 24th of the groups, fp16 results: 11008 x 4096 1x16
+// 4 / 5 / 6 / 8, 1x12 -4 / -1 / 0 / 1, 2x8 -7 / -2 / 0 / 2; 8192 x 8192 2x8 -12 / -3 / 1 / 4; 28672 x 8192 1x16 -21 / 10 / 40 /
+// 23.  512 codewords at a 16th / 32nd / 64th / 100th: 8192 x 8192 1 / 5 / 7 / 8, 28672 x 8192 -21 / -10 / -4 / -1 (of 440).  Four
+// codebooks at the same: 11008 x 4096 -15 / -2 / 4 / 5, 8192 x 8192 -24 / -9 / -3 / 2.  fp32 codebooks to fp16 results at an 8th:
+// 8192 x 8192 1x8 3, 2x8 11.  Three codebooks or more: fp32 results need the whole SM (28672 x 8192 4x8 636 one after the other,
+// 699 side by side), and layers with few groups lose (196608 groups, fp32 codebooks, a 100th: 3x8 60 and 82, 4x8 74 and 85;
+// 131072, fp16: 4x8 72 and 78; from 262144 on side by side is 0 to 6 us less).
+inline bool step_dequant_first(const pvt_layer& L, uint64_t k, uint64_t G, int32_t out_dtype) {
+  const int M = L.num_codebooks;
+  if (M >= 3 && (out_dtype != PVT_F16 || G < 250000)) return false;
+  if (M == 4) return k <= G / 64;
+  if (M <= 2 && L.codebook_dtype == PVT_F32 && out_dtype == PVT_F16) return k <= G / 8;
+  if (M == 1 && L.group_dim == kGroupDim && L.codebook_size <= (int32_t)kM1SmallCodebook && k > 300000) return false;
+  return k <= G / 16;
+}
+
 // where a search writes the weights of the groups it re-encodes as well (null: nowhere)
 struct WeightsOut {
   void* W_hat;

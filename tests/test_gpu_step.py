@@ -8,8 +8,16 @@ from paper_2405_14852_b200.vstep import VStepLayer
 pytestmark = pytest.mark.gpu
 
 CASES = [  # rows, cols, codebooks, codewords, group, codebook type, codes, k
-    (64, 72, 1, 200, 8, torch.float16, torch.uint8, 72),          # the most that are dequantised first: an eighth
-    (64, 72, 1, 200, 8, torch.float32, torch.uint8, 73),          # one more
+    (64, 72, 1, 200, 8, torch.float16, torch.uint8, 72),          # more than are dequantised first
+    (64, 72, 1, 200, 8, torch.float32, torch.uint8, 73),          # (fp32 codebooks and fp16 weights: the most are an eighth; one more)
+    (64, 72, 1, 200, 8, torch.float32, torch.uint8, 72),          # (the most)
+    (64, 72, 1, 200, 8, torch.float16, torch.uint8, 36),          # the most of the others: a sixteenth; one more
+    (64, 72, 1, 200, 8, torch.float16, torch.uint8, 37),
+    (1000, 2008, 3, 256, 8, torch.float16, torch.uint8, 1000),    # three and four codebooks with enough groups
+    (1000, 2008, 4, 256, 8, torch.float32, torch.uint8, 3921),    # a 64th
+    (16384, 4096, 1, 100, 8, torch.float16, torch.uint8, 300000),  # the most groups of a small codebook, and one more
+    (16384, 4096, 1, 100, 8, torch.float16, torch.uint8, 300001),
+    (11264, 8192, 1, 65536, 8, torch.float16, torch.int16, 700000),  # a search in spatial order
     (3, 8, 1, 2, 8, torch.float16, torch.uint8, 1),
     (16, 8, 1, 2, 8, torch.float16, torch.uint8, 2),              # fewer groups than threads of a block
     (300, 1000, 1, 5000, 8, torch.float16, torch.int16, 1000),
@@ -20,7 +28,7 @@ CASES = [  # rows, cols, codebooks, codewords, group, codebook type, codes, k
     (129, 264, 2, 100, 8, torch.float32, torch.uint8, 400),
     (1000, 1000, 3, 256, 8, torch.float16, torch.uint8, 1000),
     (1000, 1000, 3, 31, 8, torch.float32, torch.uint8, 1000),
-    (500, 1600, 4, 256, 8, torch.float16, torch.uint8, 777),      # the least groups of three and four codebooks
+    (500, 1600, 4, 256, 8, torch.float16, torch.uint8, 777),      # three and four codebooks: too few groups
     (500, 520, 4, 256, 8, torch.float32, torch.uint8, 777),
     (1000, 1000, 4, 256, 8, torch.float32, torch.uint8, 777),
     (129, 272, 1, 1500, 16, torch.float16, torch.int16, 200),
