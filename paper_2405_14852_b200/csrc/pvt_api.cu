@@ -429,8 +429,10 @@ int pvt_vstep_block(const pvt_layer* layers, const uint64_t* k, int32_t n_layers
     const bool whole = one_kernel(L, k[i], G), first = out && step_dequant_first(L, k[i], G, out_dtype);
     if (good_ws && (whole || first) && apart(L, k[i], idx_out[i], out, out_dtype, ws, ws_bytes)) {
       const WeightsOut weights{out, out_dtype == PVT_F16};
-      cudaError_t e = whole ? launch_step_m1_small(L, G, idx_out[i], weights, ws, sm_count(), stream)
+      const bool after = whole && out && step_weights_after(L, G, out_dtype);
+      cudaError_t e = whole ? launch_step_m1_small(L, G, idx_out[i], after ? WeightsOut{} : weights, ws, sm_count(), stream)
                             : launch_select(L, G, k[i], idx_out[i], ws, sm_count(), stream, out, out_dtype);
+      if (e == cudaSuccess && after) e = launch_dequant(L, G, out, out_dtype, nullptr, sm_count(), stream);
       if (e != cudaSuccess) return fail_cuda(e);
       if (whole) continue;
       const int rc = encode(&L, idx_out[i], k[i], nullptr, ws, ws_bytes, weights, cuda_stream);

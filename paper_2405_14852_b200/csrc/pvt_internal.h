@@ -132,6 +132,15 @@ inline bool step_dequant_first(const pvt_layer& L, uint64_t k, uint64_t G, int32
   return k <= G / 16;
 }
 
+// Whether a step over every group of a layer with one small codebook leaves the weights to a kernel after its search: in large
+// layers, where eight lanes with an element each store more slowly than 16 bytes per lane.  From the search itself / after it in
+// us: fp16 weights, 256 fp16 codewords, 262144 groups 71.7 / 71.8, 524288 129.6 / 129.0, 1048576 243.7 / 239.6, 5636096 1246 /
+// 1216, 29360128 6437 / 6282; 1000 codewords 524288 332 / 333, 2097152 1201 / 1199, 29360128 16400 / 16362.  fp32 weights, 256
+// codewords: 1048576 243.3 / 242.9, 2097152 473.1 / 470.1, 29360128 6403 / 6348; 512: 2097152 710 / 709; 700: 895 / 896.
+inline bool step_weights_after(const pvt_layer& L, uint64_t G, int32_t out_dtype) {
+  return out_dtype == PVT_F16 ? G >= 500000 : L.codebook_size <= 512 && G >= 1000000;
+}
+
 // where a search writes the weights of the groups it re-encodes as well (null: nowhere)
 struct WeightsOut {
   void* W_hat;

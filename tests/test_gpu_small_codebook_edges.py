@@ -1,7 +1,7 @@
 """Search over one small codebook at the edges of its kernel: blocks of 16 codewords, the largest codebook of either type
 (binary32 up to 1024 codewords, fp16 below 1024), the smallest of the kernels beyond (fp16: the tensor engine, binary32:
 the FP32 engine), tiles of 32 and 64 targets, both splits of the targets.  A step over
-every group is one kernel: it leaves what the three calls leave."""
+every group is one kernel, with another for the weights of large layers: it leaves what the three calls leave."""
 import os
 import re
 
@@ -47,6 +47,8 @@ def test_small_codebook_search_at_its_edges(K, f16, k):
     (1024, False, 148, 2048, "float32"),  # two targets per team from here on
     (100, True, 641, 1000, "float16"),
     (300, False, 64, 72, None),           # no weights
+    (200, True, 1000, 4000, "float16"),   # weights after the search: the least groups
+    (200, False, 2000, 4000, "float32"),
     (64, False, 64, 72, "in place"),      # the weights take the place of W
 ])
 def test_a_step_over_every_group_is_the_three_calls(K, f16, rows, cols, out):

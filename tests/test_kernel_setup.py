@@ -44,7 +44,8 @@ int main() {
     pvt_layer L = {};
     L.group_dim = dg, L.num_codebooks = M, L.codebook_size = K, L.codebook_dtype = f16 ? PVT_F16 : PVT_F32;
     const uint64_t G = (uint64_t)rows * cols / dg;
-    std::printf("%d ", (int)pvt::step_dequant_first(L, G / part, G, out_f16 ? PVT_F16 : PVT_F32));
+    const int32_t out = out_f16 ? PVT_F16 : PVT_F32;
+    std::printf("%d ", (int)(part == 1 ? pvt::step_weights_after(L, G, out) : pvt::step_dequant_first(L, G / part, G, out)));
   }
 }
 """
@@ -76,6 +77,20 @@ FASTER_FIRST = [
     (8192, 8192, 2, 256, 8, 0, 1, 8), (28672, 8192, 1, 256, 8, 0, 1, 32), (28672, 8192, 1, 512, 8, 1, 1, 200),
     (11008, 4096, 4, 256, 8, 1, 1, 100), (256, 512, 1, 256, 8, 1, 0, 100), (512, 1024, 2, 256, 8, 0, 1, 48),
 ]
+
+
+# the same of steps over every group: weights from the search itself, and from a kernel after it
+FASTER_INSIDE = [(256, 256, 1, 256, 8, 0, 0, 1), (1024, 2048, 1, 256, 8, 1, 1, 1), (4096, 4096, 1, 1000, 8, 1, 0, 1),
+                 (2048, 2048, 1, 4, 8, 1, 0, 1)]
+FASTER_AFTER = [(2048, 2048, 1, 4, 8, 1, 1, 1), (4096, 4096, 1, 256, 8, 1, 1, 1), (28672, 8192, 1, 1000, 8, 1, 1, 1),
+                (4096, 4096, 1, 256, 8, 0, 0, 1), (28672, 8192, 1, 512, 8, 1, 0, 1)]
+
+
+@pytest.mark.skipif(shutil.which("nvcc") is None, reason="no nvcc")
+def test_weights_of_all_groups_come_from_the_faster_kernel(tmp_path):
+    given = "\n".join(" ".join(map(str, case)) for case in FASTER_INSIDE + FASTER_AFTER)
+    got = [int(x) for x in run(tmp_path, RULE, given).split()]
+    assert got == [0] * len(FASTER_INSIDE) + [1] * len(FASTER_AFTER)
 
 
 @pytest.mark.skipif(shutil.which("nvcc") is None, reason="no nvcc")
