@@ -71,6 +71,8 @@ def check_encode(L, idx_np, beam=None):
     enc = oracle.encode(t, L.codebooks, codes2[idx_np.astype(np.int64)], L.beam)
     got_codes, err, status = run_encode(L, idx_np)
     assert status == 0
+    # the same codes where no errors are asked for (the search may then leave binary64 out for a codeword that is alone)
+    assert np.array_equal(run_encode(L, idx_np, want_err=False)[0], got_codes)
     got2 = got_codes.reshape(-1, L.num_codebooks)
     exact, band = helpers.check_codes_against_oracle(t, L.codebooks, got2[idx_np.astype(np.int64)], enc, REL)
     # locality: everything outside idx is untouched, bit for bit

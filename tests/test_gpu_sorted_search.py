@@ -51,6 +51,14 @@ def check(parts, idx, again=False, other="fp32", fill=None):
         got.append((own, err))
     assert torch.equal(got[0][0], got[1][0])
     assert torch.equal(got[0][1], got[1][1])
+    # without errors to report, a codeword that binary32 tells from all others is taken as it is
+    own = codes.clone()
+    L = VStepLayer(rows, cols, W, g, scale, books, own, max_k=idx.numel())
+    for _ in range(1 + again):
+        L.encode(idx)
+    torch.cuda.synchronize()
+    assert L.status() == 0
+    assert torch.equal(own, got[0][0])
 
 
 @pytest.mark.parametrize("K,more", [
