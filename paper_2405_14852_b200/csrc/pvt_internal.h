@@ -154,8 +154,7 @@ cudaError_t launch_select(const pvt_layer& L, uint64_t G, uint64_t k, uint32_t* 
 // the same selection on other keys: 0 squared update norm, 1 the same while a straight-through buffer takes the
 // step, 2 uniformly random keys, 3 keys of a draw in proportion to the squared update norm (seeded)
 cudaError_t launch_select_keyed(const pvt_layer& L, uint64_t G, uint64_t k, uint32_t* idx_out, void* ws, int sm_count,
-                                cudaStream_t stream, int key_mode, float* buffer, uint64_t seed, void* W_hat = nullptr,
-                                int32_t out_dtype = 0);
+                                cudaStream_t stream, int key_mode, float* buffer, uint64_t seed);
 cudaError_t launch_encode_m1(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,
                              WeightsOut out, void* ws, int sm_count, cudaStream_t stream);
 cudaError_t launch_encode_m1_small(const pvt_layer& L, uint64_t G, const uint32_t* idx, uint64_t k, float* err_out,

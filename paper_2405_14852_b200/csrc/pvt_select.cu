@@ -363,14 +363,10 @@ cudaError_t launch_group(int mode, const SelParams& p, int sm_count, cudaStream_
 
 }  // namespace
 
-cudaError_t launch_select(const pvt_layer& L, uint64_t G, uint64_t k, uint32_t* idx_out, void* ws, int sm_count,
-                          cudaStream_t stream, void* W_hat, int32_t out_dtype) {
-  return launch_select_keyed(L, G, k, idx_out, ws, sm_count, stream, kKeyNorm, nullptr, 0, W_hat, out_dtype);
-}
-
-cudaError_t launch_select_keyed(const pvt_layer& L, uint64_t G, uint64_t k, uint32_t* idx_out, void* ws, int sm_count,
-                                cudaStream_t stream, int key_mode, float* buffer, uint64_t seed, void* W_hat,
-                                int32_t out_dtype) {
+namespace {
+// (W_hat: with the plain norms only)
+cudaError_t launch_passes(const pvt_layer& L, uint64_t G, uint64_t k, uint32_t* idx_out, void* ws, int sm_count,
+                          cudaStream_t stream, int key_mode, float* buffer, uint64_t seed, void* W_hat, int32_t out_dtype) {
   timing_begin(kKernSelect, stream);
   cudaError_t err;
   if (k == G && key_mode != kKeyNormBuffer) {  // every group is taken: the ascending index list itself
@@ -422,6 +418,17 @@ cudaError_t launch_select_keyed(const pvt_layer& L, uint64_t G, uint64_t k, uint
   count_launches(1);
   timing_end(kKernSelect, stream);
   return err;
+}
+}  // namespace
+
+cudaError_t launch_select(const pvt_layer& L, uint64_t G, uint64_t k, uint32_t* idx_out, void* ws, int sm_count,
+                          cudaStream_t stream, void* W_hat, int32_t out_dtype) {
+  return launch_passes(L, G, k, idx_out, ws, sm_count, stream, kKeyNorm, nullptr, 0, W_hat, out_dtype);
+}
+
+cudaError_t launch_select_keyed(const pvt_layer& L, uint64_t G, uint64_t k, uint32_t* idx_out, void* ws, int sm_count,
+                                cudaStream_t stream, int key_mode, float* buffer, uint64_t seed) {
+  return launch_passes(L, G, k, idx_out, ws, sm_count, stream, key_mode, buffer, seed, nullptr, 0);
 }
 
 }  // namespace pvt

@@ -37,7 +37,11 @@ int main() {
 
 RULE = r"""
 #include <cstdio>
+#include <type_traits>
 #include "pvt_internal.h"
+// weights beside the selection: by the plain norms, no other keys
+static_assert(!std::is_invocable_v<decltype(pvt::launch_select_keyed), const pvt_layer&, uint64_t, uint64_t, uint32_t*, void*, int,
+                                   cudaStream_t, int, float*, uint64_t, void*, int32_t>);
 int main() {
   int rows, cols, M, K, dg, f16, out_f16, part;
   while (std::scanf("%d %d %d %d %d %d %d %d", &rows, &cols, &M, &K, &dg, &f16, &out_f16, &part) == 8) {
