@@ -362,14 +362,18 @@ def device_peaks(local, clocks=None):
     return peaks
 
 
-def evaluated_share(layer):
-    """Share of the (target, codeword) pairs that the tensor engine evaluates.  With many targets and many codewords
-    (m1_sorted in csrc/pvt_internal.h) it searches in spatial order and leaves out what a tile of targets cannot reach: for
-    normally distributed weights and 65536 codewords a simulation of the lists gives 0.53, 0.43 and 0.39 for 1, 8 and 28
-    times 2^20 targets, which this goes through."""
-    if layer.M != 1 or layer.K <= 32768 or layer.k * layer.K * layer.K < 3e15:
-        return 1.0
-    return 0.53 * (layer.k / 2.0 ** 20) ** -0.095
+def evaluated_share(runner):
+    """Share of the (target, codeword) pairs that the search evaluates in a step, as the kernel counts them: with many targets
+    and many codewords the tensor engine searches in spatial order and leaves out what a tile of targets cannot reach.  A search
+    of each layer by itself, outside the timed region."""
+    B, pairs = runner.B, 0.0
+    runner.restore_codes()
+    for l in runner.layers:
+        B.pvt_vstep_select(l.desc, l.k, l.idx, runner.ws)
+        B.pvt_vstep_encode(l.desc, l.idx, l.k, None, runner.ws)
+        pairs += l.pairs * B.pvt_evaluated_share(l.desc, l.k, runner.ws)
+    runner.restore_codes()
+    return pairs / runner.pairs
 
 
 def search_roofline(engine, pairs_per_step, enc_ms, enc_n, steps, peaks, traffic, share=1.0):
@@ -394,8 +398,8 @@ def search_roofline(engine, pairs_per_step, enc_ms, enc_n, steps, peaks, traffic
             r["evaluated_share"] = share
             r["achieved_by_definition"] = achieved / share
             r["note"] = ("the definition of the search counts every codeword for every target; in spatial order the kernel "
-                         "evaluates an estimated share of these pairs (evaluated_share), and achieved and the fractions "
-                         "count only those; pairs_per_s counts all")
+                         "evaluates a share of these pairs (evaluated_share, from its own counts), and achieved and the "
+                         "fractions count only those; pairs_per_s counts all")
     else:
         r = {"kernel": {"fp32": "encode_m1_kernel (exhaustive search, FP32 pipe)",
                         "small": "encode_m1_small_kernel (exhaustive search, small codebook)",
@@ -537,7 +541,7 @@ def run_ours(args):
         peaks = device_peaks(local, clocks)
         ffma_measured = B.pvt_probe_fp32_tflops()  # the FP32 pipe, measured in this job
         enc_ms, enc_n = t["kern"][B.PVT_KERNEL_ENCODE_MAIN]
-        share = sum(l.pairs * evaluated_share(l) for l in runner.layers) / runner.pairs if engine == "tensor" else 1.0
+        share = evaluated_share(runner) if engine == "tensor" else 1.0
         roofline = search_roofline(engine, runner.pairs, enc_ms, enc_n, steps, peaks,
                                    recorded_traffic(engine, runner.k, share < 1.0), share)
         roofline["fp32_fma_microbenchmark_tflops"] = ffma_measured
@@ -652,7 +656,7 @@ def sweep_record(args, dev, peaks, flush_l2, block_layers):
                 engine = engine_of(layer, args.search)
                 enc_ms, enc_n = t["kern"][B.PVT_KERNEL_ENCODE_MAIN]
                 r = search_roofline(engine, runner.pairs, enc_ms, enc_n, 3, peaks, None,
-                                    evaluated_share(layer) if engine == "tensor" else 1.0)
+                                    evaluated_share(runner) if engine == "tensor" else 1.0)
                 st = stage_record(runner, t, 3, peaks, layer.W_hat.element_size())
                 rec = {"workload": f"{name}_tau{tau}", "k": layer.k, "ms_per_step": t["ms_per_step"],
                        "graph_replay": t["graphed"],

@@ -418,6 +418,11 @@ int pvt_probe_fp32_tflops(float* scratch, size_t scratch_floats, float* tflops_o
 /* Kernels this process has launched through the library so far (memsets not counted). */
 unsigned long long pvt_launch_count(void);
 int pvt_timing_read(int kernel_id, float* total_ms, int* launches);
+/* Where a search of k groups of this layer counts what it goes over: the byte offset in the workspace of
+ * ceil(k / 256) uint32, valid until the workspace's next use, or 0 if the search evaluates every codeword for every
+ * target (or the layer is invalid).  Entry i: for the i-th 256 targets, the groups of 128 codewords that were
+ * evaluated beyond the 32 nearest. */
+size_t pvt_search_counts(const pvt_layer* layer, uint64_t k);
 
 /*
  * Test hook for the give-up path of the on-chip waits (no counterpart in the paper).  Every wait of

@@ -120,6 +120,8 @@ def lib():
         L.pvt_probe_fp32_tflops.restype = ctypes.c_int
         L.pvt_probe_fp32_tflops.argtypes = [vp, sz, ctypes.POINTER(ctypes.c_float), vp]
         L.pvt_launch_count.restype = ctypes.c_ulonglong
+        L.pvt_search_counts.restype = sz
+        L.pvt_search_counts.argtypes = [lp, u64]
         L.pvt_timing_read.restype = ctypes.c_int
         L.pvt_timing_read.argtypes = [ctypes.c_int, ctypes.POINTER(ctypes.c_float), ctypes.POINTER(ctypes.c_int)]
         _lib = L
@@ -402,3 +404,14 @@ def pvt_timing_read(kernel_id: int):
     ms, n = ctypes.c_float(0.0), ctypes.c_int(0)
     _check(lib().pvt_timing_read(kernel_id, ctypes.byref(ms), ctypes.byref(n)), "pvt_timing_read")
     return float(ms.value), int(n.value)
+
+
+def pvt_evaluated_share(layer: pvt_layer, k: int, ws: torch.Tensor) -> float:
+    """Share of the (target, codeword) pairs that the search of k groups which used the workspace last has evaluated; waits
+    for it."""
+    at = int(lib().pvt_search_counts(ctypes.byref(layer), k))
+    if at == 0:
+        return 1.0
+    tiles, steps = -(-k // 256), -(-layer.codebook_size // 128)
+    beyond = int(ws[at:at + 4 * tiles].view(torch.int32).sum())
+    return (beyond + 32 * tiles) / (tiles * steps)

@@ -519,6 +519,13 @@ void pvt_set_m1_search(int mode) {
   if (mode == PVT_M1_AUTO || mode == PVT_M1_FP32 || mode == PVT_M1_TENSOR) set_m1_search(mode);
 }
 
+size_t pvt_search_counts(const pvt_layer* layer, uint64_t k) {
+  uint64_t G = 0;
+  if (check_layer(layer, &G) != PVT_OK || check_quantiser(layer) != PVT_OK || k < 1 || k > G) return 0;
+  if (!encode_m1_use_tc(*layer, k)) return 0;
+  return encode_m1_tc_layout((uint32_t)layer->codebook_size, k, sm_count(), layer->group_dim).counts_off;
+}
+
 unsigned long long pvt_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
 
 void pvt_test_wait_limit(uint32_t max_polls, int64_t withhold_copy) {

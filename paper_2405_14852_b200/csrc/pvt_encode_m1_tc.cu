@@ -162,7 +162,7 @@ size_t sorted_scratch(char* base, void* records, uint32_t K, uint64_t k, uint32_
   out.place = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * k));
   out.tile_step = reinterpret_cast<uint16_t*>(take(sizeof(uint16_t) * n_tiles));
   out.lists = reinterpret_cast<uint16_t*>(take(sizeof(uint16_t) * n_tiles * (size_t)m1::list_stride(n_steps)));
-  out.counts = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * n_tiles));
+  out.counts = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * n_tiles));  // (the last: counts_off)
   out.keys = reinterpret_cast<uint2*>(records);  // (8 bytes per target, done with before the first record of 32)
   if (s) *s = out;
   return at;
@@ -170,7 +170,7 @@ size_t sorted_scratch(char* base, void* records, uint32_t K, uint64_t k, uint32_
 }  // namespace
 
 EncodeM1TcLayout encode_m1_tc_layout(uint32_t K, uint64_t k, int sm_count, int group_dim) {
-  EncodeM1TcLayout e;
+  EncodeM1TcLayout e = {};
   e.n_steps = (K + kTcStepCw - 1) / kTcStepCw;
   e.n_tiles = (uint32_t)((k + kTcTile - 1) / kTcTile);
   uint32_t best_s = 1;
@@ -204,6 +204,7 @@ EncodeM1TcLayout encode_m1_tc_layout(uint32_t K, uint64_t k, int sm_count, int g
   if (e.sorted) {
     e.sorted_off = e.bytes;
     e.bytes = sorted_scratch(nullptr, nullptr, K, k, e.n_tiles, e.n_steps, nullptr) + e.bytes;
+    e.counts_off = e.bytes - align_up(sizeof(uint32_t) * e.n_tiles, kWsAlign);
   }
   return e;
 }

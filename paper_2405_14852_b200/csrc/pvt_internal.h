@@ -87,6 +87,7 @@ struct EncodeM1TcLayout {
   size_t exc_off;     // u32 [K]: codewords the image cannot represent, by block
   size_t gbest_off, margin_off, rec_off;
   size_t sorted_off;  // scratch of the search in spatial order
+  size_t counts_off;  // its u32 [n_tiles]: steps of the second sweep
   size_t bytes;
   bool sorted;
   uint32_t n_steps;   // 128-codeword steps

@@ -209,6 +209,18 @@ def test_many_equal_targets_do_not_queue():
     assert equal < 1.25 * spread
 
 
+def test_the_search_counts_what_it_evaluates():
+    W, g, scale, books, codes = layer(4096, 2048, 65536, 11)
+    k = enough(65536) + 100
+    L = VStepLayer(4096, 2048, W, g, scale, books, codes, max_k=k)
+    L.encode(torch.arange(k, dtype=torch.int32, device="cuda"))
+    assert 0.4 < B.pvt_evaluated_share(L.desc, k, L.reserve(k)) < 0.7  # normally distributed weights
+    assert B.pvt_evaluated_share(L.desc, enough(65536) // 2, L.reserve(k)) == 1.0
+    books[0].copy_(books[0][:1].expand_as(books[0]))
+    L.encode(torch.arange(k, dtype=torch.int32, device="cuda"))
+    assert B.pvt_evaluated_share(L.desc, k, L.reserve(k)) == 1.0  # equal codewords: all of them
+
+
 def test_an_index_out_of_range_is_reported():
     W, g, scale, books, codes = layer(4096, 2048, 65536, 3)
     idx = torch.arange(enough(65536), dtype=torch.int32, device="cuda")
