@@ -102,6 +102,8 @@ typedef struct pvt_layer {
  * and this k (the larger of the two needs).  Returns 0 if the layer or k is
  * invalid.  The workspace must be 256-byte aligned; its first 256 bytes hold the
  * status word and must be cleared once with pvt_workspace_init before first use.
+ * It grows with k where one large fp16 codebook is searched for many groups: 52 bytes
+ * for each of the k (all groups of 28672 x 8192, 65536 codewords: 1.5 GB).
  */
 size_t pvt_workspace_bytes(const pvt_layer* layer, uint64_t k);
 
@@ -221,9 +223,11 @@ int pvt_vstep_sample(const pvt_layer* layer, uint64_t k, int32_t rule, uint64_t 
  *          the last the `beam` smallest partial tuples under (||t - c1 - ... -
  *          cm||^2, tuple) are kept; the pool is the last stage's beam*K tuples
  *          plus the previous tuple.
- *   A fast binary32 score shortlists candidates; the decision among shortlisted
- *   candidates is taken on binary64 distances sum_i (t_i - c_i)^2 accumulated in
- *   index order, so ties break exactly as stated above.
+ *   A fast score shortlists candidates; the decision among them is that of the
+ *   binary64 distances sum_i (t_i - c_i)^2 accumulated in index order, so ties
+ *   break exactly as stated above.  (They are formed wherever binary32 distances,
+ *   whose error is bounded, do not already leave one codeword, and whenever
+ *   err_out asks for them.)
  *   Groups not in idx keep their codes bit for bit.
  * idx: device, k uint32, each < G, no duplicates (duplicates race benignly: the
  * same value is written twice).  err_out: device, k floats or NULL; receives the
@@ -302,12 +306,12 @@ int pvt_dequant(const pvt_layer* layer, void* W_hat, int32_t out_dtype, uint32_t
  * independent): for i = 0 .. n_layers-1, in order, on the one stream,
  *     pvt_vstep_select(layers[i], k[i]) -> idx_out[i];  pvt_vstep_encode(layers[i], idx_out[i], k[i]);
  *     pvt_dequant(layers[i]) -> W_hat[i]   (skipped when W_hat or W_hat[i] is NULL).
- * A convenience that adds no arithmetic of its own; a layer's W_hat is scratch until the call's work on it is done (it may
- * be filled from the codes before the step, and the chosen groups again after the search).  layers, k, idx_out, W_hat: HOST arrays of n_layers
- * entries (descriptors, subspace sizes, device pointers to k[i] uint32, device pointers to rows x cols of
- * out_dtype).  ws: one device workspace shared by all layers, at least pvt_block_workspace_bytes (the largest
- * per-layer need), header cleared by pvt_workspace_init; status bits of all layers accumulate in it.
- * Every layer is validated before anything is enqueued; return codes as the three calls.
+ * A convenience that adds no arithmetic of its own; a layer's W_hat is scratch until the call's work on it is done
+ * (it may be filled from the codes before the step, and the chosen groups again after the search).  layers, k,
+ * idx_out, W_hat: HOST arrays of n_layers entries (descriptors, subspace sizes, device pointers to k[i] uint32, device
+ * pointers to rows x cols of out_dtype).  ws: one device workspace shared by all layers, at least
+ * pvt_block_workspace_bytes (the largest per-layer need), header cleared by pvt_workspace_init; status bits of all layers
+ * accumulate in it.  Every layer is validated before anything is enqueued; return codes as the three calls.
  */
 size_t pvt_block_workspace_bytes(const pvt_layer* layers, const uint64_t* k, int32_t n_layers);
 int pvt_vstep_block(const pvt_layer* layers, const uint64_t* k, int32_t n_layers, uint32_t* const* idx_out,
@@ -402,10 +406,10 @@ void pvt_set_m1_search(int mode);
  * pvt_timing_read waits for the recorded events of one kernel class, returns
  * their summed duration and count, and forgets them.
  */
-#define PVT_KERNEL_SELECT 0      /* all kernels of pvt_vstep_select */
+#define PVT_KERNEL_SELECT 0      /* all kernels of pvt_vstep_select; in pvt_vstep_block also the weights beside them */
 #define PVT_KERNEL_ENCODE_MAIN 1 /* the search kernel of pvt_vstep_encode */
 #define PVT_KERNEL_ENCODE_AUX 2  /* codebook expansion before the M = 1 search */
-#define PVT_KERNEL_DEQUANT 3     /* the kernel of pvt_dequant */
+#define PVT_KERNEL_DEQUANT 3     /* the kernel of pvt_dequant (none in pvt_vstep_block where others write the weights) */
 #define PVT_KERNEL_ENCODE_RESCORE 4 /* exact rescoring and code write after the M = 1 search */
 #define PVT_KERNEL_PSTEP_GRAD 5  /* the kernel of pvt_pstep_grad */
 #define PVT_KERNEL_ADAM 6        /* the kernel of pvt_adam_update */

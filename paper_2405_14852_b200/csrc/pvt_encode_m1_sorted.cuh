@@ -14,9 +14,9 @@ constexpr uint32_t kSortedNear = 32;         // steps of the first sweep
 __host__ __device__ constexpr uint32_t list_stride(uint32_t n_steps) { return (n_steps + 7) / 8 * 8; }
 
 // What orders the steps by their distance from step `own` (its bit pattern; infinite where there is no step).  The keys of all
-// kSortedSteps steps differ, so that they have the ranks 0, 1, 2, ...: the own one is zero, every other at least kSortedSteps with
-// the step's number in its last bits.  (Without that least one step 0 would tie with `own` where the centres of their boxes are
-// the same, as in a codebook of equal codewords, and a rank would have no step.)
+// kSortedSteps steps differ, so that they have the ranks 0, 1, 2, ...: the own one is zero, every other at least kSortedSteps
+// with the step's number in its last bits.  (Without that least one step 0 would tie with `own` where the centres of their
+// boxes are the same, as in a codebook of equal codewords, and a rank would have no step.)
 __host__ __device__ constexpr uint32_t near_key(uint32_t distance_bits, uint32_t step, uint32_t own) {
   const uint32_t rounded = distance_bits & ~(kSortedSteps - 1);
   return step == own ? 0u : (rounded < kSortedSteps ? kSortedSteps : rounded) | step;

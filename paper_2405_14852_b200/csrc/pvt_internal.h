@@ -104,7 +104,8 @@ constexpr int kM1TensorCodebook = 1024;
 // near stored codes in ms, 65536 codewords: every codeword 1.47 / 1.97 / 2.71 / 5.15, in spatial order 1.51 / 1.84 / 2.36 /
 // 3.94; 50000: 1.21 / 1.60 / 2.20 / 4.14 and 1.35 / 1.65 / 2.11 / 3.43; 40000: 1.05 / 1.37 / 1.87 / 3.49 and 1.24 / 1.50 /
 // 1.94 / 3.17; 33000: 0.92 / 1.20 / 1.63 / 3.04 and 1.17 / 1.41 / 1.79 / 2.95.  The two meet where targets times the square of
-// the codewords is 1.7e15 to 2.6e15 (normally distributed weights; where less can be left out they meet later).
+// the codewords is 1.7e15 to 2.6e15 (normally distributed weights; where less can be left out they meet later: Laplace weights,
+// 700000 / 800000 / 900000 / 1000000 targets 1.80 / 2.09 / 2.27 / 2.55 and 1.92 / 2.14 / 2.31 / 2.53).
 inline bool m1_sorted(uint32_t K, uint64_t k) {
   return K > 32768 && k >= 3000000000000000ull / ((uint64_t)K * K);
 }
@@ -119,11 +120,11 @@ EncodeM1TcLayout encode_m1_tc_layout(uint32_t K, uint64_t k, int sm_count, int g
 // more in the largest layers and from fp32 codebooks to fp16 results); it costs a second write of the chosen groups, in pieces.
 // us one after the other less us side by side, at an 8th / 12th / 16th / 24th of the groups, fp16 results: 11008 x 4096 1x16
 // 4 / 5 / 6 / 8, 1x12 -4 / -1 / 0 / 1, 2x8 -7 / -2 / 0 / 2; 8192 x 8192 2x8 -12 / -3 / 1 / 4; 28672 x 8192 1x16 -21 / 10 / 40 /
-// 23.  512 codewords at a 16th / 32nd / 64th / 100th: 8192 x 8192 1 / 5 / 7 / 8, 28672 x 8192 -21 / -10 / -4 / -1 (of 440).  Four
-// codebooks at the same: 11008 x 4096 -15 / -2 / 4 / 5, 8192 x 8192 -24 / -9 / -3 / 2.  fp32 codebooks to fp16 results at an 8th:
-// 8192 x 8192 1x8 3, 2x8 11.  Three codebooks or more: fp32 results need the whole SM (28672 x 8192 4x8 636 one after the other,
-// 699 side by side), and layers with few groups lose (196608 groups, fp32 codebooks, a 100th: 3x8 60 and 82, 4x8 74 and 85;
-// 131072, fp16: 4x8 72 and 78; from 262144 on side by side is 0 to 6 us less).
+// 23.  512 codewords at a 16th / 32nd / 64th / 100th: 8192 x 8192 1 / 5 / 7 / 8, 28672 x 8192 -21 / -10 / -4 / -1 (of 440).
+// Four codebooks at the same: 11008 x 4096 -15 / -2 / 4 / 5, 8192 x 8192 -24 / -9 / -3 / 2.  fp32 codebooks to fp16 results at
+// an 8th: 8192 x 8192 1x8 3, 2x8 11.  Three codebooks or more: fp32 results need the whole SM (28672 x 8192 4x8 636 one after
+// the other, 699 side by side), and layers with few groups lose (196608 groups, fp32 codebooks, a 100th: 3x8 60 and 82, 4x8 74
+// and 85; 131072, fp16: 4x8 72 and 78; from 262144 on side by side is 0 to 6 us less).
 inline bool step_dequant_first(const pvt_layer& L, uint64_t k, uint64_t G, int32_t out_dtype) {
   const int M = L.num_codebooks;
   if (M >= 3 && (out_dtype != PVT_F16 || G < 250000)) return false;

@@ -186,7 +186,7 @@ def unlike_groups(W, g, scale, book, codes):
 @pytest.mark.parametrize("change", [one_codeword, unlike_groups])
 def test_codewords_too_many_to_remember_are_gone_over_once(change):
     """Where more codewords are near than a record holds, all that it stands for are evaluated, and none twice: the search in
-    spatial order takes no longer than the one of every codeword (1.7 times as long when it visited them all for each record)."""
+    spatial order takes no longer than the one of every codeword (1.7 times as long when it visited all for each record)."""
     K = 60000
     parts = layer(4096, 2048, K, 9, change)
     every = torch.arange(enough(K), dtype=torch.int32, device="cuda")

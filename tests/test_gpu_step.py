@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 
 CASES = [  # rows, cols, codebooks, codewords, group, codebook type, codes, k
     (64, 72, 1, 200, 8, torch.float16, torch.uint8, 72),          # more than are dequantised first
-    (64, 72, 1, 200, 8, torch.float32, torch.uint8, 73),          # (fp32 codebooks and fp16 weights: the most are an eighth; one more)
+    (64, 72, 1, 200, 8, torch.float32, torch.uint8, 73),          # (fp32 codebooks, fp16 weights: one above an eighth)
     (64, 72, 1, 200, 8, torch.float32, torch.uint8, 72),          # (the most)
     (64, 72, 1, 200, 8, torch.float16, torch.uint8, 36),          # the most of the others: a sixteenth; one more
     (64, 72, 1, 200, 8, torch.float16, torch.uint8, 37),

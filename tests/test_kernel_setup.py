@@ -40,8 +40,8 @@ RULE = r"""
 #include <type_traits>
 #include "pvt_internal.h"
 // weights beside the selection: by the plain norms, no other keys
-static_assert(!std::is_invocable_v<decltype(pvt::launch_select_keyed), const pvt_layer&, uint64_t, uint64_t, uint32_t*, void*, int,
-                                   cudaStream_t, int, float*, uint64_t, void*, int32_t>);
+static_assert(!std::is_invocable_v<decltype(pvt::launch_select_keyed), const pvt_layer&, uint64_t, uint64_t, uint32_t*,
+                                   void*, int, cudaStream_t, int, float*, uint64_t, void*, int32_t>);
 int main() {
   int rows, cols, M, K, dg, f16, out_f16, part;
   while (std::scanf("%d %d %d %d %d %d %d %d", &rows, &cols, &M, &K, &dg, &f16, &out_f16, &part) == 8) {
@@ -58,8 +58,8 @@ int main() {
 def run(tmp_path, program, given=""):
     src, exe = tmp_path / "program.cu", tmp_path / "program"
     src.write_text(program)
-    subprocess.run(["nvcc", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-I", os.path.join(ROOT, "include"), "-I",
-                    os.path.join(ROOT, "paper_2405_14852_b200", "csrc"), "-o", str(exe), str(src)], check=True)
+    subprocess.run(["nvcc", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-I", os.path.join(ROOT, "include"),
+                    "-I", os.path.join(ROOT, "paper_2405_14852_b200", "csrc"), "-o", str(exe), str(src)], check=True)
     return subprocess.run([str(exe)], check=True, capture_output=True, text=True, input=given).stdout
 
 
