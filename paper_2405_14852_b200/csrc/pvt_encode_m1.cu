@@ -386,7 +386,6 @@ __global__ void __launch_bounds__(256, DG == 8 && CB_F16 ? 5 : 3) rescore_m1_ker
     else
       form_target16(p, j, t);
   }
-  const uint32_t subs_per_unit = p.unit_cw / SUB;
   double best_d = __longlong_as_double(0x7ff0000000000000ll);
   uint32_t best_code = 0xffffffffu;
 
@@ -437,9 +436,9 @@ __global__ void __launch_bounds__(256, DG == 8 && CB_F16 ? 5 : 3) rescore_m1_ker
   const uint32_t in1 = __ballot_sync(kFull, active && __uint_as_float(raw1.x) <= limit);
   const uint32_t slices = ((in0 >> gshift) & 0xffu) | (((in1 >> gshift) & 0xffu) << kRsLanes);
   auto sweep = [&](bool on, auto&& take) {
-    auto visit = [&](uint32_t sub) {
+    auto visit = [&](uint32_t first, uint32_t many) {
 #pragma unroll 1
-      for (uint32_t at = sub * SUB + l; at < (sub + 1) * SUB; at += kRsEach * kRsLanes) {
+      for (uint32_t at = first + l; at < first + many; at += kRsEach * kRsLanes) {
         Raw raw[kRsEach];
 #pragma unroll
         for (int q = 0; q < kRsEach; ++q)
@@ -470,22 +469,20 @@ __global__ void __launch_bounds__(256, DG == 8 && CB_F16 ? 5 : 3) rescore_m1_ker
       if (cnt == kCandOverflow) {
         if (SORTED && limit > -__builtin_huge_valf()) {
           // the steps that the record stands for; no step is in both lists of a tile
-          const StepLists& from = sl ? p.lists : p.near_lists;
-          const uint32_t tile = (uint32_t)(n / p.tile), row = from.rows ? from.rows[tile] : tile;
-          const uint16_t* steps = from.steps + (size_t)row * from.stride;
-          const uint32_t many = from.counts ? from.counts[tile] : from.most;
-          for (uint32_t i = 0; i < many; ++i) {
-            const uint32_t step = min((uint32_t)steps[i], p.n_units - 1);
-            for (uint32_t q = 0; q < subs_per_unit; ++q) visit(step * subs_per_unit + q);
-          }
+          const uint32_t tile = (uint32_t)(n >> 8);
+          const uint16_t* step = sl ? p.lists.steps + (size_t)tile * p.lists.stride
+                                    : p.near_lists.steps + (size_t)p.near_lists.rows[tile] * p.near_lists.stride;
+          const uint16_t* const end = step + (sl ? p.lists.counts[tile] : p.near_lists.most);
+#pragma unroll 1
+          for (; step != end; ++step) visit(min((uint32_t)*step, p.n_units - 1) * p.unit_cw, p.unit_cw);
         } else {  // (in spatial order: a target that the tensor cores cannot serve, against the whole codebook)
           uint32_t u_lo = 0, u_hi = p.n_units;
           if (!SORTED) slice_units(p, (uint32_t)sl, &u_lo, &u_hi);
-          for (uint32_t sub = u_lo * subs_per_unit; sub < u_hi * subs_per_unit; ++sub) visit(sub);
+          visit(u_lo * p.unit_cw, (u_hi - u_lo) * p.unit_cw);
         }
       } else {
         for (uint32_t q = 0; q < cnt; ++q) {
-          visit(ids[0] & 0xfffu);
+          visit((ids[0] & 0xfffu) * SUB, SUB);
           if (q & 1u) {
             ids[0] = ids[1];
             ids[1] = ids[2];

@@ -22,7 +22,7 @@
 // codebook 0.2, the targets 0.4.  What it gives depends on the weights.  Search of 8388608 targets in ms, every codeword / in
 // spatial order: normal 20.7 / 12.9, uniform 20.7 / 8.8, correlated elements 22.1 / 6.4, Laplace 20.8 / 16.4, groups of unlike
 // size 20.8 / 15.2, a codebook ten times smaller than the targets 22.8 / 20.5, half of the targets zero 20.9 / 15.2; where more
-// codewords are near than a record holds, log-normal sizes of groups 363 / 85, equal codewords 2143 / 1995.
+// codewords are near than a record holds, log-normal sizes of groups 363 / 81, equal codewords 2143 / 1914.
 // The tree is built by a block per node with the keys in shared memory (seven launches, 150 us) and by sorting nodes of 512
 // positions; with nodes of 4096 sorted and the keys read again for every pass the codebook took 0.49 ms.  Tried for the boxes:
 // bounds from the tree's planes alone (keeps 0.03 more steps), the box of 32 targets in place of the targets (0.82 of the
